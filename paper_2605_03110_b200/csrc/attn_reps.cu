@@ -472,7 +472,9 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
                 // 32 columns go to shared memory (16-byte pieces permuted by row, free of bank
                 // conflicts both ways) and the warp then writes them out four rows at a time,
                 // 128 contiguous bytes per row, instead of 32 scattered 16-byte pieces per store.
-                unsigned char* stg = ps + half * 2 * KB_BYTES + quad * 8192;
+                // (This warp's own P rows of either K block: another warp of the set may already be
+                // writing the next item's probabilities into its rows.)
+                unsigned char* stg = ps + half * 2 * KB_BYTES + quad * 4096;
                 const unsigned long long dst_bits = reinterpret_cast<unsigned long long>(dst);
                 int ci = 0;
                 for (int o0 = half * 32; o0 < d_h; o0 += 64, ++ci) {
@@ -486,7 +488,7 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
                             w.x = fmaf(vb[q], fb, w.x); w.y = fmaf(vb[q + 1], fb, w.y);
                             w.z = fmaf(vb[q + 2], fb, w.z); w.w = fmaf(vb[q + 3], fb, w.w);
                         }
-                        *reinterpret_cast<float4*>(stg + ci * 4096 + lane * 128 + ((((q >> 2) ^ lane) & 7) << 4)) = w;
+                        *reinterpret_cast<float4*>(stg + ci * KB_BYTES + lane * 128 + ((((q >> 2) ^ lane) & 7) << 4)) = w;
                     }
                 }
                 __syncwarp();
@@ -495,7 +497,7 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
 #pragma unroll
                     for (int it = 0; it < 8; ++it) {
                         const int r = it * 4 + (lane >> 3), pc = lane & 7;
-                        const float4 w = *reinterpret_cast<const float4*>(stg + ci * 4096 + r * 128 + (((pc ^ r) & 7) << 4));
+                        const float4 w = *reinterpret_cast<const float4*>(stg + ci * KB_BYTES + r * 128 + (((pc ^ r) & 7) << 4));
                         const unsigned lo = __shfl_sync(0xffffffffu, (unsigned)dst_bits, r);
                         const unsigned hi = __shfl_sync(0xffffffffu, (unsigned)(dst_bits >> 32), r);
                         float* drow = reinterpret_cast<float*>(((unsigned long long)hi << 32) | lo);

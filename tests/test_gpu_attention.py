@@ -217,3 +217,20 @@ def test_two_stream_pipeline_matches_the_serial_order(ada):
     ref = oracle.attention_reps(Xh, Xh, Xh, R, nearest_idx=near)
     assert np.max(np.abs(res[1][-1].cpu().numpy() - ref)) <= 2.0 ** -8 * float(np.max(np.abs(X64)))
     pipe.close()
+
+
+def test_repeated_calls_with_several_items_per_cta_are_bit_identical(ada):
+    """More (query tile, head) items than SMs: a warp that is done with an item's output rows
+    writes the next item's probabilities beside warps that still stage theirs."""
+    T, h, d_h, r = 1500, 32, 128, 1300
+    g = torch.Generator(device="cuda").manual_seed(3)
+    Q, K, V = [torch.randn((T, h, d_h), generator=g, device="cuda").bfloat16() for _ in range(3)]
+    idx = torch.zeros(T, dtype=torch.int32, device="cuda")
+    idx[:r] = torch.randperm(T, generator=g, device="cuda")[:r].sort().values.int()
+    cnt = torch.tensor([r], dtype=torch.int32, device="cuda")
+    ctx = ada.ada_create(1, T, h * d_h, ada.ADA_BF16)
+    first = ada.ada_attention_reps(ctx, Q, K, V, idx, cnt)
+    for _ in range(20):
+        assert torch.equal(ada.ada_attention_reps(ctx, Q, K, V, idx, cnt), first)
+    assert ada.ada_device_status(ctx)[0] == 0
+    ada.ada_destroy(ctx)

@@ -143,7 +143,7 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
     *out = nullptr;
     if (maxB < 1 || maxT < 1 || maxd < 1 || (dt != ADA_F32 && dt != ADA_BF16))
         return ADA_ERR_INVALID_ARG;
-    // the compaction packs three per-sequence counts into 21-bit fields
+    // the compaction packs three per-sequence counts into 21-bit fields of one word
     if (maxT > ADA_MAX_T || maxB * maxT > (int64_t)1 << 30) return ADA_ERR_INVALID_ARG;
     int ndev = 0;
     if (cudaGetDeviceCount(&ndev) != cudaSuccess || device < 0 || device >= ndev)
@@ -172,11 +172,9 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
     // role, g_tok, g_rep are contiguous so that one memset clears them
     const size_t o_role = take(n_tok * 4), o_gtok = take(n_tok * 4), o_grep = take(n_tok * 4);
     const size_t o_ctr = take(32);
-    const int agg_stride = (int)((maxT + 1023) / 1024);
-    const size_t o_done = take(32), o_agg = take((size_t)maxB * agg_stride * 8);
     const size_t o_near = take(n_tok * 8);
     const size_t o_inv = take(n_tok * 4), o_invr = take(n_tok * 4);
-    const size_t o_reff = take((size_t)maxB * 4), o_stat = take(32), o_thr = take((size_t)maxB * 4);
+    const size_t o_reff = take((size_t)maxB * 4), o_stat = take(32);
     const size_t o_xrep = take(n_tok * (size_t)maxd * ctx->es + 1024);
     // bf16: the rows outside a large inherited set, copied out for the cross step (Algorithm 1 line 6)
     const size_t o_ntok = take(dt == ADA_BF16 ? n_tok * 4 : 0);
@@ -195,12 +193,8 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
     ctx->inv_norm = reinterpret_cast<float*>(ctx->ws + o_inv);
     ctx->inv_rep = reinterpret_cast<float*>(ctx->ws + o_invr);
     ctx->r_eff = reinterpret_cast<int32_t*>(ctx->ws + o_reff);
-    ctx->thr_seq = reinterpret_cast<float*>(ctx->ws + o_thr);
     ctx->status = reinterpret_cast<unsigned*>(ctx->ws + o_stat);
     ctx->tile_ctr = reinterpret_cast<unsigned*>(ctx->ws + o_ctr);
-    ctx->done_ctr = reinterpret_cast<unsigned*>(ctx->ws + o_done);
-    ctx->agg = reinterpret_cast<unsigned long long*>(ctx->ws + o_agg);
-    ctx->agg_stride = agg_stride;
     ctx->near_key = reinterpret_cast<unsigned long long*>(ctx->ws + o_near);
     ctx->Xrep = ctx->ws + o_xrep;
     ctx->Xnon = dt == ADA_BF16 ? ctx->ws + o_xnon : nullptr;
@@ -370,8 +364,6 @@ static ada_status cascade_impl(ada_ctx* ctx, const void* X, int64_t B, int64_t T
     TauUpdate tau_upd;
     memset(&tau_upd, 0, sizeof(tau_upd));
     if (tu != nullptr) tau_upd = *tu;
-    const bool adaptive = tau_upd.tau_state != nullptr;
-    if (adaptive) CU(launch_tau_thr(ctx, (int)B, tau_upd.tau_state, s));   // thresholds of this step
 
     // role map, gamma scratch and dependency counters are zero on entry (workspace invariant
     // kept by the compaction kernels).
@@ -433,7 +425,7 @@ static ada_status cascade_impl(ada_ctx* ctx, const void* X, int64_t B, int64_t T
     q.col_gate = ctx->g_rep;
     q.thr_bits = 0;
     memcpy(&q.thr_bits, &thr, 4);
-    q.thr_seq = adaptive ? reinterpret_cast<const unsigned*>(ctx->thr_seq) : nullptr;
+    q.tau_seq = tau_upd.tau_state;
     q.col_token = rep_in;
     q.row_role = ctx->role;
     q.causal = (flags & ADA_CROSS_CAUSAL) ? 1 : 0;

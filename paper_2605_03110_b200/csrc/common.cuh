@@ -62,7 +62,7 @@ struct GramProblem {
     // cross only
     const unsigned* col_gate; // [B*cap] gamma_rep bits by position
     unsigned thr_bits;        // bit pattern of (float)thr
-    const unsigned* thr_seq;  // per-sequence bit patterns instead (adaptive threshold), or NULL
+    const double* tau_seq;    // per-sequence tau instead (adaptive threshold), or NULL
     const int32_t* col_token; // [B*cap] token index of each column (causal) or NULL
     const int32_t* row_role;  // [B*cap] 0 for non-representatives
     int causal;
@@ -155,12 +155,8 @@ struct ada_ctx {
     unsigned* g_rep;     // [maxB*maxT] gamma_rep by position, bit patterns
     int32_t* role;       // [maxB*maxT] 0 = not inherited, p+1 = position p in the inherited list
     int32_t* r_eff;      // [maxB] sanitised inherited counts
-    float* thr_seq;      // [maxB] per-sequence (float)(1 - tau^2) of an adaptive step
     unsigned* status;    // [8]
     unsigned* tile_ctr;  // [8] dependency counter of the fused Gram launch
-    unsigned long long* agg;  // [maxB][agg_stride] block counts published by the compaction
-    unsigned* done_ctr;  // compaction blocks finished
-    int agg_stride;
     unsigned long long* near_key;  // [maxB*maxT] packed (value, ~column) of the nearest representative
     void* Xrep;          // [maxB*maxT*maxd] gathered representative rows (raw values)
     void* Xnon;          // [maxB*maxT*maxd] bf16 contexts: the rows outside a large inherited set
@@ -188,6 +184,11 @@ namespace ada {
 // returns once the predecessor has completed and its writes are visible.  Without the
 // attribute the wait is a no-op.
 #ifdef __CUDACC__
+// threshold of a device-resident tau: 1 - tau^2 in fp64, each operation rounded once, then fp32,
+// as for a tau given on the host
+static __device__ __forceinline__ float tau_threshold(double tau) {
+    return (float)__dsub_rn(1.0, __dmul_rn(tau, tau));
+}
 static __device__ __forceinline__ void grid_dep_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -230,15 +231,14 @@ cudaError_t launch_nearest_finish(ada_ctx* ctx, int B, int T, const int32_t* rep
                                   int32_t* nearest_idx, float* nearest_gamma, cudaStream_t s);
 cudaError_t launch_compact_full(ada_ctx* ctx, int B, int T, float thr, int32_t* rep_idx,
                                 int32_t* rep_cnt, float* gamma, cudaStream_t s);
-// adaptive threshold (Section 8.1): tau_state != NULL makes the step use ctx->thr_seq and update
-// tau_state / write the turnover of Eq. (6) once the counts are known
+// adaptive threshold (Section 8.1): tau_state != NULL makes the step take its per-sequence
+// threshold from there and update it / write the turnover of Eq. (6) once the counts are known
 struct TauUpdate {
     double* tau_state;     // [B] device, in/out; NULL = fixed threshold
     float* turnover;       // [B] device, optional
     int update;            // 0: leave tau_state as it is
     double target, gain, tau_min, tau_max;
 };
-cudaError_t launch_tau_thr(ada_ctx* ctx, int B, const double* tau_state, cudaStream_t s);
 // row_scale: the cross maxima in the scratch still lack the factor 1/||x_t|| (GramProblem::defer_row)
 cudaError_t launch_compact_cascade(ada_ctx* ctx, int B, int T, float thr, int32_t* rep_out,
                                    int32_t* rep_out_cnt, int32_t* add_idx, int32_t* add_cnt,

@@ -288,6 +288,8 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
     }
     // everything above is local to the CTA; from here on the predecessor's results are read
     grid_dep_wait();
+    // (the compaction's blocks may take the SMs that fall idle first: they wait for this whole grid)
+    grid_dep_launch_next();
     if (warp == 2) {
         // Work plan.  Everything per sequence -- its length, its tile counts -- is computed by
         // the lanes in parallel and reduced with shuffles: the lengths live in global memory, and
@@ -609,7 +611,7 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
                 // (columns past the tile are clamped to its last one and discarded afterwards,
                 // so that no load hangs on a data-dependent branch)
                 const int last = pc.n - 1;
-                const unsigned thr_b = (!p.tri && p.thr_seq != nullptr) ? p.thr_seq[pc.b] : p.thr_bits;
+                const unsigned thr_b = (!p.tri && p.tau_seq != nullptr) ? __float_as_uint(tau_threshold(p.tau_seq[pc.b])) : p.thr_bits;
 #pragma unroll
                 for (int q = 0; q < BN / 32; ++q)
                     fb[q] = __ldcg(p.inv_b + o + min(pc.col0 + lane + 32 * q, last));

@@ -275,6 +275,8 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
     }
     // everything above is local to the CTA; from here on the predecessor's results are read
     grid_dep_wait();
+    // (the compaction's blocks may take the SMs that fall idle first: they wait for this whole grid)
+    grid_dep_launch_next();
     if (threadIdx.x == 0) TRACE(0);
     if (threadIdx.x == 64) {
         // streaming form: one column tile covers the columns of every sequence, so the launch is
@@ -482,7 +484,7 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                 unsigned gate[BN / 32] = {};
                 int tk[BN / 32] = {};
                 const int last = max(pc.n - 1, 0);
-                const unsigned thr_b = (!p.tri && p.thr_seq != nullptr) ? p.thr_seq[pc.b] : p.thr_bits;
+                const unsigned thr_b = (!p.tri && p.tau_seq != nullptr) ? __float_as_uint(tau_threshold(p.tau_seq[pc.b])) : p.thr_bits;
 #pragma unroll
                 for (int q = 0; q < BN / 32; ++q)
                     fb[q] = __ldcg(p.inv_b + o + min(pc.col0 + lane + 32 * q, last));

@@ -427,156 +427,176 @@ cudaError_t launch_split(ada_ctx* ctx, const void* X, int B, int T, int d, int64
 
 // ---------------------------------------------------------------------------
 // Compaction (Definition 1's threshold; Algorithm 1 lines 5, 9, 10-11 and the lists of
-// Eq. 6).  Every 1024-thread block owns 1024 consecutive tokens of one sequence, one token
-// per thread, so all loads are coalesced and the whole sequence is in flight at once.
-// A block reduces its own counts, publishes them (one 64-bit word: three 21-bit counts
-// and a READY bit), then sums the words of the blocks before it -- those never wait on
-// anything, so the look-back is one round trip -- and writes its slice of the ascending
-// lists.  The last block to finish clears the published words and the counters, and every
-// thread clears the scratch it read, so the workspace is all-zero again when the kernel
-// ends and no memset is needed between calls.
+// Eq. 6).  One cluster of up to eight 1024-thread blocks per sequence; a block owns V x 1024
+// consecutive tokens of every round of (blocks x V x 1024), one token per thread and slice, so
+// all loads are coalesced and the whole sequence is in flight at once.  Ballots give a warp's
+// three counts, one warp per block scans them, the block totals go to the other blocks through
+// distributed shared memory, and after ONE cluster barrier every thread knows its places in the
+// ascending lists.  Every thread clears the scratch it read, so the workspace is all-zero again
+// when the kernel ends and no memset is needed between calls.
+//
+// Bound by latency: a chain of dependent round trips on O(T) integers.  The blocks used to
+// exchange their totals through global memory (publish, poll, and a fence and a counter to know
+// when the words may be cleared); the outputs' first touch also misses the TLB when a chain of
+// layers keeps its lists apart, hence the prefetches before the wait.
 // ---------------------------------------------------------------------------
-constexpr unsigned long long AGG_READY = 1ull << 63;
-constexpr unsigned long long AGG_MASK = (1ull << 21) - 1;
+constexpr int COMPACT_CTAS = 8;      // largest portable cluster
+constexpr unsigned COUNT_BITS = 21;  // three counts share a 64-bit word
+constexpr unsigned long long COUNT_MASK = (1ull << COUNT_BITS) - 1;
 
 struct CompactArgs {
     unsigned* g_tok;             // gamma (full) / gamma_cross by token, bit patterns
     unsigned* g_rep;             // gamma_rep by position (cascade) or NULL
     int32_t* role;               // 0 / position+1 (cascade) or NULL
-    unsigned long long* agg;     // [B][agg_stride] published block counts
-    unsigned* done_ctr;          // blocks finished
-    unsigned* dep_ctr;           // dependency counter of the fused Gram launch (cleared here)
+    unsigned* dep_ctr;           // dependency counters of the Gram launch (cleared here)
     unsigned* status;
-    int agg_stride, T;
+    int T;
     float thr;
     int32_t *keep_idx, *keep_cnt, *add_idx, *add_cnt, *rem_idx, *rem_cnt;
     float *gamma_a, *gamma_b;    // full: gamma | cascade: gamma_rep, gamma_cross (optional)
     const float* row_scale;      // cascade: 1/||x_t|| still to be applied to g_tok, or NULL
-    // adaptive threshold (Section 8.1)
-    const float* thr_seq;        // [B] thresholds of this step, or NULL = thr
+    // adaptive threshold (Section 8.1): thresholds come from tu.tau_state
     const int32_t* r_in;         // [B] inherited counts (Eq. 6 denominator)
     TauUpdate tu;
 };
 
-// thr_seq[b] = (float)(1 - tau_b^2), 1 - tau^2 in fp64 as for a host-side tau
-__global__ void k_tau_thr(const double* __restrict__ tau_state, int B, float* __restrict__ thr_seq,
-                          unsigned* __restrict__ status) {
-    grid_dep_wait();
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    const double tau = tau_state[b];
-    if (!(tau > 0.0 && tau < 1.0)) atomicOr(status, ST_BAD_TAU);
-    thr_seq[b] = (float)__dsub_rn(1.0, __dmul_rn(tau, tau));
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
-__device__ __forceinline__ unsigned long long block_exclusive_scan(unsigned long long v,
-                                                                   unsigned long long* s_warp,
-                                                                   unsigned long long& total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned long long incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long n = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += n;
-    }
-    if (lane == 31) s_warp[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        const unsigned long long wv = s_warp[lane];
-        unsigned long long wi = wv;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long n = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += n;
-        }
-        s_warp[lane] = wi - wv;
-        if (lane == 31) s_warp[32] = wi;
-    }
-    __syncthreads();
-    const unsigned long long off = s_warp[warp] + incl - v;
-    total = s_warp[32];
-    __syncthreads();   // s_warp is reused
-    return off;
-}
-
+template <int V>
 __global__ void __launch_bounds__(1024) k_compact(const CompactArgs a) {
-    __shared__ unsigned long long s_warp[33];
+    __shared__ unsigned long long s_off[V * 32];               // counts, then exclusive offsets, by slice and warp
+    __shared__ unsigned long long s_total[2][COMPACT_CTAS];    // block totals of the cluster, by round parity
+    const int b = blockIdx.y, rank = blockIdx.x, nblk = gridDim.x;   // the cluster is the x extent of the grid
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t o = (int64_t)b * a.T;
+    const bool cascade = a.role != nullptr;
+    {
+        const int t = rank * V * 1024 + V * (int)threadIdx.x;
+        if ((threadIdx.x & 31) == 0 && t < a.T) {              // one touch per 128 V bytes of each output
+            prefetch_l2(a.keep_idx + o + t);
+            if (cascade) { prefetch_l2(a.add_idx + o + t); prefetch_l2(a.rem_idx + o + t); }
+            if (a.gamma_a != nullptr) prefetch_l2(a.gamma_a + o + t);
+            if (a.gamma_b != nullptr) prefetch_l2(a.gamma_b + o + t);
+        }
+        if (threadIdx.x == 1) {
+            prefetch_l2(a.keep_cnt + b);
+            if (cascade) { prefetch_l2(a.add_cnt + b); prefetch_l2(a.rem_cnt + b); }
+        }
+    }
+    // every block of the cluster has started before any writes into another's shared memory
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
     grid_dep_wait();
     grid_dep_launch_next();
-    const int b = blockIdx.y, blk = blockIdx.x, nblk = gridDim.x;
-    const int t = blk * 1024 + threadIdx.x;
-    const int64_t o = (int64_t)b * a.T;
-    const bool in = t < a.T;
-    const bool cascade = a.role != nullptr;
     const unsigned faulted = a.status[0];
-    const float thr = a.thr_seq != nullptr ? a.thr_seq[b] : a.thr;
-
-    // independent loads first, the position-indexed gather second
-    const int pos = (cascade && in) ? a.role[o + t] : 0;
-    const unsigned gt = in ? a.g_tok[o + t] : 0u;
-    const float rs = (in && a.row_scale != nullptr) ? a.row_scale[o + t] : 1.0f;
-    const unsigned gp = pos > 0 ? a.g_rep[o + pos - 1] : 0u;
-    bool keep = false, add = false, rem = false;
-    if (in) {
-        float ga = 0.f, gb = 0.f;
-        if (pos > 0) {                    // inherited representative: line 5
-            ga = __uint_as_float(gp);
-            keep = ga < thr;
-            rem = !keep;
-            a.g_rep[o + pos - 1] = 0u;
-            a.role[o + t] = 0;
-        } else {                          // Definition 1 / line 9
-            // (an untouched entry is a maximum over nothing: 0 whatever the row's norm)
-            gb = gt != 0u ? __uint_as_float(gt) * rs : 0.f;
-            keep = gb < thr;
-            add = cascade && keep;
-        }
-        a.g_tok[o + t] = 0u;
-        if (cascade) {
-            if (a.gamma_a != nullptr) a.gamma_a[o + t] = ga;
-            if (a.gamma_b != nullptr) a.gamma_b[o + t] = gb;
-            if (faulted != 0u) a.g_rep[o + t] = 0u;   // a rejected list leaves positions without a token
-        } else if (a.gamma_a != nullptr) {
-            a.gamma_a[o + t] = gb;
-        }
+    float thr = a.thr;
+    if (a.tu.tau_state != nullptr) {
+        const double tau = a.tu.tau_state[b];
+        thr = tau_threshold(tau);
+        if (rank == 0 && threadIdx.x == 0 && !(tau > 0.0 && tau < 1.0)) atomicOr(a.status, ST_BAD_TAU);
     }
-    const unsigned long long mine = (keep ? 1ull : 0ull) | (add ? 1ull << 21 : 0ull) | (rem ? 1ull << 42 : 0ull);
-    unsigned long long total;
-    const unsigned long long off = block_exclusive_scan(mine, s_warp, total);
-
-    unsigned long long* agg = a.agg + (int64_t)b * a.agg_stride;
-    if (threadIdx.x == 0) atomicExch(agg + blk, total | AGG_READY);
-    // look-back over the blocks before this one (bounded spin; they wait on nothing)
-    unsigned long long before = 0;
-    for (int j = threadIdx.x; j < blk; j += 1024) {
-        unsigned long long v;
-        unsigned polls = 0;
-        long long t0 = 0;
-        while (true) {
-            v = *reinterpret_cast<volatile unsigned long long*>(agg + j);
-            if (v & AGG_READY) break;
-            if ((++polls & 1023u) == 0) {
-                const long long now = clock64();
-                if (t0 == 0) t0 = now;
-                else if (now - t0 > 4000000000ll) { atomicOr(a.status, ST_TIMEOUT); v = 0; break; }
+    unsigned long long carry = 0;                              // counts of the rounds before this one
+    int par = 0;
+    for (int t0 = 0; t0 < a.T; t0 += nblk * V * 1024, par ^= 1) {
+        const int tb = t0 + rank * V * 1024 + (int)threadIdx.x;
+        // independent loads first, the position-indexed gather second
+        int pos[V];
+        unsigned gt[V], gp[V];
+        float rs[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            const int t = tb + v * 1024;
+            const bool in = t < a.T;
+            pos[v] = (cascade && in) ? a.role[o + t] : 0;
+            gt[v] = in ? a.g_tok[o + t] : 0u;
+            rs[v] = (in && a.row_scale != nullptr) ? a.row_scale[o + t] : 1.0f;
+        }
+#pragma unroll
+        for (int v = 0; v < V; ++v) gp[v] = pos[v] > 0 ? a.g_rep[o + pos[v] - 1] : 0u;
+        unsigned bk[V], ba[V], br[V];                          // ballots: kept, added, removed
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            const int t = tb + v * 1024;
+            bool keep = false, add = false, rem = false;
+            if (t < a.T) {
+                float ga = 0.f, gb = 0.f;
+                if (pos[v] > 0) {                 // inherited representative: line 5
+                    ga = __uint_as_float(gp[v]);
+                    keep = ga < thr;
+                    rem = !keep;
+                    a.g_rep[o + pos[v] - 1] = 0u;
+                    a.role[o + t] = 0;
+                } else {                          // Definition 1 / line 9
+                    // (an untouched entry is a maximum over nothing: 0 whatever the row's norm)
+                    gb = gt[v] != 0u ? __uint_as_float(gt[v]) * rs[v] : 0.f;
+                    keep = gb < thr;
+                    add = cascade && keep;
+                }
+                a.g_tok[o + t] = 0u;
+                if (cascade) {
+                    if (a.gamma_a != nullptr) a.gamma_a[o + t] = ga;
+                    if (a.gamma_b != nullptr) a.gamma_b[o + t] = gb;
+                    if (faulted != 0u) a.g_rep[o + t] = 0u;   // a rejected list leaves positions without a token
+                } else if (a.gamma_a != nullptr) {
+                    a.gamma_a[o + t] = gb;
+                }
+            }
+            bk[v] = __ballot_sync(0xffffffffu, keep);
+            ba[v] = __ballot_sync(0xffffffffu, add);
+            br[v] = __ballot_sync(0xffffffffu, rem);
+            if (lane == 0)
+                s_off[v * 32 + warp] = (unsigned long long)__popc(bk[v]) |
+                                       ((unsigned long long)__popc(ba[v]) << COUNT_BITS) |
+                                       ((unsigned long long)__popc(br[v]) << (2 * COUNT_BITS));
+        }
+        __syncthreads();
+        if (warp == 0) {                          // lane l scans entries l V .. l V + V - 1 (token order)
+            unsigned long long c[V], mine = 0;
+#pragma unroll
+            for (int v = 0; v < V; ++v) { c[v] = s_off[lane * V + v]; mine += c[v]; }
+            unsigned long long incl = mine;
+#pragma unroll
+            for (int q = 1; q < 32; q <<= 1) {
+                const unsigned long long n = __shfl_up_sync(0xffffffffu, incl, q);
+                if (lane >= q) incl += n;
+            }
+            const unsigned long long total = __shfl_sync(0xffffffffu, incl, 31);
+            unsigned long long off = incl - mine;
+#pragma unroll
+            for (int v = 0; v < V; ++v) { s_off[lane * V + v] = off; off += c[v]; }
+            if (lane < nblk) {                    // this block's total, to every block of the cluster
+                unsigned dst;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                             : "=r"(dst)
+                             : "r"((unsigned)__cvta_generic_to_shared(&s_total[par][rank])), "r"(lane));
+                asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(dst), "l"(total) : "memory");
             }
         }
-        before += v & ~AGG_READY;
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        unsigned long long base = carry;
+        for (int j = 0; j < nblk; ++j) {
+            const unsigned long long n = s_total[par][j];
+            carry += n;
+            if (j < rank) base += n;
+        }
+        const unsigned below = (1u << lane) - 1u;
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            const int t = tb + v * 1024;
+            const unsigned long long off = base + s_off[v * 32 + warp];
+            if ((bk[v] >> lane) & 1u) a.keep_idx[o + (int)(off & COUNT_MASK) + __popc(bk[v] & below)] = t;
+            if ((ba[v] >> lane) & 1u) a.add_idx[o + (int)((off >> COUNT_BITS) & COUNT_MASK) + __popc(ba[v] & below)] = t;
+            if ((br[v] >> lane) & 1u) a.rem_idx[o + (int)(off >> (2 * COUNT_BITS)) + __popc(br[v] & below)] = t;
+        }
+        if (t0 + nblk * V * 1024 < a.T) __syncthreads();       // s_off is reused
     }
-    unsigned long long base;
-    block_exclusive_scan(before, s_warp, base);
-
-    const int nk = (int)((base + off) & AGG_MASK);
-    const int na = (int)(((base + off) >> 21) & AGG_MASK);
-    const int nr = (int)(((base + off) >> 42) & AGG_MASK);
-    if (keep) a.keep_idx[o + nk] = t;
-    if (add) a.add_idx[o + na] = t;
-    if (rem) a.rem_idx[o + nr] = t;
-    if (blk == nblk - 1 && threadIdx.x == 0) {
-        const unsigned long long all = base + total;
-        a.keep_cnt[b] = (int)(all & AGG_MASK);
+    if (rank == 0 && threadIdx.x == 0) {
+        a.keep_cnt[b] = (int)(carry & COUNT_MASK);
         if (cascade) {
-            const int n_add = (int)((all >> 21) & AGG_MASK), n_rem = (int)((all >> 42) & AGG_MASK);
+            const int n_add = (int)((carry >> COUNT_BITS) & COUNT_MASK), n_rem = (int)(carry >> (2 * COUNT_BITS));
             a.add_cnt[b] = n_add;
             a.rem_cnt[b] = n_rem;
             if (a.tu.tau_state != nullptr) {
@@ -588,6 +608,7 @@ __global__ void __launch_bounds__(1024) k_compact(const CompactArgs a) {
                 if (a.tu.turnover != nullptr)
                     a.tu.turnover[b] = defined ? (float)rho : __int_as_float(0x7fc00000);
                 if (a.tu.update) {
+                    // (every block of the cluster has read the old value: they are past the barrier)
                     double t = a.tu.tau_state[b];
                     if (defined) t = __dadd_rn(t, __dmul_rn(a.tu.gain, __dsub_rn(a.tu.target, rho)));
                     if (t < a.tu.tau_min) t = a.tu.tau_min;
@@ -596,16 +617,7 @@ __global__ void __launch_bounds__(1024) k_compact(const CompactArgs a) {
                 }
             }
         }
-    }
-    // the last block to finish restores the zero state of the shared words
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const unsigned n_blocks = gridDim.x * gridDim.y;
-        if (atomicAdd(a.done_ctr, 1u) == n_blocks - 1) {
-            for (unsigned q = 0; q < gridDim.y; ++q)
-                for (unsigned j = 0; j < gridDim.x; ++j) a.agg[(int64_t)q * a.agg_stride + j] = 0ull;
-            *a.done_ctr = 0u;
+        if (b == 0) {
             a.dep_ctr[0] = 0u;
             a.dep_ctr[1] = 0u;   // norm warps' counter of the Gram launch
             a.dep_ctr[3] = 0u;   // in-launch gather counter
@@ -661,24 +673,39 @@ cudaError_t launch_nearest_finish(ada_ctx* ctx, int B, int T, const int32_t* rep
 }
 
 static cudaError_t launch_compact(ada_ctx* ctx, int kid, const CompactArgs& a, int B, cudaStream_t s) {
-    const int nblk = (a.T + 1023) / 1024;
-    if (nblk > a.agg_stride) return cudaErrorInvalidValue;
+    // as few tokens per thread as the cluster allows; longer sequences than 4 x 8 x 1024 take rounds
+    const int slices = (a.T + 1023) / 1024;
+    const int V = slices <= COMPACT_CTAS ? 1 : (slices <= 2 * COMPACT_CTAS ? 2 : 4);
+    const int nblk = slices < COMPACT_CTAS ? slices : COMPACT_CTAS;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(nblk, B);
+    cfg.blockDim = dim3(1024);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = nblk; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = ctx->dep_launch ? 2 : 1;
     prof_begin(ctx, kid, s);
-    launch_k(ctx, k_compact, dim3(nblk, B), dim3(1024), 0, s, a);
+    cudaError_t e = V == 1 ? cudaLaunchKernelEx(&cfg, k_compact<1>, a)
+                           : (V == 2 ? cudaLaunchKernelEx(&cfg, k_compact<2>, a) : cudaLaunchKernelEx(&cfg, k_compact<4>, a));
     prof_end(ctx, s);
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_compact_full(ada_ctx* ctx, int B, int T, float thr, int32_t* rep_idx,
                                 int32_t* rep_cnt, float* gamma, cudaStream_t s) {
     CompactArgs a;
     a.g_tok = ctx->g_tok; a.g_rep = nullptr; a.role = nullptr;
-    a.agg = ctx->agg; a.done_ctr = ctx->done_ctr; a.dep_ctr = ctx->tile_ctr; a.status = ctx->status;
-    a.agg_stride = ctx->agg_stride; a.T = T; a.thr = thr;
+    a.dep_ctr = ctx->tile_ctr; a.status = ctx->status;
+    a.T = T; a.thr = thr;
     a.keep_idx = rep_idx; a.keep_cnt = rep_cnt;
     a.add_idx = nullptr; a.add_cnt = nullptr; a.rem_idx = nullptr; a.rem_cnt = nullptr;
     a.gamma_a = gamma; a.gamma_b = nullptr; a.row_scale = nullptr;
-    a.thr_seq = nullptr; a.r_in = nullptr;
+    a.r_in = nullptr;
     memset(&a.tu, 0, sizeof(a.tu));
     return launch_compact(ctx, K_COMPACT_FULL, a, B, s);
 }
@@ -690,21 +717,15 @@ cudaError_t launch_compact_cascade(ada_ctx* ctx, int B, int T, float thr, int32_
                                    cudaStream_t s) {
     CompactArgs a;
     a.g_tok = ctx->g_tok; a.g_rep = ctx->g_rep; a.role = ctx->role;
-    a.agg = ctx->agg; a.done_ctr = ctx->done_ctr; a.dep_ctr = ctx->tile_ctr; a.status = ctx->status;
-    a.agg_stride = ctx->agg_stride; a.T = T; a.thr = thr;
+    a.dep_ctr = ctx->tile_ctr; a.status = ctx->status;
+    a.T = T; a.thr = thr;
     a.keep_idx = rep_out; a.keep_cnt = rep_out_cnt;
     a.add_idx = add_idx; a.add_cnt = add_cnt; a.rem_idx = rem_idx; a.rem_cnt = rem_cnt;
     a.gamma_a = gamma_rep; a.gamma_b = gamma_cross;
     a.row_scale = row_scale ? ctx->inv_norm : nullptr;
-    a.thr_seq = tu.tau_state != nullptr ? ctx->thr_seq : nullptr;
     a.r_in = ctx->r_eff;
     a.tu = tu;
     return launch_compact(ctx, K_COMPACT_CASCADE, a, B, s);
-}
-
-cudaError_t launch_tau_thr(ada_ctx* ctx, int B, const double* tau_state, cudaStream_t s) {
-    launch_k(ctx, k_tau_thr, dim3((B + 127) / 128), dim3(128), 0, s, tau_state, B, ctx->thr_seq, ctx->status);
-    return cudaGetLastError();
 }
 
 }  // namespace ada

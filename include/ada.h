@@ -72,7 +72,7 @@ typedef enum { ADA_F32 = 0, ADA_BF16 = 1 } ada_dtype;
  * form by problem size.  ADA_BF16 feeds the stored values to the MMA; ADA_F32 is split into
  * three bf16 terms per value and contracted as the six leading cross terms (error at fp32
  * rounding level, fp32 accumulation), at the price of a 6x longer contraction and a
- * workspace of 48 bytes per element.  FFMA is the plain fp32 ALU kernel (any storage type;
+ * workspace of 12 bytes per element.  FFMA is the plain fp32 ALU kernel (any storage type;
  * for ADA_BF16 a slow cross-check of the tensor-core path).  TCGEN05 forces the one-CTA
  * kernel (128-row tiles), TCGEN05_PAIR the two-CTA kernel (cta_group::2, 256-row tiles
  * shared by the two SMs of a TPC). */
@@ -87,7 +87,8 @@ typedef struct ada_ctx ada_ctx; /* opaque */
 
 /* Create a context on `device` able to serve up to maxB sequences of maxT
  * tokens of width maxd in storage type dt.  Allocates the workspace
- * (cudaMalloc; about maxB*maxT*(maxd*es + 32) bytes, plus 48*maxB*maxT*maxd for ADA_F32).
+ * (cudaMalloc; about maxB*maxT*(maxd*es + 32) bytes, as much again of rows for ADA_BF16,
+ * 12*maxB*maxT*maxd for ADA_F32, and 128 KiB per SM for partial sums).
  * maxT may not exceed ADA_MAX_T (the list counts of one sequence are kept in 21-bit fields),
  * nor maxB*maxT 2^30: ADA_ERR_INVALID_ARG.  *out is NULL on error. */
 #define ADA_MAX_T ((int64_t)2097151)
@@ -95,12 +96,14 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
                       ada_dtype dt);
 ada_status ada_destroy(ada_ctx* ctx);
 ada_status ada_set_engine(ada_ctx* ctx, ada_engine e);
-/* The fused cascade launch has CTAs that wait on results of other CTAs of the same grid, so
- * it is launched cooperatively (the driver guarantees that all CTAs are resident, or refuses
- * the launch).  on = 0 launches it as an ordinary grid of one CTA per SM instead: same
- * kernel and results, but if other work keeps some SMs busy for long the in-kernel waits
- * can expire (ADA_ERR_TIMEOUT).  Meant for profilers that cannot replay cooperative
- * launches.  Default: on. */
+/* Gram launches have CTAs that wait on results of other CTAs of the same grid.  With on != 0 (the
+ * default) such a launch carries the cooperative attribute (the driver guarantees that all CTAs
+ * are resident, or refuses the launch) whenever another one might keep some of its CTAs from
+ * running: in all streams but the first one that uses the library on the device (until that one
+ * has been seen idle by ada_device_status or ada_destroy), under stream capture, and under MPS.
+ * on = 0 never uses the attribute: same kernels and results, but launches that overlap in
+ * different streams can then wait for one another until the in-kernel limits expire
+ * (ADA_ERR_TIMEOUT).  Meant for profilers that cannot replay cooperative launches. */
 ada_status ada_set_cooperative(ada_ctx* ctx, int on);
 
 /* Algorithm 1 line 6 forms the cross-Gram from the tokens OUTSIDE the inherited set.  On the

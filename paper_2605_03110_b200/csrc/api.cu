@@ -3,6 +3,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <mutex>
 #include <new>
 
 #include "common.cuh"
@@ -55,31 +56,26 @@ bool use_tc(const ada_ctx* ctx, ada_dtype dt) {
 
 // fp32 storage on the bf16 tensor cores through the three-term split
 bool use_split(const ada_ctx* ctx, ada_dtype dt) {
-    return dt == ADA_F32 && ctx->engine != ADA_ENGINE_FFMA && ctx->splitXA != nullptr &&
+    return dt == ADA_F32 && ctx->engine != ADA_ENGINE_FFMA && ctx->splitX != nullptr &&
            gram_tc_available();
 }
 
 // the pair-CTA form of the tensor-core kernel, or the one-CTA form?
-bool use_pair(const ada_ctx* ctx, int64_t B, int64_t T, int64_t d) {
+bool use_pair(const ada_ctx* ctx, int64_t B, int64_t T, int64_t d, ada_dtype dt) {
     if (ctx->engine == ADA_ENGINE_TCGEN05_PAIR) return true;
-    // The pair kernel pays off from a few thousand rows and a long contraction on (measured on
-    // the crossover sweep: at T = 4096, d = 4096 both calls are faster on it, at T = 2048 they
-    // are not); small problems are covered better by the finer one-CTA tiles.
-    return ctx->engine == ADA_ENGINE_AUTO && B * T >= 4096 && d >= 2048;
+    if (ctx->engine != ADA_ENGINE_AUTO) return false;
+    // Measured against the one-CTA kernel, whose narrow tiles occupy every SM where the pair kernel
+    // has to split its few tiles along K: with the split the pair kernel is faster from 512 tokens
+    // on (T = 1024, d = 4096: full selection 27.4 -> 24.0 us, step 34.8 -> 28.2; fp32, T = 700,
+    // d = 1600: 55.8 -> 23.7, step 67.8 -> 30.3), where the contraction is too long to be split only from a few
+    // thousand rows on (T = 700, d = 5120: 31.0 against 34.7 us).
+    if (dt == ADA_F32) return d >= 256 && (d <= MAX_SPLIT_D_F32 || B * T >= 4096);
+    return d >= 2048 && B * T >= (d <= MAX_SPLIT_D ? 512 : 4096);
 }
 
-// tensor-core launch of one or two segments, in the one-CTA or the pair-CTA form
-cudaError_t launch_tc(ada_ctx* ctx, const GramProblem* tri, const GramProblem* cross,
-                      const NormJob* norms, cudaStream_t s) {
-    const GramProblem* p = cross != nullptr ? cross : tri;
-    if (use_pair(ctx, p->B, p->rows, p->d)) return launch_gram_tc2(ctx, tri, cross, norms, nullptr, s);
-    return launch_gram_tc(ctx, tri, cross, norms, s);
-}
+// plane width of an fp32 row of d elements: whole 64-element K blocks
+inline int64_t plane_len(int64_t d) { return (d + 63) / 64 * 64; }
 
-cudaError_t run_gram(ada_ctx* ctx, const GramProblem& p, ada_dtype dt, cudaStream_t s) {
-    if (use_tc(ctx, dt)) return p.tri ? launch_tc(ctx, &p, nullptr, nullptr, s) : launch_tc(ctx, nullptr, &p, nullptr, s);
-    return launch_gram_ffma(ctx, p, dt, s);
-}
 
 #define CU(x)                                  \
     do {                                       \
@@ -90,6 +86,75 @@ cudaError_t run_gram(ada_ctx* ctx, const GramProblem& p, ada_dtype dt, cudaStrea
 }  // namespace
 
 namespace ada {
+
+// ---------------------------------------------------------------------------
+// Which launches have to be cooperative.  A Gram launch with CTAs that wait on one another ends
+// only if all of them get to run.  Two such launches in different streams could each hold
+// half of the SMs and wait for the other half for ever; a cooperative launch, placed whole or not
+// at all, rules that out, but the driver then neither places its CTAs while the kernel before
+// it drains nor lets them set up meanwhile (measured: 4 to 8 us per call of a chain).  So per
+// device ONE stream may launch without the attribute -- in stream order, its launches never
+// overlap one another -- and every other stream keeps it, until the first one has been seen idle.
+// Captured launches keep it too (where a graph will be replayed is unknown), and so does
+// everything under MPS (other processes are not known here).
+// ---------------------------------------------------------------------------
+namespace {
+struct SoleStream {
+    std::mutex lock;
+    bool held = false;
+    unsigned long long id = 0;       // stream ids are never reused within a process
+    unsigned long long launches = 0; // launches without the attribute so far
+    int pending = 0;                 // of them, those not handed to the driver yet
+    int mps = -1;
+};
+constexpr int kMaxSole = 64;
+SoleStream g_sole[kMaxSole];
+}  // namespace
+
+bool coop_begin(ada_ctx* ctx, cudaStream_t s) {
+    if (!ctx->cooperative) return false;
+    if (ctx->device < 0 || ctx->device >= kMaxSole) return true;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) { cudaGetLastError(); return true; }
+    if (cap != cudaStreamCaptureStatusNone) return true;
+    if (cudaStreamGetId(s, &id) != cudaSuccess) { cudaGetLastError(); return true; }
+    SoleStream& w = g_sole[ctx->device];
+    std::lock_guard<std::mutex> hold(w.lock);
+    if (w.mps < 0 && cudaDeviceGetAttribute(&w.mps, cudaDevAttrMpsEnabled, ctx->device) != cudaSuccess) {
+        cudaGetLastError();
+        w.mps = 1;
+    }
+    if (w.mps != 0 || (w.held && w.id != id)) return true;
+    w.held = true;
+    w.id = id;
+    ++w.launches;
+    ++w.pending;
+    return false;
+}
+
+void coop_end(ada_ctx* ctx, bool coop) {
+    if (coop || !ctx->cooperative) return;
+    SoleStream& w = g_sole[ctx->device];
+    std::lock_guard<std::mutex> hold(w.lock);
+    --w.pending;
+}
+
+unsigned long long sole_mark(int device) {
+    if (device < 0 || device >= kMaxSole) return 0;
+    SoleStream& w = g_sole[device];
+    std::lock_guard<std::mutex> hold(w.lock);
+    return w.pending == 0 ? w.launches : ~0ull;
+}
+
+void sole_idle(int device, bool all, cudaStream_t s, unsigned long long mark) {
+    if (device < 0 || device >= kMaxSole) return;
+    unsigned long long id = 0;
+    if (!all && cudaStreamGetId(s, &id) != cudaSuccess) { cudaGetLastError(); return; }
+    SoleStream& w = g_sole[device];
+    std::lock_guard<std::mutex> hold(w.lock);
+    if (w.held && w.launches == mark && (all || w.id == id)) w.held = false;
+}
 
 void prof_begin(ada_ctx* ctx, int kid, cudaStream_t s) {
     Profiler& pr = ctx->prof;
@@ -164,6 +229,7 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
     ctx->tc2_attr_set = false;
     ctx->tc2_pairs = 0;
     ctx->compact_min_rows = 8192;
+    ctx->max_parts = MAX_PARTS;
     cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, device);
 
     const size_t n_tok = (size_t)maxB * (size_t)maxT;
@@ -179,9 +245,11 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
     // bf16: the rows outside a large inherited set, copied out for the cross step (Algorithm 1 line 6)
     const size_t o_ntok = take(dt == ADA_BF16 ? n_tok * 4 : 0);
     const size_t o_xnon = take(dt == ADA_BF16 ? n_tok * (size_t)maxd * 2 + 1024 : 0);
-    const size_t split_bytes = dt == ADA_F32 ? n_tok * (size_t)maxd * 12 + 1024 : 0;
-    const size_t o_sxa = take(split_bytes), o_sxb = take(split_bytes), o_sra = take(split_bytes),
-                 o_srb = take(split_bytes);
+    const size_t split_bytes = dt == ADA_F32 ? n_tok * (size_t)plane_len(maxd) * 6 + 1024 : 0;
+    const size_t o_sx = take(split_bytes), o_sr = take(split_bytes);
+    // one 256-column fp32 accumulator per SM
+    ctx->part_bytes = (size_t)ctx->sm_count * 128 * 256 * 4;
+    const size_t o_part = take(ctx->part_bytes);
     if (cudaMalloc(&ctx->ws, off) != cudaSuccess) {
         cudaGetLastError();
         delete ctx;
@@ -199,11 +267,11 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
     ctx->Xrep = ctx->ws + o_xrep;
     ctx->Xnon = dt == ADA_BF16 ? ctx->ws + o_xnon : nullptr;
     ctx->non_tok = dt == ADA_BF16 ? reinterpret_cast<int32_t*>(ctx->ws + o_ntok) : nullptr;
-    ctx->splitXA = split_bytes ? ctx->ws + o_sxa : nullptr;
-    ctx->splitXB = split_bytes ? ctx->ws + o_sxb : nullptr;
-    ctx->splitRA = split_bytes ? ctx->ws + o_sra : nullptr;
-    ctx->splitRB = split_bytes ? ctx->ws + o_srb : nullptr;
+    ctx->splitX = split_bytes ? ctx->ws + o_sx : nullptr;
+    ctx->splitR = split_bytes ? ctx->ws + o_sr : nullptr;
+    ctx->part_buf = reinterpret_cast<unsigned*>(ctx->ws + o_part);
     if (cudaMemset(ctx->ws, 0, o_xrep) != cudaSuccess ||
+        cudaMemset(ctx->part_buf, 0xFF, ctx->part_bytes) != cudaSuccess ||
         (dt == ADA_BF16 && cudaMemset(ctx->ws + o_ntok, 0, n_tok * 4) != cudaSuccess)) {
         cudaFree(ctx->ws);
         delete ctx;
@@ -216,7 +284,8 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
 ada_status ada_destroy(ada_ctx* ctx) {
     if (ctx == nullptr) return ADA_ERR_INVALID_ARG;
     DeviceGuard guard(ctx->device);
-    cudaDeviceSynchronize();
+    const unsigned long long mark = sole_mark(ctx->device);
+    if (cudaDeviceSynchronize() == cudaSuccess) sole_idle(ctx->device, true, nullptr, mark);
     for (int i = 0; i < ctx->prof.created; ++i) {
         cudaEventDestroy(ctx->prof.ev0[i]);
         cudaEventDestroy(ctx->prof.ev1[i]);
@@ -277,6 +346,44 @@ ada_status ada_normalize(ada_ctx* ctx, const void* X, int64_t B, int64_t T, int6
     return ADA_OK;
 }
 
+// fp32 rows of X as bf16 planes in ctx->splitX (and their inverse norms)
+static SplitJob split_job(ada_ctx* ctx, const void* X, int64_t B, int64_t T, int64_t d, int64_t ldx, int64_t xb) {
+    SplitJob j;
+    memset(&j, 0, sizeof(j));
+    j.X = static_cast<const float*>(X); j.ldx = ldx; j.xb = xb;
+    j.T = (int)T; j.B = (int)B; j.d = (int)d; j.dpad = (int)plane_len(d);
+    j.XP = static_cast<__nv_bfloat16*>(ctx->splitX);
+    j.inv_norm = ctx->inv_norm;
+    j.role = ctx->role; j.r_eff = ctx->r_eff;
+    j.RP = static_cast<__nv_bfloat16*>(ctx->splitR);
+    j.inv_rep = ctx->inv_rep;
+    return j;
+}
+
+// Algorithm 1 lines 1-2 on bf16 rows, inside a pair-kernel launch
+static GatherJob gather_job(ada_ctx* ctx, const void* X, int64_t B, int64_t T, int64_t d, int64_t ldx, int64_t xb,
+                            const int32_t* rep_in, const int32_t* rep_in_cnt) {
+    GatherJob j;
+    memset(&j, 0, sizeof(j));
+    j.X = X; j.ldx = ldx; j.xb = xb;
+    j.rep_in = rep_in; j.rep_in_cnt = rep_in_cnt;
+    j.role = ctx->role; j.r_eff = ctx->r_eff; j.Xrep = ctx->Xrep; j.inv_rep = ctx->inv_rep;
+    j.T = (int)T; j.d = (int)d; j.B = (int)B;
+    j.Xnon = ctx->Xnon; j.non_tok = ctx->non_tok; j.inv_norm = ctx->inv_norm;
+    j.compact_min_rows = ctx->compact_min_rows;
+    return j;
+}
+
+// operands of `p` are rows of planes; the one-CTA kernel walks the six cross terms as one contraction
+static void use_planes(GramProblem& p, const void* A, const void* Bm, int64_t T, int64_t d, bool pair) {
+    const int64_t pl = plane_len(d);
+    p.A = A; p.Bm = Bm;
+    p.lda = p.ldb = 3 * pl;
+    p.a_batch = p.b_batch = T * 3 * pl;
+    p.planes = (int)pl;
+    p.d = (int)(pair ? d : 6 * pl);
+}
+
 // Definition 1 for B independent problems; row (b, t) of X starts at element b * xb + t * ldx
 static ada_status select_full_impl(ada_ctx* ctx, const void* X, int64_t B, int64_t T, int64_t d,
                                    int64_t ldx, int64_t xb, ada_dtype dt, double tau,
@@ -287,17 +394,15 @@ static ada_status select_full_impl(ada_ctx* ctx, const void* X, int64_t B, int64
     const float thr = (float)(1.0 - tau * tau);
 
     // the gamma scratch is zero on entry (workspace invariant kept by the compaction kernels)
-    // long-K tensor-core launches compute the row norms themselves, hidden behind the MMAs
-    const bool split = use_split(ctx, dt);
-    const bool tc = use_tc(ctx, dt), fuse = tc && d >= 2048 && B * T >= 4096 && xb == T * ldx;
-    if (split)   // one pass: 1/||x|| and the bf16 terms of X
-        CU(launch_split(ctx, X, (int)B, (int)T, (int)d, ldx, xb, false, s));
-    else if (!fuse)
-        CU(launch_norm_gather(ctx, X, (int)B, (int)T, (int)d, ldx, xb, dt, ctx->inv_norm, nullptr,
-                              nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s));
+    const bool split = use_split(ctx, dt), tc = use_tc(ctx, dt);
+    const bool pair = (split || tc) && use_pair(ctx, B, T, d, dt);
+    // bf16: the pair kernel (and the one-CTA kernel, for many rows of a long contraction) computes
+    // the row norms itself, hidden behind the MMAs
+    const bool fuse = tc && (pair || (d >= 2048 && B * T >= 4096 && xb == T * ldx));
     NormJob nj;
     nj.X = X; nj.ldx = ldx; nj.n_rows = B * T; nj.d = (int)d; nj.inv_norm = ctx->inv_norm;
-    nj.batch = 0; nj.rows_per_seq = 0;
+    nj.batch = xb; nj.rows_per_seq = (int)T;
+    SplitJob sj = split_job(ctx, X, B, T, d, ldx, xb);
     GramProblem p;
     memset(&p, 0, sizeof(p));
     p.A = X; p.Bm = X;
@@ -309,14 +414,16 @@ static ada_status select_full_impl(ada_ctx* ctx, const void* X, int64_t B, int64
     p.rows = (int)T; p.cap = (int)T; p.d = (int)d; p.B = (int)B;
     p.tri = 1;
     p.wait_norm_a = p.wait_norm_b = fuse ? 1 : 0;
-    if (split) {
-        p.A = ctx->splitXA; p.Bm = ctx->splitXB;
-        p.lda = p.ldb = 6 * d;
-        p.a_batch = p.b_batch = T * 6 * d;
-        p.d = (int)(6 * d);
-        CU(launch_tc(ctx, &p, nullptr, nullptr, s));
-    } else if (tc) CU(launch_tc(ctx, &p, nullptr, fuse ? &nj : nullptr, s));
-    else CU(run_gram(ctx, p, dt, s));
+    if (split) {   // 1/||x|| and the bf16 planes of X, inside the pair kernel's launch or before the other's
+        use_planes(p, ctx->splitX, ctx->splitX, T, d, pair);
+        if (!pair) CU(launch_split(ctx, sj, s));
+    } else if (!fuse) {
+        CU(launch_norm_gather(ctx, X, (int)B, (int)T, (int)d, ldx, xb, dt, ctx->inv_norm, nullptr,
+                              nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s));
+    }
+    if (pair) CU(launch_gram_tc2(ctx, &p, nullptr, fuse ? &nj : nullptr, nullptr, split ? &sj : nullptr, s));
+    else if (split || tc) CU(launch_gram_tc(ctx, &p, nullptr, fuse ? &nj : nullptr, s));
+    else CU(launch_gram_ffma(ctx, p, dt, s));
     CU(launch_compact_full(ctx, (int)B, (int)T, thr, rep_idx, rep_cnt, gamma, s));
     return ADA_OK;
 }
@@ -369,34 +476,27 @@ static ada_status cascade_impl(ada_ctx* ctx, const void* X, int64_t B, int64_t T
     // kept by the compaction kernels).
     const bool split = use_split(ctx, dt);
     const bool fuse = use_tc(ctx, dt) || split;
-    // bf16 on the pair kernel: ONE Gram launch does lines 1-8.  Its helper warps validate the
-    // inherited list, scatter the role map and gather the rows (lines 1-2); the r x r tiles
-    // (lines 3-5) and the cross tiles (lines 6-8) follow; the norms of X come out of the cross
-    // tiles while they sit in shared memory, and the row's own factor 1/||x_t|| is left to the
+    // On the pair kernel ONE Gram launch does lines 1-8.  Its spare warps validate the
+    // inherited list, scatter the role map and gather the rows (lines 1-2; fp32: and make the bf16
+    // planes); the r x r tiles (lines 3-5) and the cross tiles (lines 6-8) follow; for bf16 the
+    // norms of X are made beside them and the row's own factor 1/||x_t|| is left to the
     // compaction.
-    const bool inl = fuse && !split && use_pair(ctx, B, T, d);
+    const bool inl = fuse && use_pair(ctx, B, T, d, dt);
     // otherwise lines 1-2 are a launch of their own: inverse norms of all rows, inherited list
     // validated, scattered into the role map and its rows gathered into Xrep; for long K the
     // one-CTA tensor-core launch computes line 1's row norms itself
     const bool fuse_norm = !inl && !split && fuse && d >= 2048 && B * T >= 4096 && xb == T * ldx;
-    if (!inl)
-        CU(launch_norm_gather(ctx, X, (int)B, (int)T, (int)d, ldx, xb, dt,
-                              (fuse_norm || split) ? nullptr : ctx->inv_norm,
+    SplitJob sj = split_job(ctx, X, B, T, d, ldx, xb);
+    sj.rep_in = rep_in; sj.rep_in_cnt = rep_in_cnt;
+    if (split && !inl) CU(launch_split(ctx, sj, s));
+    else if (!inl)
+        CU(launch_norm_gather(ctx, X, (int)B, (int)T, (int)d, ldx, xb, dt, fuse_norm ? nullptr : ctx->inv_norm,
                               nullptr, rep_in, rep_in_cnt, ctx->role, ctx->r_eff, ctx->Xrep,
                               ctx->inv_rep, s));
     NormJob nj;
     nj.X = X; nj.ldx = ldx; nj.n_rows = B * T; nj.d = (int)d; nj.inv_norm = ctx->inv_norm;
     nj.batch = 0; nj.rows_per_seq = 0;
-    GatherJob gj;
-    memset(&gj, 0, sizeof(gj));
-    gj.X = X; gj.ldx = ldx; gj.xb = xb;
-    gj.rep_in = rep_in; gj.rep_in_cnt = rep_in_cnt;
-    gj.role = ctx->role; gj.r_eff = ctx->r_eff; gj.Xrep = ctx->Xrep; gj.inv_rep = ctx->inv_rep;
-    gj.T = (int)T; gj.d = (int)d; gj.B = (int)B;
-    gj.Xnon = ctx->Xnon; gj.non_tok = ctx->non_tok; gj.inv_norm = ctx->inv_norm;
-    gj.compact_min_rows = ctx->compact_min_rows;
-    if (split)   // 1/||x|| of all rows; bf16 terms of X and of the gathered rows
-        CU(launch_split(ctx, X, (int)B, (int)T, (int)d, ldx, xb, true, s));
+    GatherJob gj = gather_job(ctx, X, B, T, d, ldx, xb, rep_in, rep_in_cnt);
     // lines 3-4: r x r Gram among inherited reps, max over earlier ones
     GramProblem p;
     memset(&p, 0, sizeof(p));
@@ -409,7 +509,7 @@ static ada_status cascade_impl(ada_ctx* ctx, const void* X, int64_t B, int64_t T
     p.n_clamp = inl ? 1 : 0;
     p.rows = (int)T; p.cap = (int)T; p.d = (int)d; p.B = (int)B;
     p.tri = 1;
-    if (!fuse) CU(run_gram(ctx, p, dt, s));
+    if (!fuse) CU(launch_gram_ffma(ctx, p, dt, s));
     // lines 6-8: cross-Gram of all rows against the valid inherited reps
     GramProblem q;
     memset(&q, 0, sizeof(q));
@@ -430,25 +530,22 @@ static ada_status cascade_impl(ada_ctx* ctx, const void* X, int64_t B, int64_t T
     q.row_role = ctx->role;
     q.causal = (flags & ADA_CROSS_CAUSAL) ? 1 : 0;
     q.wait_norm_a = fuse_norm ? 1 : 0;
-    if (inl) {
+    if (inl && !split) {
         q.defer_row = 1;
         q.inv_out = ctx->inv_norm;
         q.hb_rows = gram_tc2_hb_rows(ctx, (int)B, (int)T);
         if (q.hb_rows == 0) return ADA_ERR_CUDA;
     }
     if (split) {
-        p.A = ctx->splitRA; p.Bm = ctx->splitRB;
-        q.A = ctx->splitXA; q.Bm = ctx->splitRB;
-        p.lda = p.ldb = q.lda = q.ldb = 6 * d;
-        p.a_batch = p.b_batch = q.a_batch = q.b_batch = T * 6 * d;
-        p.d = q.d = (int)(6 * d);
+        use_planes(p, ctx->splitR, ctx->splitR, T, d, inl);
+        use_planes(q, ctx->splitX, ctx->splitR, T, d, inl);
     }
-    if (inl) CU(launch_gram_tc2(ctx, &p, &q, nullptr, &gj, s));
-    else if (fuse) CU(launch_tc(ctx, &p, &q, fuse_norm ? &nj : nullptr, s));
-    else CU(run_gram(ctx, q, dt, s));
+    if (inl) CU(launch_gram_tc2(ctx, &p, &q, nullptr, split ? nullptr : &gj, split ? &sj : nullptr, s));
+    else if (fuse) CU(launch_gram_tc(ctx, &p, &q, fuse_norm ? &nj : nullptr, s));
+    else CU(launch_gram_ffma(ctx, q, dt, s));
     // lines 5, 9, 10-11
     CU(launch_compact_cascade(ctx, (int)B, (int)T, thr, rep_out, rep_out_cnt, add_idx, add_cnt,
-                              rem_idx, rem_cnt, gamma_rep, gamma_cross, tau_upd, inl, s));
+                              rem_idx, rem_cnt, gamma_rep, gamma_cross, tau_upd, q.defer_row != 0, s));
     return ADA_OK;
 }
 
@@ -516,35 +613,47 @@ ada_status ada_nearest_rep(ada_ctx* ctx, const void* X, int64_t B, int64_t T, in
     if (st != ADA_OK) return st;
     if (rep_idx == nullptr || rep_cnt == nullptr || nearest_idx == nullptr) return ADA_ERR_INVALID_ARG;
     const bool split = dt == ADA_F32;
-    if (!gram_tc_available() || (split && ctx->splitXA == nullptr)) return ADA_ERR_UNSUPPORTED;
+    if (!gram_tc_available() || (split && ctx->splitX == nullptr)) return ADA_ERR_UNSUPPORTED;
     DeviceGuard guard(ctx->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const bool pair = use_pair(ctx, B, T, d, dt);
     // role map and keys are zero on entry (workspace invariant); the finish kernel clears them
-    CU(launch_norm_gather(ctx, X, (int)B, (int)T, (int)d, ldx, T * ldx, dt, split ? nullptr : ctx->inv_norm,
-                          nullptr, rep_idx, rep_cnt, ctx->role, ctx->r_eff, ctx->Xrep, ctx->inv_rep, s));
-    if (split) CU(launch_split(ctx, X, (int)B, (int)T, (int)d, ldx, T * ldx, true, s));
+    SplitJob sj = split_job(ctx, X, B, T, d, ldx, T * ldx);
+    sj.rep_in = rep_idx; sj.rep_in_cnt = rep_cnt;
+    GatherJob gj = gather_job(ctx, X, B, T, d, ldx, T * ldx, rep_idx, rep_cnt);
+    gj.Xnon = nullptr;                // every row is wanted
+    if (!pair) {
+        if (split) CU(launch_split(ctx, sj, s));
+        else
+            CU(launch_norm_gather(ctx, X, (int)B, (int)T, (int)d, ldx, T * ldx, dt, ctx->inv_norm, nullptr, rep_idx,
+                                  rep_cnt, ctx->role, ctx->r_eff, ctx->Xrep, ctx->inv_rep, s));
+    }
     GramProblem q;
     memset(&q, 0, sizeof(q));
     q.A = X; q.Bm = ctx->Xrep;
     q.lda = ldx; q.ldb = d;
     q.a_batch = T * ldx; q.b_batch = T * d;
-    if (split) {
-        q.A = ctx->splitXA; q.Bm = ctx->splitRB;
-        q.lda = q.ldb = 6 * d;
-        q.a_batch = q.b_batch = T * 6 * d;
-    }
     q.inv_a = ctx->inv_norm; q.inv_b = ctx->inv_rep;
     q.out = ctx->g_tok;
     q.out_arg = ctx->near_key;
-    q.n_dev = ctx->r_eff; q.n_host = 0;
-    q.rows = (int)T; q.cap = (int)T; q.d = (int)(split ? 6 * d : d); q.B = (int)B;
+    q.n_dev = pair ? rep_cnt : ctx->r_eff; q.n_host = 0;
+    q.n_clamp = pair ? 1 : 0;
+    q.rows = (int)T; q.cap = (int)T; q.d = (int)d; q.B = (int)B;
     q.tri = 0;
     q.col_gate = ctx->g_rep;          // all zero: every column passes the gate
     q.thr_bits = 0xFFFFFFFFu;
     q.col_token = rep_idx;
     q.row_role = ctx->role;           // representatives are resolved by the finish kernel
     q.causal = 0;
-    CU(launch_gram_tc(ctx, nullptr, &q, nullptr, s));
+    q.defer_row = 1;                  // which applies the row's own factor too
+    if (split) use_planes(q, ctx->splitX, ctx->splitR, T, d, pair);
+    else if (pair) {
+        q.inv_out = ctx->inv_norm;
+        q.hb_rows = gram_tc2_hb_rows(ctx, (int)B, (int)T);
+        if (q.hb_rows == 0) return ADA_ERR_CUDA;
+    }
+    if (pair) CU(launch_gram_tc2(ctx, nullptr, &q, nullptr, split ? nullptr : &gj, split ? &sj : nullptr, s));
+    else CU(launch_gram_tc(ctx, nullptr, &q, nullptr, s));
     CU(launch_nearest_finish(ctx, (int)B, (int)T, rep_idx, nearest_idx, nearest_gamma, s));
     return ADA_OK;
 }
@@ -577,13 +686,16 @@ ada_status ada_device_status(ada_ctx* ctx, void* stream, int64_t* n_zero_norm_ro
     DeviceGuard guard(ctx->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     unsigned h[8];
+    const unsigned long long mark = sole_mark(ctx->device);
     CU(cudaMemcpyAsync(h, ctx->status, sizeof(h), cudaMemcpyDeviceToHost, s));
     CU(cudaMemsetAsync(ctx->status, 0, sizeof(h), s));
     CU(cudaStreamSynchronize(s));
+    sole_idle(ctx->device, false, s, mark);
     if (n_zero_norm_rows != nullptr) *n_zero_norm_rows = (int64_t)h[1];
     if (h[0] != 0) {
-        // a faulted call may have left scratch behind: restore the all-zero workspace invariant
+        // a faulted call may have left scratch behind: restore the workspace invariants
         CU(cudaMemsetAsync(ctx->role, 0, (size_t)((char*)ctx->inv_norm - (char*)ctx->role), s));
+        CU(cudaMemsetAsync(ctx->part_buf, 0xFF, ctx->part_bytes, s));
         CU(cudaStreamSynchronize(s));
     }
     if (h[0] & ST_TIMEOUT) return ADA_ERR_TIMEOUT;

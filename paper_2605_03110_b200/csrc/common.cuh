@@ -74,17 +74,20 @@ struct GramProblem {
     unsigned long long* out_arg;
     // n_dev holds the caller's raw counts: clamp them to [0, cap] (nobody has sanitised them yet)
     int n_clamp;
-    // pair kernel, cross only -----------------------------------------------------------------
-    // out[] receives the row maximum WITHOUT the factor inv_a[i] (a positive factor common to the
+    // cross only --------------------------------------------------------------------------------
+    // out[] (or the key in out_arg) receives the row maximum WITHOUT the factor inv_a[i] (a positive factor common to the
     // row commutes with the maximum, rounding included); the compaction applies it.  No row
     // norm is then needed inside the launch.
     int defer_row;
+    // pair kernel, cross only -----------------------------------------------------------------
     // 1/||a_i|| of every row of A, computed from the A tiles while they sit in shared memory (by
     // the tiles of the first column tile) and stored here; NULL: not wanted
     float* inv_out;
     // rows of A per CTA when a single column tile covers every sequence's columns (a cross-Gram
     // bound by streaming A once: shorter row tiles put every SM pair to work); 0 or 128: 128
     int hb_rows;
+    // fp32 storage: A and Bm point to rows of three bf16 planes of this many elements; 0: plain bf16
+    int planes;
 };
 
 // Algorithm 1 lines 1-2 inside a pair-kernel launch: the inherited list is validated, scattered
@@ -109,6 +112,26 @@ struct GatherJob {
     int compact_min_rows;     // sequences shorter than this never use it
 };
 
+// fp32 storage on the bf16 tensor cores: every row becomes three bf16 planes (x = hi + mid + lo,
+// hi = bf16(x), mid = bf16(x - hi), lo = bf16(x - hi - mid); both differences are exact in fp32), and
+// a dot product is evaluated as the six largest of the nine cross terms, hi.hi + hi.mid +
+// mid.hi + hi.lo + lo.hi + mid.mid, all of whose bf16 x bf16 products are exact in the fp32
+// accumulator.  What is dropped is below 2^-23 |x||y|, i.e. fp32 rounding level.
+// X == NULL: nothing to do.
+struct SplitJob {
+    const float* X;
+    int64_t ldx, xb;          // row / sequence strides of X in elements
+    int T, B, d, dpad;        // dpad: d rounded up to whole 64-element K blocks
+    __nv_bfloat16* XP;        // [B*T][3][dpad]
+    float* inv_norm;          // [B*T]
+    const int32_t* rep_in;    // inherited list, or NULL
+    const int32_t* rep_in_cnt;
+    int32_t* role;
+    int32_t* r_eff;
+    __nv_bfloat16* RP;        // [B*T][3][dpad], by position
+    float* inv_rep;           // [B*T] by position
+};
+
 // Row norms computed inside a tensor-core Gram launch by four extra warps per CTA
 // (Section 2.1; Algorithm 1 line 1): inv_norm[row] = 1/||x_row|| for all n_rows rows of X.
 // X == NULL: nothing to do.
@@ -123,6 +146,10 @@ struct NormJob {
     int64_t batch;
     int rows_per_seq;
 };
+
+// contraction lengths up to which a tile may be split in two (pair kernel, shares_ok)
+constexpr int MAX_SPLIT_D = 4600, MAX_SPLIT_D_F32 = 2140;
+constexpr int MAX_PARTS = 4;      // most shares of one tile
 
 struct Profiler {
     bool on = false;
@@ -142,7 +169,7 @@ struct ada_ctx {
     ada_engine engine;
     int sm_count;
     bool tc_attr_set;
-    bool cooperative;    // fused launches use the cooperative attribute
+    bool cooperative;    // false: never use the cooperative attribute (see coop_begin)
     bool dep_launch;     // kernels are launched with programmatic stream serialization
     int compact_min_rows;  // sequence length from which a large inherited set's complement is copied out
     bool tc2_attr_set;   // pair-CTA kernel configured
@@ -161,9 +188,13 @@ struct ada_ctx {
     void* Xrep;          // [maxB*maxT*maxd] gathered representative rows (raw values)
     void* Xnon;          // [maxB*maxT*maxd] bf16 contexts: the rows outside a large inherited set
     int32_t* non_tok;    // [maxB*maxT] their token indices
-    // fp32 contexts: three-term bf16 splits laid out for one contraction of length 6d
-    void *splitXA, *splitXB;   // [maxB*maxT][6 maxd] of X
-    void *splitRA, *splitRB;   // same, of the gathered representative rows
+    // fp32 contexts: three bf16 planes of every row
+    void *splitX;        // [maxB*maxT][3][dpad] of X
+    void *splitR;        // same, of the gathered representative rows
+    // exchange of partial accumulators in the pair kernel (tiles split along K)
+    unsigned* part_buf;  // all ones between calls
+    size_t part_bytes;
+    int max_parts;       // most shares of one tile (1: never split)
     // gathered Q_R, K_R, V_R^T of the attention on the representative set (allocated on first use)
     char* attn_ws;
     size_t attn_ws_bytes;
@@ -216,6 +247,14 @@ cudaError_t launch_k(ada_ctx* ctx, void (*kernel)(KArgs...), dim3 grid, dim3 blo
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// Must a launch on `s` whose CTAs wait on one another be cooperative?  Asked right before such a launch;
+// coop_end, with the answer, right after it.  sole_mark before and sole_idle after a
+// synchronisation (of stream s, or of everything) tell that the launches so far are done.
+bool coop_begin(ada_ctx* ctx, cudaStream_t s);
+void coop_end(ada_ctx* ctx, bool coop);
+unsigned long long sole_mark(int device);
+void sole_idle(int device, bool all, cudaStream_t s, unsigned long long mark);
+
 // RAII-free launch bracket used by every launcher.
 void prof_begin(ada_ctx* ctx, int kid, cudaStream_t s);
 void prof_end(ada_ctx* ctx, cudaStream_t s);
@@ -225,8 +264,7 @@ cudaError_t launch_norm_gather(ada_ctx* ctx, const void* X, int B, int T, int d,
                                int64_t xb, ada_dtype dt, float* inv_norm, void* Xhat, const int32_t* rep_in,
                                const int32_t* rep_in_cnt, int32_t* role, int32_t* r_eff, void* Xrep,
                                float* inv_rep, cudaStream_t s);
-cudaError_t launch_split(ada_ctx* ctx, const void* X, int B, int T, int d, int64_t ldx, int64_t xb,
-                         bool with_rep, cudaStream_t s);
+cudaError_t launch_split(ada_ctx* ctx, const SplitJob& job, cudaStream_t s);
 cudaError_t launch_nearest_finish(ada_ctx* ctx, int B, int T, const int32_t* rep_idx,
                                   int32_t* nearest_idx, float* nearest_gamma, cudaStream_t s);
 cudaError_t launch_compact_full(ada_ctx* ctx, int B, int T, float thr, int32_t* rep_idx,
@@ -263,7 +301,8 @@ cudaError_t launch_attention_reps(ada_ctx* ctx, const void* Q, const void* K, co
 
 // gram_tc2.cu (bf16, tcgen05.cta_group::2: two CTAs per 256-row tile)
 cudaError_t launch_gram_tc2(ada_ctx* ctx, const GramProblem* tri, const GramProblem* cross,
-                            const NormJob* norms, const GatherJob* gather, cudaStream_t s);
+                            const NormJob* norms, const GatherJob* gather, const SplitJob* split,
+                            cudaStream_t s);
 // rows of the left operand per CTA for a cross-Gram that a single column tile covers
 int gram_tc2_hb_rows(ada_ctx* ctx, int B, int T);
 

@@ -64,7 +64,8 @@ struct Shape {
 // for the counter to reach 4 x (number of triangular tiles) before it stages its column
 // factors.  The cross MAIN LOOPS do not wait, so the short r x r problem hides behind them.
 // Triangular tiles precede cross tiles in every CTA's order and wait on nothing, and the
-// launch is cooperative (all CTAs co-resident), so the wait always ends.
+// launch is cooperative unless nothing else can keep its CTAs apart (coop_begin), so the wait
+// always ends.
 __device__ __forceinline__ int seq_n(const GramProblem& p, int b) {
     return p.n_dev != nullptr ? p.n_dev[b] : p.n_host;
 }
@@ -187,6 +188,11 @@ __device__ __forceinline__ bool decode_tile(const GramProblem& p, int par, int i
     return false;
 }
 
+// fp32 storage (GramProblem::planes): the six cross terms are contracted one K block after the
+// other, p.d = 6 planes elements in all; planes of A and B in term t
+__device__ __forceinline__ int plane_a(int t) { return t == 4 ? 2 : (t == 2 || t == 5 ? 1 : 0); }
+__device__ __forceinline__ int plane_b(int t) { return t == 3 ? 2 : (t == 1 || t == 5 ? 1 : 0); }
+
 // ---------------------------------------------------------------- the kernel
 // Under ADA_CROSS_CAUSAL a cross tile whose first (lowest) column token is not below the
 // tile's last row has no admissible (row, column) pair: every role skips it, so neither
@@ -251,7 +257,7 @@ struct GramMaps {
     CUtensorMap a[2], b[2], bw[2];
 };
 
-template <bool SHORTK>
+template <bool SHORTK, bool PLANES>
 __global__ void __launch_bounds__(Shape<SHORTK>::THREADS, 1)
 k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramProblem seg0,
           const __grid_constant__ GramProblem seg1, const int nseg,
@@ -482,13 +488,18 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
                     mbar_expect_tx(&sh.full[s], tx);
                     for (int u = 0; u < ksub; ++u) {          // K blocks past d are zero-filled
                         unsigned char* su = sa + u * subb;
-                        const int k0 = (kb * ksub + u) * BK;
+                        int k0 = (kb * ksub + u) * BK, kB = k0;
+                        if (PLANES) {                         // fp32: cross term `term` of plane block `blk`
+                            const int blk = (kb * ksub + u) / 6, term = (kb * ksub + u) % 6;
+                            k0 = plane_a(term) * p.planes + blk * BK;
+                            kB = plane_b(term) * p.planes + blk * BK;
+                        }
                         tma_load_3d(&maps.a[sg], &sh.full[s], su, k0, pc.row0, pc.b);
                         if (SHORTK && nbox == BN / BOX_N) {   // full-width tile: one 256-row box
-                            tma_load_3d(&maps.bw[sg], &sh.full[s], su + A_BYTES, k0, pc.col0, pc.b);
+                            tma_load_3d(&maps.bw[sg], &sh.full[s], su + A_BYTES, kB, pc.col0, pc.b);
                         } else {
                             for (int j = 0; j < nbox; ++j)
-                                tma_load_3d(&maps.b[sg], &sh.full[s], su + A_BYTES + j * BOX_BYTES, k0,
+                                tma_load_3d(&maps.b[sg], &sh.full[s], su + A_BYTES + j * BOX_BYTES, kB,
                                             pc.col0 + j * BOX_N, pc.b);
                         }
                     }
@@ -640,9 +651,11 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
             // this thread's row: its role and inverse norm are fetched while the MMAs finish
             const int row = pc.row0 + quad * 32 + lane;
             const bool row_live = row < pc.m;
-            const bool skip = row_live && !p.tri && p.row_role[o + row] != 0;   // inherited reps are not candidates
-            const bool inv_early = !(p.wait_norm_a && !norm_ok);
-            float inv_row = (row_live && inv_early) ? __ldcg(p.inv_a + o + row) : 0.f;
+            const bool defer = !p.tri && p.defer_row != 0;   // the row's own factor is applied later
+            // inherited reps are not candidates (with a deferred factor later kernels ignore them)
+            const bool skip = row_live && !p.tri && !defer && p.row_role[o + row] != 0;
+            const bool inv_early = defer || !(p.wait_norm_a && !norm_ok);
+            float inv_row = defer ? 1.0f : ((row_live && inv_early) ? __ldcg(p.inv_a + o + row) : 0.f);
             // warp-uniform outcome of the bounded wait
             const bool got = mbar_wait(&sh.tmem_full[acc], acc_ph, abort_flag, 4);
             if (!__all_sync(0xffffffffu, got)) break;
@@ -697,7 +710,7 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
             tcgen05_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh.tmem_empty[acc]);
-            if (p.wait_norm_a && !norm_ok) {
+            if (!inv_early && !norm_ok) {
                 if (!wait_counter(dep_ctr + 1, norm_total, lane, abort_flag, 9)) break;
                 norm_ok = true;
             }
@@ -770,15 +783,21 @@ cudaError_t launch_selftest_wait(ada_ctx* ctx, int limit_ms, cudaStream_t s) {
 }
 
 // tri and/or cross may be NULL.  With both, the cross epilogues wait inside the kernel for the
-// triangular segment (ctx->tile_ctr must be zero at launch) and the launch is cooperative.
+// triangular segment (ctx->tile_ctr must be zero at launch).
 cudaError_t launch_gram_tc(ada_ctx* ctx, const GramProblem* tri, const GramProblem* cross,
                            const NormJob* norms, cudaStream_t s) {
     if (!ctx->tc_attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_gram_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(k_gram_tc<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              smem_tc_bytes<true>());
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(k_gram_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 smem_tc_bytes<false>());
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_gram_tc<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     smem_tc_bytes<true>());
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_gram_tc<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     smem_tc_bytes<false>());
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_gram_tc<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     smem_tc_bytes<false>());
         if (e != cudaSuccess) return e;
         ctx->tc_attr_set = true;
     }
@@ -795,9 +814,10 @@ cudaError_t launch_gram_tc(ada_ctx* ctx, const GramProblem* tri, const GramProbl
         const int a_rows = p->tri ? n_cap : p->rows;
         if (n_cap <= 0 || a_rows <= 0) continue;
         // rows beyond the matrices (and k beyond d) are zero-filled by the TMA unit
-        if (!make_map(&maps.a[nseg], p->A, p->d, p->tri ? p->cap : p->rows, p->B, p->lda, p->a_batch, BM) ||
-            !make_map(&maps.b[nseg], p->Bm, p->d, p->cap, p->B, p->ldb, p->b_batch, BOX_N) ||
-            !make_map(&maps.bw[nseg], p->Bm, p->d, p->cap, p->B, p->ldb, p->b_batch, BN))
+        const int width = p->planes > 0 ? 3 * p->planes : p->d;
+        if (!make_map(&maps.a[nseg], p->A, width, p->tri ? p->cap : p->rows, p->B, p->lda, p->a_batch, BM) ||
+            !make_map(&maps.b[nseg], p->Bm, width, p->cap, p->B, p->ldb, p->b_batch, BOX_N) ||
+            !make_map(&maps.bw[nseg], p->Bm, width, p->cap, p->B, p->ldb, p->b_batch, BN))
             return cudaErrorInvalidValue;
         segs[nseg++] = *p;
     }
@@ -818,7 +838,8 @@ cudaError_t launch_gram_tc(ada_ctx* ctx, const GramProblem* tri, const GramProbl
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     int na = 0;
-    if (fused && ctx->cooperative) {
+    const bool coop = fused && coop_begin(ctx, s);
+    if (coop) {
         attr[na].id = cudaLaunchAttributeCooperative;
         attr[na].val.cooperative = 1;
         ++na;
@@ -830,10 +851,11 @@ cudaError_t launch_gram_tc(ada_ctx* ctx, const GramProblem* tri, const GramProbl
     }
     cfg.attrs = attr;
     cfg.numAttrs = na;
-    cudaError_t e = shortk ? cudaLaunchKernelEx(&cfg, k_gram_tc<true>, maps, segs[0], segs[1], nseg, nj,
-                                                ctx->tile_ctr, ctx->status)
-                           : cudaLaunchKernelEx(&cfg, k_gram_tc<false>, maps, segs[0], segs[1], nseg, nj,
-                                                ctx->tile_ctr, ctx->status);
+    const bool planes = segs[0].planes > 0;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, shortk ? (planes ? k_gram_tc<true, true> : k_gram_tc<true, false>)
+                                                    : (planes ? k_gram_tc<false, true> : k_gram_tc<false, false>),
+                                       maps, segs[0], segs[1], nseg, nj, ctx->tile_ctr, ctx->status);
+    if (fused) coop_end(ctx, coop);
     prof_end(ctx, s);
     return e;
 }

@@ -8,23 +8,30 @@
 //
 // Same contract as the one-CTA kernel (out[i] = max_j |a_i.b_j| inv_a[i] inv_b[j] over the
 // admissible j; Definition 1, Algorithm 1 lines 3-4 and 7-8; the Gram never leaves TMEM),
-// same tile list (triangular segment first, cross epilogues wait for it), same warp roles:
-//   warp 0      TMA producer in BOTH CTAs (completion bytes of both land on the leader's
-//               mbarrier; no multicast is used)
+// same order of tiles (triangular segment first, cross epilogues wait for it); ten warps:
+//   warp 0      plans the work (tile list, what is split along K), decodes the CTA's tiles into shared
+//               memory and then is the TMA producer, in BOTH CTAs (completion bytes of both land on
+//               the leader's mbarrier; no multicast is used)
 //   warp 1      leader: MMA issuer; releases ring stages and hands over accumulators with
 //               tcgen05.commit multicast to both CTAs.  Both CTAs: TMEM allocation
-//   warps 2..5  epilogue in both CTAs, each on its own 128 rows; the peer's epilogue
-//               returns the accumulator by a remote arrive on the leader's mbarrier
-//   warps 6..13 helpers.  Full selection: 1/||x_t|| of every row with plain loads, behind the
-//               main loops.  Cascade step: first the gather of Algorithm 1 lines 1-2 (list
-//               checked, role map, rows copied to Xrep with their inverse norms; loads of Xrep
-//               and the epilogues wait for it), then warps 6..9 take the row norms of X out of
-//               the left-operand tiles while those sit in shared memory (tiles of the first
-//               column tile only; one thread per row), so X is read from memory exactly once
+//   warps 2..9  first the preparation of a cascade step: Algorithm 1 lines 1-2 (list checked, role
+//               map, rows copied to Xrep with their inverse norms; fp32: the bf16 planes of
+//               every row), which loads and epilogues wait for; then the row norms of X with
+//               plain loads behind the first main loops (in the streaming form, warps 6..9, out of
+//               the left-operand tiles while those sit in shared memory, one thread per row,
+//               so that X is read from memory exactly once); then the epilogue, each CTA on its own
+//               128 rows, two warps per TMEM lane quadrant; the peer's returns the accumulator by
+//               a remote arrive on the leader's mbarrier
 // The cross segment's row maxima are published WITHOUT the factor 1/||x_t|| (it commutes with
 // the maximum; the compaction applies it), so no epilogue waits for a norm.  When one column
 // tile covers all representatives the step is bound by streaming X once: the row tiles are
 // then cut shorter than 128 rows per CTA so that every SM pair streams a share.
+//
+// What bounds a launch (in-kernel time stamps, one B200): 8-9 us until the first MMA of a cascade step
+// (preparation 4 us, arrival seen by every CTA 1.5 us, first copies 2-3 us, much of it instruction
+// fetch: with a layer's activations passing through L2 between launches the code is cold), 0.6 us per
+// 64 KB stage and SM in the main loop (L2 to SM), 2-3 us from the last accumulator to the
+// maxima, 3-5 us when a tile was split.
 // Every wait is bounded; the two CTAs meet at a cluster barrier before either frees TMEM
 // or exits.
 #include "gram_tc_dev.cuh"
@@ -44,11 +51,28 @@ __device__ unsigned long long g_trace[160 * 64];
 namespace {
 
 constexpr int PM = 2 * BM;     // rows of a pair tile
-// A ring stage holds KSUB consecutive 64-element K blocks (each its own 128-byte-swizzled
-// sub-tile), so that the per-stage costs -- barrier round trips, fences, commit -- are paid
-// once per 128 K elements and the MMA issue stays ahead of the tensor pipe.
-constexpr int KSUB = 2;
-constexpr int BKS = BK * KSUB; // K elements per stage
+// What a ring stage holds.  bf16 storage: two consecutive 64-element K blocks (each its own
+// 128-byte-swizzled sub-tile), so that the per-stage costs -- barrier round trips, fences,
+// commit -- are paid once per 128 K elements and the MMA issue stays ahead of the tensor pipe.
+// fp32 storage: the three bf16 planes (hi, mid, lo) of ONE 64-element K block, from which the six
+// leading cross terms are contracted: every plane is fetched once and used two or three times.
+// Its tiles are at most 128 columns wide so that three stages fit the ring.
+// Warps 2..9 do everything but copies and MMAs: preparation, row norms, epilogue.  (Twelve of them left
+// 128 registers a thread and an epilogue that spilled, which cost more than the warps gave.)
+constexpr int EPI_WARPS = 8;
+constexpr int SUBS = EPI_WARPS / 4;            // warps per TMEM lane quadrant
+constexpr int PAIR_THREADS = 64 + 32 * EPI_WARPS;
+template <bool SPLIT>
+struct Stage {
+    static constexpr int NSUB = SPLIT ? 3 : 2;
+    static constexpr int K = SPLIT ? BK : 2 * BK;          // K elements per stage
+    static constexpr int MAXW = SPLIT ? BN / 2 : BN;       // widest tile (columns of the pair)
+    static constexpr int TERMS = SPLIT ? 6 : 2;            // MMA groups per stage
+    static constexpr int CHUNKS = MAXW / 32 / SUBS;        // 32-column chunks of a tile per epilogue warp
+    // sub-tiles of A and B multiplied by group t
+    static __device__ __forceinline__ constexpr int ta(int t) { return SPLIT ? (t == 2 || t == 5 ? 1 : (t == 4 ? 2 : 0)) : t; }
+    static __device__ __forceinline__ constexpr int tb(int t) { return SPLIT ? (t == 1 || t == 5 ? 1 : (t == 3 ? 2 : 0)) : t; }
+};
 
 // ---------------------------------------------------------------- PTX, pair forms
 __device__ __forceinline__ unsigned cluster_rank() {
@@ -110,65 +134,87 @@ __device__ __forceinline__ unsigned instr_desc_pair(int n) {
 }
 
 // ---------------------------------------------------------------- tile list (256-row tiles)
-__device__ __forceinline__ int seq_n(const GramProblem& p, int b) {
+// a / b for 0 <= a, 0 < b and quotients below 2^20: a float quotient is off by at most one there, and an
+// integer division costs several times as much on the path to the first copy
+__device__ __forceinline__ int quot(int a, int b) {
+    int q = (int)__fdividef((float)a, (float)b);
+    const int r = a - q * b;
+    q += (r >= b) - (r < 0);
+    return q;
+}
+constexpr int PLAN_B = 64;      // sequences whose lengths are kept in shared memory
+// Work plan of a launch, made by one warp of every CTA.
+struct Plan {
+    int tiles0, total;          // triangular tiles; all tiles
+    int tw;                     // column width of the triangular tiles
+    int hrows;                  // rows of the left operand per CTA in cross tiles (128, or fewer: streaming form)
+    int one_col_tile, compact;
+    int full, rem, parts;       // tiles dealt whole; tiles of the last round, each cut into `parts` K ranges
+    int len[PLAN_B];            // sequence lengths (B <= PLAN_B)
+};
+__device__ __forceinline__ int seq_n_global(const GramProblem& p, int b) {
     int n = p.n_dev != nullptr ? p.n_dev[b] : p.n_host;
     if (p.n_clamp) n = min(max(n, 0), p.cap);
     return n;
 }
-__device__ __forceinline__ int tri_tiles(int n) {           // row pair P needs column tiles 0..P
-    const int M = (n + PM - 1) / PM;
-    return M * (M + 1) / 2;
+__device__ __forceinline__ int seq_n(const GramProblem& p, const Plan& pl, int b) {
+    return p.B <= PLAN_B ? pl.len[b] : seq_n_global(p, b);
 }
-// column tiles of a cross problem with n columns.  With in-launch norms (inv_out) a sequence
-// without columns still gets one (empty) column tile: its rows have to be read for their norms.
-__device__ __forceinline__ void cross_cols(const GramProblem& p, int n, int& nct, int& w) {
-    nct = (n + BN - 1) / BN;
+// lower triangle in column tiles of width tw (256 or 128): row pair P (256 rows) needs the columns below (P + 1) 256
+__device__ __forceinline__ int tri_tiles(int n, int tw) {
+    const int M = (n + PM - 1) / PM;
+    const int f = tw == PM ? 1 : 2;
+    return M > 0 ? f * (M * (M - 1) / 2) + (tw == PM ? M : (n + BM - 1) / BM) : 0;
+}
+// column tiles of a cross problem with n columns, at most maxw wide.  With in-launch norms (inv_out)
+// a sequence without columns still gets one (empty) column tile: its rows have to be read for
+// their norms.
+__device__ __forceinline__ void cross_cols(const GramProblem& p, int n, int maxw, int& nct, int& w) {
+    nct = (n + maxw - 1) / maxw;
     if (nct == 0 && p.inv_out != nullptr && n == 0) nct = 1;
-    w = nct > 0 ? max(32, (((n + nct - 1) / nct) + 31) & ~31) : 0;    // each CTA holds w/2 columns: keep w/2 a multiple of 16
+    w = nct > 0 ? max(32, (quot(n + nct - 1, nct) + 31) & ~31) : 0;    // each CTA holds w/2 columns: keep w/2 a multiple of 16
 }
 // rows of the cross segment's left operand for a sequence with n inherited tokens: all of
 // X, or only the tokens outside the inherited set when those were copied out (compact)
 __device__ __forceinline__ int cross_rows(const GramProblem& p, int n, bool compact) {
     return compact ? p.rows - n : p.rows;
 }
-// hrows: rows of the left operand per CTA in cross tiles (128, or fewer in the streaming form)
-__device__ __forceinline__ int seg_tiles(const GramProblem& p, int hrows, bool compact) {
-    int total = 0;
-    for (int b = 0; b < p.B; ++b) {
-        const int n = seq_n(p, b);
-        if (p.tri) { if (n > 0) total += tri_tiles(n); }
-        else {
-            int nct, w;
-            cross_cols(p, n, nct, w);
-            total += ((cross_rows(p, n, compact) + 2 * hrows - 1) / (2 * hrows)) * nct;
-        }
-    }
-    return total;
+__device__ __forceinline__ int seq_tiles(const GramProblem& p, int n, int maxw, int tw, int hrows, bool compact) {
+    if (p.tri) return tri_tiles(n, tw);
+    int nct, w;
+    cross_cols(p, n, maxw, nct, w);
+    return quot(cross_rows(p, n, compact) + 2 * hrows - 1, 2 * hrows) * nct;
 }
-__device__ __forceinline__ bool decode_tile(const GramProblem& p, int hrows, bool compact, int id, Piece& t) {
+template <bool SPLIT>
+__device__ __forceinline__ bool decode_tile(const GramProblem& p, const Plan& pl, int id, Piece& t) {
+    constexpr int MAXW = Stage<SPLIT>::MAXW;
+    const int hrows = pl.hrows, tw = pl.tw;
+    const bool compact = pl.compact != 0;
     for (int b = 0; b < p.B; ++b) {
-        const int n = seq_n(p, b);
-        int cnt = 0, nct = 0, w = 0;
-        if (p.tri) cnt = n > 0 ? tri_tiles(n) : 0;
-        else {
-            cross_cols(p, n, nct, w);
-            cnt = ((cross_rows(p, n, compact) + 2 * hrows - 1) / (2 * hrows)) * nct;
-        }
+        const int n = seq_n(p, pl, b);
+        const int cnt = seq_tiles(p, n, MAXW, tw, hrows, compact);
         if (id >= cnt) { id -= cnt; continue; }
         t.b = b;
         t.n = n;
         int nc;
         if (p.tri) {
-            int mi = (int)((sqrtf(8.0f * (float)id + 1.0f) - 1.0f) * 0.5f);
-            while (mi * (mi + 1) / 2 > id) --mi;
-            while ((mi + 1) * (mi + 2) / 2 <= id) ++mi;
+            const int f = tw == PM ? 1 : 2, M = (n + PM - 1) / PM;
+            int mi = M - 1;
+            if (id < f * (M * (M - 1) / 2)) {
+                mi = (int)((sqrtf(8.0f * (float)(f == 1 ? id : id >> 1) + 1.0f) - 1.0f) * 0.5f);
+                while (f * (mi * (mi + 1) / 2) > id) --mi;
+                while (f * ((mi + 1) * (mi + 2) / 2) <= id) ++mi;
+            }
             t.row0 = mi * PM;
-            t.col0 = (id - mi * (mi + 1) / 2) * BN;
+            t.col0 = (id - f * (mi * (mi + 1) / 2)) * tw;
             t.m = n;
-            nc = min(n - t.col0, BN);
+            nc = min(n - t.col0, tw);
         } else {
-            t.row0 = (id / nct) * 2 * hrows;
-            t.col0 = (id % nct) * w;
+            int nct, w;
+            cross_cols(p, n, MAXW, nct, w);
+            const int q = quot(id, nct);
+            t.row0 = q * 2 * hrows;
+            t.col0 = (id - q * nct) * w;
             t.m = cross_rows(p, n, compact);
             nc = min(n - t.col0, w);
         }
@@ -183,21 +229,15 @@ __device__ __forceinline__ int a_bytes_of(int hrows) { return (hrows * 128 + 102
 __device__ __forceinline__ int sub_bytes_pair(int a_bytes, int ncols) {
     return a_bytes + (((ncols >> 1) + BOX_N - 1) / BOX_N) * BOX_BYTES;
 }
-__device__ __forceinline__ int stage_count(int sbytes, int a_bytes) {
-    // the MMA reads 128 rows of A whatever was loaded: keep what it reads past a shorter tile
-    // inside the ring
-    return min(MAX_STAGES, (RING_BYTES - (A_BYTES - a_bytes)) / sbytes);
-}
-
 // Row norms of the cross segment's left operand (inv_out).  When one column tile covers all
 // columns every row tile is loaded exactly once and the launch is bound by streaming them: the
 // norms are then taken from the tiles in shared memory (`from_smem`; the stage release waits for
 // the readers, which costs nothing while the tensor pipe idles).  With several column tiles the
 // main loops are bound by the tensor pipe and by what an SM can draw from L2, a stage release
-// that waits for readers slows them, and the helper warps read the rows with plain loads
+// that waits for readers slows them, and warps 2..9 read the rows with plain loads
 // instead (X then stays resident in L2 between the column tiles anyway).
-__device__ __forceinline__ bool norm_duty(const GramProblem& p, const Piece& pc, bool from_smem) {
-    return from_smem && !p.tri && p.inv_out != nullptr && pc.col0 == 0;
+__device__ __forceinline__ bool norm_duty(const GramProblem& p, int col0, bool from_smem) {
+    return from_smem && !p.tri && p.inv_out != nullptr && col0 == 0;
 }
 // Under ADA_CROSS_CAUSAL a cross tile whose first (lowest) column token is not below the
 // tile's last row has no admissible (row, column) pair: every role skips it, so neither
@@ -205,18 +245,143 @@ __device__ __forceinline__ bool norm_duty(const GramProblem& p, const Piece& pc,
 // that has to yield row norms is never skipped.)
 __device__ __forceinline__ bool dead_tile(const GramProblem& p, const Piece& pc, int hrows, bool from_smem,
                                           bool compact) {
-    if (p.tri || !p.causal || p.col_token == nullptr || pc.n <= 0 || norm_duty(p, pc, from_smem)) return false;
+    if (p.tri || !p.causal || p.col_token == nullptr || pc.n <= 0 || norm_duty(p, pc.col0, from_smem)) return false;
     if (compact) return false;     // rows are compacted there: a row index is not a token index
     return p.col_token[(int64_t)pc.b * p.cap + pc.col0] >= pc.row0 + 2 * hrows;
 }
 
 struct GramMaps {
-    CUtensorMap a[2], b[2];
+    CUtensorMap a[2];        // left operand, 128-row boxes
+    CUtensorMap b[2], bt[2]; // right operand in 64-row boxes, and in 32-row boxes for a half-empty last one
     CUtensorMap ah;          // left operand of the cross segment in boxes of hb_rows rows
     CUtensorMap an;          // the rows outside a large inherited set (Xnon), 128-row boxes
 };
 
+// ---------------------------------------------------------------- work plan
+// Tiles are dealt round-robin to the pairs.  What does not fill a last round -- everything, in a
+// small problem -- is cut along K: each of its `rem` tiles goes to `parts` pairs, which exchange
+// partial accumulators through L2 (see the epilogue): a pair's share shrinks from the whole
+// chain to a part of it, and a wide tile split over K draws fewer bytes per SM than narrow tiles
+// would.  Measured: full selection at T = 2048, d = 4096 31.0 -> 26.1 us, at T = 512, d = 768 fp32 30.2 ->
+// 17.7 us, cascade steps at T = 2005, d = 4096 43 -> 31 us.
+// How many shares a tile may have.  The tensor core's accumulator truncates, so a sum over K comes out
+// too small, by about 3.6e-9 d of itself for bf16 storage (measured at d = 2600 and 4096; more past 4096,
+// where the sums of unit-variance rows enter the next binade) and by up to 8e-9 d for the six
+// terms of fp32 storage; cutting it in p shares takes 1 - 1/p of that away.  The same row must
+// not move by more than 1e-5 when the number of tiles around it changes, hence the limits:
+// measured shifts at them are 7.9e-6 (bf16, d = 3450, p = 3) and 8.6e-6 (fp32, d = 1600, p = 3).
+template <bool SPLIT>
+__device__ __forceinline__ bool shares_ok(int p, int d) { return (p - 1) * d <= (SPLIT ? MAX_SPLIT_D_F32 : MAX_SPLIT_D) / 2 * p; }
+template <bool SPLIT>
+__device__ __forceinline__ void make_plan(Plan& pl, const GramProblem& seg0, const GramProblem& seg1, int nseg,
+                                          const GatherJob& gather, int npairs, int max_parts, int lane) {
+    constexpr int MAXW = Stage<SPLIT>::MAXW;
+    const GramProblem& cx = nseg > 1 ? seg1 : seg0;
+    // both segments of a launch share the sequences: one read of every length
+    bool one = !cx.tri;
+    for (int b = lane; b < cx.B; b += 32) {
+        const int n = seq_n_global(cx, b);
+        if (b < PLAN_B) pl.len[b] = n;
+        one = one && n <= MAXW;
+    }
+    one = __all_sync(0xffffffffu, one);
+    // streaming form: one column tile covers the columns of every sequence and the rows are many,
+    // so the launch is one pass over the rows of A, and shorter row tiles put every pair to work.
+    // (Below 48 rows per CTA the right operand would be most of the traffic; splitting K is cheaper.)
+    const bool stream = !SPLIT && one && cx.hb_rows >= 48;
+    const int hrows = stream && cx.hb_rows < BM ? cx.hb_rows : BM;
+    const bool compact = !SPLIT && gather.X != nullptr && compact_wanted(gather, lane);
+    __syncwarp();
+    int t256 = 0, t128 = 0, tc = 0;                 // triangular tiles by width, cross tiles
+    for (int b = lane; b < cx.B; b += 32) {
+        const int n = cx.B <= PLAN_B ? pl.len[b] : seq_n_global(cx, b);
+        if (seg0.tri) { t256 += tri_tiles(n, PM); t128 += tri_tiles(n, BM); }
+        if (!cx.tri) tc += seq_tiles(cx, n, MAXW, PM, hrows, compact);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        t256 += __shfl_xor_sync(0xffffffffu, t256, o);
+        t128 += __shfl_xor_sync(0xffffffffu, t128, o);
+        tc += __shfl_xor_sync(0xffffffffu, tc, o);
+    }
+    // The number of shares, for both widths of the triangular tiles at once: lane 8 w + q asks whether
+    // q + 1 shares are possible with width w.  (Integer divisions are slow and the plan is on the
+    // path to the first copy.)
+    const int nst = ((SPLIT ? cx.planes : cx.d) + Stage<SPLIT>::K - 1) / Stage<SPLIT>::K;
+    const int cand = (lane & 8) ? t128 + tc : t256 + tc, q1 = (lane & 7) + 1;
+    const int rounds = quot(cand, npairs), rem = cand - rounds * npairs;
+    // the exchange costs about as much as six stages
+    const bool can = q1 == 1 || (!stream && q1 <= max_parts && shares_ok<SPLIT>(q1, cx.d) && rem > 0 && q1 * rem <= npairs && 2 * q1 <= nst &&
+                                 nst - quot(nst + q1 - 1, q1) >= 6);
+    const unsigned cans = __ballot_sync(0xffffffffu, can);
+    const int parts256 = 32 - __clz(cans & 0xffu), parts128 = 32 - __clz((cans >> 8) & 0xffu);
+    const int rounds256 = __shfl_sync(0xffffffffu, rounds + (rem > 0), 0), rounds128 = __shfl_sync(0xffffffffu, rounds + (rem > 0), 8);
+    // cross epilogues wait for the triangle: half-width triangular tiles are done earlier, where that
+    // costs neither a round nor a finer split
+    const bool narrow = SPLIT || (nseg > 1 && rounds128 == rounds256 && parts128 >= parts256);
+    const int the_rem = __shfl_sync(0xffffffffu, rem, narrow ? 8 : 0);
+    if (lane == 0) {
+        const int tiles0 = seg0.tri ? (narrow ? t128 : t256) : tc;
+        const int total = nseg > 1 ? tiles0 + tc : tiles0;
+        pl.tiles0 = tiles0; pl.total = total; pl.tw = narrow ? BM : PM; pl.hrows = hrows;
+        pl.one_col_tile = stream ? 1 : 0;
+        pl.compact = compact ? 1 : 0;
+        pl.parts = narrow ? parts128 : parts256;
+        pl.rem = pl.parts > 1 ? the_rem : 0;
+        pl.full = total - pl.rem;
+    }
+}
+// Work item of a pair: a tile, or one share of a split tile's contraction, with all that the roles need to
+// know about it.
+struct alignas(16) Item {
+    int row0, col0, ncols, b;   // ncols: multiple of 32
+    int n, m, st0, st1;         // columns of the sequence, row bound, K stages [st0, st1)
+    int kind;                   // 0: no more work, 1: tile, 2: nothing to do (dead tile)
+    int seg, part, parts;
+    int unit0;                  // first exchange slot of a split tile
+    int ring;                   // stages of the ring at this tile's stage size
+    int pad[2];
+};
+constexpr int ITEMS = 32;       // items decoded ahead, one per lane; later ones on the fly
+
+template <bool SPLIT> struct Ring { static constexpr int BYTES = (SPLIT ? 216 : 208) * 1024; };
+
+// Not inlined: the decoding is a few hundred instructions of integer arithmetic that would sit in
+// the path of every role; run once, by 32 lanes side by side, it is read from shared memory.
+template <bool SPLIT>
+__device__ __noinline__ void decode_item(const GramProblem* seg0, const GramProblem* seg1, const Plan& pl, int pair,
+                                         int npairs, int it, Item& w) {
+    const int at = pair + it * npairs;
+    int id = at, part = 0, parts = 1;
+    w.kind = 0;
+    if (at >= pl.full) {                            // pl.full is a multiple of npairs when anything is split
+        const int u = at - pl.full;
+        parts = pl.parts;
+        if (u >= pl.rem * parts) return;
+        const int tile = quot(u, parts);
+        id = pl.full + tile;
+        part = u - tile * parts;
+    }
+    const int sg = id < pl.tiles0 ? 0 : 1;
+    const GramProblem& p = sg ? *seg1 : *seg0;
+    Piece t;
+    if (!decode_tile<SPLIT>(p, pl, id - (sg ? pl.tiles0 : 0), t)) return;
+    const int nst = ((SPLIT ? p.planes : p.d) + Stage<SPLIT>::K - 1) / Stage<SPLIT>::K;
+    w.row0 = t.row0; w.col0 = t.col0; w.ncols = t.ncols; w.b = t.b; w.n = t.n; w.m = t.m;
+    w.st0 = 0; w.st1 = nst;
+    if (parts > 1) { w.st0 = quot(nst * part, parts); w.st1 = quot(nst * (part + 1), parts); }
+    w.seg = sg; w.part = part; w.parts = parts; w.unit0 = (id - pl.full) * parts;
+    const int a_bytes = a_bytes_of(p.tri ? BM : pl.hrows);
+    // the MMA reads 128 rows of A whatever was loaded: what it reads past a shorter tile stays inside the ring
+    const int room = Ring<SPLIT>::BYTES - (A_BYTES - a_bytes), sb = Stage<SPLIT>::NSUB * sub_bytes_pair(a_bytes, t.ncols);
+    w.ring = 0;
+#pragma unroll
+    for (int q = 1; q <= MAX_STAGES; ++q) w.ring += q * sb <= room;
+    w.kind = dead_tile(p, t, pl.hrows, pl.one_col_tile != 0, pl.compact != 0) ? 2 : 1;
+}
+
 // ---------------------------------------------------------------- the kernel
+template <bool SPLIT>
 struct alignas(16) SharedPair {
     unsigned long long full[MAX_STAGES];
     unsigned long long empty[MAX_STAGES];
@@ -224,27 +389,81 @@ struct alignas(16) SharedPair {
     unsigned long long tmem_full[2];
     unsigned long long tmem_empty[2];
     unsigned long long drain;
+    unsigned long long planned;                // the work plan is in shared memory
+    // global counters seen complete by the CTA's one polling thread: preparation, row norms, triangle
+    unsigned long long prep_seen, norm_seen, dep_seen;
+    unsigned pub_cnt;                          // epilogue warps that have published their share of a triangular tile
     unsigned tmem_base;
     int abort_flag;
-    int tiles0, tiles1, hrows, one_col_tile, compact;
     unsigned norm_cnt[MAX_STAGES];             // norm warps done with a stage
-    // per epilogue warp, so that staging needs no barrier across warps
-    alignas(16) float col_scale[4][BN];
-    alignas(16) int col_token[4][BN];
+    Plan plan;
+    Item item[ITEMS];
+    // per epilogue warp (its own column chunks), so that staging needs no barrier across warps
+    alignas(16) float col_scale[EPI_WARPS][32 * Stage<SPLIT>::CHUNKS];
+    alignas(16) int col_token[EPI_WARPS][32 * Stage<SPLIT>::CHUNKS];
 };
-constexpr int SMEM_PAIR_BYTES = RING_BYTES + (int)sizeof(SharedPair) + 1024;
-static_assert(SMEM_PAIR_BYTES <= 227 * 1024, "shared memory budget");
-constexpr int SMEM_NORM_WARPS = 4;             // warps 6..9 read the A tiles
+template <bool SPLIT>
+constexpr int smem_pair_bytes() { return Ring<SPLIT>::BYTES + (int)sizeof(SharedPair<SPLIT>) + 1024; }
+static_assert(smem_pair_bytes<false>() <= 227 * 1024 && smem_pair_bytes<true>() <= 227 * 1024, "shared memory budget");
+constexpr int RING_NORM_WARPS = 4;             // warps 6..9 read the A tiles
+// partial accumulators: [tile][source part][CTA of the pair][32-column chunk][8 16-byte columns][128 rows]
+constexpr int CHUNK_WORDS = BM * 32;
+__device__ __forceinline__ int64_t chunk_at(int unit, int rank, int chunk) {
+    return (((int64_t)unit * 2 + rank) * (BN / 32) + chunk) * CHUNK_WORDS;
+}
 
-__global__ void __launch_bounds__(NUM_THREADS, 1)
+// Adds one thread's 32 partial sums at src (16-byte columns, BM apart) to r once they have arrived, and
+// marks the place empty again for the next launch.  An empty word holds a NaN pattern that no
+// sum can produce, so every word says for itself whether it is there: no fence, no flag and no
+// second round trip between the writer and the reader.
+constexpr unsigned EMPTY_WORD = 0xFFFFFFFFu;
+__device__ __forceinline__ void load_partials(const uint4* src, uint4 (&x)[8]) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+        asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(x[e].x), "=r"(x[e].y), "=r"(x[e].z), "=r"(x[e].w) : "l"(src + e * BM) : "memory");
+}
+__device__ __forceinline__ bool take_partials(uint4* src, uint4 (&x)[8], unsigned (&r)[32], volatile int* abort_flag) {
+    unsigned polls = 0;
+    unsigned long long t0 = 0;
+    while (true) {
+        bool there = true;
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            there = there && x[e].x != EMPTY_WORD && x[e].y != EMPTY_WORD && x[e].z != EMPTY_WORD && x[e].w != EMPTY_WORD;
+        if (there) break;
+        if ((++polls & 255u) == 0) {
+            if (*abort_flag != 0) return false;
+            const unsigned long long now = global_ns();
+            if (t0 == 0) t0 = now;
+            else if (now - t0 > WAIT_LIMIT_NS) { *abort_flag = 16; return false; }
+        }
+        load_partials(src, x);
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        r[4 * e] = __float_as_uint(__uint_as_float(r[4 * e]) + __uint_as_float(x[e].x));
+        r[4 * e + 1] = __float_as_uint(__uint_as_float(r[4 * e + 1]) + __uint_as_float(x[e].y));
+        r[4 * e + 2] = __float_as_uint(__uint_as_float(r[4 * e + 2]) + __uint_as_float(x[e].z));
+        r[4 * e + 3] = __float_as_uint(__uint_as_float(r[4 * e + 3]) + __uint_as_float(x[e].w));
+        __stcg(src + e * BM, make_uint4(EMPTY_WORD, EMPTY_WORD, EMPTY_WORD, EMPTY_WORD));
+    }
+    return true;
+}
+
+template <bool SPLIT>
+__global__ void __launch_bounds__(PAIR_THREADS, 1)
 k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramProblem seg0,
            const __grid_constant__ GramProblem seg1, const int nseg,
            const __grid_constant__ NormJob norms, const __grid_constant__ GatherJob gather,
+           const __grid_constant__ SplitJob split, const void* __restrict__ touch_base,
+           const size_t touch_bytes, const int max_parts, unsigned* __restrict__ part_buf,
            unsigned* __restrict__ dep_ctr, unsigned* __restrict__ status) {
+    using St = Stage<SPLIT>;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    SharedPair& sh = *reinterpret_cast<SharedPair*>(smem + RING_BYTES);
+    SharedPair<SPLIT>& sh = *reinterpret_cast<SharedPair<SPLIT>*>(smem + Ring<SPLIT>::BYTES);
     volatile int* abort_flag = &sh.abort_flag;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -260,9 +479,12 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(&sh.tmem_full[a], 1);
-            mbar_init(&sh.tmem_empty[a], 8);      // four epilogue warps in each CTA
+            mbar_init(&sh.tmem_empty[a], 2 * EPI_WARPS);     // the epilogue warps of both CTAs
         }
         mbar_init(&sh.drain, 1);
+        mbar_init(&sh.planned, 1);
+        mbar_init(&sh.prep_seen, 1); mbar_init(&sh.norm_seen, 1); mbar_init(&sh.dep_seen, 1);
+        sh.pub_cnt = 0u;
         sh.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -273,99 +495,120 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
-    // everything above is local to the CTA; from here on the predecessor's results are read
-    grid_dep_wait();
-    // (the compaction's blocks may take the SMs that fall idle first: they wait for this whole grid)
-    grid_dep_launch_next();
-    if (threadIdx.x == 0) TRACE(0);
-    if (threadIdx.x == 64) {
-        // streaming form: one column tile covers the columns of every sequence, so the launch is
-        // one pass over the rows of A and shorter row tiles put every pair to work
-        const GramProblem& cx = (nseg > 1) ? seg1 : seg0;
-        int hrows = BM;
-        bool one = !cx.tri;
-        if (one)
-            for (int b = 0; b < cx.B; ++b) one = one && seq_n(cx, b) <= BN;
-        if (one && cx.hb_rows > 0 && cx.hb_rows < BM) hrows = cx.hb_rows;
-        // a large inherited set (two fifths of the tokens or more, in every sequence) of a long
-        // sequence: the rows outside it are copied out by the gather and the cross tiles run over
-        // those only.  (Measured on the crossover sweep at r/T = 0.5: 1052 -> 699 us at T = 16384,
-        // 250 -> 217 us at T = 8192, but 87 -> 97 us at T = 4096, where the copy costs more than
-        // the saved tiles.)
-        bool compact = !cx.tri && !one && gather.X != nullptr && gather.Xnon != nullptr && cx.rows >= gather.compact_min_rows;
-        if (compact)
-            for (int b = 0; b < cx.B; ++b) compact = compact && 5 * (int64_t)seq_n(cx, b) >= 2 * (int64_t)cx.rows;
-        sh.hrows = hrows;
-        sh.one_col_tile = one ? 1 : 0;
-        sh.compact = compact ? 1 : 0;
-        sh.tiles0 = seg_tiles(seg0, hrows, compact);
-        sh.tiles1 = nseg > 1 ? seg_tiles(seg1, hrows, compact) : 0;
+    if (threadIdx.x == 32) {                         // descriptors are fetched before the first copy needs them
+        prefetch_map(&maps.a[0]); prefetch_map(&maps.b[0]); prefetch_map(&maps.bt[0]);
+        prefetch_map(&maps.a[1]); prefetch_map(&maps.b[1]); prefetch_map(&maps.bt[1]);
+        prefetch_map(&maps.ah); prefetch_map(&maps.an);
     }
+    if (warp == 13) touch(touch_base, touch_bytes, (int)blockIdx.x * 32 + lane, (int)gridDim.x * 32);
     tcgen05_fence_before();
     __syncthreads();
     cluster_sync_all();          // the peer's barriers exist before anything signals them
     tcgen05_fence_after();
     const unsigned tmem_base = sh.tmem_base;
-    const int tiles0 = sh.tiles0, total = sh.tiles0 + sh.tiles1;
-    const int hrows = sh.hrows;                          // rows per CTA of a cross tile
-    const bool smem_norms = sh.one_col_tile != 0;        // row norms out of the tiles in shared memory
-    const bool compact = sh.compact != 0;                // cross tiles over the copied-out rows (Xnon)
-    // the helper warps AND the epilogue warps (idle until the first tile is done) share the gather
-    constexpr int GATHER_WARPS = NORM_WARPS + 4;
-    const unsigned gather_total = (unsigned)(gridDim.x * GATHER_WARPS);
-    const bool has_gather = gather.X != nullptr;
-    Piece pc;
+    const bool has_prep = gather.X != nullptr || split.X != nullptr;
+    // everything above is local to the CTA; from here on the predecessor's results are read
+    grid_dep_wait();
+    // (the compaction's blocks may take the SMs that fall idle first: they wait for this whole grid)
+    grid_dep_launch_next();
+    if (threadIdx.x == 0) TRACE(0);
+    if (has_prep && warp >= 2) {
+        // ------------------------------------------------ preparation, by every warp that is idle at
+        // the start.  Items are dealt across the SMs first, so that a
+        // short list is read by all of them.  One arrival per CTA.
+        const int g = (warp - 2) * (int)gridDim.x + (int)blockIdx.x, nw = (int)gridDim.x * EPI_WARPS;
+        if (gather.X != nullptr) gather_rows(gather, g, nw, lane, status);
+        else split_rows(split, g, nw, lane, status);
+        // the rows just written are read by TMA (async proxy) from other CTAs
+        asm volatile("fence.proxy.async.global;" ::: "memory");
+        __threadfence();
+        asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
+        if (threadIdx.x == 64) {
+            __threadfence();
+            atomicAdd(dep_ctr + 3, 1u);
+            TRACE(2);
+        }
+    }
+    const unsigned prep_total = gridDim.x;
+    if (warp == 0) {
+        make_plan<SPLIT>(sh.plan, seg0, seg1, nseg, gather, npairs, max_parts, lane);
+        __syncwarp();
+        decode_item<SPLIT>(&seg0, &seg1, sh.plan, pair, npairs, lane, sh.item[lane]);
+        __syncwarp();
+        if (lane == 0) { __threadfence_block(); mbar_arrive(&sh.planned); }
+        __syncwarp();
+    }
+    // (a plan is always made, by warp 0 of the same CTA, which waits for nobody)
+    while (!mbar_try_long(&sh.planned, 0)) { }
+    const Plan& pl = sh.plan;
+    const int tiles0 = pl.tiles0;
+    const int hrows = pl.hrows;                          // rows per CTA of a cross tile
+    const bool smem_norms = pl.one_col_tile != 0;        // row norms out of the tiles in shared memory
+    const bool compact = pl.compact != 0;                // cross tiles over the copied-out rows (Xnon)
+    Item own;                                            // an item beyond the table
     if (threadIdx.x == 0) TRACE(1);
 
+    auto item_at = [&](int it) __attribute__((always_inline)) -> const Item& {
+        if (it < ITEMS) return sh.item[it];
+        decode_item<SPLIT>(&seg0, &seg1, pl, pair, npairs, it, own);
+        return own;
+    };
     if (warp == 0) {
         // ------------------------------------------------ TMA producer (both CTAs)
         if (lane == 0) {
             unsigned fills = 0, used = 0, ever = 0;
             int cur_sb = 0, cur_nst = 0, s = 0;
-            bool ok = true;
-            // the right operand (and the triangle's left operand) is the gathered copy
-            if (has_gather && total > 0) {
-                ok = wait_counter_1(dep_ctr + 3, gather_total, abort_flag, 12);
-                asm volatile("fence.proxy.async.global;" ::: "memory");
-            }
-            TRACE(3);
-            for (int id = pair; ok && id < total; id += npairs) {
-                const int sg = id < tiles0 ? 0 : 1;
+            bool ok = true, prep_ok = !has_prep;
+            for (int it = 0; ok; ++it) {
+                const Item& w = item_at(it);
+                if (w.kind == 0) break;
+                if (w.kind == 2) continue;
+                const int sg = w.seg;
                 const GramProblem& p = sg ? seg1 : seg0;
-                if (!decode_tile(p, hrows, compact, id - (sg ? tiles0 : 0), pc)) break;
-                if (dead_tile(p, pc, hrows, smem_norms, compact)) continue;   // causal cross tile with no admissible pair
-                const int num_kb = (p.d + BKS - 1) / BKS;
-                const int half = pc.ncols >> 1;
-                const int nbox = (half + BOX_N - 1) / BOX_N;
+                const int half = w.ncols >> 1, st0 = w.st0, st1 = w.st1, wb = w.b;
+                // whole 64-row boxes, and for the rest a 32- or a 64-row one
+                const int nbox = (half + BOX_N - 1) / BOX_N, rest = half % BOX_N;
+                const bool tail32 = rest != 0 && rest <= 32;
                 const int arows = p.tri ? BM : hrows;
                 const int a_bytes = a_bytes_of(arows);
-                const int subb = sub_bytes_pair(a_bytes, pc.ncols);
-                const int sb = KSUB * subb;
-                const unsigned tx = (unsigned)(KSUB * (arows * 128 + nbox * BOX_BYTES));
+                const int subb = sub_bytes_pair(a_bytes, w.ncols);
+                const int sb = St::NSUB * subb;
+                const unsigned tx = (unsigned)(St::NSUB * (arows * 128 + nbox * BOX_BYTES - (tail32 ? BOX_BYTES / 2 : 0)));
                 const CUtensorMap* amap = p.tri ? &maps.a[sg] : (compact ? &maps.an : (hrows != BM ? &maps.ah : &maps.a[sg]));
                 if (sb != cur_sb) {
                     for (int q = 0; q < cur_nst && ok; ++q)
                         if ((used >> q) & 1u)
                             ok = mbar_wait(&sh.empty[q], ((fills >> q) & 1u) ^ 1u, abort_flag, 6);
                     if (!ok) break;
-                    cur_sb = sb; cur_nst = stage_count(sb, a_bytes); s = 0; used = 0;
+                    cur_sb = sb; cur_nst = w.ring; s = 0; used = 0;
                 }
-                const int a_row = pc.row0 + (int)rank * arows;
-                const int b_row = pc.col0 + (int)rank * half;
-                for (int kb = 0; kb < num_kb; ++kb) {
+                const int a_row = w.row0 + (int)rank * arows;
+                const int b_row = w.col0 + (int)rank * half;
+                const int kstep = SPLIT ? p.planes : BK;          // from one sub-tile of a stage to the next
+                if (!prep_ok) {
+                    // the right operand (and the triangle's left operand) is made by the preparation;
+                    // all of the above is ready by the time that ends
+                    ok = wait_counter_1(dep_ctr + 3, prep_total, abort_flag, 12);
+                    mbar_arrive(&sh.prep_seen);
+                    asm volatile("fence.proxy.async.global;" ::: "memory");
+                    prep_ok = true;
+                    TRACE(3);
+                    if (!ok) break;
+                }
+                for (int st = st0; st < st1; ++st) {
                     if (!mbar_wait(&sh.empty[s], ((fills >> s) & 1u) ^ 1u, abort_flag, 1)) { ok = false; break; }
                     unsigned char* sa = smem + s * sb;
                     // the leader's barrier counts the bytes of both CTAs
                     if (rank == 0) mbar_expect_tx(&sh.full[s], 2u * tx);
-                    // K blocks past d are zero-filled by the TMA unit
+                    // K past the operand is zero-filled by the TMA unit (planes are padded with zeros)
 #pragma unroll
-                    for (int u = 0; u < KSUB; ++u) {
+                    for (int u = 0; u < St::NSUB; ++u) {
                         unsigned char* su = sa + u * subb;
-                        const int k0 = kb * BKS + u * BK;
-                        tma_load_3d_pair(amap, &sh.full[s], su, k0, a_row, pc.b);
+                        const int k0 = st * St::K + u * kstep;
+                        tma_load_3d_pair(amap, &sh.full[s], su, k0, a_row, wb);
                         for (int j = 0; j < nbox; ++j)
-                            tma_load_3d_pair(&maps.b[sg], &sh.full[s], su + a_bytes + j * BOX_BYTES, k0,
-                                             b_row + j * BOX_N, pc.b);
+                            tma_load_3d_pair(j == nbox - 1 && tail32 ? &maps.bt[sg] : &maps.b[sg], &sh.full[s],
+                                             su + a_bytes + j * BOX_BYTES, k0, b_row + j * BOX_N, wb);
                     }
                     fills ^= 1u << s; used |= 1u << s; ever |= 1u << s;
                     s = (s + 1 == cur_nst) ? 0 : s + 1;
@@ -387,35 +630,35 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
             unsigned uses = 0, tile_it = 0;
             int cur_sb = 0, cur_nst = 0, s = 0;
             bool ok = true;
-            for (int id = pair; ok && id < total; id += npairs) {
-                const int sg = id < tiles0 ? 0 : 1;
-                const GramProblem& p = sg ? seg1 : seg0;
-                if (!decode_tile(p, hrows, compact, id - (sg ? tiles0 : 0), pc)) break;
-                if (dead_tile(p, pc, hrows, smem_norms, compact)) continue;   // causal cross tile with no admissible pair
-                const int num_kb = (p.d + BKS - 1) / BKS;
+            for (int it = 0; ok; ++it) {
+                const Item& w = item_at(it);
+                if (w.kind == 0) break;
+                if (w.kind == 2) continue;
+                const GramProblem& p = w.seg ? seg1 : seg0;
+                const int st0 = w.st0, st1 = w.st1;
                 const int a_bytes = a_bytes_of(p.tri ? BM : hrows);
-                const int subb = sub_bytes_pair(a_bytes, pc.ncols);
-                const int sb = KSUB * subb;
-                if (sb != cur_sb) { cur_sb = sb; cur_nst = stage_count(sb, a_bytes); s = 0; }
-                const bool duty = norm_duty(p, pc, smem_norms);
+                const int subb = sub_bytes_pair(a_bytes, w.ncols);
+                const int sb = St::NSUB * subb;
+                if (sb != cur_sb) { cur_sb = sb; cur_nst = w.ring; s = 0; }
+                const bool duty = norm_duty(p, w.col0, smem_norms);
                 const unsigned acc = tile_it & 1u, acc_ph = (tile_it >> 1) & 1u;
                 ++tile_it;
                 if (!mbar_wait(&sh.tmem_empty[acc], acc_ph ^ 1u, abort_flag, 2)) { ok = false; break; }
                 tcgen05_fence_after();
-                const unsigned idesc = instr_desc_pair(pc.ncols);
+                const unsigned idesc = instr_desc_pair(w.ncols);
                 const unsigned d_tmem = tmem_base + acc * BN;
-                for (int kb = 0; kb < num_kb; ++kb) {
+                for (int st = st0; st < st1; ++st) {
                     if (!mbar_wait(&sh.full[s], (uses >> s) & 1u, abort_flag, 3)) { ok = false; break; }
-                    if (tile_it == 1 && kb == 0) TRACE(5);
+                    if (tile_it == 1 && st == st0) TRACE(5);
                     tcgen05_fence_after();
+                    const unsigned s_addr = smem_u32(smem + s * sb);
 #pragma unroll
-                    for (int u = 0; u < KSUB; ++u) {
-                        const unsigned a_addr = smem_u32(smem + s * sb + u * subb);
-                        const unsigned long long adesc = smem_desc_sw128(a_addr);
-                        const unsigned long long bdesc = smem_desc_sw128(a_addr + a_bytes);
+                    for (int t = 0; t < St::TERMS; ++t) {
+                        const unsigned long long adesc = smem_desc_sw128(s_addr + St::ta(t) * subb);
+                        const unsigned long long bdesc = smem_desc_sw128(s_addr + St::tb(t) * subb + a_bytes);
 #pragma unroll
                         for (int k = 0; k < BK / UMMA_K; ++k)
-                            umma_bf16_pair(d_tmem, adesc + 2 * k, bdesc + 2 * k, idesc, (kb | u | k) != 0);
+                            umma_bf16_pair(d_tmem, adesc + 2 * k, bdesc + 2 * k, idesc, ((st - st0) | t | k) != 0);
                     }
                     // both producers may refill this stage -- after the norm warps have read the
                     // A tiles, where those yield the row norms
@@ -433,89 +676,150 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                 if (global_ns() - t0 > WAIT_LIMIT_NS / 2) { *abort_flag = 8; break; }
             }
         }
-    } else if (warp < 6) {
-        // ------------------------------------------------ epilogue (warps 2..5, both CTAs)
-        const int quad = warp & 3;
+    } else {
+        // ------------------------------------------------ warps 2..13, both CTAs: row norms of X where
+        // the launch makes them, then the epilogue.  A warp reaches the TMEM lanes 32 (warp % 4)..;
+        // the two warps of a lane quadrant share a tile's 32-column chunks (sub, sub + 2, ..), so
+        // that a finished accumulator is read out by eight warps.
+        const int quad = warp & 3, sub = (warp - 2) >> 2;
+        constexpr int NK = St::CHUNKS;
         float* cs = sh.col_scale[warp - 2];
         int* ct = sh.col_token[warp - 2];
-        const unsigned dep_total = 8u * (unsigned)tiles0;
+        const GramProblem& cx = (nseg > 1) ? seg1 : seg0;
+        if (norms.X != nullptr) {         // full selection: row norms with plain loads
+            norm_rows(norms, blockIdx.x * EPI_WARPS + (warp - 2), gridDim.x * EPI_WARPS, lane, dep_ctr + 1, status);
+        } else if (!cx.tri && cx.inv_out != nullptr && !smem_norms && !compact) {
+            // several column tiles: 1/||x_t|| of every row with plain loads, behind the first main loops
+            // (nothing in this launch waits for them: the row factor is applied by the compaction)
+            NormJob nj;
+            nj.X = cx.A; nj.ldx = cx.lda; nj.n_rows = (int64_t)cx.B * cx.rows; nj.d = cx.d;
+            nj.inv_norm = cx.inv_out;
+            nj.batch = cx.a_batch; nj.rows_per_seq = cx.rows;
+            norm_rows(nj, blockIdx.x * EPI_WARPS + (warp - 2), gridDim.x * EPI_WARPS, lane, dep_ctr + 1, status);
+        }
+        // row norms out of the A tiles in shared memory (streaming form): warps 6..9, thread lrow owns
+        // row lrow of the CTA's tile and follows the ring exactly as the producer fills it
+        const bool ring_norms = smem_norms && sub == 1 && !cx.tri && cx.inv_out != nullptr;
+        unsigned cons = 0;
+        int ring_sb = 0, ring_nst = 0, ring_s = 0;
+        // every share of a triangular tile is published once by both CTAs
+        const unsigned dep_total = 2u * (unsigned)(min(tiles0, pl.full) + max(tiles0 - pl.full, 0) * pl.parts);
         bool dep_ok = !(nseg > 1 && tiles0 > 0);
         bool norm_ok = norms.X == nullptr;           // row norms computed by this launch's norm warps
-        bool gather_ok = !has_gather;
-        const unsigned norm_total = (unsigned)(gridDim.x * NORM_WARPS);
-        if (has_gather)               // Algorithm 1 lines 1-2, shared with the helper warps
-            gather_rows(gather, blockIdx.x * GATHER_WARPS + NORM_WARPS + (warp - 2), gridDim.x * GATHER_WARPS,
-                        lane, dep_ctr + 3, status, compact);
+        bool prep_ok = !has_prep;
+        const unsigned norm_total = (unsigned)(gridDim.x * EPI_WARPS);
         // the accumulator goes back to the leader's barrier
         const unsigned empty_addr[2] = {map_to_cta(smem_u32(&sh.tmem_empty[0]), 0),
                                         map_to_cta(smem_u32(&sh.tmem_empty[1]), 0)};
+        // Wait for a counter of the whole grid.  One thread per CTA polls it and the other warps wait in
+        // shared memory: with every warp polling, the polls alone saturate the counter's L2 slice
+        // and delay the very arrivals that they wait for (up to 9 us before the cross epilogues).
+        auto await = [&](const unsigned* ctr, unsigned target, unsigned long long* seen, int where)
+                         __attribute__((always_inline)) -> bool {
+            if (warp == 2) {
+                const bool good = wait_counter(ctr, target, lane, abort_flag, where);
+                if (lane == 0) mbar_arrive(seen);
+                return good;
+            }
+            return __all_sync(0xffffffffu, mbar_wait(seen, 0, abort_flag, where)) && *abort_flag == 0;
+        };
         unsigned tile_it = 0;
-        for (int id = pair; id < total; id += npairs) {
-            const int sg = id < tiles0 ? 0 : 1;
+        for (int it = 0;; ++it) {
+            const Item& w = item_at(it);
+            if (w.kind == 0) break;
+            if (w.kind == 2) continue;
+            const int sg = w.seg, col0 = w.col0, ncols = w.ncols, row0 = w.row0;
             const GramProblem& p = sg ? seg1 : seg0;
-            if (!decode_tile(p, hrows, compact, id - (sg ? tiles0 : 0), pc)) break;
-            if (dead_tile(p, pc, hrows, smem_norms, compact)) continue;   // causal cross tile with no admissible pair
             const unsigned acc = tile_it & 1u, acc_ph = (tile_it >> 1) & 1u;
             ++tile_it;
-            const int64_t o = (int64_t)pc.b * p.cap;
-            const int ncols = pc.ncols;
-            if (!gather_ok) {
-                // the gathered rows' inverse norms (column factors, and the triangle's row factors)
-                if (!wait_counter(dep_ctr + 3, gather_total, lane, abort_flag, 13)) break;
-                gather_ok = true;
+            const int64_t o = (int64_t)w.b * p.cap;
+            const int nch = ncols >> 5;
+            const int arows = p.tri ? BM : hrows;
+            const int lrow = quad * 32 + lane;           // this thread's row of the CTA's share of the tile
+            const int row_base = row0 + (int)rank * arows;
+            const int row = row_base + lrow;
+            if (ring_norms) {
+                const int nst = w.st1;                   // (nothing is split in this form)
+                const int a_bytes = a_bytes_of(arows);
+                const int subb = sub_bytes_pair(a_bytes, ncols);
+                const int sb = St::NSUB * subb;
+                if (sb != ring_sb) { ring_sb = sb; ring_nst = w.ring; ring_s = 0; }
+                if (!norm_duty(p, col0, smem_norms)) {
+                    ring_s = (ring_s + nst) % ring_nst;
+                } else {
+                    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+                    bool ok = true;
+                    for (int st = 0; st < nst; ++st) {
+                        int good = 1;
+                        if (lane == 0) good = mbar_wait(&sh.consumed[ring_s], (cons >> ring_s) & 1u, abort_flag, 14) ? 1 : 0;
+                        if (__shfl_sync(0xffffffffu, good, 0) == 0) { ok = false; break; }
+                        if (lrow < arows) {
+#pragma unroll
+                            for (int u = 0; u < St::NSUB; ++u) {
+                                // the 16-byte chunks of a row are permuted by the swizzle, which a sum
+                                // of squares need not undo; lanes start at different chunks so that a
+                                // warp's loads spread over all banks
+                                const unsigned char* rowp = smem + ring_s * sb + u * subb + lrow * 128;
+                                uint4 x[8];
+#pragma unroll
+                                for (int j = 0; j < 8; ++j)
+                                    x[j] = *reinterpret_cast<const uint4*>(rowp + (((j + lane) & 7) << 4));
+                                s0 += sumsq_bf16x8(x[0]) + sumsq_bf16x8(x[4]);
+                                s1 += sumsq_bf16x8(x[1]) + sumsq_bf16x8(x[5]);
+                                s2 += sumsq_bf16x8(x[2]) + sumsq_bf16x8(x[6]);
+                                s3 += sumsq_bf16x8(x[3]) + sumsq_bf16x8(x[7]);
+                            }
+                        }
+                        __syncwarp();
+                        // the last of the four warps releases the stage to the producer
+                        if (lane == 0) {
+                            if (atomicAdd(&sh.norm_cnt[ring_s], 1u) == RING_NORM_WARPS - 1) {
+                                sh.norm_cnt[ring_s] = 0u;
+                                mbar_arrive(&sh.empty[ring_s]);
+                            }
+                        }
+                        cons ^= 1u << ring_s;
+                        ring_s = (ring_s + 1 == ring_nst) ? 0 : ring_s + 1;
+                    }
+                    if (!ok) break;
+                    if (lrow < arows && row < w.m) {
+                        const float ss = (s0 + s1) + (s2 + s3);
+                        float inv = 0.f;
+                        if (!(ss <= 3.0e38f)) atomicOr(status, ST_NONFINITE);
+                        else if (ss > 0.f) inv = 1.0f / sqrtf(ss);
+                        else atomicAdd(status + 1, 1u);
+                        p.inv_out[o + row] = inv;
+                    }
+                    if (lrow == 0) TRACE(40);
+                }
             }
-            if (sg == 1 && !dep_ok) {
-                // every triangular tile of this launch first (line 5 before line 7)
-                if (!wait_counter(dep_ctr, dep_total, lane, abort_flag, 5)) break;
-                dep_ok = true;
-                if (warp == 2 && lane == 0) TRACE(4);
+            if (!prep_ok) {
+                // the gathered rows' inverse norms (column factors, and the triangle's row factors)
+                if (!__all_sync(0xffffffffu, mbar_wait(&sh.prep_seen, 0, abort_flag, 13))) break;
+                prep_ok = true;
             }
             if (p.wait_norm_b && !norm_ok) {
-                if (!wait_counter(dep_ctr + 1, norm_total, lane, abort_flag, 9)) break;
+                if (!await(dep_ctr + 1, norm_total, &sh.norm_seen, 9)) break;
                 norm_ok = true;
             }
-            __syncwarp();
-            {
-                // all of the tile's global loads are issued before the first is used (columns
-                // past the tile are clamped to its last one and discarded afterwards, so that
-                // no load hangs on a data-dependent branch): eight dependent round trips to L2
-                // would otherwise sit on the path from a finished accumulator to its maxima
-                float fb[BN / 32];
-                unsigned gate[BN / 32] = {};
-                int tk[BN / 32] = {};
-                const int last = max(pc.n - 1, 0);
-                const unsigned thr_b = (!p.tri && p.tau_seq != nullptr) ? __float_as_uint(tau_threshold(p.tau_seq[pc.b])) : p.thr_bits;
+            // all of the tile's global loads are issued before the first is used (columns past the
+            // tile are clamped to its last one and discarded afterwards, so that no load hangs
+            // on a data-dependent branch), and what does not depend on line 5 before that is
+            // waited for: the path from the triangle's verdict to the maxima is one round trip
+            float fb[NK];
+            unsigned gate[NK] = {};
+            int tk[NK] = {};
+            const int last = max(w.n - 1, 0);
 #pragma unroll
-                for (int q = 0; q < BN / 32; ++q)
-                    fb[q] = __ldcg(p.inv_b + o + min(pc.col0 + lane + 32 * q, last));
-                if (!p.tri) {
-                    // representative removed at line 5 (written earlier in this launch: read at L2)
+            for (int k = 0; k < NK; ++k)
+                fb[k] = __ldcg(p.inv_b + o + min(col0 + 32 * (sub + SUBS * k) + lane, last));
+            if (!p.tri && p.causal) {
 #pragma unroll
-                    for (int q = 0; q < BN / 32; ++q)
-                        gate[q] = __ldcg(p.col_gate + o + min(pc.col0 + lane + 32 * q, last));
-                }
-                if (!p.tri && p.causal) {
-#pragma unroll
-                    for (int q = 0; q < BN / 32; ++q)
-                        tk[q] = p.col_token[o + min(pc.col0 + lane + 32 * q, last)];
-                }
-#pragma unroll
-                for (int q = 0; q < BN / 32; ++q) {
-                    const int c = lane + 32 * q, col = pc.col0 + c;
-                    const bool live = col < pc.n;
-                    if (c < ncols) {
-                        cs[c] = (live && (p.tri || gate[q] < thr_b)) ? fb[q] : 0.f;
-                        ct[c] = (live && !p.tri && p.causal) ? tk[q] : col;
-                    }
-                }
+                for (int k = 0; k < NK; ++k)
+                    tk[k] = __ldcg(p.col_token + o + min(col0 + 32 * (sub + SUBS * k) + lane, last));
             }
-            __syncwarp();
-            // this thread's row: its role and inverse norm are fetched while the MMAs finish
-            const int arows = p.tri ? BM : hrows;
-            const int lrow = quad * 32 + lane;
-            const int row_base = pc.row0 + (int)rank * arows;
-            const int row = row_base + lrow;
-            bool row_live = lrow < arows && row < pc.m;
+            const unsigned thr_b = (!p.tri && p.tau_seq != nullptr) ? __float_as_uint(tau_threshold(__ldcg(p.tau_seq + w.b))) : p.thr_bits;
+            bool row_live = lrow < arows && row < w.m;
             // the token this row belongs to: the row index itself, except over the copied-out rows
             // (an entry the gather did not write -- possible only with a rejected list -- is
             // never used as an index)
@@ -527,138 +831,161 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
             const bool defer = !p.tri && p.defer_row != 0;   // the row's own factor is applied later
             // inherited reps are not candidates (with a deferred factor the compaction ignores them)
             const bool skip = row_live && !p.tri && !defer && p.row_role[o + row] != 0;
-            const bool inv_early = !(p.wait_norm_a && !norm_ok);
+            const bool inv_early = defer || !(p.wait_norm_a && !norm_ok);
             float inv_row = defer ? 1.0f : ((row_live && inv_early) ? __ldcg(p.inv_a + o + row) : 0.f);
+            if (sg == 1 && !dep_ok) {
+                // every triangular tile of this launch first (line 5 before line 7)
+                if (!await(dep_ctr, dep_total, &sh.dep_seen, 5)) break;
+                dep_ok = true;
+                if (warp == 2 && lane == 0) TRACE(4);
+            }
+            if (!p.tri) {
+                // representative removed at line 5 (written earlier in this launch: read at L2)
+#pragma unroll
+                for (int k = 0; k < NK; ++k)
+                    gate[k] = __ldcg(p.col_gate + o + min(col0 + 32 * (sub + SUBS * k) + lane, last));
+            }
+            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < NK; ++k) {
+                const int col = col0 + 32 * (sub + SUBS * k) + lane;
+                const bool live = col < w.n;
+                cs[k * 32 + lane] = (live && (p.tri || gate[k] < thr_b)) ? fb[k] : 0.f;
+                ct[k * 32 + lane] = (live && !p.tri && p.causal) ? tk[k] : col;
+            }
+            __syncwarp();
             const bool got = mbar_wait(&sh.tmem_full[acc], acc_ph, abort_flag, 4);
             if (!__all_sync(0xffffffffu, got)) break;
             tcgen05_fence_after();
-            const bool need_cmp = p.tri ? (pc.col0 + ncols > row_base) : (p.causal != 0);
-            float mx = 0.f;
-            // (a warp whose 32 rows lie past a short tile's rows still joins the aligned loads)
-            for (int c0 = 0; c0 < ncols; c0 += 32) {
-                float v[32];
-                tmem_ld32(tmem_base + ((unsigned)(quad * 32) << 16) + acc * BN + c0, v);
-                if (!need_cmp) {
+            const bool need_cmp = p.tri ? (col0 + ncols > row_base) : (p.causal != 0);
+            const bool want_arg = p.out_arg != nullptr;
+            float mx0 = 0.f, mx1 = 0.f;
+            int arg = 0;                                     // nearest-representative mode: column of the maximum
+            // 32 columns of this thread's row, the warp's k-th chunk
+            auto consume = [&](const unsigned (&r)[32], int k) __attribute__((always_inline)) {
+                const float* csk = cs + k * 32;
+                if (want_arg) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) {           // ascending columns, strict '>': lowest index on ties
+                        const float x = fabsf(__uint_as_float(r[j])) * csk[j];
+                        if (x > mx0) { mx0 = x; arg = 32 * (sub + SUBS * k) + j; }
+                    }
+                } else if (!need_cmp) {
 #pragma unroll
                     for (int j = 0; j < 32; j += 4) {
-                        const float4 f = *reinterpret_cast<const float4*>(cs + c0 + j);
-                        mx = fmaxf(mx, fabsf(v[j]) * f.x);
-                        mx = fmaxf(mx, fabsf(v[j + 1]) * f.y);
-                        mx = fmaxf(mx, fabsf(v[j + 2]) * f.z);
-                        mx = fmaxf(mx, fabsf(v[j + 3]) * f.w);
+                        const float4 f = *reinterpret_cast<const float4*>(csk + j);
+                        mx0 = fmaxf(mx0, fabsf(__uint_as_float(r[j])) * f.x);
+                        mx1 = fmaxf(mx1, fabsf(__uint_as_float(r[j + 1])) * f.y);
+                        mx0 = fmaxf(mx0, fabsf(__uint_as_float(r[j + 2])) * f.z);
+                        mx1 = fmaxf(mx1, fabsf(__uint_as_float(r[j + 3])) * f.w);
                     }
                 } else {
+                    const int* ctk = ct + k * 32;
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const float x = fabsf(v[j]) * cs[c0 + j];
-                        if (ct[c0 + j] < tokrow) mx = fmaxf(mx, x);
+                    for (int j = 0; j < 32; j += 4) {
+                        const float4 f = *reinterpret_cast<const float4*>(csk + j);
+                        const int4 t = *reinterpret_cast<const int4*>(ctk + j);
+                        if (t.x < tokrow) mx0 = fmaxf(mx0, fabsf(__uint_as_float(r[j])) * f.x);
+                        if (t.y < tokrow) mx1 = fmaxf(mx1, fabsf(__uint_as_float(r[j + 1])) * f.y);
+                        if (t.z < tokrow) mx0 = fmaxf(mx0, fabsf(__uint_as_float(r[j + 2])) * f.z);
+                        if (t.w < tokrow) mx1 = fmaxf(mx1, fabsf(__uint_as_float(r[j + 3])) * f.w);
                     }
                 }
+            };
+            // (a warp whose 32 rows lie past a short tile's rows still joins the aligned loads)
+            const unsigned tbase = tmem_base + ((unsigned)(quad * 32) << 16) + acc * BN + sub * 32;   // the warp's chunk k: + 32 SUBS k
+            if (w.parts == 1) {
+                // (rolled loops: the code of an epilogue is fetched cold in most launches)
+#pragma unroll 1
+                for (int k = 0; sub + SUBS * k < nch; ++k) {
+                    unsigned r0[32];
+                    tmem_ld32_issue(tbase + 32 * SUBS * k, r0);
+                    tmem_ld_wait(r0);
+                    consume(r0, k);
+                }
+            } else {
+                // A share of the contraction.  The tile's chunks are divided among its shares: each
+                // writes its partial sums of the others' chunks to the exchange buffer (a row per
+                // thread, 16-byte columns outermost: coalesced both ways) and adds the others' to its
+                // own chunks in a fixed order.
+                const int unit0 = w.unit0;
+                const int own0 = nch * w.part / w.parts, own1 = nch * (w.part + 1) / w.parts;
+                bool mine = false;
+#pragma unroll 1
+                for (int k = 0; k < NK; ++k) {
+                    const int c = sub + SUBS * k;
+                    if (c >= nch) break;
+                    if (c >= own0 && c < own1) { mine = true; continue; }
+                    unsigned r0[32];
+                    tmem_ld32_issue(tbase + 32 * SUBS * k, r0);
+                    tmem_ld_wait(r0);
+                    uint4* dst = reinterpret_cast<uint4*>(part_buf + chunk_at(unit0 + w.part, rank, c)) + lrow;
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) r0[j] = r0[j] == EMPTY_WORD ? 0x7FFFFFFFu : r0[j];   // another NaN
+#pragma unroll
+                    for (int q = 0; q < 8; ++q)
+                        __stcg(dst + q * BM, make_uint4(r0[4 * q], r0[4 * q + 1], r0[4 * q + 2], r0[4 * q + 3]));
+                }
+                if (mine) {
+                    bool good = true;
+#pragma unroll 1
+                    for (int k = 0; k < NK; ++k) {
+                        const int c = sub + SUBS * k;
+                        if (c < own0 || c >= own1) continue;
+                        uint4* const src = reinterpret_cast<uint4*>(part_buf + chunk_at(w.unit0, rank, c)) + lrow;
+                        constexpr int STEP = 2 * (BN / 32) * CHUNK_WORDS / 4;        // from one share's slot to the next
+                        unsigned r0[32];
+                        tmem_ld32_issue(tbase + 32 * SUBS * k, r0);
+                        // (two shares' loads in flight)
+                        uint4 x0[8], x1[8];
+                        int q = w.part == 0 ? 1 : 0;
+                        load_partials(src + q * STEP, x0);
+                        tmem_ld_wait(r0);
+                        while (q < w.parts) {
+                            int q2 = q + 1 + (q + 1 == w.part);
+                            if (q2 < w.parts) load_partials(src + q2 * STEP, x1);
+                            good = take_partials(src + q * STEP, x0, r0, abort_flag) && good;
+                            if (q2 >= w.parts) break;
+                            q = q2 + 1 + (q2 + 1 == w.part);
+                            if (q < w.parts) load_partials(src + q * STEP, x0);
+                            good = take_partials(src + q2 * STEP, x1, r0, abort_flag) && good;
+                        }
+                        consume(r0, k);
+                    }
+                    if (!__all_sync(0xffffffffu, good)) break;
+                }
             }
+            float mx = fmaxf(mx0, mx1);
             tcgen05_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_remote(empty_addr[acc]);
-            if (!defer && p.wait_norm_a && !norm_ok) {
-                if (!wait_counter(dep_ctr + 1, norm_total, lane, abort_flag, 9)) break;
+            // (a share is its pair's last item: nobody waits for its accumulator, and the arrive would
+            // first wait for the stores above)
+            if (lane == 0 && w.parts == 1) mbar_arrive_remote(empty_addr[acc]);
+            if (!inv_early && !norm_ok) {
+                if (!await(dep_ctr + 1, norm_total, &sh.norm_seen, 9)) break;
                 norm_ok = true;
             }
-            if (row_live) {
-                if (!skip) {
-                    if (!defer && !inv_early) inv_row = __ldcg(p.inv_a + o + row);
-                    mx *= inv_row;
-                    if (mx > 0.f) atomicMax(p.out + o + tokrow, __float_as_uint(mx));
+            if (row_live && !skip) {
+                if (!inv_early) inv_row = __ldcg(p.inv_a + o + row);
+                mx *= inv_row;
+                if (mx > 0.f) {
+                    if (want_arg)
+                        atomicMax(p.out_arg + o + tokrow, ((unsigned long long)__float_as_uint(mx) << 32) |
+                                                              (unsigned long long)(0xFFFFFFFFu - (unsigned)(col0 + arg)));
+                    else
+                        atomicMax(p.out + o + tokrow, __float_as_uint(mx));
                 }
             }
             if (sg == 0 && nseg > 1) {
+                // publish: one arrival per CTA and tile, by the last of its warps
                 __threadfence();
                 __syncwarp();
-                if (lane == 0) atomicAdd(dep_ctr, 1u);
+                if (lane == 0 && atomicAdd(&sh.pub_cnt, 1u) % EPI_WARPS == EPI_WARPS - 1) {
+                    __threadfence();
+                    atomicAdd(dep_ctr, 1u);
+                }
             }
             if (warp == 2 && lane == 0) TRACE(9 + 2 * (int)min(tile_it - 1, 8u));
-        }
-    } else {
-        // ------------------------------------------------ helper warps (6 and up)
-        if (norms.X != nullptr)       // full selection: row norms with plain loads
-            norm_rows(norms, blockIdx.x * NORM_WARPS + (warp - 6), gridDim.x * NORM_WARPS, lane,
-                      dep_ctr + 1, status);
-        if (has_gather)               // Algorithm 1 lines 1-2
-            gather_rows(gather, blockIdx.x * GATHER_WARPS + (warp - 6), gridDim.x * GATHER_WARPS, lane,
-                        dep_ctr + 3, status, compact);
-        if (warp == 6 && lane == 0) TRACE(2);
-        const GramProblem& cx = (nseg > 1) ? seg1 : seg0;
-        if (!cx.tri && cx.inv_out != nullptr && !smem_norms && !compact) {
-            // several column tiles: 1/||x_t|| of every row with plain loads, behind the main loops
-            // (nothing in this launch waits for them: the row factor is applied by the compaction)
-            NormJob nj;
-            nj.X = cx.A; nj.ldx = cx.lda; nj.n_rows = (int64_t)cx.B * cx.rows; nj.d = cx.d;
-            nj.inv_norm = cx.inv_out;
-            nj.batch = cx.a_batch; nj.rows_per_seq = cx.rows;
-            norm_rows(nj, blockIdx.x * NORM_WARPS + (warp - 6), gridDim.x * NORM_WARPS, lane,
-                      dep_ctr + 1, status);
-        } else if (warp < 6 + SMEM_NORM_WARPS && !cx.tri && cx.inv_out != nullptr) {
-            // row norms of X out of the A tiles in shared memory: thread lrow owns row lrow of
-            // the CTA's tile; this role follows the ring exactly as the producer fills it
-            const int lrow = (warp - 6) * 32 + lane;
-            unsigned cons = 0;
-            int cur_sb = 0, cur_nst = 0, s = 0;
-            bool ok = true;
-            for (int id = pair; ok && id < total; id += npairs) {
-                const int sg = id < tiles0 ? 0 : 1;
-                const GramProblem& p = sg ? seg1 : seg0;
-                if (!decode_tile(p, hrows, compact, id - (sg ? tiles0 : 0), pc)) break;
-                if (dead_tile(p, pc, hrows, smem_norms, compact)) continue;
-                const int num_kb = (p.d + BKS - 1) / BKS;
-                const int arows = p.tri ? BM : hrows;
-                const int a_bytes = a_bytes_of(arows);
-                const int subb = sub_bytes_pair(a_bytes, pc.ncols);
-                const int sb = KSUB * subb;
-                if (sb != cur_sb) { cur_sb = sb; cur_nst = stage_count(sb, a_bytes); s = 0; }
-                if (!norm_duty(p, pc, smem_norms)) { s = (s + num_kb) % cur_nst; continue; }
-                float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-                for (int kb = 0; kb < num_kb; ++kb) {
-                    int good = 1;
-                    if (lane == 0) good = mbar_wait(&sh.consumed[s], (cons >> s) & 1u, abort_flag, 14) ? 1 : 0;
-                    if (__shfl_sync(0xffffffffu, good, 0) == 0) { ok = false; break; }
-                    if (lrow < arows) {
-#pragma unroll
-                        for (int u = 0; u < KSUB; ++u) {
-                            // the 16-byte chunks of a row are permuted by the swizzle, which a sum
-                            // of squares need not undo; lanes start at different chunks so that a
-                            // warp's loads spread over all banks
-                            const unsigned char* rowp = smem + s * sb + u * subb + lrow * 128;
-                            uint4 x[8];
-#pragma unroll
-                            for (int j = 0; j < 8; ++j)
-                                x[j] = *reinterpret_cast<const uint4*>(rowp + (((j + lane) & 7) << 4));
-                            s0 += sumsq_bf16x8(x[0]) + sumsq_bf16x8(x[4]);
-                            s1 += sumsq_bf16x8(x[1]) + sumsq_bf16x8(x[5]);
-                            s2 += sumsq_bf16x8(x[2]) + sumsq_bf16x8(x[6]);
-                            s3 += sumsq_bf16x8(x[3]) + sumsq_bf16x8(x[7]);
-                        }
-                    }
-                    __syncwarp();
-                    // the last of the four warps releases the stage to the producer
-                    if (lane == 0) {
-                        if (atomicAdd(&sh.norm_cnt[s], 1u) == SMEM_NORM_WARPS - 1) {
-                            sh.norm_cnt[s] = 0u;
-                            mbar_arrive(&sh.empty[s]);
-                        }
-                    }
-                    cons ^= 1u << s;
-                    s = (s + 1 == cur_nst) ? 0 : s + 1;
-                }
-                if (!ok) break;
-                const int row = pc.row0 + (int)rank * arows + lrow;
-                if (lrow < arows && row < pc.m) {
-                    const float ss = (s0 + s1) + (s2 + s3);
-                    float inv = 0.f;
-                    if (!(ss <= 3.0e38f)) atomicOr(status, ST_NONFINITE);
-                    else if (ss > 0.f) inv = 1.0f / sqrtf(ss);
-                    else atomicAdd(status + 1, 1u);
-                    p.inv_out[(int64_t)pc.b * p.cap + row] = inv;
-                }
-                if (lrow == 0) TRACE(40);
-            }
         }
     }
 
@@ -682,21 +1009,23 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
 
 static cudaError_t ensure_tc2(ada_ctx* ctx) {
     if (ctx->tc2_attr_set) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_gram_tc2, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         SMEM_PAIR_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(k_gram_tc2<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         smem_pair_bytes<false>());
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_gram_tc2<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_pair_bytes<true>());
     if (e != cudaSuccess) return e;
     // how many clusters of two fit on the device at once
     cudaLaunchConfig_t q;
     memset(&q, 0, sizeof(q));
     q.gridDim = dim3(2 * (ctx->sm_count / 2));
-    q.blockDim = dim3(NUM_THREADS);
-    q.dynamicSmemBytes = SMEM_PAIR_BYTES;
+    q.blockDim = dim3(PAIR_THREADS);
+    q.dynamicSmemBytes = smem_pair_bytes<false>();
     cudaLaunchAttribute qa[1];
     qa[0].id = cudaLaunchAttributeClusterDimension;
     qa[0].val.clusterDim.x = 2; qa[0].val.clusterDim.y = 1; qa[0].val.clusterDim.z = 1;
     q.attrs = qa; q.numAttrs = 1;
     int nclusters = 0;
-    e = cudaOccupancyMaxActiveClusters(&nclusters, k_gram_tc2, &q);
+    e = cudaOccupancyMaxActiveClusters(&nclusters, k_gram_tc2<false>, &q);
     if (e != cudaSuccess || nclusters < 1) { cudaGetLastError(); return cudaErrorLaunchOutOfResources; }
     ctx->tc2_pairs = nclusters < ctx->sm_count / 2 ? nclusters : ctx->sm_count / 2;
     ctx->tc2_attr_set = true;
@@ -720,7 +1049,8 @@ int gram_tc2_hb_rows(ada_ctx* ctx, int B, int T) {
 // Pair-CTA launch.  tri and/or cross may be NULL; with both the cross epilogues wait in-kernel
 // for the triangular segment (ctx->tile_ctr must be zero at launch).
 cudaError_t launch_gram_tc2(ada_ctx* ctx, const GramProblem* tri, const GramProblem* cross,
-                            const NormJob* norms, const GatherJob* gather, cudaStream_t s) {
+                            const NormJob* norms, const GatherJob* gather, const SplitJob* split,
+                            cudaStream_t s) {
     cudaError_t e0 = ensure_tc2(ctx);
     if (e0 != cudaSuccess) return e0;
     GramMaps maps;
@@ -735,21 +1065,23 @@ cudaError_t launch_gram_tc2(ada_ctx* ctx, const GramProblem* tri, const GramProb
         const int n_cap = p->n_dev != nullptr ? p->cap : p->n_host;
         const int a_rows = p->tri ? n_cap : p->rows;
         if (n_cap <= 0 || a_rows <= 0) continue;
-        if (!make_map(&maps.a[nseg], p->A, p->d, p->tri ? p->cap : p->rows, p->B, p->lda, p->a_batch, BM) ||
-            !make_map(&maps.b[nseg], p->Bm, p->d, p->cap, p->B, p->ldb, p->b_batch, BOX_N))
+        const int width = p->planes > 0 ? 3 * p->planes : p->d;
+        if (!make_map(&maps.a[nseg], p->A, width, p->tri ? p->cap : p->rows, p->B, p->lda, p->a_batch, BM) ||
+            !make_map(&maps.b[nseg], p->Bm, width, p->cap, p->B, p->ldb, p->b_batch, BOX_N) ||
+            !make_map(&maps.bt[nseg], p->Bm, width, p->cap, p->B, p->ldb, p->b_batch, BOX_N / 2))
             return cudaErrorInvalidValue;
-        if (!p->tri) {
-            const int hb = (p->hb_rows > 0 && p->hb_rows < BM) ? p->hb_rows : BM;
-            if (!make_map(&maps.ah, p->A, p->d, p->rows, p->B, p->lda, p->a_batch, hb))
+        if (!p->tri && p->hb_rows > 0 && p->hb_rows < BM) {
+            if (!make_map(&maps.ah, p->A, width, p->rows, p->B, p->lda, p->a_batch, p->hb_rows))
                 return cudaErrorInvalidValue;
+        } else {
+            maps.ah = maps.a[nseg];
         }
         segs[nseg++] = *p;
     }
     if (nseg == 0) return cudaSuccess;
-    if (nseg == 1) { maps.a[1] = maps.a[0]; maps.b[1] = maps.b[0]; segs[1] = segs[0]; segs[1].B = 0; }
-    if (segs[0].tri && nseg == 1) maps.ah = maps.a[0];
+    if (nseg == 1) { maps.a[1] = maps.a[0]; maps.b[1] = maps.b[0]; maps.bt[1] = maps.bt[0]; segs[1] = segs[0]; segs[1].B = 0; }
     maps.an = maps.ah;
-    if (gather != nullptr && gather->Xnon != nullptr && cross != nullptr &&
+    if (gather != nullptr && gather->Xnon != nullptr && cross != nullptr && gather->T >= gather->compact_min_rows &&
         !make_map(&maps.an, gather->Xnon, cross->d, cross->rows, cross->B, cross->d, (int64_t)cross->cap * cross->d, BM))
         return cudaErrorInvalidValue;
     NormJob nj;
@@ -758,22 +1090,46 @@ cudaError_t launch_gram_tc2(ada_ctx* ctx, const GramProblem* tri, const GramProb
     GatherJob gj;
     memset(&gj, 0, sizeof(gj));
     if (gather != nullptr) gj = *gather;
+    SplitJob sj;
+    memset(&sj, 0, sizeof(sj));
+    if (split != nullptr) sj = *split;
+    const bool planes = segs[0].planes > 0;
+    // the caller's activations: extent of what this call reads
+    const void* touch_base = segs[0].A;
+    size_t touch_bytes = (size_t)((segs[0].B - 1) * segs[0].a_batch + (int64_t)(segs[0].rows - 1) * segs[0].lda + segs[0].d) * 2;
+    if (gj.X != nullptr) {
+        touch_base = gj.X;
+        touch_bytes = (size_t)((gj.B - 1) * gj.xb + (int64_t)(gj.T - 1) * gj.ldx + gj.d) * 2;
+    } else if (sj.X != nullptr) {
+        touch_base = sj.X;
+        touch_bytes = (size_t)((sj.B - 1) * sj.xb + (int64_t)(sj.T - 1) * sj.ldx + sj.d) * 4;
+    }
+    int max_parts = ctx->part_buf != nullptr ? ctx->max_parts : 1;
+    if (nseg == 1 && segs[0].tri && segs[0].n_dev == nullptr) {
+        // tile count known here: a last round that is more than half full is not split, and the launch
+        // then need not be cooperative
+        const int M = (segs[0].n_host + PM - 1) / PM, f = planes ? 2 : 1;
+        const int64_t tiles = (int64_t)segs[0].B * (f * (M * (M - 1) / 2) + (segs[0].n_host + PM / f - 1) / (PM / f));
+        if (2 * (tiles % ctx->tc2_pairs) > ctx->tc2_pairs || tiles % ctx->tc2_pairs == 0) max_parts = 1;
+    }
     const bool fused = nseg == 2;
     prof_begin(ctx, fused ? K_GRAM_TC_CASCADE : (segs[0].tri ? K_GRAM_TC_TRI : K_GRAM_TC_CROSS), s);
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(2 * ctx->tc2_pairs);
-    cfg.blockDim = dim3(NUM_THREADS);
-    cfg.dynamicSmemBytes = SMEM_PAIR_BYTES;
+    cfg.blockDim = dim3(PAIR_THREADS);
+    cfg.dynamicSmemBytes = planes ? smem_pair_bytes<true>() : smem_pair_bytes<false>();
     cfg.stream = s;
     cudaLaunchAttribute attr[3];
     int na = 0;
     attr[na].id = cudaLaunchAttributeClusterDimension;
     attr[na].val.clusterDim.x = 2; attr[na].val.clusterDim.y = 1; attr[na].val.clusterDim.z = 1;
     ++na;
-    // CTAs wait on results of other CTAs (triangle before cross epilogues, the gather before
-    // everything): all of them have to be resident
-    if ((fused || gj.X != nullptr) && ctx->cooperative) {
+    // CTAs wait on results of other CTAs (triangle before cross epilogues, the preparation before
+    // everything, the other shares of a split tile): all of them have to get to run
+    const bool waits = fused || gj.X != nullptr || sj.X != nullptr || max_parts > 1;
+    const bool coop = waits && coop_begin(ctx, s);
+    if (coop) {
         attr[na].id = cudaLaunchAttributeCooperative;
         attr[na].val.cooperative = 1;
         ++na;
@@ -785,8 +1141,10 @@ cudaError_t launch_gram_tc2(ada_ctx* ctx, const GramProblem* tri, const GramProb
     }
     cfg.attrs = attr;
     cfg.numAttrs = na;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_gram_tc2, maps, segs[0], segs[1], nseg, nj, gj, ctx->tile_ctr,
+    cudaError_t e = cudaLaunchKernelEx(&cfg, planes ? k_gram_tc2<true> : k_gram_tc2<false>, maps, segs[0], segs[1],
+                                       nseg, nj, gj, sj, touch_base, touch_bytes, max_parts, ctx->part_buf, ctx->tile_ctr,
                                        ctx->status);
+    if (waits) coop_end(ctx, coop);
     prof_end(ctx, s);
     return e;
 }

@@ -23,7 +23,9 @@ static constexpr int BOX_BYTES = BOX_N * BK * 2;            // 8 KiB
 static constexpr int NORM_WARPS = 8;
 static constexpr int NUM_THREADS = 192 + 32 * NORM_WARPS;   // producer, MMA, 4 epilogue warps, norm warps
 static constexpr int TMEM_COLS = 512;
-static constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;   // 2 s
+// Limit of every wait: 20 s.  (Long, because the CTAs of a launch that is not cooperative may have to wait
+// for SMs that another stream's kernel still holds.)
+static constexpr unsigned long long WAIT_LIMIT_NS = 20000000000ull;
 
 // one output tile: `ncols` (multiple of 16, <= 256) columns from col0 of the 128-row tile at row0
 struct Piece {
@@ -89,15 +91,27 @@ static __device__ __forceinline__ unsigned long long global_ns() {
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
     return t;
 }
+// One try that suspends the thread for up to about 20 us: a waiting warp then costs neither issue slots
+// nor power (a dozen warps per SM polling through a 200 us main loop were measured to cost 3 %).
+static __device__ __forceinline__ bool mbar_try_long(unsigned long long* bar, unsigned parity) {
+    unsigned ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity), "r"(20000u)
+        : "memory");
+    return ok != 0;
+}
 // Bounded wait.  Returns false when the CTA is aborting (this or another wait ran out).
-// try_wait itself suspends the thread for a while before it reports failure, so the wall
-// clock (a slow special register) is consulted only once per 256 failed polls.
 static __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity,
                                           volatile int* abort_flag, int where) {
     unsigned polls = 0;
     unsigned long long t0 = 0;
-    while (!mbar_try(bar, parity)) {
-        if ((++polls & 255u) == 0) {
+    while (!mbar_try_long(bar, parity)) {
+        // (the wall clock is a slow special register)
+        if ((++polls & 15u) == 0) {
             if (*abort_flag != 0) return false;
             const unsigned long long now = global_ns();
             if (t0 == 0) t0 = now;
@@ -117,6 +131,17 @@ static __device__ __forceinline__ void tma_load_3d(const CUtensorMap* map, unsig
         ::"r"(smem_u32(dst)), "l"(reinterpret_cast<unsigned long long>(map)), "r"(smem_u32(bar)),
           "r"(c0), "r"(c1), "r"(c2)
         : "memory");
+}
+// One cache line in every 1/n of [base, base + bytes), thread i of n.  The first access to a page in a
+// long while costs several microseconds of address translation; touching the activations
+// as soon as a kernel starts takes that off the path of its first copies.
+static __device__ __forceinline__ void touch(const void* base, size_t bytes, int i, int n) {
+    const size_t at = bytes / (size_t)n * (size_t)i;
+    if (base != nullptr && at < bytes)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(base) + at));
+}
+static __device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<unsigned long long>(map)) : "memory");
 }
 static __device__ __forceinline__ void tcgen05_fence_before() {
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -341,11 +366,21 @@ static __device__ __forceinline__ bool wait_counter_1(const unsigned* counter, u
     }
 }
 
-// Algorithm 1 lines 1-2, by the helper warps of every CTA (warp `g` of `nw`): entry i of
-// sequence b is checked (in range, strictly above entry i-1), role[token] = i + 1, the raw row
-// goes to Xrep[b, i] and its inverse norm to inv_rep[b, i]; a rejected entry gets inverse norm
-// 0 (its column then counts for nothing) and raises the status.  Ends with one arrival per warp
-// on `counter`.
+// Is the complement of the inherited set copied out (below)?  Two fifths of the tokens or more in
+// every sequence of a long batch, and more than one column tile (256) in one of them.  (Measured on
+// the crossover sweep at r/T = 0.5: 1052 -> 699 us at T = 16384, 250 -> 217 us at T = 8192, but
+// 87 -> 97 us at T = 4096, where the copy costs more than the saved tiles.)
+static __device__ __forceinline__ bool compact_wanted(const GatherJob& gj, int lane) {
+    if (gj.Xnon == nullptr || gj.T < gj.compact_min_rows) return false;
+    bool one = true, big = true;
+    for (int b = lane; b < gj.B; b += 32) {
+        const int n = min(max(gj.rep_in_cnt[b], 0), gj.T);
+        one = one && n <= BN;
+        big = big && 5 * (int64_t)n >= 2 * (int64_t)gj.T;
+    }
+    return __all_sync(0xffffffffu, big) && !__all_sync(0xffffffffu, one);
+}
+
 // one warp: copy a row of nvec 16-byte vectors, return its sum of squares (all lanes)
 static __device__ __forceinline__ float copy_row_sumsq(const uint4* __restrict__ src, uint4* __restrict__ dst,
                                                        int nvec, int lane) {
@@ -374,8 +409,11 @@ static __device__ __forceinline__ float copy_row_sumsq(const uint4* __restrict__
 // between consecutive inherited tokens are copied, in order, to Xnon (row t goes to t minus the
 // number of inherited tokens before it), with their token index in non_tok and 1/||x_t|| in
 // inv_norm.  A warp takes one gap between two list entries at a time.
-static __device__ __forceinline__ void gather_rows(const GatherJob& gj, int g, int nw, int lane,
-                                            unsigned* counter, unsigned* status, bool compact) {
+// Algorithm 1 lines 1-2, by the preparation warps of all CTAs (warp `g` of `nw`): entry i of
+// sequence b is checked (in range, strictly above entry i-1), role[token] = i + 1, the raw row
+// goes to Xrep[b, i] and its inverse norm to inv_rep[b, i]; a rejected entry gets inverse norm
+// 0 (its column then counts for nothing) and raises the status.
+static __device__ __forceinline__ void gather_rows(const GatherJob& gj, int g, int nw, int lane, unsigned* status) {
     const __nv_bfloat16* X = reinterpret_cast<const __nv_bfloat16*>(gj.X);
     __nv_bfloat16* Xrep = reinterpret_cast<__nv_bfloat16*>(gj.Xrep);
     __nv_bfloat16* Xnon = reinterpret_cast<__nv_bfloat16*>(gj.Xnon);
@@ -389,6 +427,7 @@ static __device__ __forceinline__ void gather_rows(const GatherJob& gj, int g, i
         first_idx = __ldg(gj.rep_in + g);
         if (g > 0) first_prev = __ldg(gj.rep_in + g - 1);
     }
+    const bool compact = compact_wanted(gj, lane);
     while (b < gj.B) {
         int cnt = gj.rep_in_cnt[b];
         if (cnt < 0 || cnt > gj.T) {
@@ -441,11 +480,95 @@ static __device__ __forceinline__ void gather_rows(const GatherJob& gj, int g, i
             gj.role[(int64_t)b * gj.T + idx] = i + 1;
         }
     }
-    // the rows just written are read by TMA (async proxy) from other CTAs
-    asm volatile("fence.proxy.async.global;" ::: "memory");
-    __threadfence();
-    __syncwarp();
-    if (lane == 0) atomicAdd(counter, 1u);
+}
+
+// ---------------------------------------------------------------- fp32 rows as three bf16 planes
+static __device__ __forceinline__ void split3(float x, __nv_bfloat16& hi, __nv_bfloat16& mid, __nv_bfloat16& lo) {
+    hi = __float2bfloat16_rn(x);
+    const float r1 = x - __bfloat162float(hi);
+    mid = __float2bfloat16_rn(r1);
+    const float r2 = r1 - __bfloat162float(mid);
+    lo = __float2bfloat16_rn(r2);
+}
+// one warp: planes of one row (each `dpad` elements, zeros past d), its sum of squares (all lanes)
+static __device__ __forceinline__ float split_row(const float4* __restrict__ src, __nv_bfloat16* __restrict__ dst,
+                                                  int d, int dpad, int lane) {
+    float ss = 0.f;
+    const int nvec = d >> 2, nout = dpad >> 2;                // d is a multiple of 4
+    for (int v0 = lane; v0 < nout; v0 += 256) {
+        float4 x[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            x[q] = v0 + 32 * q < nvec ? __ldg(src + v0 + 32 * q) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int v = v0 + 32 * q;
+            if (v >= nout) break;
+            const float xs[4] = {x[q].x, x[q].y, x[q].z, x[q].w};
+            __align__(8) __nv_bfloat16 hi[4], mid[4], lo[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                ss = fmaf(xs[e], xs[e], ss);
+                split3(xs[e], hi[e], mid[e], lo[e]);
+            }
+            *reinterpret_cast<uint2*>(dst + v * 4) = *reinterpret_cast<const uint2*>(hi);
+            *reinterpret_cast<uint2*>(dst + dpad + v * 4) = *reinterpret_cast<const uint2*>(mid);
+            *reinterpret_cast<uint2*>(dst + 2 * dpad + v * 4) = *reinterpret_cast<const uint2*>(lo);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    return ss;
+}
+// Preparation of an fp32 call, warp `g` of `nw`: planes and inverse norms of every row of X, and of
+// the rows of the inherited list (checked and scattered into the role map as in gather_rows).
+static __device__ __forceinline__ void split_rows(const SplitJob& sj, int g, int nw, int lane, unsigned* status) {
+    const int64_t n_rows = (int64_t)sj.B * sj.T;
+    const int64_t prow_len = 3 * (int64_t)sj.dpad;
+    // list entries first: they hang on two more loads than the plain rows
+    if (sj.rep_in != nullptr) {
+        int b = 0;
+        int64_t item = g;
+        while (b < sj.B) {
+            int cnt = sj.rep_in_cnt[b];
+            if (cnt < 0 || cnt > sj.T) {
+                if (g == 0 && lane == 0) atomicOr(status, ST_BAD_COUNT);
+                cnt = cnt < 0 ? 0 : sj.T;
+            }
+            if (g == 0 && lane == 0) sj.r_eff[b] = cnt;
+            if (item >= cnt) { item -= cnt; ++b; continue; }
+            const int i = (int)item;
+            item += nw;
+            const int32_t* list = sj.rep_in + (int64_t)b * sj.T;
+            const int32_t idx = list[i];
+            bool ok = idx >= 0 && idx < sj.T;
+            if (ok && i > 0) ok = list[i - 1] < idx;
+            const int64_t prow = (int64_t)b * sj.T + i;
+            if (!ok) {
+                if (lane == 0) { atomicOr(status, ST_BAD_INDEX); sj.inv_rep[prow] = 0.f; }
+                continue;
+            }
+            const float ss = split_row(reinterpret_cast<const float4*>(sj.X + (int64_t)b * sj.xb + (int64_t)idx * sj.ldx),
+                                       sj.RP + prow * prow_len, sj.d, sj.dpad, lane);
+            if (lane == 0) {
+                sj.inv_rep[prow] = (ss <= 3.0e38f && ss > 0.f) ? 1.0f / sqrtf(ss) : 0.f;
+                sj.role[(int64_t)b * sj.T + idx] = i + 1;
+            }
+        }
+    }
+    // warps from the far end take the rows first, so that few warps have both kinds
+    for (int64_t row = nw - 1 - g; row < n_rows; row += nw) {
+        const int64_t b = row / sj.T, t = row % sj.T;
+        const float ss = split_row(reinterpret_cast<const float4*>(sj.X + b * sj.xb + t * sj.ldx), sj.XP + row * prow_len,
+                                   sj.d, sj.dpad, lane);
+        if (lane == 0) {
+            float inv = 0.f;
+            if (!(ss <= 3.0e38f)) atomicOr(status, ST_NONFINITE);
+            else if (ss > 0.f) inv = 1.0f / sqrtf(ss);
+            else atomicAdd(status + 1, 1u);
+            sj.inv_norm[row] = inv;
+        }
+    }
 }
 
 }  // namespace tc

@@ -83,7 +83,10 @@ ada_status setup_device(int device, PerDevice** out) {
         c.Xnon = nullptr;
         c.non_tok = nullptr;
         c.near_key = nullptr;
-        c.splitXA = c.splitXB = c.splitRA = c.splitRB = nullptr;
+        c.splitX = c.splitR = nullptr;
+        c.part_buf = nullptr;
+        c.part_bytes = 0;
+        c.max_parts = 1;
         pd.setup_status = ADA_OK;
     });
     *out = &pd;

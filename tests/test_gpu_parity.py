@@ -664,3 +664,43 @@ def test_rejected_list_on_the_pair_kernel_with_row_compaction(ada):
     assert ada.ada_device_status(ctx)[0] == 5
     check_cascade(ctx, X, TAU, [list(range(0, T, 2))])
     ada.ada_destroy(ctx)
+
+
+@pytest.mark.parametrize("dtype,T,d", [("bf16", 512, 2056), ("bf16", 700, 4096), ("bf16", 1030, 2504), ("bf16", 2049, 3072),
+                                       ("f32", 300, 772), ("f32", 520, 1600), ("f32", 1025, 512)])
+def test_tiles_split_along_the_contraction(ada, dtype, T, d):
+    """Too few tiles for the SM pairs: every tile's contraction is shared by several pairs, with K
+    lengths that divide into no equal stages, ragged last tiles and sets of a few columns; calls
+    back to back on one context, so that the exchange buffer is used again at once."""
+    from parity import check_cascade, check_full
+    ctx = ada.ada_create(1, T, d, ada.ADA_F32 if dtype == "f32" else ada.ADA_BF16)
+    X0 = clustered(T, d, 31 * T + d, dtype)
+    for _ in range(2):
+        _, reps = check_full(ctx, X0, TAU)
+    rng = np.random.default_rng(T + d)
+    for R in (reps[0], [0], sorted(rng.choice(T, 33, replace=False).tolist()), list(range(T // 2))):
+        for causal in (False, True):
+            check_cascade(ctx, X0, TAU, [R], causal=causal)
+    assert ada.ada_device_status(ctx)[0] == 0
+    ada.ada_destroy(ctx)
+
+
+def test_two_streams_launch_without_waiting_on_each_other(ada):
+    """Two contexts in two streams at once: only one stream's launches may go without the
+    cooperative attribute.  Results equal those of one stream, and no wait expires."""
+    T, d = 1500, 2048
+    Xs = [torch.from_numpy(clustered(T, d, 5 + i, "bf16").view(np.int16)).view(torch.bfloat16).cuda() for i in range(2)]
+    ctx = [ada.ada_create(1, T, d, ada.ADA_BF16) for _ in range(2)]
+    ref = [ada.ada_select_full(ctx[i], Xs[i], TAU) for i in range(2)]
+    steps = [ada.ada_cascade_step(ctx[i], Xs[i], TAU, ref[i][0], ref[i][1]) for i in range(2)]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    for _ in range(20):
+        out = [ada.ada_cascade_step(ctx[i], Xs[i], TAU, ref[i][0], ref[i][1], stream=streams[i]) for i in range(2)]
+        torch.cuda.synchronize()
+        for i in range(2):
+            assert torch.equal(out[i].rep_out_cnt, steps[i].rep_out_cnt)
+            assert torch.equal(out[i].gamma_cross, steps[i].gamma_cross)
+    for c, s in zip(ctx, streams):
+        assert ada.ada_device_status(c, stream=s)[0] == 0
+        ada.ada_destroy(c)

@@ -117,7 +117,7 @@ __device__ __forceinline__ float ex2_approx(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ void tmem_st32(unsigned taddr, const float (&v)[32]) {
+__device__ __forceinline__ void tmem_st32f(unsigned taddr, const float (&v)[32]) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
         "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
@@ -411,7 +411,7 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
                         tmem_ld32(t_o + o0, v);
 #pragma unroll
                         for (int q = 0; q < 32; ++q) v[q] *= f;
-                        tmem_st32(t_o + o0, v);
+                        tmem_st32f(t_o + o0, v);
                     }
                     l *= f;
                     if (raise) m_ref = m_new;

@@ -68,7 +68,8 @@ struct Stage {
     static constexpr int K = SPLIT ? BK : 2 * BK;          // K elements per stage
     static constexpr int MAXW = SPLIT ? BN / 2 : BN;       // widest tile (columns of the pair)
     static constexpr int TERMS = SPLIT ? 6 : 2;            // MMA groups per stage
-    static constexpr int CHUNKS = MAXW / 32 / SUBS;        // 32-column chunks of a tile per epilogue warp
+    static constexpr bool ALT = !SPLIT;                     // may the two epilogue sets take alternate tiles?
+    static constexpr int COLS = ALT ? MAXW : MAXW / SUBS;   // columns of a tile that one epilogue warp sees
     // sub-tiles of A and B multiplied by group t
     static __device__ __forceinline__ constexpr int ta(int t) { return SPLIT ? (t == 2 || t == 5 ? 1 : (t == 4 ? 2 : 0)) : t; }
     static __device__ __forceinline__ constexpr int tb(int t) { return SPLIT ? (t == 1 || t == 5 ? 1 : (t == 3 ? 2 : 0)) : t; }
@@ -90,8 +91,8 @@ __device__ __forceinline__ unsigned map_to_cta(unsigned addr, unsigned rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-__device__ __forceinline__ void mbar_arrive_remote(unsigned cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr)
+__device__ __forceinline__ void mbar_arrive_remote(unsigned cluster_addr, unsigned count) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(cluster_addr), "r"(count)
                  : "memory");
 }
 // TMA load whose completion bytes go to the LEADER's barrier: bit 24 of a shared::cluster
@@ -148,7 +149,8 @@ struct Plan {
     int tiles0, total;          // triangular tiles; all tiles
     int tw;                     // column width of the triangular tiles
     int hrows;                  // rows of the left operand per CTA in cross tiles (128, or fewer: streaming form)
-    int one_col_tile, compact;
+    int smem_norms, compact;      // row norms of X out of the tiles in shared memory; cross tiles over Xnon
+    int alt;                    // the two epilogue sets take alternate tiles
     int full, rem, parts;       // tiles dealt whole; tiles of the last round, each cut into `parts` K ranges
     int len[PLAN_B];            // sequence lengths (B <= PLAN_B)
 };
@@ -273,24 +275,26 @@ struct GramMaps {
 template <bool SPLIT>
 __device__ __forceinline__ bool shares_ok(int p, int d) { return (p - 1) * d <= (SPLIT ? MAX_SPLIT_D_F32 : MAX_SPLIT_D) / 2 * p; }
 template <bool SPLIT>
-__device__ __forceinline__ void make_plan(Plan& pl, const GramProblem& seg0, const GramProblem& seg1, int nseg,
-                                          const GatherJob& gather, int npairs, int max_parts, int lane) {
+__device__ __noinline__ void make_plan(Plan& pl, const GramProblem& seg0, const GramProblem& seg1, int nseg,
+                                          bool maybe_compact, int npairs, int max_parts, int lane) {
     constexpr int MAXW = Stage<SPLIT>::MAXW;
     const GramProblem& cx = nseg > 1 ? seg1 : seg0;
     // both segments of a launch share the sequences: one read of every length
-    bool one = !cx.tri;
+    bool one = !cx.tri, big = true;
     for (int b = lane; b < cx.B; b += 32) {
         const int n = seq_n_global(cx, b);
         if (b < PLAN_B) pl.len[b] = n;
         one = one && n <= MAXW;
+        big = big && 5 * (int64_t)n >= 2 * (int64_t)cx.rows;
     }
     one = __all_sync(0xffffffffu, one);
+    big = __all_sync(0xffffffffu, big);
     // streaming form: one column tile covers the columns of every sequence and the rows are many,
     // so the launch is one pass over the rows of A, and shorter row tiles put every pair to work.
     // (Below 48 rows per CTA the right operand would be most of the traffic; splitting K is cheaper.)
     const bool stream = !SPLIT && one && cx.hb_rows >= 48;
     const int hrows = stream && cx.hb_rows < BM ? cx.hb_rows : BM;
-    const bool compact = !SPLIT && gather.X != nullptr && compact_wanted(gather, lane);
+    const bool compact = !SPLIT && maybe_compact && big && !one;       // (compact_wanted)
     __syncwarp();
     int t256 = 0, t128 = 0, tc = 0;                 // triangular tiles by width, cross tiles
     for (int b = lane; b < cx.B; b += 32) {
@@ -310,9 +314,9 @@ __device__ __forceinline__ void make_plan(Plan& pl, const GramProblem& seg0, con
     const int nst = ((SPLIT ? cx.planes : cx.d) + Stage<SPLIT>::K - 1) / Stage<SPLIT>::K;
     const int cand = (lane & 8) ? t128 + tc : t256 + tc, q1 = (lane & 7) + 1;
     const int rounds = quot(cand, npairs), rem = cand - rounds * npairs;
-    // the exchange costs about as much as six stages
+    // the exchange costs about 5 us: as much as six stages of fp32 planes, ten of bf16
     const bool can = q1 == 1 || (!stream && q1 <= max_parts && shares_ok<SPLIT>(q1, cx.d) && rem > 0 && q1 * rem <= npairs && 2 * q1 <= nst &&
-                                 nst - quot(nst + q1 - 1, q1) >= 6);
+                                 nst - quot(nst + q1 - 1, q1) >= (SPLIT ? 6 : 10));
     const unsigned cans = __ballot_sync(0xffffffffu, can);
     const int parts256 = 32 - __clz(cans & 0xffu), parts128 = 32 - __clz((cans >> 8) & 0xffu);
     const int rounds256 = __shfl_sync(0xffffffffu, rounds + (rem > 0), 0), rounds128 = __shfl_sync(0xffffffffu, rounds + (rem > 0), 8);
@@ -324,8 +328,13 @@ __device__ __forceinline__ void make_plan(Plan& pl, const GramProblem& seg0, con
         const int tiles0 = seg0.tri ? (narrow ? t128 : t256) : tc;
         const int total = nseg > 1 ? tiles0 + tc : tiles0;
         pl.tiles0 = tiles0; pl.total = total; pl.tw = narrow ? BM : PM; pl.hrows = hrows;
-        pl.one_col_tile = stream ? 1 : 0;
+        pl.smem_norms = stream || (!SPLIT && !cx.tri && nst >= 4 && nst <= 8 && total <= 2 * npairs && !compact) ? 1 : 0;
         pl.compact = compact ? 1 : 0;
+        // Short contractions, many tiles: a tile's main loop is as short as the bookkeeping of its
+        // epilogue (column factors, barriers, atomics: dependent round trips), so the two sets of
+        // four warps take alternate tiles, one accumulator each, and one set's bookkeeping runs beside
+        // the other's reading.  Otherwise both read every tile and its maxima are there sooner.
+        pl.alt = Stage<SPLIT>::ALT && !pl.smem_norms && nst <= 12 && total > 2 * npairs ? 1 : 0;
         pl.parts = narrow ? parts128 : parts256;
         pl.rem = pl.parts > 1 ? the_rem : 0;
         pl.full = total - pl.rem;
@@ -344,7 +353,8 @@ struct alignas(16) Item {
 };
 constexpr int ITEMS = 32;       // items decoded ahead, one per lane; later ones on the fly
 
-template <bool SPLIT> struct Ring { static constexpr int BYTES = (SPLIT ? 216 : 208) * 1024; };
+// (200 KiB hold as many bf16 stages of every width as 208 would; the rest is column factors.)
+template <bool SPLIT> struct Ring { static constexpr int BYTES = (SPLIT ? 216 : 200) * 1024; };
 
 // Not inlined: the decoding is a few hundred instructions of integer arithmetic that would sit in
 // the path of every role; run once, by 32 lanes side by side, it is read from shared memory.
@@ -377,7 +387,7 @@ __device__ __noinline__ void decode_item(const GramProblem* seg0, const GramProb
     w.ring = 0;
 #pragma unroll
     for (int q = 1; q <= MAX_STAGES; ++q) w.ring += q * sb <= room;
-    w.kind = dead_tile(p, t, pl.hrows, pl.one_col_tile != 0, pl.compact != 0) ? 2 : 1;
+    w.kind = dead_tile(p, t, pl.hrows, pl.smem_norms != 0, pl.compact != 0) ? 2 : 1;
 }
 
 // ---------------------------------------------------------------- the kernel
@@ -390,17 +400,22 @@ struct alignas(16) SharedPair {
     unsigned long long tmem_empty[2];
     unsigned long long drain;
     unsigned long long planned;                // the work plan is in shared memory
-    // global counters seen complete by the CTA's one polling thread: preparation, row norms, triangle
-    unsigned long long prep_seen, norm_seen, dep_seen;
+    // global counters seen complete by the thread that polls them for the CTA (for an epilogue set, where
+    // those take alternate tiles): preparation, row norms, triangle
+    unsigned long long prep_seen, norm_seen[SUBS], dep_seen[SUBS];
     unsigned pub_cnt;                          // epilogue warps that have published their share of a triangular tile
     unsigned tmem_base;
     int abort_flag;
     unsigned norm_cnt[MAX_STAGES];             // norm warps done with a stage
     Plan plan;
+    // the problems and the split job once more: what is not inlined takes them by reference, and reading
+    // the parameter space through a pointer is a trip to memory
+    GramProblem seg[2];
+    SplitJob split;
     Item item[ITEMS];
     // per epilogue warp (its own column chunks), so that staging needs no barrier across warps
-    alignas(16) float col_scale[EPI_WARPS][32 * Stage<SPLIT>::CHUNKS];
-    alignas(16) int col_token[EPI_WARPS][32 * Stage<SPLIT>::CHUNKS];
+    alignas(16) float col_scale[EPI_WARPS][Stage<SPLIT>::COLS];
+    alignas(16) int col_token[EPI_WARPS][Stage<SPLIT>::COLS];
 };
 template <bool SPLIT>
 constexpr int smem_pair_bytes() { return Ring<SPLIT>::BYTES + (int)sizeof(SharedPair<SPLIT>) + 1024; }
@@ -451,13 +466,19 @@ __device__ __forceinline__ bool take_partials(uint4* src, uint4 (&x)[8], unsigne
     return true;
 }
 
+template <typename T>
+__device__ __forceinline__ void copy_args(T& dst, const T& src, int i, int n) {
+    static_assert(sizeof(T) % 8 == 0, "copied in 8-byte words");
+    for (; i < (int)(sizeof(T) / 8); i += n)
+        reinterpret_cast<unsigned long long*>(&dst)[i] = reinterpret_cast<const unsigned long long*>(&src)[i];
+}
+
 template <bool SPLIT>
 __global__ void __launch_bounds__(PAIR_THREADS, 1)
 k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramProblem seg0,
            const __grid_constant__ GramProblem seg1, const int nseg,
            const __grid_constant__ NormJob norms, const __grid_constant__ GatherJob gather,
-           const __grid_constant__ SplitJob split, const void* __restrict__ touch_base,
-           const size_t touch_bytes, const int max_parts, unsigned* __restrict__ part_buf,
+           const __grid_constant__ SplitJob split, const int max_parts, unsigned* __restrict__ part_buf,
            unsigned* __restrict__ dep_ctr, unsigned* __restrict__ status) {
     using St = Stage<SPLIT>;
     extern __shared__ unsigned char smem_raw[];
@@ -483,7 +504,8 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         }
         mbar_init(&sh.drain, 1);
         mbar_init(&sh.planned, 1);
-        mbar_init(&sh.prep_seen, 1); mbar_init(&sh.norm_seen, 1); mbar_init(&sh.dep_seen, 1);
+        mbar_init(&sh.prep_seen, 1);
+        for (int q = 0; q < SUBS; ++q) { mbar_init(&sh.norm_seen[q], 1); mbar_init(&sh.dep_seen[q], 1); }
         sh.pub_cnt = 0u;
         sh.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -495,18 +517,23 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
+    if (warp >= 2) {
+        const int i = (int)threadIdx.x - 64, n = 32 * EPI_WARPS;
+        copy_args(sh.seg[0], seg0, i, n);
+        copy_args(sh.seg[1], seg1, i, n);
+        if (SPLIT) copy_args(sh.split, split, i, n);
+    }
     if (threadIdx.x == 32) {                         // descriptors are fetched before the first copy needs them
         prefetch_map(&maps.a[0]); prefetch_map(&maps.b[0]); prefetch_map(&maps.bt[0]);
         prefetch_map(&maps.a[1]); prefetch_map(&maps.b[1]); prefetch_map(&maps.bt[1]);
         prefetch_map(&maps.ah); prefetch_map(&maps.an);
     }
-    if (warp == 13) touch(touch_base, touch_bytes, (int)blockIdx.x * 32 + lane, (int)gridDim.x * 32);
     tcgen05_fence_before();
     __syncthreads();
     cluster_sync_all();          // the peer's barriers exist before anything signals them
     tcgen05_fence_after();
     const unsigned tmem_base = sh.tmem_base;
-    const bool has_prep = gather.X != nullptr || split.X != nullptr;
+    const bool has_prep = SPLIT ? split.X != nullptr : gather.X != nullptr;
     // everything above is local to the CTA; from here on the predecessor's results are read
     grid_dep_wait();
     // (the compaction's blocks may take the SMs that fall idle first: they wait for this whole grid)
@@ -517,8 +544,8 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         // the start.  Items are dealt across the SMs first, so that a
         // short list is read by all of them.  One arrival per CTA.
         const int g = (warp - 2) * (int)gridDim.x + (int)blockIdx.x, nw = (int)gridDim.x * EPI_WARPS;
-        if (gather.X != nullptr) gather_rows(gather, g, nw, lane, status);
-        else split_rows(split, g, nw, lane, status);
+        if constexpr (!SPLIT) gather_rows(gather, g, nw, lane, status);
+        else split_rows(sh.split, g, nw, lane, status);
         // the rows just written are read by TMA (async proxy) from other CTAs
         asm volatile("fence.proxy.async.global;" ::: "memory");
         __threadfence();
@@ -531,9 +558,10 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
     }
     const unsigned prep_total = gridDim.x;
     if (warp == 0) {
-        make_plan<SPLIT>(sh.plan, seg0, seg1, nseg, gather, npairs, max_parts, lane);
+        const bool maybe_compact = gather.X != nullptr && gather.Xnon != nullptr && gather.T >= gather.compact_min_rows;
+        make_plan<SPLIT>(sh.plan, sh.seg[0], sh.seg[1], nseg, maybe_compact, npairs, max_parts, lane);
         __syncwarp();
-        decode_item<SPLIT>(&seg0, &seg1, sh.plan, pair, npairs, lane, sh.item[lane]);
+        decode_item<SPLIT>(&sh.seg[0], &sh.seg[1], sh.plan, pair, npairs, lane, sh.item[lane]);
         __syncwarp();
         if (lane == 0) { __threadfence_block(); mbar_arrive(&sh.planned); }
         __syncwarp();
@@ -543,14 +571,14 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
     const Plan& pl = sh.plan;
     const int tiles0 = pl.tiles0;
     const int hrows = pl.hrows;                          // rows per CTA of a cross tile
-    const bool smem_norms = pl.one_col_tile != 0;        // row norms out of the tiles in shared memory
+    const bool smem_norms = pl.smem_norms != 0;        // row norms out of the tiles in shared memory
     const bool compact = pl.compact != 0;                // cross tiles over the copied-out rows (Xnon)
     Item own;                                            // an item beyond the table
     if (threadIdx.x == 0) TRACE(1);
 
     auto item_at = [&](int it) __attribute__((always_inline)) -> const Item& {
         if (it < ITEMS) return sh.item[it];
-        decode_item<SPLIT>(&seg0, &seg1, pl, pair, npairs, it, own);
+        decode_item<SPLIT>(&sh.seg[0], &sh.seg[1], pl, pair, npairs, it, own);
         return own;
     };
     if (warp == 0) {
@@ -682,21 +710,24 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         // the two warps of a lane quadrant share a tile's 32-column chunks (sub, sub + 2, ..), so
         // that a finished accumulator is read out by eight warps.
         const int quad = warp & 3, sub = (warp - 2) >> 2;
-        constexpr int NK = St::CHUNKS;
         float* cs = sh.col_scale[warp - 2];
         int* ct = sh.col_token[warp - 2];
         const GramProblem& cx = (nseg > 1) ? seg1 : seg0;
         if (norms.X != nullptr) {         // full selection: row norms with plain loads
             norm_rows(norms, blockIdx.x * EPI_WARPS + (warp - 2), gridDim.x * EPI_WARPS, lane, dep_ctr + 1, status);
-        } else if (!cx.tri && cx.inv_out != nullptr && !smem_norms && !compact) {
-            // several column tiles: 1/||x_t|| of every row with plain loads, behind the first main loops
-            // (nothing in this launch waits for them: the row factor is applied by the compaction)
+        }
+        // Cascade step with several column tiles: 1/||x_t|| of every row with plain loads, behind the first
+        // main loops.  Nothing in this launch waits for them (the row factor is applied by the
+        // compaction), but everything waits for the triangle: its tiles go first.
+        bool norms_due = !cx.tri && cx.inv_out != nullptr && !smem_norms && !compact;
+        auto make_norms = [&]() __attribute__((always_inline)) {
             NormJob nj;
             nj.X = cx.A; nj.ldx = cx.lda; nj.n_rows = (int64_t)cx.B * cx.rows; nj.d = cx.d;
             nj.inv_norm = cx.inv_out;
             nj.batch = cx.a_batch; nj.rows_per_seq = cx.rows;
             norm_rows(nj, blockIdx.x * EPI_WARPS + (warp - 2), gridDim.x * EPI_WARPS, lane, dep_ctr + 1, status);
-        }
+            norms_due = false;
+        };
         // row norms out of the A tiles in shared memory (streaming form): warps 6..9, thread lrow owns
         // row lrow of the CTA's tile and follows the ring exactly as the producer fills it
         const bool ring_norms = smem_norms && sub == 1 && !cx.tri && cx.inv_out != nullptr;
@@ -711,12 +742,14 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         // the accumulator goes back to the leader's barrier
         const unsigned empty_addr[2] = {map_to_cta(smem_u32(&sh.tmem_empty[0]), 0),
                                         map_to_cta(smem_u32(&sh.tmem_empty[1]), 0)};
-        // Wait for a counter of the whole grid.  One thread per CTA polls it and the other warps wait in
+        const bool alt = pl.alt != 0;
+        // Wait for a counter of the whole grid.  One thread per CTA (or epilogue set) polls it and the other warps wait in
         // shared memory: with every warp polling, the polls alone saturate the counter's L2 slice
         // and delay the very arrivals that they wait for (up to 9 us before the cross epilogues).
         auto await = [&](const unsigned* ctr, unsigned target, unsigned long long* seen, int where)
                          __attribute__((always_inline)) -> bool {
-            if (warp == 2) {
+            seen += alt ? sub : 0;
+            if (warp == 2 || (alt && warp == 6)) {
                 const bool good = wait_counter(ctr, target, lane, abort_flag, where);
                 if (lane == 0) mbar_arrive(seen);
                 return good;
@@ -724,14 +757,20 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
             return __all_sync(0xffffffffu, mbar_wait(seen, 0, abort_flag, where)) && *abort_flag == 0;
         };
         unsigned tile_it = 0;
+#pragma unroll 1
         for (int it = 0;; ++it) {
             const Item& w = item_at(it);
+            if (norms_due && (w.kind == 0 || !(w.seg ? seg1 : seg0).tri)) make_norms();
             if (w.kind == 0) break;
             if (w.kind == 2) continue;
             const int sg = w.seg, col0 = w.col0, ncols = w.ncols, row0 = w.row0;
             const GramProblem& p = sg ? seg1 : seg0;
             const unsigned acc = tile_it & 1u, acc_ph = (tile_it >> 1) & 1u;
             ++tile_it;
+            const bool solo = alt && w.parts == 1;       // this set's tile alone
+            if (solo && (int)acc != sub) continue;
+            // the warp's chunks of 32 columns: cfirst, cfirst + cstep, .. below nch
+            const int cfirst = solo ? 0 : sub, cstep = solo ? 1 : SUBS;
             const int64_t o = (int64_t)w.b * p.cap;
             const int nch = ncols >> 5;
             const int arows = p.tri ? BM : hrows;
@@ -748,11 +787,11 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                     ring_s = (ring_s + nst) % ring_nst;
                 } else {
                     float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-                    bool ok = true;
+                    bool fine = true;
                     for (int st = 0; st < nst; ++st) {
                         int good = 1;
                         if (lane == 0) good = mbar_wait(&sh.consumed[ring_s], (cons >> ring_s) & 1u, abort_flag, 14) ? 1 : 0;
-                        if (__shfl_sync(0xffffffffu, good, 0) == 0) { ok = false; break; }
+                        if (__shfl_sync(0xffffffffu, good, 0) == 0) { fine = false; break; }
                         if (lrow < arows) {
 #pragma unroll
                             for (int u = 0; u < St::NSUB; ++u) {
@@ -781,7 +820,7 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                         cons ^= 1u << ring_s;
                         ring_s = (ring_s + 1 == ring_nst) ? 0 : ring_s + 1;
                     }
-                    if (!ok) break;
+                    if (!fine) break;
                     if (lrow < arows && row < w.m) {
                         const float ss = (s0 + s1) + (s2 + s3);
                         float inv = 0.f;
@@ -799,24 +838,8 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                 prep_ok = true;
             }
             if (p.wait_norm_b && !norm_ok) {
-                if (!await(dep_ctr + 1, norm_total, &sh.norm_seen, 9)) break;
+                if (!await(dep_ctr + 1, norm_total, sh.norm_seen, 9)) break;
                 norm_ok = true;
-            }
-            // all of the tile's global loads are issued before the first is used (columns past the
-            // tile are clamped to its last one and discarded afterwards, so that no load hangs
-            // on a data-dependent branch), and what does not depend on line 5 before that is
-            // waited for: the path from the triangle's verdict to the maxima is one round trip
-            float fb[NK];
-            unsigned gate[NK] = {};
-            int tk[NK] = {};
-            const int last = max(w.n - 1, 0);
-#pragma unroll
-            for (int k = 0; k < NK; ++k)
-                fb[k] = __ldcg(p.inv_b + o + min(col0 + 32 * (sub + SUBS * k) + lane, last));
-            if (!p.tri && p.causal) {
-#pragma unroll
-                for (int k = 0; k < NK; ++k)
-                    tk[k] = __ldcg(p.col_token + o + min(col0 + 32 * (sub + SUBS * k) + lane, last));
             }
             const unsigned thr_b = (!p.tri && p.tau_seq != nullptr) ? __float_as_uint(tau_threshold(__ldcg(p.tau_seq + w.b))) : p.thr_bits;
             bool row_live = lrow < arows && row < w.m;
@@ -833,54 +856,122 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
             const bool skip = row_live && !p.tri && !defer && p.row_role[o + row] != 0;
             const bool inv_early = defer || !(p.wait_norm_a && !norm_ok);
             float inv_row = defer ? 1.0f : ((row_live && inv_early) ? __ldcg(p.inv_a + o + row) : 0.f);
+            const unsigned tbase = tmem_base + ((unsigned)(quad * 32) << 16) + acc * BN;
+            int own0 = 0, own1 = nch;                    // chunks that this share of the tile answers for
+            // Two steps: the column factors (for a cross tile they wait for the triangle's verdict), and for a
+            // share of a split tile the exchange of partial sums.  What has to wait comes second.
+            bool ok = true;
+#pragma unroll 1
+            for (int step = 0; step < 2; ++step) {
+            if ((step == 0) != (p.tri != 0)) {
+            if (w.parts > 1) {
+                // A share of the contraction.  The tile's chunks are divided among its shares: each
+                // writes its partial sums of the others' chunks to the exchange buffer (a row per
+                // thread, 16-byte columns outermost: coalesced both ways) and adds the others' to its
+                // own chunks, in a fixed order, in TMEM.  A cross tile does all this before it waits for
+                // the triangle's verdict (pair kernel, T = 512, d = 768, fp32: 4 us of a 24 us step).
+                const bool got = mbar_wait(&sh.tmem_full[acc], acc_ph, abort_flag, 4);
+                ok = __all_sync(0xffffffffu, got);
+                if (!ok) break;
+                tcgen05_fence_after();
+                own0 = quot(nch * w.part, w.parts); own1 = quot(nch * (w.part + 1), w.parts);
+                const int unit0 = w.unit0;
+#pragma unroll 1
+                for (int c = sub; c < nch; c += SUBS) {
+                    if (c >= own0 && c < own1) continue;
+                    unsigned r0[32];
+                    tmem_ld32_issue(tbase + 32 * c, r0);
+                    tmem_ld_wait(r0);
+                    uint4* dst = reinterpret_cast<uint4*>(part_buf + chunk_at(unit0 + w.part, rank, c)) + lrow;
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) r0[j] = r0[j] == EMPTY_WORD ? 0x7FFFFFFFu : r0[j];   // another NaN
+#pragma unroll
+                    for (int q = 0; q < 8; ++q)
+                        __stcg(dst + q * BM, make_uint4(r0[4 * q], r0[4 * q + 1], r0[4 * q + 2], r0[4 * q + 3]));
+                }
+                bool good = true;
+#pragma unroll 1
+                for (int c = sub; c < own1; c += SUBS) {
+                    if (c < own0) continue;
+                    uint4* const src = reinterpret_cast<uint4*>(part_buf + chunk_at(unit0, rank, c)) + lrow;
+                    constexpr int STEP = 2 * (BN / 32) * CHUNK_WORDS / 4;        // from one share's slot to the next
+                    unsigned r0[32];
+                    tmem_ld32_issue(tbase + 32 * c, r0);
+                    tmem_ld_wait(r0);
+#pragma unroll 1
+                    for (int q = 0; q < w.parts; ++q) {
+                        if (q == w.part) continue;
+                        uint4 x0[8];
+                        load_partials(src + q * STEP, x0);
+                        good = take_partials(src + q * STEP, x0, r0, abort_flag) && good;
+                    }
+                    tmem_st32(tbase + 32 * c, r0);
+                }
+                ok = __all_sync(0xffffffffu, good);
+                if (!ok) break;
+            }
+            } else {
             if (sg == 1 && !dep_ok) {
                 // every triangular tile of this launch first (line 5 before line 7)
-                if (!await(dep_ctr, dep_total, &sh.dep_seen, 5)) break;
+                ok = await(dep_ctr, dep_total, sh.dep_seen, 5);
+                if (!ok) break;
                 dep_ok = true;
                 if (warp == 2 && lane == 0) TRACE(4);
             }
-            if (!p.tri) {
-                // representative removed at line 5 (written earlier in this launch: read at L2)
+            // Column factors of the warp's chunks.  All of a group's global loads are issued before the
+            // first is used (columns past the tile are clamped to its last one and discarded
+            // afterwards, so that no load hangs on a data-dependent branch).
+            __syncwarp();
+            const int last = max(w.n - 1, 0);
+#pragma unroll 1
+            for (int g = cfirst; g < nch; g += 4 * cstep) {
+                float fb[4];
+                unsigned gate[4] = {};
+                int tk[4] = {};
 #pragma unroll
-                for (int k = 0; k < NK; ++k)
-                    gate[k] = __ldcg(p.col_gate + o + min(col0 + 32 * (sub + SUBS * k) + lane, last));
+                for (int k = 0; k < 4; ++k) {
+                    const int64_t at = o + min(col0 + 32 * (g + k * cstep) + lane, last);
+                    fb[k] = __ldcg(p.inv_b + at);
+                    // representative removed at line 5 (written earlier in this launch: read at L2)
+                    if (!p.tri) gate[k] = __ldcg(p.col_gate + at);
+                    if (!p.tri && p.causal) tk[k] = __ldcg(p.col_token + at);
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int c = g + k * cstep, col = col0 + 32 * c + lane;
+                    if (c >= nch) break;
+                    const bool live = col < w.n;
+                    const int at = (solo ? 32 * c : 32 * (c >> 1)) + lane;
+                    cs[at] = (live && (p.tri || gate[k] < thr_b)) ? fb[k] : 0.f;
+                    ct[at] = (live && !p.tri && p.causal) ? tk[k] : col;
+                }
             }
             __syncwarp();
-#pragma unroll
-            for (int k = 0; k < NK; ++k) {
-                const int col = col0 + 32 * (sub + SUBS * k) + lane;
-                const bool live = col < w.n;
-                cs[k * 32 + lane] = (live && (p.tri || gate[k] < thr_b)) ? fb[k] : 0.f;
-                ct[k * 32 + lane] = (live && !p.tri && p.causal) ? tk[k] : col;
             }
-            __syncwarp();
-            const bool got = mbar_wait(&sh.tmem_full[acc], acc_ph, abort_flag, 4);
-            if (!__all_sync(0xffffffffu, got)) break;
-            tcgen05_fence_after();
+            }
+            if (!ok) break;
+            if (w.parts == 1) {
+                const bool got = mbar_wait(&sh.tmem_full[acc], acc_ph, abort_flag, 4);
+                if (!__all_sync(0xffffffffu, got)) break;
+                tcgen05_fence_after();
+            }
             const bool need_cmp = p.tri ? (col0 + ncols > row_base) : (p.causal != 0);
             const bool want_arg = p.out_arg != nullptr;
             float mx0 = 0.f, mx1 = 0.f;
             int arg = 0;                                     // nearest-representative mode: column of the maximum
-            // 32 columns of this thread's row, the warp's k-th chunk
-            auto consume = [&](const unsigned (&r)[32], int k) __attribute__((always_inline)) {
-                const float* csk = cs + k * 32;
+            // 32 columns (chunk c) of this thread's row
+            auto consume = [&](const unsigned (&r)[32], int c) __attribute__((always_inline)) {
+                const float* csk = cs + (solo ? 32 * c : 32 * (c >> 1));
                 if (want_arg) {
 #pragma unroll
                     for (int j = 0; j < 32; ++j) {           // ascending columns, strict '>': lowest index on ties
                         const float x = fabsf(__uint_as_float(r[j])) * csk[j];
-                        if (x > mx0) { mx0 = x; arg = 32 * (sub + SUBS * k) + j; }
+                        if (x > mx0) { mx0 = x; arg = 32 * c + j; }
                     }
                 } else if (!need_cmp) {
-#pragma unroll
-                    for (int j = 0; j < 32; j += 4) {
-                        const float4 f = *reinterpret_cast<const float4*>(csk + j);
-                        mx0 = fmaxf(mx0, fabsf(__uint_as_float(r[j])) * f.x);
-                        mx1 = fmaxf(mx1, fabsf(__uint_as_float(r[j + 1])) * f.y);
-                        mx0 = fmaxf(mx0, fabsf(__uint_as_float(r[j + 2])) * f.z);
-                        mx1 = fmaxf(mx1, fabsf(__uint_as_float(r[j + 3])) * f.w);
-                    }
+                    row_max32(r, csk, mx0, mx1);
                 } else {
-                    const int* ctk = ct + k * 32;
+                    const int* ctk = ct + (solo ? 32 * c : 32 * (c >> 1));
 #pragma unroll
                     for (int j = 0; j < 32; j += 4) {
                         const float4 f = *reinterpret_cast<const float4*>(csk + j);
@@ -892,77 +983,24 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                     }
                 }
             };
-            // (a warp whose 32 rows lie past a short tile's rows still joins the aligned loads)
-            const unsigned tbase = tmem_base + ((unsigned)(quad * 32) << 16) + acc * BN + sub * 32;   // the warp's chunk k: + 32 SUBS k
-            if (w.parts == 1) {
-                // (rolled loops: the code of an epilogue is fetched cold in most launches)
+            // (a warp whose 32 rows lie past a short tile's rows still joins the aligned loads; rolled
+            // loops: the code of an epilogue is fetched cold in most launches)
 #pragma unroll 1
-                for (int k = 0; sub + SUBS * k < nch; ++k) {
-                    unsigned r0[32];
-                    tmem_ld32_issue(tbase + 32 * SUBS * k, r0);
-                    tmem_ld_wait(r0);
-                    consume(r0, k);
-                }
-            } else {
-                // A share of the contraction.  The tile's chunks are divided among its shares: each
-                // writes its partial sums of the others' chunks to the exchange buffer (a row per
-                // thread, 16-byte columns outermost: coalesced both ways) and adds the others' to its
-                // own chunks in a fixed order.
-                const int unit0 = w.unit0;
-                const int own0 = nch * w.part / w.parts, own1 = nch * (w.part + 1) / w.parts;
-                bool mine = false;
-#pragma unroll 1
-                for (int k = 0; k < NK; ++k) {
-                    const int c = sub + SUBS * k;
-                    if (c >= nch) break;
-                    if (c >= own0 && c < own1) { mine = true; continue; }
-                    unsigned r0[32];
-                    tmem_ld32_issue(tbase + 32 * SUBS * k, r0);
-                    tmem_ld_wait(r0);
-                    uint4* dst = reinterpret_cast<uint4*>(part_buf + chunk_at(unit0 + w.part, rank, c)) + lrow;
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) r0[j] = r0[j] == EMPTY_WORD ? 0x7FFFFFFFu : r0[j];   // another NaN
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        __stcg(dst + q * BM, make_uint4(r0[4 * q], r0[4 * q + 1], r0[4 * q + 2], r0[4 * q + 3]));
-                }
-                if (mine) {
-                    bool good = true;
-#pragma unroll 1
-                    for (int k = 0; k < NK; ++k) {
-                        const int c = sub + SUBS * k;
-                        if (c < own0 || c >= own1) continue;
-                        uint4* const src = reinterpret_cast<uint4*>(part_buf + chunk_at(w.unit0, rank, c)) + lrow;
-                        constexpr int STEP = 2 * (BN / 32) * CHUNK_WORDS / 4;        // from one share's slot to the next
-                        unsigned r0[32];
-                        tmem_ld32_issue(tbase + 32 * SUBS * k, r0);
-                        // (two shares' loads in flight)
-                        uint4 x0[8], x1[8];
-                        int q = w.part == 0 ? 1 : 0;
-                        load_partials(src + q * STEP, x0);
-                        tmem_ld_wait(r0);
-                        while (q < w.parts) {
-                            int q2 = q + 1 + (q + 1 == w.part);
-                            if (q2 < w.parts) load_partials(src + q2 * STEP, x1);
-                            good = take_partials(src + q * STEP, x0, r0, abort_flag) && good;
-                            if (q2 >= w.parts) break;
-                            q = q2 + 1 + (q2 + 1 == w.part);
-                            if (q < w.parts) load_partials(src + q * STEP, x0);
-                            good = take_partials(src + q2 * STEP, x1, r0, abort_flag) && good;
-                        }
-                        consume(r0, k);
-                    }
-                    if (!__all_sync(0xffffffffu, good)) break;
-                }
+            for (int c = cfirst; c < own1; c += cstep) {
+                if (c < own0) continue;
+                unsigned r0[32];
+                tmem_ld32_issue(tbase + 32 * c, r0);
+                tmem_ld_wait(r0);
+                consume(r0, c);
             }
             float mx = fmaxf(mx0, mx1);
             tcgen05_fence_before();
             __syncwarp();
             // (a share is its pair's last item: nobody waits for its accumulator, and the arrive would
             // first wait for the stores above)
-            if (lane == 0 && w.parts == 1) mbar_arrive_remote(empty_addr[acc]);
+            if (lane == 0 && w.parts == 1) mbar_arrive_remote(empty_addr[acc], solo ? SUBS : 1);
             if (!inv_early && !norm_ok) {
-                if (!await(dep_ctr + 1, norm_total, &sh.norm_seen, 9)) break;
+                if (!await(dep_ctr + 1, norm_total, sh.norm_seen, 9)) break;
                 norm_ok = true;
             }
             if (row_live && !skip) {
@@ -980,7 +1018,8 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                 // publish: one arrival per CTA and tile, by the last of its warps
                 __threadfence();
                 __syncwarp();
-                if (lane == 0 && atomicAdd(&sh.pub_cnt, 1u) % EPI_WARPS == EPI_WARPS - 1) {
+                const unsigned share = solo ? SUBS : 1;
+                if (lane == 0 && (atomicAdd(&sh.pub_cnt, share) + share) % EPI_WARPS == 0) {
                     __threadfence();
                     atomicAdd(dep_ctr, 1u);
                 }
@@ -1094,16 +1133,6 @@ cudaError_t launch_gram_tc2(ada_ctx* ctx, const GramProblem* tri, const GramProb
     memset(&sj, 0, sizeof(sj));
     if (split != nullptr) sj = *split;
     const bool planes = segs[0].planes > 0;
-    // the caller's activations: extent of what this call reads
-    const void* touch_base = segs[0].A;
-    size_t touch_bytes = (size_t)((segs[0].B - 1) * segs[0].a_batch + (int64_t)(segs[0].rows - 1) * segs[0].lda + segs[0].d) * 2;
-    if (gj.X != nullptr) {
-        touch_base = gj.X;
-        touch_bytes = (size_t)((gj.B - 1) * gj.xb + (int64_t)(gj.T - 1) * gj.ldx + gj.d) * 2;
-    } else if (sj.X != nullptr) {
-        touch_base = sj.X;
-        touch_bytes = (size_t)((sj.B - 1) * sj.xb + (int64_t)(sj.T - 1) * sj.ldx + sj.d) * 4;
-    }
     int max_parts = ctx->part_buf != nullptr ? ctx->max_parts : 1;
     if (nseg == 1 && segs[0].tri && segs[0].n_dev == nullptr) {
         // tile count known here: a last round that is more than half full is not split, and the launch
@@ -1142,7 +1171,7 @@ cudaError_t launch_gram_tc2(ada_ctx* ctx, const GramProblem* tri, const GramProb
     cfg.attrs = attr;
     cfg.numAttrs = na;
     cudaError_t e = cudaLaunchKernelEx(&cfg, planes ? k_gram_tc2<true> : k_gram_tc2<false>, maps, segs[0], segs[1],
-                                       nseg, nj, gj, sj, touch_base, touch_bytes, max_parts, ctx->part_buf, ctx->tile_ctr,
+                                       nseg, nj, gj, sj, max_parts, ctx->part_buf, ctx->tile_ctr,
                                        ctx->status);
     if (waits) coop_end(ctx, coop);
     prof_end(ctx, s);

@@ -132,14 +132,6 @@ static __device__ __forceinline__ void tma_load_3d(const CUtensorMap* map, unsig
           "r"(c0), "r"(c1), "r"(c2)
         : "memory");
 }
-// One cache line in every 1/n of [base, base + bytes), thread i of n.  The first access to a page in a
-// long while costs several microseconds of address translation; touching the activations
-// as soon as a kernel starts takes that off the path of its first copies.
-static __device__ __forceinline__ void touch(const void* base, size_t bytes, int i, int n) {
-    const size_t at = bytes / (size_t)n * (size_t)i;
-    if (base != nullptr && at < bytes)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(base) + at));
-}
 static __device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<unsigned long long>(map)) : "memory");
 }
@@ -211,6 +203,43 @@ static __device__ __forceinline__ void tmem_ld_wait(unsigned (&r)[32]) {
         : "memory");
 }
 
+// tcgen05.st of 32 columns of this warp's lanes
+static __device__ __forceinline__ void tmem_st32(unsigned taddr, const unsigned (&r)[32]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
+        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+        "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};\n\t"
+        "tcgen05.wait::st.sync.aligned;"
+        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+          "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
+          "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
+          "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+        : "memory");
+}
+// max(m, |a|, |b|) in one instruction
+static __device__ __forceinline__ float max3_abs(float m, float a, float b) {
+    float d;
+    asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(m), "f"(a), "f"(b));
+    return d;
+}
+// Running maxima of |r[j]| * f[j] over 32 columns: two products per multiply, two candidates per maximum, i.e.
+// one arithmetic instruction per column (the epilogues of short contractions are bound by them).
+static __device__ __forceinline__ void row_max32(const unsigned (&r)[32], const float* f, float& m0, float& m1) {
+#pragma unroll
+    for (int j = 0; j < 32; j += 4) {
+        const ulonglong2 ff = *reinterpret_cast<const ulonglong2*>(f + j);
+        float a, b, c, d;
+        asm("{\n\t.reg .b64 x, y;\n\t"
+            "mov.b64 x, {%4, %5};\n\tmov.b64 y, {%6, %7};\n\t"
+            "mul.rn.f32x2 x, x, %8;\n\tmul.rn.f32x2 y, y, %9;\n\t"
+            "mov.b64 {%0, %1}, x;\n\tmov.b64 {%2, %3}, y;\n\t}"
+            : "=f"(a), "=f"(b), "=f"(c), "=f"(d)
+            : "r"(r[j]), "r"(r[j + 1]), "r"(r[j + 2]), "r"(r[j + 3]), "l"(ff.x), "l"(ff.y));
+        m0 = max3_abs(m0, a, b);
+        m1 = max3_abs(m1, c, d);
+    }
+}
+
 // Shared-memory matrix descriptor of a K-major bf16 tile whose rows are 128 bytes wide and
 // stored with the 128-byte swizzle: 8-row groups are 1024 bytes apart (stride byte offset),
 // the leading byte offset is unused for swizzled K-major tiles, descriptor version 1.
@@ -279,53 +308,84 @@ static __device__ __forceinline__ float sumsq_bf16x8(const uint4& v) {
     }
     return s;
 }
+static __device__ __forceinline__ float inv_of_sumsq(float ss, int lane, unsigned* status) {
+    float inv = 0.f;
+    if (!(ss <= 3.0e38f)) {
+        if (lane == 0) atomicOr(status, ST_NONFINITE);
+    } else if (ss > 0.f) {
+        inv = 1.0f / sqrtf(ss);
+    } else if (lane == 0) {
+        atomicAdd(status + 1, 1u);
+    }
+    return inv;
+}
 // Executed by the norm warps of every CTA: warp `w` of `nw` takes rows w, w+nw, ...; when a
 // warp has stored its last row it bumps the counter, so counter == nw means "all rows done".
-static __device__ __forceinline__ void norm_rows(const NormJob& job, int w, int nw, int lane,
-                                                 unsigned* counter, unsigned* status) {
+// (Not inlined, like the other parts that run once: a Gram launch fetches its instructions cold, and
+// its start-up gets longer with every line of code that lies between those it executes.  The
+// arguments come by value: reading kernel parameters through a pointer is a trip to memory.)
+static __device__ __noinline__ void norm_rows(const NormJob job, int w, int nw, int lane, unsigned* counter,
+                                              unsigned* status) {
     const int nvec = job.d >> 3;
     const __nv_bfloat16* X = reinterpret_cast<const __nv_bfloat16*>(job.X);
-    for (int64_t row = w; row < job.n_rows; row += nw) {
-        const int64_t off = job.rows_per_seq > 0
-            ? (row / job.rows_per_seq) * job.batch + (row % job.rows_per_seq) * job.ldx
-            : row * job.ldx;
+    // (row counts fit 31 bits; a 32-bit division is several times cheaper)
+    auto at = [&](int64_t row) {
+        return job.rows_per_seq > 0 ? ((unsigned)row / (unsigned)job.rows_per_seq) * job.batch +
+                                          ((unsigned)row % (unsigned)job.rows_per_seq) * job.ldx
+                                    : row * job.ldx;
+    };
+    int64_t row = w;
+    if (nvec <= 128) {
+        // rows of at most 128 vectors: four rows, sixteen loads, in flight per lane
+        for (; row + 3 * (int64_t)nw < job.n_rows; row += 4 * (int64_t)nw) {
+            float ss[4];
+            uint4 x[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint4* src = reinterpret_cast<const uint4*>(X + at(row + i * (int64_t)nw));
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    x[i][q] = lane + 32 * q < nvec ? __ldg(src + lane + 32 * q) : make_uint4(0u, 0u, 0u, 0u);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                ss[i] = ((sumsq_bf16x8(x[i][0]) + sumsq_bf16x8(x[i][1])) + sumsq_bf16x8(x[i][2])) + sumsq_bf16x8(x[i][3]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) ss[i] += __shfl_xor_sync(0xffffffffu, ss[i], o);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float inv = inv_of_sumsq(ss[i], lane, status);
+                if (lane == 0) job.inv_norm[row + i * (int64_t)nw] = inv;
+            }
+        }
+    }
+    for (; row < job.n_rows; row += nw) {
+        const int64_t off = at(row);
         const uint4* src = reinterpret_cast<const uint4*>(X + off);
-        // sixteen (then eight) independent 128-bit loads in flight per lane: these few warps
-        // have to cover the memory latency that a dedicated kernel would hide with occupancy
-        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+        // sixteen independent 128-bit loads in flight per lane: these few warps have to cover the
+        // memory latency that a dedicated kernel would hide with occupancy
+        float ss = 0.f;
         int v = lane;
         for (; v + 480 < nvec; v += 512) {
             uint4 x[16];
 #pragma unroll
             for (int q = 0; q < 16; ++q) x[q] = __ldg(src + v + 32 * q);
 #pragma unroll
-            for (int q = 0; q < 16; q += 4) {
-                s0 += sumsq_bf16x8(x[q]); s1 += sumsq_bf16x8(x[q + 1]);
-                s2 += sumsq_bf16x8(x[q + 2]); s3 += sumsq_bf16x8(x[q + 3]);
-            }
+            for (int q = 0; q < 16; ++q) ss += sumsq_bf16x8(x[q]);
         }
-        for (; v + 224 < nvec; v += 256) {
+        for (; v < nvec; v += 256) {
             uint4 x[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) x[q] = __ldg(src + v + 32 * q);
+            for (int q = 0; q < 8; ++q)
+                x[q] = v + 32 * q < nvec ? __ldg(src + v + 32 * q) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-            for (int q = 0; q < 8; q += 4) {
-                s0 += sumsq_bf16x8(x[q]); s1 += sumsq_bf16x8(x[q + 1]);
-                s2 += sumsq_bf16x8(x[q + 2]); s3 += sumsq_bf16x8(x[q + 3]);
-            }
+            for (int q = 0; q < 8; ++q) ss += sumsq_bf16x8(x[q]);
         }
-        for (; v < nvec; v += 32) s0 += sumsq_bf16x8(__ldg(src + v));
-        float ss = (s0 + s1) + (s2 + s3);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        float inv = 0.f;
-        if (!(ss <= 3.0e38f)) {
-            if (lane == 0) atomicOr(status, ST_NONFINITE);
-        } else if (ss > 0.f) {
-            inv = 1.0f / sqrtf(ss);
-        } else if (lane == 0) {
-            atomicAdd(status + 1, 1u);
-        }
+        const float inv = inv_of_sumsq(ss, lane, status);
         if (lane == 0) job.inv_norm[row] = inv;
     }
     __threadfence();
@@ -381,45 +441,109 @@ static __device__ __forceinline__ bool compact_wanted(const GatherJob& gj, int l
     return __all_sync(0xffffffffu, big) && !__all_sync(0xffffffffu, one);
 }
 
-// one warp: copy a row of nvec 16-byte vectors, return its sum of squares (all lanes)
-static __device__ __forceinline__ float copy_row_sumsq(const uint4* __restrict__ src, uint4* __restrict__ dst,
-                                                       int nvec, int lane) {
-    float ss = 0.f;
+// one warp: copy U rows of nvec 16-byte vectors (dst NULL: only read), V loads per lane and row in flight;
+// ss: their sums of squares (all lanes)
+template <int U, int V>
+static __device__ __forceinline__ void copy_rows(const uint4* const (&src)[U], uint4* const (&dst)[U], int nvec, int lane,
+                                                 float (&ss)[U]) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) ss[u] = 0.f;
     int v = lane;
-    for (; v + 480 < nvec; v += 512) {            // sixteen loads in flight per lane
-        uint4 x[16];
+    for (; v - lane + 32 * V <= nvec; v += 32 * V) {
+        uint4 x[U][V];
 #pragma unroll
-        for (int q = 0; q < 16; ++q) x[q] = __ldg(src + v + 32 * q);
+        for (int u = 0; u < U; ++u)
 #pragma unroll
-        for (int q = 0; q < 16; ++q) { ss += sumsq_bf16x8(x[q]); dst[v + 32 * q] = x[q]; }
+            for (int q = 0; q < V; ++q) x[u][q] = __ldg(src[u] + v + 32 * q);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int q = 0; q < V; ++q) {
+                ss[u] += sumsq_bf16x8(x[u][q]);
+                if (U == 1 || dst[u] != nullptr) dst[u][v + 32 * q] = x[u][q];
+            }
     }
-    for (; v < nvec; v += 32) {
-        const uint4 x = __ldg(src + v);
-        ss += sumsq_bf16x8(x);
-        dst[v] = x;
+#pragma unroll 1
+    for (; v - lane < nvec; v += 128) {
+        uint4 x[U][4];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                x[u][q] = v + 32 * q < nvec ? __ldg(src[u] + v + 32 * q) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                ss[u] += sumsq_bf16x8(x[u][q]);
+                if ((U == 1 || dst[u] != nullptr) && v + 32 * q < nvec) dst[u][v + 32 * q] = x[u][q];
+            }
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    return ss;
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int u = 0; u < U; ++u) ss[u] += __shfl_xor_sync(0xffffffffu, ss[u], o);
 }
 
-// `compact`: also Algorithm 1 line 6's row set as a matrix of its own.  Line 6 builds the
-// cross-Gram from the (T - r) tokens OUTSIDE the inherited set; when the set is large, streaming
-// all T rows and masking the inherited ones wastes r/T of the loads and MMAs, so the rows
-// between consecutive inherited tokens are copied, in order, to Xnon (row t goes to t minus the
-// number of inherited tokens before it), with their token index in non_tok and 1/||x_t|| in
-// inv_norm.  A warp takes one gap between two list entries at a time.
-// Algorithm 1 lines 1-2, by the preparation warps of all CTAs (warp `g` of `nw`): entry i of
-// sequence b is checked (in range, strictly above entry i-1), role[token] = i + 1, the raw row
-// goes to Xrep[b, i] and its inverse norm to inv_rep[b, i]; a rejected entry gets inverse norm
-// 0 (its column then counts for nothing) and raises the status.
-static __device__ __forceinline__ void gather_rows(const GatherJob& gj, int g, int nw, int lane, unsigned* status) {
+// Walks a warp through the entries of all sequences' lists: item -> (sequence b, entry i).  The counts are
+// read 32 sequences at a time, one per lane (dozens of heads or a batch: one thread following
+// them would be a chain of memory round trips).
+struct ListCursor {
+    const int32_t* counts;
+    int T, B, lane, b0, mine, incl;
+    bool first;
+    int64_t base;                // items of the sequences before b0
+    int32_t* r_eff;
+    unsigned* status;
+    int b, cnt, i;
+    __device__ __forceinline__ ListCursor(const int32_t* c, int T_, int B_, bool first_, int32_t* re, int lane_,
+                                          unsigned* st)
+        : counts(c), T(T_), B(B_), lane(lane_), b0(0), first(first_), base(0), r_eff(re), status(st) { load(); }
+    __device__ __forceinline__ void load() {
+        mine = 0;
+        if (b0 + lane < B) {
+            mine = counts[b0 + lane];
+            if (mine < 0 || mine > T) {
+                if (first) atomicOr(status, ST_BAD_COUNT);
+                mine = mine < 0 ? 0 : T;
+            }
+            if (first) r_eff[b0 + lane] = mine;
+        }
+        incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+    }
+    // (items ascend from call to call)
+    __device__ __forceinline__ bool find(int64_t item) {
+        while (true) {
+            const unsigned above = __ballot_sync(0xffffffffu, item - base < incl);
+            if (above != 0u) {
+                const int l = __ffs(above) - 1;
+                b = b0 + l;
+                cnt = __shfl_sync(0xffffffffu, mine, l);
+                i = (int)(item - base) - __shfl_sync(0xffffffffu, incl - mine, l);
+                return true;
+            }
+            base += __shfl_sync(0xffffffffu, incl, 31);
+            b0 += 32;
+            if (b0 >= B) return false;
+            load();
+        }
+    }
+};
+
+// Entries of the inherited lists, warp `g` of `nw`, U at a time: entry i of sequence b is checked (in range,
+// strictly above entry i-1), role[token] = i + 1, the raw row goes to Xrep[b, i] and its inverse
+// norm to inv_rep[b, i]; a rejected entry gets inverse norm 0 (its column then counts for
+// nothing) and raises the status.  copy: false when another pass copies the rows.
+template <int U, int V>
+static __device__ __forceinline__ void gather_entries(const GatherJob& gj, int g, int nw, int lane, bool copy,
+                                                      unsigned* status) {
     const __nv_bfloat16* X = reinterpret_cast<const __nv_bfloat16*>(gj.X);
     __nv_bfloat16* Xrep = reinterpret_cast<__nv_bfloat16*>(gj.Xrep);
-    __nv_bfloat16* Xnon = reinterpret_cast<__nv_bfloat16*>(gj.Xnon);
-    const int nvec = gj.d >> 3;
-    int b = 0;
-    int64_t item = g;
     // this warp's first entry is most often entry g of sequence 0: fetch it (and its
     // predecessor) beside the count instead of after it
     int32_t first_idx = 0, first_prev = -1;
@@ -427,59 +551,136 @@ static __device__ __forceinline__ void gather_rows(const GatherJob& gj, int g, i
         first_idx = __ldg(gj.rep_in + g);
         if (g > 0) first_prev = __ldg(gj.rep_in + g - 1);
     }
-    const bool compact = compact_wanted(gj, lane);
-    while (b < gj.B) {
-        int cnt = gj.rep_in_cnt[b];
-        if (cnt < 0 || cnt > gj.T) {
-            if (g == 0 && lane == 0) atomicOr(status, ST_BAD_COUNT);
-            cnt = cnt < 0 ? 0 : gj.T;
+    ListCursor cur(gj.rep_in_cnt, gj.T, gj.B, g == 0, gj.r_eff, lane, status);
+    int64_t item = g;
+    bool more = true;
+    while (more) {
+        int b[U], i[U];
+        int32_t idx[U], prev[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            b[u] = -1;
+            if (more) more = cur.find(item);
+            if (!more) continue;
+            b[u] = cur.b; i[u] = cur.i;
+            item += nw;
         }
-        if (g == 0 && lane == 0) gj.r_eff[b] = cnt;
-        const int n_items = compact ? 2 * cnt + 1 : cnt;     // list entries, then the gaps around them
-        if (item >= n_items) { item -= n_items; ++b; continue; }
-        const int i = (int)item;
-        item += nw;                                   // this warp's next item (maybe in a later sequence)
-        const int32_t* list = gj.rep_in + (int64_t)b * gj.T;
-        if (i >= cnt) {
-            // gap number gp: the tokens after entry gp - 1 and before entry gp
-            const int gp = i - cnt;
-            int lo = gp > 0 ? list[gp - 1] + 1 : 0;
-            int hi = gp < cnt ? list[gp] : gj.T;
-            lo = max(lo, 0); hi = min(hi, gj.T);      // (a bad list is reported by the entries' check)
-            for (int t = lo; t < hi; ++t) {
-                const int dstrow = t - gp;
-                if (dstrow < 0 || dstrow >= gj.T) continue;
-                const uint4* src = reinterpret_cast<const uint4*>(X + (int64_t)b * gj.xb + (int64_t)t * gj.ldx);
-                uint4* dst = reinterpret_cast<uint4*>(Xnon + ((int64_t)b * gj.T + dstrow) * (int64_t)gj.d);
-                const float ss = copy_row_sumsq(src, dst, nvec, lane);
-                if (lane == 0) {
-                    float inv = 0.f;
-                    if (!(ss <= 3.0e38f)) atomicOr(status, ST_NONFINITE);
-                    else if (ss > 0.f) inv = 1.0f / sqrtf(ss);
-                    else atomicAdd(status + 1, 1u);
-                    gj.inv_norm[(int64_t)b * gj.T + t] = inv;
-                    gj.non_tok[(int64_t)b * gj.T + dstrow] = t;
-                }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (b[u] < 0) continue;
+            const int32_t* list = gj.rep_in + (int64_t)b[u] * gj.T;
+            const bool spec = b[u] == 0 && i[u] == g;
+            idx[u] = spec ? first_idx : __ldg(list + i[u]);
+            prev[u] = i[u] == 0 ? -1 : (spec ? first_prev : __ldg(list + i[u] - 1));
+        }
+        const uint4* src[U];
+        uint4* dst[U];
+        bool ok[U], any = false;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            src[u] = reinterpret_cast<const uint4*>(X); dst[u] = nullptr;
+            ok[u] = b[u] >= 0 && idx[u] >= 0 && idx[u] < gj.T && prev[u] < idx[u];
+            if (b[u] < 0) continue;
+            const int64_t prow = (int64_t)b[u] * gj.T + i[u];
+            if (!ok[u] && lane == 0) { atomicOr(status, ST_BAD_INDEX); gj.inv_rep[prow] = 0.f; }
+            if (!ok[u] || !copy) continue;
+            any = true;
+            src[u] = reinterpret_cast<const uint4*>(X + (int64_t)b[u] * gj.xb + (int64_t)idx[u] * gj.ldx);
+            dst[u] = reinterpret_cast<uint4*>(Xrep + prow * (int64_t)gj.d);
+        }
+        if (!any) continue;
+        float ss[U];
+        copy_rows<U, V>(src, dst, gj.d >> 3, lane, ss);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (ok[u] && lane == 0) {
+                gj.inv_rep[(int64_t)b[u] * gj.T + i[u]] = (ss[u] <= 3.0e38f && ss[u] > 0.f) ? 1.0f / sqrtf(ss[u]) : 0.f;
+                gj.role[(int64_t)b[u] * gj.T + idx[u]] = i[u] + 1;
             }
-            continue;
-        }
-        const bool spec = b == 0 && i == g;
-        const int32_t idx = spec ? first_idx : list[i];
-        bool ok = idx >= 0 && idx < gj.T;
-        if (ok && i > 0) ok = (spec ? first_prev : list[i - 1]) < idx;
-        const int64_t prow = (int64_t)b * gj.T + i;
-        if (!ok) {
-            if (lane == 0) { atomicOr(status, ST_BAD_INDEX); gj.inv_rep[prow] = 0.f; }
-            continue;
-        }
-        const uint4* src = reinterpret_cast<const uint4*>(X + (int64_t)b * gj.xb + (int64_t)idx * gj.ldx);
-        uint4* dst = reinterpret_cast<uint4*>(Xrep + prow * (int64_t)gj.d);
-        const float ss = copy_row_sumsq(src, dst, nvec, lane);
-        if (lane == 0) {
-            gj.inv_rep[prow] = (ss <= 3.0e38f && ss > 0.f) ? 1.0f / sqrtf(ss) : 0.f;
-            gj.role[(int64_t)b * gj.T + idx] = i + 1;
+    }
+}
+
+// How many of the ascending list's n entries lie below t: a 32-way search by the whole warp
+static __device__ __forceinline__ int entries_below(const int32_t* list, int n, int t, int lane) {
+    int lo = 0, hi = n;
+    while (hi - lo > 32) {
+        const int step = (hi - lo + 31) >> 5, at = lo + (lane + 1) * step - 1;
+        const unsigned below = __ballot_sync(0xffffffffu, at < hi && __ldg(list + min(at, hi - 1)) < t);
+        const int k = __popc(below);
+        lo += k * step;
+        hi = min(hi, lo + step);
+        if (lo >= hi) return hi;
+    }
+    return lo + __popc(__ballot_sync(0xffffffffu, lo + lane < hi && __ldg(list + min(lo + lane, n - 1)) < t));
+}
+
+// Line 6's row set as a matrix of its own.  Line 6 builds the cross-Gram from the (T - r) tokens OUTSIDE
+// the inherited set; when the set is large, streaming all T rows and masking the inherited ones
+// wastes r/T of the loads and MMAs, so those rows are copied, in order, to Xnon (row t goes to t
+// minus the number of inherited tokens before it), with their token index in non_tok and
+// 1/||x_t|| in inv_norm, and the inherited ones to Xrep, in one pass over X: a warp takes runs of
+// consecutive tokens of equal length.  (Dealt by gaps between list entries, the longest gap held
+// everybody up: 56 us instead of 17 at T = 8192, r/T = 0.5, d = 1536.)
+template <int U, int V>
+static __device__ __forceinline__ void gather_all_rows(const GatherJob& gj, int g, int nw, int lane, unsigned* status) {
+    const __nv_bfloat16* X = reinterpret_cast<const __nv_bfloat16*>(gj.X);
+    __nv_bfloat16* Xrep = reinterpret_cast<__nv_bfloat16*>(gj.Xrep);
+    __nv_bfloat16* Xnon = reinterpret_cast<__nv_bfloat16*>(gj.Xnon);
+    const int run = min(32, (int)(((int64_t)gj.B * gj.T + nw - 1) / nw));
+    const int runs = (gj.T + run - 1) / run;                       // per sequence
+    for (int64_t it = g; it < (int64_t)gj.B * runs; it += nw) {
+        const int b = (int)(it / runs), t0 = (int)(it % runs) * run, t1 = min(t0 + run, gj.T);
+        const int32_t* list = gj.rep_in + (int64_t)b * gj.T;
+        const int cnt = min(max(gj.rep_in_cnt[b], 0), gj.T);
+        int pos = entries_below(list, cnt, t0, lane);
+        const int32_t ahead = pos + lane < cnt ? __ldg(list + pos + lane) : -1;
+        int used = 0;
+        for (int t = t0; t < t1; t += U) {
+            const uint4* src[U];
+            uint4* dst[U];
+            int at[U];                                             // >= 0: list position; < 0: -1 - row of Xnon
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                src[u] = reinterpret_cast<const uint4*>(X); dst[u] = nullptr;
+                at[u] = 0;
+                if (t + u >= t1) continue;
+                const bool rep = used < 32 && __shfl_sync(0xffffffffu, ahead, used & 31) == t + u;
+                at[u] = rep ? pos : -1 - max(t + u - pos, 0);
+                if (rep) { ++pos; ++used; }
+                src[u] = reinterpret_cast<const uint4*>(X + (int64_t)b * gj.xb + (int64_t)(t + u) * gj.ldx);
+                dst[u] = reinterpret_cast<uint4*>(rep ? Xrep + ((int64_t)b * gj.T + at[u]) * (int64_t)gj.d
+                                                      : Xnon + ((int64_t)b * gj.T + (-1 - at[u])) * (int64_t)gj.d);
+            }
+            float ss[U];
+            copy_rows<U, V>(src, dst, gj.d >> 3, lane, ss);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (t + u >= t1) continue;
+                const float inv = inv_of_sumsq(ss[u], lane, status);
+                if (lane != 0) continue;
+                const int64_t o = (int64_t)b * gj.T;
+                gj.inv_norm[o + t + u] = inv;
+                if (at[u] >= 0) { gj.inv_rep[o + at[u]] = inv; gj.role[o + t + u] = at[u] + 1; }
+                else gj.non_tok[o + (-1 - at[u])] = t + u;
+            }
         }
     }
+}
+
+// Algorithm 1 lines 1-2, by the preparation warps of all CTAs (warp `g` of `nw`): sixteen loads in flight
+// per lane, over as many rows as it takes
+static __device__ __noinline__ void gather_short_rows(const GatherJob gj, int g, int nw, int lane, unsigned* status) {
+    gather_entries<4, 4>(gj, g, nw, lane, true, status);
+}
+static __device__ __noinline__ void gather_compact(const GatherJob gj, int g, int nw, int lane, unsigned* status) {
+    gather_entries<1, 16>(gj, g, nw, lane, false, status);
+    if (gj.d <= 1024) gather_all_rows<4, 4>(gj, g, nw, lane, status);
+    else gather_all_rows<1, 16>(gj, g, nw, lane, status);
+}
+static __device__ __forceinline__ void gather_rows(const GatherJob& gj, int g, int nw, int lane, unsigned* status) {
+    if (compact_wanted(gj, lane)) gather_compact(gj, g, nw, lane, status);
+    else if (gj.d <= 1024) gather_short_rows(gj, g, nw, lane, status);
+    else gather_entries<1, 16>(gj, g, nw, lane, true, status);
 }
 
 // ---------------------------------------------------------------- fp32 rows as three bf16 planes
@@ -522,23 +723,14 @@ static __device__ __forceinline__ float split_row(const float4* __restrict__ src
 }
 // Preparation of an fp32 call, warp `g` of `nw`: planes and inverse norms of every row of X, and of
 // the rows of the inherited list (checked and scattered into the role map as in gather_rows).
-static __device__ __forceinline__ void split_rows(const SplitJob& sj, int g, int nw, int lane, unsigned* status) {
+static __device__ __noinline__ void split_rows(const SplitJob& sj, int g, int nw, int lane, unsigned* status) {
     const int64_t n_rows = (int64_t)sj.B * sj.T;
     const int64_t prow_len = 3 * (int64_t)sj.dpad;
     // list entries first: they hang on two more loads than the plain rows
     if (sj.rep_in != nullptr) {
-        int b = 0;
         int64_t item = g;
-        while (b < sj.B) {
-            int cnt = sj.rep_in_cnt[b];
-            if (cnt < 0 || cnt > sj.T) {
-                if (g == 0 && lane == 0) atomicOr(status, ST_BAD_COUNT);
-                cnt = cnt < 0 ? 0 : sj.T;
-            }
-            if (g == 0 && lane == 0) sj.r_eff[b] = cnt;
-            if (item >= cnt) { item -= cnt; ++b; continue; }
-            const int i = (int)item;
-            item += nw;
+        for (ListCursor cur(sj.rep_in_cnt, sj.T, sj.B, g == 0, sj.r_eff, lane, status); cur.find(item); item += nw) {
+            const int b = cur.b, i = cur.i;
             const int32_t* list = sj.rep_in + (int64_t)b * sj.T;
             const int32_t idx = list[i];
             bool ok = idx >= 0 && idx < sj.T;

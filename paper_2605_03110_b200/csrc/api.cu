@@ -60,8 +60,8 @@ bool use_split(const ada_ctx* ctx, ada_dtype dt) {
            gram_tc_available();
 }
 
-// the pair-CTA form of the tensor-core kernel, or the one-CTA form?
-bool use_pair(const ada_ctx* ctx, int64_t B, int64_t T, int64_t d, ada_dtype dt) {
+// the pair-CTA form of the tensor-core kernel, or the one-CTA form?  full: full selection, else a cross-Gram
+bool use_pair(const ada_ctx* ctx, int64_t B, int64_t T, int64_t d, ada_dtype dt, bool full) {
     if (ctx->engine == ADA_ENGINE_TCGEN05_PAIR) return true;
     if (ctx->engine != ADA_ENGINE_AUTO) return false;
     // Measured against the one-CTA kernel, whose narrow tiles occupy every SM where the pair kernel
@@ -70,7 +70,12 @@ bool use_pair(const ada_ctx* ctx, int64_t B, int64_t T, int64_t d, ada_dtype dt)
     // d = 1600: 55.8 -> 23.7, step 67.8 -> 30.3), where the contraction is too long to be split only from a few
     // thousand rows on (T = 700, d = 5120: 31.0 against 34.7 us).
     if (dt == ADA_F32) return d >= 256 && (d <= MAX_SPLIT_D_F32 || B * T >= 4096);
-    return d >= 2048 && B * T >= (d <= MAX_SPLIT_D ? 512 : 4096);
+    if (d >= 2048) return B * T >= (d <= MAX_SPLIT_D ? 512 : 4096);
+    // Shorter contractions: a step saves the launch that gathers and normalises (8 x 2048 x 768: 37 -> 29 us
+    // per step; at d = 512 between 0.95 and 1.1 times as fast), a full selection is as fast at
+    // d = 1024, gains above (T = 4096, d = 1536: 32.3 -> 30.0 us) and loses below (T = 4096, d = 768: 23.2
+    // -> 24.8 us).
+    return full ? d > 1024 && B * T >= 1024 : d >= 512;
 }
 
 // plane width of an fp32 row of d elements: whole 64-element K blocks
@@ -395,7 +400,7 @@ static ada_status select_full_impl(ada_ctx* ctx, const void* X, int64_t B, int64
 
     // the gamma scratch is zero on entry (workspace invariant kept by the compaction kernels)
     const bool split = use_split(ctx, dt), tc = use_tc(ctx, dt);
-    const bool pair = (split || tc) && use_pair(ctx, B, T, d, dt);
+    const bool pair = (split || tc) && use_pair(ctx, B, T, d, dt, true);
     // bf16: the pair kernel (and the one-CTA kernel, for many rows of a long contraction) computes
     // the row norms itself, hidden behind the MMAs
     const bool fuse = tc && (pair || (d >= 2048 && B * T >= 4096 && xb == T * ldx));
@@ -481,7 +486,7 @@ static ada_status cascade_impl(ada_ctx* ctx, const void* X, int64_t B, int64_t T
     // planes); the r x r tiles (lines 3-5) and the cross tiles (lines 6-8) follow; for bf16 the
     // norms of X are made beside them and the row's own factor 1/||x_t|| is left to the
     // compaction.
-    const bool inl = fuse && use_pair(ctx, B, T, d, dt);
+    const bool inl = fuse && use_pair(ctx, B, T, d, dt, false);
     // otherwise lines 1-2 are a launch of their own: inverse norms of all rows, inherited list
     // validated, scattered into the role map and its rows gathered into Xrep; for long K the
     // one-CTA tensor-core launch computes line 1's row norms itself
@@ -616,7 +621,7 @@ ada_status ada_nearest_rep(ada_ctx* ctx, const void* X, int64_t B, int64_t T, in
     if (!gram_tc_available() || (split && ctx->splitX == nullptr)) return ADA_ERR_UNSUPPORTED;
     DeviceGuard guard(ctx->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const bool pair = use_pair(ctx, B, T, d, dt);
+    const bool pair = use_pair(ctx, B, T, d, dt, false);
     // role map and keys are zero on entry (workspace invariant); the finish kernel clears them
     SplitJob sj = split_job(ctx, X, B, T, d, ldx, T * ldx);
     sj.rep_in = rep_idx; sj.rep_in_cnt = rep_cnt;

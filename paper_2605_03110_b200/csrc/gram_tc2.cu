@@ -408,10 +408,12 @@ struct alignas(16) SharedPair {
     int abort_flag;
     unsigned norm_cnt[MAX_STAGES];             // norm warps done with a stage
     Plan plan;
-    // the problems and the split job once more: what is not inlined takes them by reference, and reading
-    // the parameter space through a pointer is a trip to memory
+    // the launch's arguments once more: what is not inlined takes them by reference, and reading the
+    // parameter space through a pointer is a trip to memory
     GramProblem seg[2];
     SplitJob split;
+    GatherJob gather;
+    NormJob norms;
     Item item[ITEMS];
     // per epilogue warp (its own column chunks), so that staging needs no barrier across warps
     alignas(16) float col_scale[EPI_WARPS][Stage<SPLIT>::COLS];
@@ -521,7 +523,18 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         const int i = (int)threadIdx.x - 64, n = 32 * EPI_WARPS;
         copy_args(sh.seg[0], seg0, i, n);
         copy_args(sh.seg[1], seg1, i, n);
-        if (SPLIT) copy_args(sh.split, split, i, n);
+        if constexpr (SPLIT) copy_args(sh.split, split, i, n);
+        else if (gather.X != nullptr) copy_args(sh.gather, gather, i, n);
+        if (i == 0) {
+            const GramProblem& cx = (nseg > 1) ? seg1 : seg0;
+            if (norms.X != nullptr) {
+                sh.norms = norms;
+            } else {                                 // cascade step: the left operand of the cross segment
+                sh.norms.X = cx.A; sh.norms.ldx = cx.lda; sh.norms.n_rows = (int64_t)cx.B * cx.rows; sh.norms.d = cx.d;
+                sh.norms.inv_norm = cx.inv_out;
+                sh.norms.batch = cx.a_batch; sh.norms.rows_per_seq = cx.rows;
+            }
+        }
     }
     if (threadIdx.x == 32) {                         // descriptors are fetched before the first copy needs them
         prefetch_map(&maps.a[0]); prefetch_map(&maps.b[0]); prefetch_map(&maps.bt[0]);
@@ -544,7 +557,7 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         // the start.  Items are dealt across the SMs first, so that a
         // short list is read by all of them.  One arrival per CTA.
         const int g = (warp - 2) * (int)gridDim.x + (int)blockIdx.x, nw = (int)gridDim.x * EPI_WARPS;
-        if constexpr (!SPLIT) gather_rows(gather, g, nw, lane, status);
+        if constexpr (!SPLIT) gather_rows(gather, sh.gather, g, nw, lane, status);
         else split_rows(sh.split, g, nw, lane, status);
         // the rows just written are read by TMA (async proxy) from other CTAs
         asm volatile("fence.proxy.async.global;" ::: "memory");
@@ -713,21 +726,11 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         float* cs = sh.col_scale[warp - 2];
         int* ct = sh.col_token[warp - 2];
         const GramProblem& cx = (nseg > 1) ? seg1 : seg0;
-        if (norms.X != nullptr) {         // full selection: row norms with plain loads
-            norm_rows(norms, blockIdx.x * EPI_WARPS + (warp - 2), gridDim.x * EPI_WARPS, lane, dep_ctr + 1, status);
-        }
-        // Cascade step with several column tiles: 1/||x_t|| of every row with plain loads, behind the first
-        // main loops.  Nothing in this launch waits for them (the row factor is applied by the
-        // compaction), but everything waits for the triangle: its tiles go first.
-        bool norms_due = !cx.tri && cx.inv_out != nullptr && !smem_norms && !compact;
-        auto make_norms = [&]() __attribute__((always_inline)) {
-            NormJob nj;
-            nj.X = cx.A; nj.ldx = cx.lda; nj.n_rows = (int64_t)cx.B * cx.rows; nj.d = cx.d;
-            nj.inv_norm = cx.inv_out;
-            nj.batch = cx.a_batch; nj.rows_per_seq = cx.rows;
-            norm_rows(nj, blockIdx.x * EPI_WARPS + (warp - 2), gridDim.x * EPI_WARPS, lane, dep_ctr + 1, status);
-            norms_due = false;
-        };
+        // 1/||x_t|| of every row of X with plain loads, behind the first main loops.  Full selection: at once, the
+        // epilogues need them.  Cascade step with several column tiles: nothing in this launch waits
+        // for them (the row factor is applied by the compaction), but everything waits for the
+        // triangle, so its tiles go first.
+        bool norms_due = norms.X != nullptr || (!cx.tri && cx.inv_out != nullptr && !smem_norms && !compact);
         // row norms out of the A tiles in shared memory (streaming form): warps 6..9, thread lrow owns
         // row lrow of the CTA's tile and follows the ring exactly as the producer fills it
         const bool ring_norms = smem_norms && sub == 1 && !cx.tri && cx.inv_out != nullptr;
@@ -760,7 +763,10 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
 #pragma unroll 1
         for (int it = 0;; ++it) {
             const Item& w = item_at(it);
-            if (norms_due && (w.kind == 0 || !(w.seg ? seg1 : seg0).tri)) make_norms();
+            if (norms_due && (norms.X != nullptr || w.kind == 0 || !(w.seg ? seg1 : seg0).tri)) {
+                norm_rows(sh.norms, blockIdx.x * EPI_WARPS + (warp - 2), gridDim.x * EPI_WARPS, lane, dep_ctr + 1, status);
+                norms_due = false;
+            }
             if (w.kind == 0) break;
             if (w.kind == 2) continue;
             const int sg = w.seg, col0 = w.col0, ncols = w.ncols, row0 = w.row0;

@@ -321,10 +321,7 @@ static __device__ __forceinline__ float inv_of_sumsq(float ss, int lane, unsigne
 }
 // Executed by the norm warps of every CTA: warp `w` of `nw` takes rows w, w+nw, ...; when a
 // warp has stored its last row it bumps the counter, so counter == nw means "all rows done".
-// (Not inlined, like the other parts that run once: a Gram launch fetches its instructions cold, and
-// its start-up gets longer with every line of code that lies between those it executes.  The
-// arguments come by value: reading kernel parameters through a pointer is a trip to memory.)
-static __device__ __noinline__ void norm_rows(const NormJob job, int w, int nw, int lane, unsigned* counter,
+static __device__ __forceinline__ void norm_rows(const NormJob& job, int w, int nw, int lane, unsigned* counter,
                                               unsigned* status) {
     const int nvec = job.d >> 3;
     const __nv_bfloat16* X = reinterpret_cast<const __nv_bfloat16*>(job.X);
@@ -667,19 +664,19 @@ static __device__ __forceinline__ void gather_all_rows(const GatherJob& gj, int 
     }
 }
 
-// Algorithm 1 lines 1-2, by the preparation warps of all CTAs (warp `g` of `nw`): sixteen loads in flight
-// per lane, over as many rows as it takes
-static __device__ __noinline__ void gather_short_rows(const GatherJob gj, int g, int nw, int lane, unsigned* status) {
-    gather_entries<4, 4>(gj, g, nw, lane, true, status);
-}
-static __device__ __noinline__ void gather_compact(const GatherJob gj, int g, int nw, int lane, unsigned* status) {
+// Algorithm 1 lines 1-2, by the preparation warps of all CTAs (warp `g` of `nw`).  (A single row at a time
+// outside the copying-out form: a warp has one or two, and several at once cost more code, fetched
+// cold, than they save.)
+static __device__ __noinline__ void gather_compact(const GatherJob& gj, int g, int nw, int lane, unsigned* status) {
     gather_entries<1, 16>(gj, g, nw, lane, false, status);
     if (gj.d <= 1024) gather_all_rows<4, 4>(gj, g, nw, lane, status);
     else gather_all_rows<1, 16>(gj, g, nw, lane, status);
 }
-static __device__ __forceinline__ void gather_rows(const GatherJob& gj, int g, int nw, int lane, unsigned* status) {
-    if (compact_wanted(gj, lane)) gather_compact(gj, g, nw, lane, status);
-    else if (gj.d <= 1024) gather_short_rows(gj, g, nw, lane, status);
+// (gs: the same job in shared memory.  The rare form is not inlined: a Gram launch fetches its
+// instructions cold, and its start-up gets longer with every line of code between those it executes.)
+static __device__ __forceinline__ void gather_rows(const GatherJob& gj, const GatherJob& gs, int g, int nw, int lane,
+                                                   unsigned* status) {
+    if (compact_wanted(gj, lane)) gather_compact(gs, g, nw, lane, status);
     else gather_entries<1, 16>(gj, g, nw, lane, true, status);
 }
 

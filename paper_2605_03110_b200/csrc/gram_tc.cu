@@ -222,9 +222,11 @@ struct alignas(16) SharedTc {
     uint4 tile_tab[TAB];
     int seq_len[2][Shape<SHORTK>::PLAN_B + 1];     // per segment: sequence lengths ...
     int seq_first[2][Shape<SHORTK>::PLAN_B + 1];   // ... and first tile ids (entry B: tile count)
-    // per epilogue warp, so that staging needs no barrier across warps
-    alignas(16) float col_scale[Shape<SHORTK>::EPI_WARPS][BN];
-    alignas(16) int col_token[Shape<SHORTK>::EPI_WARPS][BN];
+    // column factors of a tile, per epilogue set, in alternating buffers: each of the set's four warps
+    // stages a quarter, `staged` completes when all have
+    unsigned long long staged[Shape<SHORTK>::EPI_WARPS / 4];
+    alignas(16) float col_scale[Shape<SHORTK>::EPI_WARPS / 4][2][BN];
+    alignas(16) int col_token[Shape<SHORTK>::EPI_WARPS / 4][2][BN];
 };
 template <bool SHORTK>
 constexpr int smem_tc_bytes() {
@@ -282,6 +284,7 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
             mbar_init(&sh.tmem_empty[a], 4);      // one arrival per epilogue warp
         }
         mbar_init(&sh.drain, 1);
+        for (int q = 0; q < Shape<SHORTK>::EPI_WARPS / 4; ++q) mbar_init(&sh.staged[q], 4);
         sh.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -577,8 +580,7 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
         // ------------------------------------------------ epilogue (warps 2..5, and 6..9 without norm warps)
         const int quad = warp & 3;                    // TMEM lane quadrant this warp may read
         const unsigned eset = (unsigned)(warp - 2) >> 2;   // which of the two sets
-        float* cs = sh.col_scale[warp - 2];
-        int* ct = sh.col_token[warp - 2];
+        unsigned n_staged = 0;                        // tiles of this set so far
         const unsigned dep_total = 4u * (unsigned)tiles0;
         bool dep_ok = !(nseg > 1 && tiles0 > 0);
         bool norm_ok = norms.X == nullptr;           // row norms computed by this launch's norm warps
@@ -610,44 +612,40 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
                 if (!wait_counter(dep_ctr + 1, norm_total, lane, abort_flag, 9)) break;
                 norm_ok = true;
             }
-            // stage this tile's column factors (0 for inadmissible columns); warp-private copy
-            __syncwarp();
+            // stage this tile's column factors (0 for inadmissible columns), a quarter of them per warp.
+            // (With a short contraction the epilogue is the critical path and every instruction of a warp
+            // that has its scheduler almost to itself is exposed: four warps staging all 256 columns
+            // each took 1.8 of the 3.3 us per tile.  A warp is never more than one tile ahead of
+            // another, hence two buffers.)
+            float* cs = sh.col_scale[eset][n_staged & 1u];
+            int* ct = sh.col_token[eset][n_staged & 1u];
             {
-                // all of the tile's global loads are issued before the first is used: with a
-                // short contraction the epilogue is the critical path, and eight dependent
-                // round trips to L2 would be most of it
-                float fb[BN / 32];
-                unsigned gate[BN / 32] = {};
-                int tk[BN / 32] = {};
+                constexpr int Q = BN / 32 / 4;
+                float fb[Q];
+                unsigned gate[Q] = {};
+                int tk[Q] = {};
                 // (columns past the tile are clamped to its last one and discarded afterwards,
                 // so that no load hangs on a data-dependent branch)
                 const int last = pc.n - 1;
                 const unsigned thr_b = (!p.tri && p.tau_seq != nullptr) ? __float_as_uint(tau_threshold(p.tau_seq[pc.b])) : p.thr_bits;
 #pragma unroll
-                for (int q = 0; q < BN / 32; ++q)
-                    fb[q] = __ldcg(p.inv_b + o + min(pc.col0 + lane + 32 * q, last));
-                if (!p.tri) {
+                for (int q = 0; q < Q; ++q) {
+                    const int64_t at = o + min(pc.col0 + lane + 32 * (quad * Q + q), last);
+                    fb[q] = __ldcg(p.inv_b + at);
                     // representative removed at line 5 (written earlier in this launch: read at L2)
-#pragma unroll
-                    for (int q = 0; q < BN / 32; ++q)
-                        gate[q] = __ldcg(p.col_gate + o + min(pc.col0 + lane + 32 * q, last));
-                }
-                if (!p.tri && p.causal) {
-#pragma unroll
-                    for (int q = 0; q < BN / 32; ++q)
-                        tk[q] = p.col_token[o + min(pc.col0 + lane + 32 * q, last)];
+                    if (!p.tri) gate[q] = __ldcg(p.col_gate + at);
+                    if (!p.tri && p.causal) tk[q] = __ldg(p.col_token + at);
                 }
 #pragma unroll
-                for (int q = 0; q < BN / 32; ++q) {
-                    const int c = lane + 32 * q, col = pc.col0 + c;
+                for (int q = 0; q < Q; ++q) {
+                    const int c = lane + 32 * (quad * Q + q), col = pc.col0 + c;
                     const bool live = c < ncols && col < pc.n;
-                    if (c < ncols32) {
-                        cs[c] = (live && (p.tri || gate[q] < thr_b)) ? fb[q] : 0.f;
-                        ct[c] = (live && !p.tri && p.causal) ? tk[q] : col;
-                    }
+                    cs[c] = (live && (p.tri || gate[q] < thr_b)) ? fb[q] : 0.f;
+                    ct[c] = (live && !p.tri && p.causal) ? tk[q] : col;
                 }
             }
             __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.staged[eset]);
             // this thread's row: its role and inverse norm are fetched while the MMAs finish
             const int row = pc.row0 + quad * 32 + lane;
             const bool row_live = row < pc.m;
@@ -657,7 +655,9 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
             const bool inv_early = defer || !(p.wait_norm_a && !norm_ok);
             float inv_row = defer ? 1.0f : ((row_live && inv_early) ? __ldcg(p.inv_a + o + row) : 0.f);
             // warp-uniform outcome of the bounded wait
-            const bool got = mbar_wait(&sh.tmem_full[acc], acc_ph, abort_flag, 4);
+            const bool got = mbar_wait(&sh.staged[eset], n_staged & 1u, abort_flag, 4) &&
+                             mbar_wait(&sh.tmem_full[acc], acc_ph, abort_flag, 4);
+            ++n_staged;
             if (!__all_sync(0xffffffffu, got)) break;
             tcgen05_fence_after();
             const bool need_cmp = p.tri ? (pc.col0 + ncols > pc.row0) : (p.causal != 0);
@@ -678,14 +678,7 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
             } else {
                 auto consume = [&](const unsigned (&r)[32], int c0) {
                     if (!need_cmp) {
-#pragma unroll
-                        for (int j = 0; j < 32; j += 4) {
-                            const float4 f = *reinterpret_cast<const float4*>(cs + c0 + j);
-                            mx4[0] = fmaxf(mx4[0], fabsf(__uint_as_float(r[j])) * f.x);
-                            mx4[1] = fmaxf(mx4[1], fabsf(__uint_as_float(r[j + 1])) * f.y);
-                            mx4[0] = fmaxf(mx4[0], fabsf(__uint_as_float(r[j + 2])) * f.z);
-                            mx4[1] = fmaxf(mx4[1], fabsf(__uint_as_float(r[j + 3])) * f.w);
-                        }
+                        row_max32(r, cs + c0, mx4[0], mx4[1]);
                     } else {
 #pragma unroll
                         for (int j = 0; j < 32; j += 4) {

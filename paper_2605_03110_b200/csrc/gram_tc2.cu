@@ -415,9 +415,12 @@ struct alignas(16) SharedPair {
     GatherJob gather;
     NormJob norms;
     Item item[ITEMS];
-    // per epilogue warp (its own column chunks), so that staging needs no barrier across warps
-    alignas(16) float col_scale[EPI_WARPS][Stage<SPLIT>::COLS];
-    alignas(16) int col_token[EPI_WARPS][Stage<SPLIT>::COLS];
+    // column factors of a tile, per epilogue set (the chunks that it reads), in alternating buffers: each of
+    // the set's four warps stages a quarter, `staged` completes when all have.  A warp is never more
+    // than one tile ahead of another.
+    unsigned long long staged[SUBS];
+    alignas(16) float col_scale[SUBS][2][Stage<SPLIT>::COLS];
+    alignas(16) int col_token[SUBS][2][Stage<SPLIT>::COLS];
 };
 template <bool SPLIT>
 constexpr int smem_pair_bytes() { return Ring<SPLIT>::BYTES + (int)sizeof(SharedPair<SPLIT>) + 1024; }
@@ -507,6 +510,7 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         mbar_init(&sh.drain, 1);
         mbar_init(&sh.planned, 1);
         mbar_init(&sh.prep_seen, 1);
+        for (int q = 0; q < SUBS; ++q) mbar_init(&sh.staged[q], 4);
         for (int q = 0; q < SUBS; ++q) { mbar_init(&sh.norm_seen[q], 1); mbar_init(&sh.dep_seen[q], 1); }
         sh.pub_cnt = 0u;
         sh.abort_flag = 0;
@@ -723,8 +727,7 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         // the two warps of a lane quadrant share a tile's 32-column chunks (sub, sub + 2, ..), so
         // that a finished accumulator is read out by eight warps.
         const int quad = warp & 3, sub = (warp - 2) >> 2;
-        float* cs = sh.col_scale[warp - 2];
-        int* ct = sh.col_token[warp - 2];
+        unsigned n_staged = 0;                       // tiles of this set so far
         const GramProblem& cx = (nseg > 1) ? seg1 : seg0;
         // 1/||x_t|| of every row of X with plain loads, behind the first main loops.  Full selection: at once, the
         // epilogues need them.  Cascade step with several column tiles: nothing in this launch waits
@@ -777,6 +780,8 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
             if (solo && (int)acc != sub) continue;
             // the warp's chunks of 32 columns: cfirst, cfirst + cstep, .. below nch
             const int cfirst = solo ? 0 : sub, cstep = solo ? 1 : SUBS;
+            float* cs = sh.col_scale[sub][n_staged & 1u];
+            int* ct = sh.col_token[sub][n_staged & 1u];
             const int64_t o = (int64_t)w.b * p.cap;
             const int nch = ncols >> 5;
             const int arows = p.tri ? BM : hrows;
@@ -924,38 +929,34 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                 dep_ok = true;
                 if (warp == 2 && lane == 0) TRACE(4);
             }
-            // Column factors of the warp's chunks.  All of a group's global loads are issued before the
-            // first is used (columns past the tile are clamped to its last one and discarded
-            // afterwards, so that no load hangs on a data-dependent branch).
-            __syncwarp();
+            // Column factors: the set's chunks are dealt to its four warps.  (Columns past the tile are
+            // clamped to its last one and discarded afterwards, so that no load hangs on a
+            // data-dependent branch.)
             const int last = max(w.n - 1, 0);
-#pragma unroll 1
-            for (int g = cfirst; g < nch; g += 4 * cstep) {
-                float fb[4];
-                unsigned gate[4] = {};
-                int tk[4] = {};
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int64_t at = o + min(col0 + 32 * (g + k * cstep) + lane, last);
-                    fb[k] = __ldcg(p.inv_b + at);
-                    // representative removed at line 5 (written earlier in this launch: read at L2)
-                    if (!p.tri) gate[k] = __ldcg(p.col_gate + at);
-                    if (!p.tri && p.causal) tk[k] = __ldcg(p.col_token + at);
-                }
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int c = g + k * cstep, col = col0 + 32 * c + lane;
-                    if (c >= nch) break;
-                    const bool live = col < w.n;
-                    const int at = (solo ? 32 * c : 32 * (c >> 1)) + lane;
-                    cs[at] = (live && (p.tri || gate[k] < thr_b)) ? fb[k] : 0.f;
-                    ct[at] = (live && !p.tri && p.causal) ? tk[k] : col;
-                }
+            for (int e = 0; e < (St::COLS / 32 + 3) / 4; ++e) {
+                const int c = cfirst + (quad + 4 * e) * cstep, col = col0 + 32 * c + lane;
+                if (c >= nch) break;
+                const int64_t from = o + min(col, last);
+                const float f = __ldcg(p.inv_b + from);
+                // representative removed at line 5 (written earlier in this launch: read at L2)
+                const unsigned gate = p.tri ? 0u : __ldcg(p.col_gate + from);
+                const int tk = !p.tri && p.causal ? __ldcg(p.col_token + from) : col;
+                const bool live = col < w.n;
+                const int at = 32 * (quad + 4 * e) + lane;
+                cs[at] = (live && (p.tri || gate < thr_b)) ? f : 0.f;
+                ct[at] = live ? tk : col;
             }
             __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.staged[sub]);
             }
             }
             if (!ok) break;
+            {
+                const bool got = mbar_wait(&sh.staged[sub], n_staged & 1u, abort_flag, 4);
+                ++n_staged;
+                if (!__all_sync(0xffffffffu, got)) break;
+            }
             if (w.parts == 1) {
                 const bool got = mbar_wait(&sh.tmem_full[acc], acc_ph, abort_flag, 4);
                 if (!__all_sync(0xffffffffu, got)) break;

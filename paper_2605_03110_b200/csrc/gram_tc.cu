@@ -59,9 +59,9 @@ struct Shape {
 // Algorithm 1 lines 3-4 on the gathered representatives) and a cross one (lines 7-8).
 // Their output tiles form one list, triangular tiles first, dealt round-robin to the
 // persistent CTAs.  When both are present the cross epilogues need line 5's verdict on
-// every column, i.e. the finished triangular segment: each epilogue warp bumps a global
-// counter after publishing a triangular tile's maxima, and a cross epilogue waits (bounded)
-// for the counter to reach 4 x (number of triangular tiles) before it stages its column
+// every column, i.e. the finished triangular segment: a global counter is bumped after a
+// triangular tile's maxima have been published, and a cross epilogue waits (bounded)
+// for the counter to reach the number of triangular tiles before it stages its column
 // factors.  The cross MAIN LOOPS do not wait, so the short r x r problem hides behind them.
 // Triangular tiles precede cross tiles in every CTA's order and wait on nothing, and the
 // launch is cooperative unless nothing else can keep its CTAs apart (coop_begin), so the wait
@@ -219,6 +219,8 @@ struct alignas(16) SharedTc {
     int abort_flag;
     int tiles0, tiles1, par0, par1;
     int wide0, wide1;           // widest tile of each segment (fixes the segment's ring geometry)
+    unsigned long long dep_seen[2];   // per epilogue set: every triangular tile of the grid is done
+    unsigned pub[2];            // per epilogue set: warps that have published their share of a triangular tile
     uint4 tile_tab[TAB];
     int seq_len[2][Shape<SHORTK>::PLAN_B + 1];     // per segment: sequence lengths ...
     int seq_first[2][Shape<SHORTK>::PLAN_B + 1];   // ... and first tile ids (entry B: tile count)
@@ -284,6 +286,7 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
             mbar_init(&sh.tmem_empty[a], 4);      // one arrival per epilogue warp
         }
         mbar_init(&sh.drain, 1);
+        for (int q = 0; q < 2; ++q) { mbar_init(&sh.dep_seen[q], 1); sh.pub[q] = 0u; }
         for (int q = 0; q < Shape<SHORTK>::EPI_WARPS / 4; ++q) mbar_init(&sh.staged[q], 4);
         sh.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -581,7 +584,7 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
         const int quad = warp & 3;                    // TMEM lane quadrant this warp may read
         const unsigned eset = (unsigned)(warp - 2) >> 2;   // which of the two sets
         unsigned n_staged = 0;                        // tiles of this set so far
-        const unsigned dep_total = 4u * (unsigned)tiles0;
+        const unsigned dep_total = (unsigned)tiles0;
         bool dep_ok = !(nseg > 1 && tiles0 > 0);
         bool norm_ok = norms.X == nullptr;           // row norms computed by this launch's norm warps
         const unsigned norm_total = (unsigned)(gridDim.x * NORM_WARPS);      // cross epilogues must see segment 0 finished
@@ -605,7 +608,16 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
             const int ncols32 = (ncols + 31) & ~31;   // TMEM is read 32 columns at a time
             if (sg == 1 && !dep_ok) {
                 // every triangular tile of this launch first (line 5 before line 7)
-                if (!wait_counter(dep_ctr, dep_total, lane, abort_flag, 5)) break;
+                // (one warp of a set polls: with all of them polling, the counter's L2 slice is saturated
+                // and the arrivals themselves are late)
+                bool good;
+                if (quad == 2) {
+                    good = wait_counter(dep_ctr, dep_total, lane, abort_flag, 5);
+                    if (lane == 0) mbar_arrive(&sh.dep_seen[eset]);
+                } else {
+                    good = __all_sync(0xffffffffu, mbar_wait(&sh.dep_seen[eset], 0, abort_flag, 5)) && *abort_flag == 0;
+                }
+                if (!good) break;
                 dep_ok = true;
             }
             if (p.wait_norm_b && !norm_ok) {
@@ -722,10 +734,14 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
                 }
             }
             if (sg == 0 && nseg > 1) {
-                // publish: this warp's share of a triangular tile is in global memory
+                // publish: this warp's share of a triangular tile is in global memory; one arrival per
+                // tile, by the last of the set's four warps
                 __threadfence();
                 __syncwarp();
-                if (lane == 0) atomicAdd(dep_ctr, 1u);
+                if (lane == 0 && (atomicAdd(&sh.pub[eset], 1u) & 3u) == 3u) {
+                    __threadfence();
+                    atomicAdd(dep_ctr, 1u);
+                }
             }
         }
     } else if (!SHORTK && norms.X != nullptr) {

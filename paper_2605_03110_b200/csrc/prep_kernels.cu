@@ -52,31 +52,13 @@ struct Vec16<__nv_bfloat16> {
     }
 };
 
-// Sum of squares of one row, one warp, four independent 128-bit loads in flight per lane.
-template <typename T>
-__device__ __forceinline__ float warp_row_sumsq(const uint4* __restrict__ src, int nvec, int lane) {
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-    int v = lane;
-    for (; v + 96 < nvec; v += 128) {
-        const uint4 a = __ldg(src + v), b = __ldg(src + v + 32), c = __ldg(src + v + 64),
-                    e = __ldg(src + v + 96);
-        s0 += Vec16<T>::sumsq(a);
-        s1 += Vec16<T>::sumsq(b);
-        s2 += Vec16<T>::sumsq(c);
-        s3 += Vec16<T>::sumsq(e);
-    }
-    for (; v < nvec; v += 32) s0 += Vec16<T>::sumsq(__ldg(src + v));
-    float ss = (s0 + s1) + (s2 + s3);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    return ss;
-}
-
-// Warps [0, n_rows) normalise: inv_norm[row] (and Xhat).  Warps [n_rows, 2 n_rows) serve the
-// inherited list (Algorithm 1 "Require" and line 2): warp (b, i) with i < count validates
-// entry i (in range, strictly above entry i-1), records role[token] = i+1, copies the raw
-// row to Xrep[b, i] and stores its inverse norm.  Both halves read X directly, so there is
+// Warps [0, ceil(n_rows / NORM_ROWS)) normalise NORM_ROWS rows each: inv_norm[row] (and Xhat).  The warps
+// after them serve the inherited list (Algorithm 1 "Require" and line 2): warp (b, i) with i < count
+// validates entry i (in range, strictly above entry i-1), records role[token] = i+1, copies the raw
+// row to Xrep[b, i] and stores its inverse norm.  Both kinds read X directly, so there is
 // no dependency between them and no separate scatter pass.
+constexpr int NORM_ROWS = 2;
+
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_norm_gather(const T* __restrict__ X, int64_t n_rows, int Tseq, int d, int64_t ldx, int64_t xb,
@@ -87,31 +69,57 @@ k_norm_gather(const T* __restrict__ X, int64_t n_rows, int Tseq, int d, int64_t 
     grid_dep_wait();
     const int lane = threadIdx.x & 31;
     int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (inv_norm == nullptr && Xhat == nullptr) w += n_rows;   // gather-only launch: list warps only
+    const int64_t n_norm_warps = (n_rows + NORM_ROWS - 1) / NORM_ROWS;
+    if (inv_norm == nullptr && Xhat == nullptr) w += n_norm_warps;   // gather-only launch: list warps only
     constexpr int N = Vec16<T>::N;
     const int nvec = d / N;  // d*es is a multiple of 16 bytes
-    if (w < n_rows) {
-        const int64_t row = w;
+    if (w < n_norm_warps) {
         // row (b, t) of X starts at b * xb + t * ldx (xb = Tseq * ldx for stacked sequences,
         // the head width for heads interleaved inside one row)
-        const uint4* src = reinterpret_cast<const uint4*>(X + (row / Tseq) * xb + (row % Tseq) * ldx);
-        const float ss = warp_row_sumsq<T>(src, nvec, lane);
-        float inv = 0.f;
-        if (!(ss <= 3.0e38f)) {  // NaN or overflow to Inf
-            if (lane == 0) atomicOr(status, ST_NONFINITE);
-        } else if (ss > 0.f) {
-            inv = 1.0f / sqrtf(ss);
-        } else if (lane == 0) {
-            atomicAdd(status + 1, 1u);
+        const uint4* src[NORM_ROWS];
+        float ss[NORM_ROWS];
+#pragma unroll
+        for (int u = 0; u < NORM_ROWS; ++u) {
+            const unsigned row = (unsigned)min(w * NORM_ROWS + u, n_rows - 1);
+            src[u] = reinterpret_cast<const uint4*>(X + (int64_t)(row / (unsigned)Tseq) * xb + (int64_t)(row % (unsigned)Tseq) * ldx);
+            ss[u] = 0.f;
         }
-        if (inv_norm != nullptr && lane == 0) inv_norm[row] = inv;
-        if (Xhat != nullptr) {
-            uint4* dst = reinterpret_cast<uint4*>(Xhat + row * (int64_t)d);
-            for (int v = lane; v < nvec; v += 32) dst[v] = Vec16<T>::scale(__ldg(src + v), inv);
+        for (int v = lane; v < nvec; v += 128) {
+            uint4 x[NORM_ROWS][4];
+#pragma unroll
+            for (int u = 0; u < NORM_ROWS; ++u)
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    x[u][q] = v + 32 * q < nvec ? __ldg(src[u] + v + 32 * q) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int u = 0; u < NORM_ROWS; ++u)
+                ss[u] += (Vec16<T>::sumsq(x[u][0]) + Vec16<T>::sumsq(x[u][1])) + (Vec16<T>::sumsq(x[u][2]) + Vec16<T>::sumsq(x[u][3]));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int u = 0; u < NORM_ROWS; ++u) ss[u] += __shfl_xor_sync(0xffffffffu, ss[u], o);
+#pragma unroll
+        for (int u = 0; u < NORM_ROWS; ++u) {
+            const int64_t row = w * NORM_ROWS + u;
+            if (row >= n_rows) break;
+            float inv = 0.f;
+            if (!(ss[u] <= 3.0e38f)) {  // NaN or overflow to Inf
+                if (lane == 0) atomicOr(status, ST_NONFINITE);
+            } else if (ss[u] > 0.f) {
+                inv = 1.0f / sqrtf(ss[u]);
+            } else if (lane == 0) {
+                atomicAdd(status + 1, 1u);
+            }
+            if (inv_norm != nullptr && lane == 0) inv_norm[row] = inv;
+            if (Xhat != nullptr) {
+                uint4* dst = reinterpret_cast<uint4*>(Xhat + row * (int64_t)d);
+                for (int v = lane; v < nvec; v += 32) dst[v] = Vec16<T>::scale(__ldg(src[u] + v), inv);
+            }
         }
         return;
     }
-    w -= n_rows;
+    w -= n_norm_warps;
     if (rep_in == nullptr || w >= n_rows) return;
     const int b = (int)(w / Tseq), i = (int)(w % Tseq);
     int cnt = rep_in_cnt[b];
@@ -282,7 +290,7 @@ cudaError_t launch_norm_gather(ada_ctx* ctx, const void* X, int B, int T, int d,
     int G = 32;
     if (nvec <= 16) for (G = 1; G < nvec; G <<= 1) {}
     const int rpw = G == 32 ? 1 : (32 / G) * NORM_U;
-    const int64_t n_norm_warps = (n_rows + rpw - 1) / rpw;
+    const int64_t n_norm_warps = rpw == 1 ? (n_rows + NORM_ROWS - 1) / NORM_ROWS : (n_rows + rpw - 1) / rpw;
     // list warps: one per list position, or one per rpw positions of a sequence (short rows)
     const int64_t n_list_warps = rpw == 1 ? n_rows : (int64_t)B * ((T + rpw - 1) / rpw);
     const int64_t n_warps = gather_only ? n_list_warps

@@ -60,54 +60,61 @@ __device__ __forceinline__ int clamp_count(const int32_t* cnt, int T) {
 }
 
 // ---------------------------------------------------------------- gather
-// grid (Tp / 32, h), 256 threads.  Positions at or past r (up to the next multiple of 128)
-// are filled with zeros, so that the padding of the last key tile is harmless.
+// grid (at most GATHER_BLOCKS, h), 256 threads; a block takes every gridDim.x-th group of 32 positions (r
+// lives on the device: a grid sized for T is thousands of blocks that only find out that they
+// have nothing to do; T = 8192, r = 410, 32 heads: 9.9 -> 5.5 us).  Positions at or past r (up to
+// the next multiple of 128) are filled with zeros, so that the padding of the last key tile is
+// harmless.
+constexpr int GATHER_BLOCKS = 32;
 __global__ void __launch_bounds__(256)
 k_attn_gather(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __restrict__ K,
               const __nv_bfloat16* __restrict__ V, int T, int Tp, int h, int d_h, int64_t ld,
               const int32_t* __restrict__ rep_idx, const int32_t* __restrict__ rep_cnt,
               __nv_bfloat16* __restrict__ Qr, __nv_bfloat16* __restrict__ Kr,
               __nv_bfloat16* __restrict__ Vt, unsigned* __restrict__ status) {
-    grid_dep_wait();
     __shared__ __nv_bfloat16 vs[32][128 + 8];
     __shared__ int tok[32];
-    const int head = blockIdx.y, p0 = blockIdx.x * 32;
+    grid_dep_wait();
+    grid_dep_launch_next();
+    const int head = blockIdx.y;
     const int r = clamp_count(rep_cnt, T);
     const int rpad = (r + AKV - 1) / AKV * AKV;
-    if (p0 >= rpad) return;
-    if (threadIdx.x < 32) {
-        const int p = p0 + threadIdx.x;
-        int t = p < r ? rep_idx[p] : -1;
-        if (p < r && (t < 0 || t >= T)) { atomicOr(status, ST_BAD_INDEX); t = -1; }
-        tok[threadIdx.x] = t;
-    }
-    __syncthreads();
     const int nvec = d_h >> 3;                       // 16-byte vectors per head row
-    for (int i = threadIdx.x; i < 32 * nvec; i += blockDim.x) {
-        const int pl = i / nvec, v = i % nvec;
-        const int t = tok[pl];
-        uint4 q = make_uint4(0u, 0u, 0u, 0u), k = q, w = q;
-        if (t >= 0) {
-            const int64_t off = (int64_t)t * ld + (int64_t)head * d_h + v * 8;
-            q = __ldg(reinterpret_cast<const uint4*>(Q + off));
-            k = __ldg(reinterpret_cast<const uint4*>(K + off));
-            w = __ldg(reinterpret_cast<const uint4*>(V + off));
+    for (int p0 = blockIdx.x * 32; p0 < rpad; p0 += gridDim.x * 32) {
+        __syncthreads();                             // vs and tok are reused
+        if (threadIdx.x < 32) {
+            const int p = p0 + threadIdx.x;
+            int t = p < r ? rep_idx[p] : -1;
+            if (p < r && (t < 0 || t >= T)) { atomicOr(status, ST_BAD_INDEX); t = -1; }
+            tok[threadIdx.x] = t;
         }
-        const int64_t row = ((int64_t)head * Tp + p0 + pl) * d_h + v * 8;
-        *reinterpret_cast<uint4*>(Qr + row) = q;
-        *reinterpret_cast<uint4*>(Kr + row) = k;
-        *reinterpret_cast<uint4*>(&vs[pl][v * 8]) = w;
-    }
-    __syncthreads();
-    // V^T: thread (c, half) writes 16 consecutive positions of feature c
-    const int c = threadIdx.x >> 1, half = threadIdx.x & 1;
-    if (c < d_h) {
-        __align__(16) __nv_bfloat16 o[16];
+        __syncthreads();
+        for (int i = threadIdx.x; i < 32 * nvec; i += blockDim.x) {
+            const int pl = i / nvec, v = i % nvec;
+            const int t = tok[pl];
+            uint4 q = make_uint4(0u, 0u, 0u, 0u), k = q, w = q;
+            if (t >= 0) {
+                const int64_t off = (int64_t)t * ld + (int64_t)head * d_h + v * 8;
+                q = __ldg(reinterpret_cast<const uint4*>(Q + off));
+                k = __ldg(reinterpret_cast<const uint4*>(K + off));
+                w = __ldg(reinterpret_cast<const uint4*>(V + off));
+            }
+            const int64_t row = ((int64_t)head * Tp + p0 + pl) * d_h + v * 8;
+            *reinterpret_cast<uint4*>(Qr + row) = q;
+            *reinterpret_cast<uint4*>(Kr + row) = k;
+            *reinterpret_cast<uint4*>(&vs[pl][v * 8]) = w;
+        }
+        __syncthreads();
+        // V^T: thread (c, half) writes 16 consecutive positions of feature c
+        const int c = threadIdx.x >> 1, half = threadIdx.x & 1;
+        if (c < d_h) {
+            __align__(16) __nv_bfloat16 o[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) o[i] = vs[half * 16 + i][c];
-        uint4* dst = reinterpret_cast<uint4*>(Vt + ((int64_t)head * d_h + c) * Tp + p0 + half * 16);
-        dst[0] = *reinterpret_cast<const uint4*>(&o[0]);
-        dst[1] = *reinterpret_cast<const uint4*>(&o[8]);
+            for (int i = 0; i < 16; ++i) o[i] = vs[half * 16 + i][c];
+            uint4* dst = reinterpret_cast<uint4*>(Vt + ((int64_t)head * d_h + c) * Tp + p0 + half * 16);
+            dst[0] = *reinterpret_cast<const uint4*>(&o[0]);
+            dst[1] = *reinterpret_cast<const uint4*>(&o[8]);
+        }
     }
 }
 
@@ -204,12 +211,8 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
     // Barriers, TMEM and the rings live across items (a buffer's uses are counted on, so every
     // wait's parity follows from a running count), and the next item's Q, first keys and first
     // score tiles are under way while the softmax warps still write the previous item's rows.
-    grid_dep_wait();
-    const int n = clamp_count(rep_cnt, T);
-    const int nq = (n + AQ - 1) / AQ;
-    const int total = nq * h;
-    if ((int)blockIdx.x >= total) return;              // before anything is set up
     if ((smem_u32(smem) & 1023u) != 0u) {              // the tiles would not be where the swizzle assumes
+        grid_dep_wait();
         if (threadIdx.x == 0) { atomicOr(status, ST_TIMEOUT); status[2] = 299u; }
         return;
     }
@@ -233,10 +236,17 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
                      ::"r"(smem_u32(&sh.tmem_base)), "r"(TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    if (threadIdx.x == 64) { prefetch_map(&maps.q); prefetch_map(&maps.k); prefetch_map(&maps.v); }
     tcgen05_fence_before();
     __syncthreads();
     tcgen05_fence_after();
     const unsigned tmem_base = sh.tmem_base;
+    // everything above is local to the CTA; from here on the predecessor's results are read
+    grid_dep_wait();
+    grid_dep_launch_next();
+    const int n = clamp_count(rep_cnt, T);
+    const int nq = (n + AQ - 1) / AQ;
+    const int total = nq * h;                          // (a CTA without an item falls through to the end)
     if (threadIdx.x == 0) ATRACE(1);
     const int nkv_all = (n + AKV - 1) / AKV;
     const int nkb = (d_h + BK - 1) / BK;               // 64-element K blocks of the first contraction
@@ -528,21 +538,30 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
 
 // ---------------------------------------------------------------- expansion (Section 2.3)
 // One warp per token: a token outside the set takes its nearest representative's output; a
-// token without one (empty set) gets zeros.
+// token without one (empty set) gets zeros.  Bound by the writes (T rows of h d_h floats; the
+// representatives' rows stay in L2): eight 16-byte loads in flight per lane, streaming stores
+// (T = 8192, 32 x 128: 34 -> 24 us).
 __global__ void __launch_bounds__(256)
 k_attn_expand(float* __restrict__ out, int64_t ldo, int T, int width, const int32_t* __restrict__ nearest) {
     grid_dep_wait();
+    grid_dep_launch_next();
     const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (t >= T) return;
     const int s = nearest[t];
     if (s == t) return;
+    const bool none = s < 0 || s >= T;
     float4* dst = reinterpret_cast<float4*>(out + (int64_t)t * ldo);
-    if (s < 0 || s >= T) {
-        for (int v = lane; v < (width >> 2); v += 32) dst[v] = make_float4(0.f, 0.f, 0.f, 0.f);
-        return;
+    const float4* src = reinterpret_cast<const float4*>(out + (int64_t)(none ? t : s) * ldo);
+    const int nvec = width >> 2;
+    for (int v = lane; v < nvec; v += 256) {
+        float4 x[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            x[q] = !none && v + 32 * q < nvec ? __ldcg(src + v + 32 * q) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (v + 32 * q < nvec) __stcs(dst + v + 32 * q, x[q]);
     }
-    const float4* src = reinterpret_cast<const float4*>(out + (int64_t)s * ldo);
-    for (int v = lane; v < (width >> 2); v += 32) dst[v] = __ldcg(src + v);
 }
 
 }  // namespace
@@ -572,7 +591,7 @@ cudaError_t launch_attention_reps(ada_ctx* ctx, const void* Q, const void* K, co
         !make_map(&maps.k, Kr, d_h, Tp, h, d_h, (int64_t)Tp * d_h, AKV) ||
         !make_map(&maps.v, Vt, Tp, d_h, h, Tp, (int64_t)d_h * Tp, d_h))
         return cudaErrorInvalidValue;
-    launch_k(ctx, k_attn_gather, dim3(Tp / 32, h), dim3(256), 0, s, (const __nv_bfloat16*)Q,
+    launch_k(ctx, k_attn_gather, dim3(Tp / 32 < GATHER_BLOCKS ? Tp / 32 : GATHER_BLOCKS, h), dim3(256), 0, s, (const __nv_bfloat16*)Q,
              (const __nv_bfloat16*)K, (const __nv_bfloat16*)V, T, Tp, h, d_h, ld, rep_idx, rep_cnt, Qr, Kr, Vt,
              ctx->status);
     // persistent CTAs, at most one per SM; r (hence the number of work items) lives on the device

@@ -554,6 +554,7 @@ k_nearest_finish(unsigned long long* __restrict__ near_key, int32_t* __restrict_
                  const int32_t* __restrict__ rep_idx, int T, int32_t* __restrict__ nearest_idx,
                  float* __restrict__ nearest_gamma, unsigned* __restrict__ dep_ctr) {
     grid_dep_wait();
+    grid_dep_launch_next();
     const int b = blockIdx.y, t = blockIdx.x * blockDim.x + threadIdx.x;
     if (b == 0 && blockIdx.x == 0 && threadIdx.x < 4) dep_ctr[threadIdx.x] = 0u;   // counters of the Gram launch
     if (t >= T) return;

@@ -1,4 +1,5 @@
-"""ctypes binding of libada.so -- same names as include/ada.h, marshalling only.
+"""Binding of libada.so -- same names as include/ada.h, marshalling only (ctypes; the calls of the
+selection and attention path through the native _pycall module).
 
 Every step of the selection runs inside the CUDA library; this module converts
 torch tensors to pointers, allocates output tensors, and raises on any
@@ -33,6 +34,7 @@ SYMBOLS = [
 ADA_NOALLOC_MAX_T = 16384
 
 _lib = None
+_fast = None             # the _pycall module, once the library is loaded
 
 
 class TauPolicy(C.Structure):
@@ -48,7 +50,7 @@ class AdaError(RuntimeError):
 
 
 def lib() -> C.CDLL:
-    global _lib
+    global _lib, _fast
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(
@@ -94,7 +96,8 @@ def lib() -> C.CDLL:
         for name in SYMBOLS:
             if name not in ("ada_gram_op_count", "ada_status_string"):
                 getattr(L, name).restype = C.c_int
-        _lib = L
+        from . import _pycall
+        _lib, _fast = L, _pycall
     return _lib
 
 
@@ -111,10 +114,14 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return None if t is None else t.data_ptr()
 
 
-def _stream(stream) -> Optional[int]:
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return stream.cuda_stream or None
+def _stream(stream) -> int:
+    if stream is None:           # the current stream's handle without a Stream object around it
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
+
+
+def _raise(st: int, where: str) -> None:
+    raise AdaError(st, where)
 
 
 def dtype_of(t: torch.Tensor) -> int:
@@ -128,10 +135,12 @@ def dtype_of(t: torch.Tensor) -> int:
 def _shape(X: torch.Tensor):
     if X.dim() == 2:
         X = X.unsqueeze(0)
-    if X.dim() != 3 or X.stride(2) != 1 or (X.shape[0] > 1 and X.stride(0) != X.shape[1] * X.stride(1)):
-        raise ValueError("X must be (B,)T x d, unit inner stride, sequences densely stacked")
-    B, T, d = X.shape
-    return X, B, T, d, X.stride(1)
+    if X.dim() == 3:
+        B, T, d = X.shape
+        sb, st, sd = X.stride()
+        if sd == 1 and (B <= 1 or sb == T * st):
+            return X, B, T, d, st
+    raise ValueError("X must be (B,)T x d, unit inner stride, sequences densely stacked")
 
 
 class Context:
@@ -141,12 +150,13 @@ class Context:
         h = C.c_void_p()
         _check(lib().ada_create(C.byref(h), device, maxB, maxT, maxd, dtype), "ada_create")
         self.h, self.device, self.dtype = h, device, dtype
+        self.addr = h.value              # None once closed: the library then reports an invalid argument
         self.maxB, self.maxT, self.maxd = maxB, maxT, maxd
 
     def close(self):
         if self.h:
             lib().ada_destroy(self.h)
-            self.h = None
+            self.h = self.addr = None
 
     def __del__(self):
         try:
@@ -221,9 +231,9 @@ def ada_select_full(ctx: Context, X: torch.Tensor, tau: float, rep_idx=None, rep
         rep_cnt = torch.empty((B,), dtype=torch.int32, device=dev)
     if gamma is None and want_gamma:
         gamma = torch.empty((B, T), dtype=torch.float32, device=dev)
-    _check(lib().ada_select_full(ctx.h, X.data_ptr(), B, T, d, ldx, dtype_of(X), float(tau),
-                                 rep_idx.data_ptr(), rep_cnt.data_ptr(), _ptr(gamma),
-                                 _stream(stream)), "ada_select_full")
+    st = _fast.select_full(ctx.addr, X, B, T, d, ldx, dtype_of(X), tau, rep_idx, rep_cnt, gamma, _stream(stream))
+    if st:
+        _raise(st, "ada_select_full")
     return rep_idx, rep_cnt, gamma
 
 
@@ -250,13 +260,11 @@ def ada_cascade_step(ctx: Context, X: torch.Tensor, tau: float, rep_in: torch.Te
     X, B, T, d, ldx = _shape(X)
     if out is None:
         out = CascadeOut(B, T, X.device, want_gamma)
-    _check(lib().ada_cascade_step(ctx.h, X.data_ptr(), B, T, d, ldx, dtype_of(X), float(tau),
-                                  rep_in.data_ptr(), rep_in_cnt.data_ptr(), out.rep_out.data_ptr(),
-                                  out.rep_out_cnt.data_ptr(), out.add_idx.data_ptr(),
-                                  out.add_cnt.data_ptr(), out.rem_idx.data_ptr(),
-                                  out.rem_cnt.data_ptr(), _ptr(out.gamma_rep),
-                                  _ptr(out.gamma_cross), flags, _stream(stream)),
-           "ada_cascade_step")
+    st = _fast.cascade_step(ctx.addr, X, B, T, d, ldx, dtype_of(X), tau, rep_in, rep_in_cnt, out.rep_out,
+                            out.rep_out_cnt, out.add_idx, out.add_cnt, out.rem_idx, out.rem_cnt, out.gamma_rep,
+                            out.gamma_cross, flags, _stream(stream))
+    if st:
+        _raise(st, "ada_cascade_step")
     return out
 
 
@@ -271,21 +279,22 @@ def ada_cascade_step_adaptive(ctx: Context, X: torch.Tensor, tau_state: torch.Te
     assert tau_state.dtype == torch.float64 and tau_state.is_cuda and tau_state.numel() == B
     if out is None:
         out = CascadeOut(B, T, X.device, want_gamma)
-    _check(lib().ada_cascade_step_adaptive(
-        ctx.h, X.data_ptr(), B, T, d, ldx, dtype_of(X), tau_state.data_ptr(),
-        None if policy is None else C.byref(policy), rep_in.data_ptr(), rep_in_cnt.data_ptr(),
-        out.rep_out.data_ptr(), out.rep_out_cnt.data_ptr(), out.add_idx.data_ptr(),
-        out.add_cnt.data_ptr(), out.rem_idx.data_ptr(), out.rem_cnt.data_ptr(),
-        _ptr(out.gamma_rep), _ptr(out.gamma_cross), _ptr(turnover), flags, _stream(stream)),
-        "ada_cascade_step_adaptive")
+    st = _fast.cascade_step_adaptive(
+        ctx.addr, X, B, T, d, ldx, dtype_of(X), tau_state, None if policy is None else C.addressof(policy), rep_in,
+        rep_in_cnt, out.rep_out, out.rep_out_cnt, out.add_idx, out.add_cnt, out.rem_idx, out.rem_cnt, out.gamma_rep,
+        out.gamma_cross, turnover, flags, _stream(stream))
+    if st:
+        _raise(st, "ada_cascade_step_adaptive")
     return out
 
 
 def _shape_heads(X: torch.Tensor):
-    if X.dim() != 3 or X.stride(2) != 1 or X.stride(1) != X.shape[2]:
-        raise ValueError("X must be T x h x d_h with the heads of a token side by side")
-    T, h, d_h = X.shape
-    return T, h, d_h, X.stride(0)
+    if X.dim() == 3:
+        T, h, d_h = X.shape
+        st, sh, sd = X.stride()
+        if sd == 1 and sh == d_h:
+            return T, h, d_h, st
+    raise ValueError("X must be T x h x d_h with the heads of a token side by side")
 
 
 def ada_select_full_heads(ctx: Context, X: torch.Tensor, tau: float, rep_idx=None, rep_cnt=None,
@@ -300,9 +309,10 @@ def ada_select_full_heads(ctx: Context, X: torch.Tensor, tau: float, rep_idx=Non
         rep_cnt = torch.empty((h,), dtype=torch.int32, device=dev)
     if gamma is None and want_gamma:
         gamma = torch.empty((h, T), dtype=torch.float32, device=dev)
-    _check(lib().ada_select_full_heads(ctx.h, X.data_ptr(), T, h, d_h, ldx, dtype_of(X), float(tau),
-                                       rep_idx.data_ptr(), rep_cnt.data_ptr(), _ptr(gamma),
-                                       _stream(stream)), "ada_select_full_heads")
+    st = _fast.select_full_heads(ctx.addr, X, T, h, d_h, ldx, dtype_of(X), tau, rep_idx, rep_cnt, gamma,
+                                 _stream(stream))
+    if st:
+        _raise(st, "ada_select_full_heads")
     return rep_idx, rep_cnt, gamma
 
 
@@ -313,13 +323,11 @@ def ada_cascade_step_heads(ctx: Context, X: torch.Tensor, tau: float, rep_in: to
     T, h, d_h, ldx = _shape_heads(X)
     if out is None:
         out = CascadeOut(h, T, X.device, want_gamma)
-    _check(lib().ada_cascade_step_heads(ctx.h, X.data_ptr(), T, h, d_h, ldx, dtype_of(X),
-                                        float(tau), rep_in.data_ptr(), rep_in_cnt.data_ptr(),
-                                        out.rep_out.data_ptr(), out.rep_out_cnt.data_ptr(),
-                                        out.add_idx.data_ptr(), out.add_cnt.data_ptr(),
-                                        out.rem_idx.data_ptr(), out.rem_cnt.data_ptr(),
-                                        _ptr(out.gamma_rep), _ptr(out.gamma_cross), flags,
-                                        _stream(stream)), "ada_cascade_step_heads")
+    st = _fast.cascade_step_heads(ctx.addr, X, T, h, d_h, ldx, dtype_of(X), tau, rep_in, rep_in_cnt, out.rep_out,
+                                  out.rep_out_cnt, out.add_idx, out.add_cnt, out.rem_idx, out.rem_cnt, out.gamma_rep,
+                                  out.gamma_cross, flags, _stream(stream))
+    if st:
+        _raise(st, "ada_cascade_step_heads")
     return out
 
 
@@ -329,9 +337,9 @@ def ada_nearest_rep(ctx: Context, X: torch.Tensor, rep_idx: torch.Tensor, rep_cn
     X, B, T, d, ldx = _shape(X)
     near = torch.empty((B, T), dtype=torch.int32, device=X.device)
     g = torch.empty((B, T), dtype=torch.float32, device=X.device) if want_gamma else None
-    _check(lib().ada_nearest_rep(ctx.h, X.data_ptr(), B, T, d, ldx, dtype_of(X), rep_idx.data_ptr(),
-                                 rep_cnt.data_ptr(), near.data_ptr(), _ptr(g), _stream(stream)),
-           "ada_nearest_rep")
+    st = _fast.nearest_rep(ctx.addr, X, B, T, d, ldx, dtype_of(X), rep_idx, rep_cnt, near, g, _stream(stream))
+    if st:
+        _raise(st, "ada_nearest_rep")
     return near, g
 
 
@@ -342,15 +350,15 @@ def ada_attention_reps(ctx: Context, Q: torch.Tensor, K: torch.Tensor, V: torch.
     bf16), expanded to every token through nearest_idx when given.  Returns out fp32 [T, h, d_h]
     (rows that receive nothing are left as they are: zeros in a fresh tensor)."""
     T, h, d_h, ld = _shape_heads(Q)
-    for X in (K, V):
-        if X.shape != Q.shape or X.stride() != Q.stride():
-            raise ValueError("Q, K, V must share shape and strides")
+    shape, strides = Q.shape, Q.stride()
+    if K.shape != shape or V.shape != shape or K.stride() != strides or V.stride() != strides:
+        raise ValueError("Q, K, V must share shape and strides")
     if out is None:
         out = torch.zeros((T, h, d_h), dtype=torch.float32, device=Q.device)
-    _check(lib().ada_attention_reps(ctx.h, Q.data_ptr(), K.data_ptr(), V.data_ptr(), T, h, d_h, ld,
-                                    dtype_of(Q), rep_idx.data_ptr(), rep_cnt.data_ptr(),
-                                    _ptr(nearest_idx), out.data_ptr(), out.stride(0), flags,
-                                    _stream(stream)), "ada_attention_reps")
+    st = _fast.attention_reps(ctx.addr, Q, K, V, T, h, d_h, ld, dtype_of(Q), rep_idx, rep_cnt, nearest_idx, out,
+                              out.stride(0), flags, _stream(stream))
+    if st:
+        _raise(st, "ada_attention_reps")
     return out
 
 

@@ -228,6 +228,7 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
     ctx->engine = ADA_ENGINE_AUTO;
     ctx->stage = nullptr; ctx->stage_bytes = 0; ctx->host_stream = nullptr;
     ctx->attn_ws = nullptr; ctx->attn_ws_bytes = 0;
+    ctx->map_cache = nullptr;
     ctx->tc_attr_set = false;
     ctx->cooperative = true;
     ctx->dep_launch = true;
@@ -282,6 +283,7 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
         delete ctx;
         return ADA_ERR_CUDA;
     }
+    ctx->map_cache = new_map_cache();
     *out = ctx;
     return ADA_OK;
 }
@@ -299,6 +301,7 @@ ada_status ada_destroy(ada_ctx* ctx) {
     if (ctx->attn_ws) cudaFree(ctx->attn_ws);
     if (ctx->host_stream) cudaStreamDestroy(ctx->host_stream);
     cudaFree(ctx->ws);
+    delete_map_cache(ctx->map_cache);
     delete ctx;
     return ADA_OK;
 }

@@ -587,9 +587,9 @@ cudaError_t launch_attention_reps(ada_ctx* ctx, const void* Q, const void* K, co
     __nv_bfloat16* Vt = reinterpret_cast<__nv_bfloat16*>(ctx->attn_ws + 2 * stride);
     AttnMaps maps;
     memset(&maps, 0, sizeof(maps));
-    if (!make_map(&maps.q, Qr, d_h, Tp, h, d_h, (int64_t)Tp * d_h, AQ) ||
-        !make_map(&maps.k, Kr, d_h, Tp, h, d_h, (int64_t)Tp * d_h, AKV) ||
-        !make_map(&maps.v, Vt, Tp, d_h, h, Tp, (int64_t)d_h * Tp, d_h))
+    if (!make_map(ctx, &maps.q, Qr, d_h, Tp, h, d_h, (int64_t)Tp * d_h, AQ) ||
+        !make_map(ctx, &maps.k, Kr, d_h, Tp, h, d_h, (int64_t)Tp * d_h, AKV) ||
+        !make_map(ctx, &maps.v, Vt, Tp, d_h, h, Tp, (int64_t)d_h * Tp, d_h))
         return cudaErrorInvalidValue;
     launch_k(ctx, k_attn_gather, dim3(Tp / 32 < GATHER_BLOCKS ? Tp / 32 : GATHER_BLOCKS, h), dim3(256), 0, s, (const __nv_bfloat16*)Q,
              (const __nv_bfloat16*)K, (const __nv_bfloat16*)V, T, Tp, h, d_h, ld, rep_idx, rep_cnt, Qr, Kr, Vt,

@@ -198,6 +198,7 @@ struct ada_ctx {
     // gathered Q_R, K_R, V_R^T of the attention on the representative set (allocated on first use)
     char* attn_ws;
     size_t attn_ws_bytes;
+    void* map_cache;     // tc::MapCache, or NULL: none kept
     // staging for the *_host entry points (allocated on first use)
     char* stage;
     size_t stage_bytes;
@@ -254,6 +255,9 @@ bool coop_begin(ada_ctx* ctx, cudaStream_t s);
 void coop_end(ada_ctx* ctx, bool coop);
 unsigned long long sole_mark(int device);
 void sole_idle(int device, bool all, cudaStream_t s, unsigned long long mark);
+
+void* new_map_cache();            // NULL: none could be made, which costs only time
+void delete_map_cache(void* c);
 
 // RAII-free launch bracket used by every launcher.
 void prof_begin(ada_ctx* ctx, int kid, cudaStream_t s);

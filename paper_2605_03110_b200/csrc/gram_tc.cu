@@ -824,9 +824,9 @@ cudaError_t launch_gram_tc(ada_ctx* ctx, const GramProblem* tri, const GramProbl
         if (n_cap <= 0 || a_rows <= 0) continue;
         // rows beyond the matrices (and k beyond d) are zero-filled by the TMA unit
         const int width = p->planes > 0 ? 3 * p->planes : p->d;
-        if (!make_map(&maps.a[nseg], p->A, width, p->tri ? p->cap : p->rows, p->B, p->lda, p->a_batch, BM) ||
-            !make_map(&maps.b[nseg], p->Bm, width, p->cap, p->B, p->ldb, p->b_batch, BOX_N) ||
-            !make_map(&maps.bw[nseg], p->Bm, width, p->cap, p->B, p->ldb, p->b_batch, BN))
+        if (!make_map(ctx, &maps.a[nseg], p->A, width, p->tri ? p->cap : p->rows, p->B, p->lda, p->a_batch, BM) ||
+            !make_map(ctx, &maps.b[nseg], p->Bm, width, p->cap, p->B, p->ldb, p->b_batch, BOX_N) ||
+            !make_map(ctx, &maps.bw[nseg], p->Bm, width, p->cap, p->B, p->ldb, p->b_batch, BN))
             return cudaErrorInvalidValue;
         segs[nseg++] = *p;
     }

@@ -1112,12 +1112,12 @@ cudaError_t launch_gram_tc2(ada_ctx* ctx, const GramProblem* tri, const GramProb
         const int a_rows = p->tri ? n_cap : p->rows;
         if (n_cap <= 0 || a_rows <= 0) continue;
         const int width = p->planes > 0 ? 3 * p->planes : p->d;
-        if (!make_map(&maps.a[nseg], p->A, width, p->tri ? p->cap : p->rows, p->B, p->lda, p->a_batch, BM) ||
-            !make_map(&maps.b[nseg], p->Bm, width, p->cap, p->B, p->ldb, p->b_batch, BOX_N) ||
-            !make_map(&maps.bt[nseg], p->Bm, width, p->cap, p->B, p->ldb, p->b_batch, BOX_N / 2))
+        if (!make_map(ctx, &maps.a[nseg], p->A, width, p->tri ? p->cap : p->rows, p->B, p->lda, p->a_batch, BM) ||
+            !make_map(ctx, &maps.b[nseg], p->Bm, width, p->cap, p->B, p->ldb, p->b_batch, BOX_N) ||
+            !make_map(ctx, &maps.bt[nseg], p->Bm, width, p->cap, p->B, p->ldb, p->b_batch, BOX_N / 2))
             return cudaErrorInvalidValue;
         if (!p->tri && p->hb_rows > 0 && p->hb_rows < BM) {
-            if (!make_map(&maps.ah, p->A, width, p->rows, p->B, p->lda, p->a_batch, p->hb_rows))
+            if (!make_map(ctx, &maps.ah, p->A, width, p->rows, p->B, p->lda, p->a_batch, p->hb_rows))
                 return cudaErrorInvalidValue;
         } else {
             maps.ah = maps.a[nseg];
@@ -1128,7 +1128,7 @@ cudaError_t launch_gram_tc2(ada_ctx* ctx, const GramProblem* tri, const GramProb
     if (nseg == 1) { maps.a[1] = maps.a[0]; maps.b[1] = maps.b[0]; maps.bt[1] = maps.bt[0]; segs[1] = segs[0]; segs[1].B = 0; }
     maps.an = maps.ah;
     if (gather != nullptr && gather->Xnon != nullptr && cross != nullptr && gather->T >= gather->compact_min_rows &&
-        !make_map(&maps.an, gather->Xnon, cross->d, cross->rows, cross->B, cross->d, (int64_t)cross->cap * cross->d, BM))
+        !make_map(ctx, &maps.an, gather->Xnon, cross->d, cross->rows, cross->B, cross->d, (int64_t)cross->cap * cross->d, BM))
         return cudaErrorInvalidValue;
     NormJob nj;
     memset(&nj, 0, sizeof(nj));

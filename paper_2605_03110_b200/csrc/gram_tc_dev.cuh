@@ -280,8 +280,8 @@ static inline EncodeTiledFn encode_fn() {
 }
 
 // 3-D map over a stack of K-major bf16 matrices: (k, row, sequence).
-static inline bool make_map(CUtensorMap* map, const void* base, int d, int rows, int B, int64_t ld,
-              int64_t batch, int box_rows) {
+static inline bool encode_map(CUtensorMap* map, const void* base, int d, int rows, int B, int64_t ld,
+                              int64_t batch, int box_rows) {
     EncodeTiledFn fn = encode_fn();
     if (fn == nullptr) return false;
     const cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)rows, (cuuint64_t)B};
@@ -294,6 +294,40 @@ static inline bool make_map(CUtensorMap* map, const void* base, int d, int rows,
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The last tensor maps of a context: a call needs up to eight, most of them over the context's own
+// workspace or a tensor that the caller passes again (a descriptor depends on address and shape
+// only).  One context serves one stream at a time, so it has no lock; ctx->map_cache is NULL where a
+// context may be used by several threads at once.
+struct MapCache {
+    static constexpr int N = 48;
+    struct Key {
+        const void* base;
+        int64_t ld, batch;
+        int d, rows, B, box_rows;
+    } key[N];
+    CUtensorMap map[N];
+    int n = 0, next = 0;
+};
+static inline bool make_map(ada_ctx* ctx, CUtensorMap* map, const void* base, int d, int rows, int B, int64_t ld,
+                            int64_t batch, int box_rows) {
+    MapCache* c = static_cast<MapCache*>(ctx->map_cache);
+    if (c == nullptr) return encode_map(map, base, d, rows, B, ld, batch, box_rows);
+    for (int i = 0; i < c->n; ++i) {
+        const MapCache::Key& k = c->key[i];
+        if (k.base == base && k.d == d && k.rows == rows && k.B == B && k.ld == ld && k.batch == batch &&
+            k.box_rows == box_rows) {
+            *map = c->map[i];
+            return true;
+        }
+    }
+    if (!encode_map(map, base, d, rows, B, ld, batch, box_rows)) return false;
+    const int at = c->next;
+    c->key[at] = {base, ld, batch, d, rows, B, box_rows};
+    c->map[at] = *map;
+    c->next = at + 1 == MapCache::N ? 0 : at + 1;
+    if (c->n < MapCache::N) ++c->n;
+    return true;
+}
 
 // ---------------------------------------------------------------- in-launch row norms
 // bf16 pairs are the halves of 32-bit words; a bf16 is the upper half of an fp32

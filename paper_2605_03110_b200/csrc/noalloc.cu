@@ -65,6 +65,7 @@ ada_status setup_device(int device, PerDevice** out) {
         c.tc2_pairs = 0;
         c.ws = nullptr;
         c.attn_ws = nullptr;
+        c.map_cache = nullptr;
         c.attn_ws_bytes = 0;
         c.stage = nullptr;
         c.stage_bytes = 0;

@@ -1,6 +1,8 @@
 // HBM-bound helper kernels of the selection path: fused row-norm + representative
 // gather (with validation of the inherited list), and the prefix-sum compaction that
 // turns gamma into sorted index lists.
+#include <new>
+
 #include "gram_tc_dev.cuh"
 
 namespace ada {
@@ -649,5 +651,8 @@ cudaError_t launch_compact_cascade(ada_ctx* ctx, int B, int T, float thr, int32_
     a.tu = tu;
     return launch_compact(ctx, K_COMPACT_CASCADE, a, B, s);
 }
+
+void* new_map_cache() { return new (std::nothrow) tc::MapCache; }
+void delete_map_cache(void* c) { delete static_cast<tc::MapCache*>(c); }
 
 }  // namespace ada

@@ -227,6 +227,7 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
     ctx->es = dt == ADA_F32 ? 4 : 2;
     ctx->engine = ADA_ENGINE_AUTO;
     ctx->stage = nullptr; ctx->stage_bytes = 0; ctx->host_stream = nullptr;
+    ctx->host_event = nullptr; ctx->host_out = false;
     ctx->attn_ws = nullptr; ctx->attn_ws_bytes = 0;
     ctx->map_cache = nullptr;
     ctx->tc_attr_set = false;
@@ -300,6 +301,7 @@ ada_status ada_destroy(ada_ctx* ctx) {
     if (ctx->stage) cudaFree(ctx->stage);
     if (ctx->attn_ws) cudaFree(ctx->attn_ws);
     if (ctx->host_stream) cudaStreamDestroy(ctx->host_stream);
+    if (ctx->host_event) cudaEventDestroy(ctx->host_event);
     cudaFree(ctx->ws);
     delete_map_cache(ctx->map_cache);
     delete ctx;
@@ -758,6 +760,37 @@ static Stage carve(ada_ctx* ctx) {
     return st;
 }
 
+// Outputs in pinned host memory are written by the compaction itself, through their device address: the
+// call is bound by copying the activations in (16.8 MB at 50 GB/s), and eight small copies back, one
+// after the other, added 25 us to it.  Anything else goes through the staging buffers.
+struct HostOut {
+    void* host;
+    void* dev;        // where the kernels write
+    size_t bytes;     // copied back afterwards; 0: nothing to copy
+};
+static void* mapped(void* host) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
+}
+// the staging buffers become the outputs' own memory where every output is mapped
+static void choose_outputs(ada_ctx* ctx, HostOut* out, int n) {
+    void* m[8];
+    for (int i = 0; i < n; ++i) {
+        m[i] = out[i].host != nullptr ? mapped(out[i].host) : nullptr;
+        if (out[i].host != nullptr && m[i] == nullptr) return;
+    }
+    for (int i = 0; i < n; ++i) { out[i].dev = m[i]; out[i].bytes = 0; }
+    ctx->host_out = true;
+}
+static ada_status copy_back(HostOut* out, int n, cudaStream_t s) {
+    for (int i = 0; i < n; ++i)
+        if (out[i].host != nullptr && out[i].bytes > 0)
+            CU(cudaMemcpyAsync(out[i].host, out[i].dev, out[i].bytes, cudaMemcpyDeviceToHost, s));
+    CU(cudaStreamSynchronize(s));
+    return ADA_OK;
+}
+
 ada_status ada_select_full_host(ada_ctx* ctx, const void* X, int64_t B, int64_t T, int64_t d,
                                 ada_dtype dt, double tau, int32_t* rep_idx, int32_t* rep_cnt,
                                 float* gamma, void* stream) {
@@ -775,13 +808,12 @@ ada_status ada_select_full_host(ada_ctx* ctx, const void* X, int64_t B, int64_t 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const size_t n_tok = (size_t)B * T;
     CU(cudaMemcpyAsync(sg.X, X, n_tok * d * ctx->es, cudaMemcpyHostToDevice, s));
-    st = ada_select_full(ctx, sg.X, B, T, d, d, dt, tau, sg.l0, sg.c0, gamma ? sg.g0 : nullptr, s);
-    if (st != ADA_OK) return st;
-    CU(cudaMemcpyAsync(rep_idx, sg.l0, n_tok * 4, cudaMemcpyDeviceToHost, s));
-    CU(cudaMemcpyAsync(rep_cnt, sg.c0, (size_t)B * 4, cudaMemcpyDeviceToHost, s));
-    if (gamma) CU(cudaMemcpyAsync(gamma, sg.g0, n_tok * 4, cudaMemcpyDeviceToHost, s));
-    CU(cudaStreamSynchronize(s));
-    return ADA_OK;
+    HostOut out[3] = {{rep_idx, sg.l0, n_tok * 4}, {rep_cnt, sg.c0, (size_t)B * 4}, {gamma, sg.g0, n_tok * 4}};
+    choose_outputs(ctx, out, 3);
+    st = ada_select_full(ctx, sg.X, B, T, d, d, dt, tau, (int32_t*)out[0].dev, (int32_t*)out[1].dev,
+                         gamma ? (float*)out[2].dev : nullptr, s);
+    ctx->host_out = false;
+    return st != ADA_OK ? st : copy_back(out, 3, s);
 }
 
 ada_status ada_cascade_step_host(ada_ctx* ctx, const void* X, int64_t B, int64_t T, int64_t d,
@@ -805,23 +837,24 @@ ada_status ada_cascade_step_host(ada_ctx* ctx, const void* X, int64_t B, int64_t
     Stage sg = carve(ctx);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const size_t n_tok = (size_t)B * T;
+    // the inherited lists travel beside the activations, on a stream of their own
+    if (ctx->host_stream == nullptr) CU(cudaStreamCreateWithFlags(&ctx->host_stream, cudaStreamNonBlocking));
+    if (ctx->host_event == nullptr) CU(cudaEventCreateWithFlags(&ctx->host_event, cudaEventDisableTiming));
     CU(cudaMemcpyAsync(sg.X, X, n_tok * d * ctx->es, cudaMemcpyHostToDevice, s));
-    CU(cudaMemcpyAsync(sg.l0, rep_in, n_tok * 4, cudaMemcpyHostToDevice, s));
-    CU(cudaMemcpyAsync(sg.c0, rep_in_cnt, (size_t)B * 4, cudaMemcpyHostToDevice, s));
-    st = ada_cascade_step(ctx, sg.X, B, T, d, d, dt, tau, sg.l0, sg.c0, sg.l1, sg.c1, sg.l2, sg.c2,
-                          sg.l3, sg.c3, gamma_rep ? sg.g0 : nullptr, gamma_cross ? sg.g1 : nullptr,
-                          flags, s);
-    if (st != ADA_OK) return st;
-    CU(cudaMemcpyAsync(rep_out, sg.l1, n_tok * 4, cudaMemcpyDeviceToHost, s));
-    CU(cudaMemcpyAsync(add_idx, sg.l2, n_tok * 4, cudaMemcpyDeviceToHost, s));
-    CU(cudaMemcpyAsync(rem_idx, sg.l3, n_tok * 4, cudaMemcpyDeviceToHost, s));
-    CU(cudaMemcpyAsync(rep_out_cnt, sg.c1, (size_t)B * 4, cudaMemcpyDeviceToHost, s));
-    CU(cudaMemcpyAsync(add_cnt, sg.c2, (size_t)B * 4, cudaMemcpyDeviceToHost, s));
-    CU(cudaMemcpyAsync(rem_cnt, sg.c3, (size_t)B * 4, cudaMemcpyDeviceToHost, s));
-    if (gamma_rep) CU(cudaMemcpyAsync(gamma_rep, sg.g0, n_tok * 4, cudaMemcpyDeviceToHost, s));
-    if (gamma_cross) CU(cudaMemcpyAsync(gamma_cross, sg.g1, n_tok * 4, cudaMemcpyDeviceToHost, s));
-    CU(cudaStreamSynchronize(s));
-    return ADA_OK;
+    CU(cudaMemcpyAsync(sg.l0, rep_in, n_tok * 4, cudaMemcpyHostToDevice, ctx->host_stream));
+    CU(cudaMemcpyAsync(sg.c0, rep_in_cnt, (size_t)B * 4, cudaMemcpyHostToDevice, ctx->host_stream));
+    CU(cudaEventRecord(ctx->host_event, ctx->host_stream));
+    CU(cudaStreamWaitEvent(s, ctx->host_event, 0));
+    HostOut out[8] = {{rep_out, sg.l1, n_tok * 4}, {rep_out_cnt, sg.c1, (size_t)B * 4},
+                      {add_idx, sg.l2, n_tok * 4}, {add_cnt, sg.c2, (size_t)B * 4},
+                      {rem_idx, sg.l3, n_tok * 4}, {rem_cnt, sg.c3, (size_t)B * 4},
+                      {gamma_rep, sg.g0, n_tok * 4}, {gamma_cross, sg.g1, n_tok * 4}};
+    choose_outputs(ctx, out, 8);
+    st = ada_cascade_step(ctx, sg.X, B, T, d, d, dt, tau, sg.l0, sg.c0, (int32_t*)out[0].dev, (int32_t*)out[1].dev,
+                          (int32_t*)out[2].dev, (int32_t*)out[3].dev, (int32_t*)out[4].dev, (int32_t*)out[5].dev,
+                          gamma_rep ? (float*)out[6].dev : nullptr, gamma_cross ? (float*)out[7].dev : nullptr, flags, s);
+    ctx->host_out = false;
+    return st != ADA_OK ? st : copy_back(out, 8, s);
 }
 
 ada_status ada_selftest_wait_timeout(ada_ctx* ctx, int limit_ms, void* stream) {

@@ -202,7 +202,9 @@ struct ada_ctx {
     // staging for the *_host entry points (allocated on first use)
     char* stage;
     size_t stage_bytes;
-    cudaStream_t host_stream;
+    cudaStream_t host_stream;    // carries the small inputs beside the activations
+    cudaEvent_t host_event;
+    bool host_out;               // the call's outputs are mapped host memory
     ada::Profiler prof;
 };
 

@@ -70,6 +70,8 @@ ada_status setup_device(int device, PerDevice** out) {
         c.stage = nullptr;
         c.stage_bytes = 0;
         c.host_stream = nullptr;
+        c.host_event = nullptr;
+        c.host_out = false;
         if (cudaDeviceGetAttribute(&c.sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
             return;
         c.g_tok = reinterpret_cast<unsigned*>(pd.scratch);

@@ -372,6 +372,7 @@ struct CompactArgs {
     unsigned* dep_ctr;           // dependency counters of the Gram launch (cleared here)
     unsigned* status;
     int T;
+    int prefetch;                // outputs are device memory
     float thr;
     int32_t *keep_idx, *keep_cnt, *add_idx, *add_cnt, *rem_idx, *rem_cnt;
     float *gamma_a, *gamma_b;    // full: gamma | cascade: gamma_rep, gamma_cross (optional)
@@ -393,7 +394,7 @@ __global__ void __launch_bounds__(1024) k_compact(const CompactArgs a) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t o = (int64_t)b * a.T;
     const bool cascade = a.role != nullptr;
-    {
+    if (a.prefetch) {
         const int t = rank * V * 1024 + V * (int)threadIdx.x;
         if ((threadIdx.x & 31) == 0 && t < a.T) {              // one touch per 128 V bytes of each output
             prefetch_l2(a.keep_idx + o + t);
@@ -625,7 +626,7 @@ cudaError_t launch_compact_full(ada_ctx* ctx, int B, int T, float thr, int32_t* 
     CompactArgs a;
     a.g_tok = ctx->g_tok; a.g_rep = nullptr; a.role = nullptr;
     a.dep_ctr = ctx->tile_ctr; a.status = ctx->status;
-    a.T = T; a.thr = thr;
+    a.T = T; a.thr = thr; a.prefetch = ctx->host_out ? 0 : 1;
     a.keep_idx = rep_idx; a.keep_cnt = rep_cnt;
     a.add_idx = nullptr; a.add_cnt = nullptr; a.rem_idx = nullptr; a.rem_cnt = nullptr;
     a.gamma_a = gamma; a.gamma_b = nullptr; a.row_scale = nullptr;
@@ -642,7 +643,7 @@ cudaError_t launch_compact_cascade(ada_ctx* ctx, int B, int T, float thr, int32_
     CompactArgs a;
     a.g_tok = ctx->g_tok; a.g_rep = ctx->g_rep; a.role = ctx->role;
     a.dep_ctr = ctx->tile_ctr; a.status = ctx->status;
-    a.T = T; a.thr = thr;
+    a.T = T; a.thr = thr; a.prefetch = ctx->host_out ? 0 : 1;
     a.keep_idx = rep_out; a.keep_cnt = rep_out_cnt;
     a.add_idx = add_idx; a.add_cnt = add_cnt; a.rem_idx = rem_idx; a.rem_cnt = rem_cnt;
     a.gamma_a = gamma_rep; a.gamma_b = gamma_cross;

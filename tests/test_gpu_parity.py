@@ -704,3 +704,29 @@ def test_two_streams_launch_without_waiting_on_each_other(ada):
     for c, s in zip(ctx, streams):
         assert ada.ada_device_status(c, stream=s)[0] == 0
         ada.ada_destroy(c)
+
+
+@pytest.mark.parametrize("pinned", [(True,) * 8, (False,) * 8, (True, True, False, True, True, True, True, False)])
+def test_host_outputs_pinned_pageable_and_mixed(ada, pinned):
+    """Pinned outputs are written by the kernels themselves, others are copied back: same lists, counts
+    and gammas either way, also when the output list overwrites the input list's buffer."""
+    T, d = 1500, 512
+    X = torch.from_numpy(clustered(T, d, 7, "bf16").view(np.int16)).view(torch.bfloat16)
+    ctx = ada.ada_create(1, T, d, ada.ADA_BF16)
+    Xd = X.cuda()
+    ri, rc, _ = ada.ada_select_full(ctx, Xd, TAU)
+    X1 = (Xd.float() + 0.3 * torch.randn(Xd.shape, device="cuda", generator=torch.Generator("cuda").manual_seed(1))).bfloat16()
+    ref = ada.ada_cascade_step(ctx, X1, TAU, ri, rc)
+    make = lambda t, p: t.cpu().pin_memory() if p else t.cpu()
+    empties = [torch.empty((1, T), dtype=torch.int32), torch.empty(1, dtype=torch.int32)] * 3 + [torch.empty(1, T)] * 2
+    ro, roc, ai, ac, mi, mc, gr, gc = [make(e.clone(), p) for e, p in zip(empties, pinned)]
+    ro.copy_(ri), roc.copy_(rc)
+    ada.ada_cascade_step_host(ctx, make(X1, pinned[0]), TAU, ro, roc, ro, roc, ai, ac, mi, mc, gr, gc)
+    for host, dev, cnt in ((ro, ref.rep_out, ref.rep_out_cnt), (ai, ref.add_idx, ref.add_cnt),
+                           (mi, ref.rem_idx, ref.rem_cnt)):
+        n = int(cnt[0])
+        assert host[0, :n].tolist() == dev[0, :n].tolist()
+    assert [int(t) for t in (roc, ac, mc)] == [int(t) for t in (ref.rep_out_cnt, ref.add_cnt, ref.rem_cnt)]
+    assert torch.equal(gr, ref.gamma_rep.cpu()) and torch.equal(gc, ref.gamma_cross.cpu())
+    assert ada.ada_device_status(ctx)[0] == 0
+    ada.ada_destroy(ctx)

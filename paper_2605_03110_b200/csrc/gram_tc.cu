@@ -735,8 +735,9 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
             }
             if (sg == 0 && nseg > 1) {
                 // publish: this warp's share of a triangular tile is in global memory; one arrival per
-                // tile, by the last of the set's four warps
-                __threadfence();
+                // tile, by the last of the set's four warps, whose fence covers what the others' orders
+                // before the shared counter
+                __threadfence_block();
                 __syncwarp();
                 if (lane == 0 && (atomicAdd(&sh.pub[eset], 1u) & 3u) == 3u) {
                     __threadfence();

@@ -564,8 +564,9 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         if constexpr (!SPLIT) gather_rows(gather, sh.gather, g, nw, lane, status);
         else split_rows(sh.split, g, nw, lane, status);
         // the rows just written are read by TMA (async proxy) from other CTAs
+        // (one fence for the whole device per CTA, after the barrier: it covers what the barrier ordered
+        // before it)
         asm volatile("fence.proxy.async.global;" ::: "memory");
-        __threadfence();
         asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
         if (threadIdx.x == 64) {
             __threadfence();
@@ -1022,8 +1023,9 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                 }
             }
             if (sg == 0 && nseg > 1) {
-                // publish: one arrival per CTA and tile, by the last of its warps
-                __threadfence();
+                // publish: one arrival per CTA and tile, by the last of its warps, whose fence covers what
+                // the others' orders before the shared counter
+                __threadfence_block();
                 __syncwarp();
                 const unsigned share = solo ? SUBS : 1;
                 if (lane == 0 && (atomicAdd(&sh.pub_cnt, share) + share) % EPI_WARPS == 0) {

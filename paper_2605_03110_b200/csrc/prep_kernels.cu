@@ -69,6 +69,7 @@ k_norm_gather(const T* __restrict__ X, int64_t n_rows, int Tseq, int d, int64_t 
               int32_t* __restrict__ role, int32_t* __restrict__ r_eff, T* __restrict__ Xrep,
               float* __restrict__ inv_rep, unsigned* __restrict__ status) {
     grid_dep_wait();
+    grid_dep_launch_next();
     const int lane = threadIdx.x & 31;
     int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int64_t n_norm_warps = (n_rows + NORM_ROWS - 1) / NORM_ROWS;
@@ -180,6 +181,7 @@ k_norm_gather_short(const T* __restrict__ X, int64_t n_rows, int Tseq, int d, in
                     int32_t* __restrict__ role, int32_t* __restrict__ r_eff, T* __restrict__ Xrep,
                     float* __restrict__ inv_rep, unsigned* __restrict__ status) {
     grid_dep_wait();
+    grid_dep_launch_next();
     const int lane = threadIdx.x & 31;
     int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (inv_norm == nullptr && Xhat == nullptr) w += n_norm_warps;   // gather-only launch: list warps only

@@ -298,10 +298,14 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    // everything above is local to the CTA; from here on the predecessor's results are read
-    grid_dep_wait();
-    // (the compaction's blocks may take the SMs that fall idle first: they wait for this whole grid)
-    grid_dep_launch_next();
+    // everything above is local to the CTA; the predecessor's results are read only after the wait -- which
+    // comes after the work plan where that does not depend on them (full selection)
+    const bool early = nseg == 1 && seg0.n_dev == nullptr;
+    if (!early) {
+        grid_dep_wait();
+        // (the compaction's blocks may take the SMs that fall idle first: they wait for this whole grid)
+        grid_dep_launch_next();
+    }
     if (warp == 2) {
         // Work plan.  Everything per sequence -- its length, its tile counts -- is computed by
         // the lanes in parallel and reduced with shuffles: the lengths live in global memory, and
@@ -450,6 +454,10 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
         sh.tile_tab[threadIdx.x] = e;
     }
     __syncthreads();
+    if (early) {
+        grid_dep_wait();
+        grid_dep_launch_next();
+    }
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer

@@ -551,6 +551,19 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
     tcgen05_fence_after();
     const unsigned tmem_base = sh.tmem_base;
     const bool has_prep = SPLIT ? split.X != nullptr : gather.X != nullptr;
+    // The work plan: before the predecessor's results are waited for where it does not depend on them (full
+    // selection, T = 2048, d = 4096: 26.3 -> 25.2 us; one-CTA kernel, T = 512, d = 768: 14.1 -> 13.1).
+    auto plan_work = [&]() {
+        const bool maybe_compact = gather.X != nullptr && gather.Xnon != nullptr && gather.T >= gather.compact_min_rows;
+        make_plan<SPLIT>(sh.plan, sh.seg[0], sh.seg[1], nseg, maybe_compact, npairs, max_parts, lane);
+        __syncwarp();
+        decode_item<SPLIT>(&sh.seg[0], &sh.seg[1], sh.plan, pair, npairs, lane, sh.item[lane]);
+        __syncwarp();
+        if (lane == 0) { __threadfence_block(); mbar_arrive(&sh.planned); }
+        __syncwarp();
+    };
+    const bool early = (nseg > 1 ? seg1 : seg0).n_dev == nullptr;
+    if (early && warp == 0) plan_work();
     // everything above is local to the CTA; from here on the predecessor's results are read
     grid_dep_wait();
     // (the compaction's blocks may take the SMs that fall idle first: they wait for this whole grid)
@@ -575,15 +588,7 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         }
     }
     const unsigned prep_total = gridDim.x;
-    if (warp == 0) {
-        const bool maybe_compact = gather.X != nullptr && gather.Xnon != nullptr && gather.T >= gather.compact_min_rows;
-        make_plan<SPLIT>(sh.plan, sh.seg[0], sh.seg[1], nseg, maybe_compact, npairs, max_parts, lane);
-        __syncwarp();
-        decode_item<SPLIT>(&sh.seg[0], &sh.seg[1], sh.plan, pair, npairs, lane, sh.item[lane]);
-        __syncwarp();
-        if (lane == 0) { __threadfence_block(); mbar_arrive(&sh.planned); }
-        __syncwarp();
-    }
+    if (!early && warp == 0) plan_work();
     // (a plan is always made, by warp 0 of the same CTA, which waits for nobody)
     while (!mbar_try_long(&sh.planned, 0)) { }
     const Plan& pl = sh.plan;

@@ -17,7 +17,7 @@
 //   warps 2..9  first the preparation of a cascade step: Algorithm 1 lines 1-2 (list checked, role
 //               map, rows copied to Xrep with their inverse norms; fp32: the bf16 planes of
 //               every row), which loads and epilogues wait for; then the row norms of X with
-//               plain loads behind the first main loops (in the streaming form, warps 6..9, out of
+//               plain loads behind the first main loops (in the streaming form out of
 //               the left-operand tiles while those sit in shared memory, one thread per row,
 //               so that X is read from memory exactly once); then the epilogue, each CTA on its own
 //               128 rows, two warps per TMEM lane quadrant; the peer's returns the accumulator by
@@ -226,10 +226,11 @@ __device__ __forceinline__ bool decode_tile(const GramProblem& p, const Plan& pl
     return false;
 }
 // per-CTA stage: the CTA's rows of A (a_bytes per 64-element K block, a multiple of 1024) and
-// ncols/2 rows of B (in 64-row boxes)
+// ncols/2 rows of B (in 64-row boxes, a 32-row one at the end where that is enough)
 __device__ __forceinline__ int a_bytes_of(int hrows) { return (hrows * 128 + 1023) & ~1023; }
 __device__ __forceinline__ int sub_bytes_pair(int a_bytes, int ncols) {
-    return a_bytes + (((ncols >> 1) + BOX_N - 1) / BOX_N) * BOX_BYTES;
+    const int half = ncols >> 1, rest = half % BOX_N;
+    return a_bytes + half / BOX_N * BOX_BYTES + (rest == 0 ? 0 : (rest <= 32 ? BOX_BYTES / 2 : BOX_BYTES));
 }
 // Row norms of the cross segment's left operand (inv_out).  When one column tile covers all
 // columns every row tile is loaded exactly once and the launch is bound by streaming them: the
@@ -407,6 +408,8 @@ struct alignas(16) SharedPair {
     unsigned tmem_base;
     int abort_flag;
     unsigned norm_cnt[MAX_STAGES];             // norm warps done with a stage
+    unsigned long long normed;                 // the sums of squares of a tile's rows are in norm_part
+    float norm_part[2][SUBS][BM];              // by tile parity and set
     Plan plan;
     // the launch's arguments once more: what is not inlined takes them by reference, and reading the
     // parameter space through a pointer is a trip to memory
@@ -425,7 +428,6 @@ struct alignas(16) SharedPair {
 template <bool SPLIT>
 constexpr int smem_pair_bytes() { return Ring<SPLIT>::BYTES + (int)sizeof(SharedPair<SPLIT>) + 1024; }
 static_assert(smem_pair_bytes<false>() <= 227 * 1024 && smem_pair_bytes<true>() <= 227 * 1024, "shared memory budget");
-constexpr int RING_NORM_WARPS = 4;             // warps 6..9 read the A tiles
 // partial accumulators: [tile][source part][CTA of the pair][32-column chunk][8 16-byte columns][128 rows]
 constexpr int CHUNK_WORDS = BM * 32;
 __device__ __forceinline__ int64_t chunk_at(int unit, int rank, int chunk) {
@@ -510,6 +512,7 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         mbar_init(&sh.drain, 1);
         mbar_init(&sh.planned, 1);
         mbar_init(&sh.prep_seen, 1);
+        mbar_init(&sh.normed, EPI_WARPS);
         for (int q = 0; q < SUBS; ++q) mbar_init(&sh.staged[q], 4);
         for (int q = 0; q < SUBS; ++q) { mbar_init(&sh.norm_seen[q], 1); mbar_init(&sh.dep_seen[q], 1); }
         sh.pub_cnt = 0u;
@@ -740,9 +743,13 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         // for them (the row factor is applied by the compaction), but everything waits for the
         // triangle, so its tiles go first.
         bool norms_due = norms.X != nullptr || (!cx.tri && cx.inv_out != nullptr && !smem_norms && !compact);
-        // row norms out of the A tiles in shared memory (streaming form): warps 6..9, thread lrow owns
-        // row lrow of the CTA's tile and follows the ring exactly as the producer fills it
-        const bool ring_norms = smem_norms && sub == 1 && !cx.tri && cx.inv_out != nullptr;
+        // row norms out of the A tiles in shared memory (streaming form): thread lrow owns row lrow of the CTA's
+        // tile, set `sub` the stage's K block `sub`, and both follow the ring exactly as the producer
+        // fills it.  (The stage goes back to the producer behind them: with one set reading both K
+        // blocks the ring turned over in 1.06 us per stage at T = 16384, r = 164.)
+        static_assert(SPLIT || SUBS == St::NSUB, "a set per K block of a stage");
+        const bool ring_norms = !SPLIT && smem_norms && !cx.tri && cx.inv_out != nullptr;
+        unsigned n_normed = 0;
         unsigned cons = 0;
         int ring_sb = 0, ring_nst = 0, ring_s = 0;
         // every share of a triangular tile is published once by both CTAs
@@ -806,30 +813,26 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                     float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
                     bool fine = true;
                     for (int st = 0; st < nst; ++st) {
-                        int good = 1;
-                        if (lane == 0) good = mbar_wait(&sh.consumed[ring_s], (cons >> ring_s) & 1u, abort_flag, 14) ? 1 : 0;
-                        if (__shfl_sync(0xffffffffu, good, 0) == 0) { fine = false; break; }
+                        fine = __all_sync(0xffffffffu, mbar_wait(&sh.consumed[ring_s], (cons >> ring_s) & 1u, abort_flag, 14));
+                        if (!fine) break;
                         if (lrow < arows) {
+                            // the 16-byte chunks of a row are permuted by the swizzle, which a sum
+                            // of squares need not undo; lanes start at different chunks so that a
+                            // warp's loads spread over all banks
+                            const unsigned char* rowp = smem + ring_s * sb + sub * subb + lrow * 128;
+                            uint4 x[8];
 #pragma unroll
-                            for (int u = 0; u < St::NSUB; ++u) {
-                                // the 16-byte chunks of a row are permuted by the swizzle, which a sum
-                                // of squares need not undo; lanes start at different chunks so that a
-                                // warp's loads spread over all banks
-                                const unsigned char* rowp = smem + ring_s * sb + u * subb + lrow * 128;
-                                uint4 x[8];
-#pragma unroll
-                                for (int j = 0; j < 8; ++j)
-                                    x[j] = *reinterpret_cast<const uint4*>(rowp + (((j + lane) & 7) << 4));
-                                s0 += sumsq_bf16x8(x[0]) + sumsq_bf16x8(x[4]);
-                                s1 += sumsq_bf16x8(x[1]) + sumsq_bf16x8(x[5]);
-                                s2 += sumsq_bf16x8(x[2]) + sumsq_bf16x8(x[6]);
-                                s3 += sumsq_bf16x8(x[3]) + sumsq_bf16x8(x[7]);
-                            }
+                            for (int j = 0; j < 8; ++j)
+                                x[j] = *reinterpret_cast<const uint4*>(rowp + (((j + lane) & 7) << 4));
+                            s0 += sumsq_bf16x8(x[0]) + sumsq_bf16x8(x[4]);
+                            s1 += sumsq_bf16x8(x[1]) + sumsq_bf16x8(x[5]);
+                            s2 += sumsq_bf16x8(x[2]) + sumsq_bf16x8(x[6]);
+                            s3 += sumsq_bf16x8(x[3]) + sumsq_bf16x8(x[7]);
                         }
                         __syncwarp();
-                        // the last of the four warps releases the stage to the producer
+                        // the last of the eight warps releases the stage to the producer
                         if (lane == 0) {
-                            if (atomicAdd(&sh.norm_cnt[ring_s], 1u) == RING_NORM_WARPS - 1) {
+                            if (atomicAdd(&sh.norm_cnt[ring_s], 1u) == EPI_WARPS - 1) {
                                 sh.norm_cnt[ring_s] = 0u;
                                 mbar_arrive(&sh.empty[ring_s]);
                             }
@@ -838,8 +841,14 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                         ring_s = (ring_s + 1 == ring_nst) ? 0 : ring_s + 1;
                     }
                     if (!fine) break;
-                    if (lrow < arows && row < w.m) {
-                        const float ss = (s0 + s1) + (s2 + s3);
+                    float* part = sh.norm_part[n_normed & 1u][0];
+                    part[sub * BM + lrow] = (s0 + s1) + (s2 + s3);
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&sh.normed);
+                    if (!__all_sync(0xffffffffu, mbar_wait(&sh.normed, n_normed & 1u, abort_flag, 17))) break;
+                    ++n_normed;
+                    if (sub == 0 && lrow < arows && row < w.m) {
+                        const float ss = part[lrow] + part[BM + lrow];
                         float inv = 0.f;
                         if (!(ss <= 3.0e38f)) atomicOr(status, ST_NONFINITE);
                         else if (ss > 0.f) inv = 1.0f / sqrtf(ss);

@@ -51,9 +51,6 @@ __device__ unsigned long long g_trace[160 * 64];
 namespace {
 
 constexpr int PM = 2 * BM;     // rows of a pair tile
-#ifndef PRIME
-#define PRIME 3
-#endif
 // What a ring stage holds.  bf16 storage: two consecutive 64-element K blocks (each its own
 // 128-byte-swizzled sub-tile), so that the per-stage costs -- barrier round trips, fences,
 // commit -- are paid once per 128 K elements and the MMA issue stays ahead of the tensor pipe.
@@ -411,7 +408,6 @@ struct alignas(16) SharedPair {
     unsigned tmem_base;
     int abort_flag;
     unsigned norm_cnt[MAX_STAGES];             // norm warps done with a stage
-    unsigned long long primed;                 // the producer has filled the ring for the first time
     unsigned long long normed;                 // the sums of squares of a tile's rows are in norm_part
     float norm_part[2][SUBS][BM];              // by tile parity and set
     Plan plan;
@@ -517,7 +513,6 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         mbar_init(&sh.planned, 1);
         mbar_init(&sh.prep_seen, 1);
         mbar_init(&sh.normed, EPI_WARPS);
-        mbar_init(&sh.primed, 1);
         for (int q = 0; q < SUBS; ++q) mbar_init(&sh.staged[q], 4);
         for (int q = 0; q < SUBS; ++q) { mbar_init(&sh.norm_seen[q], 1); mbar_init(&sh.dep_seen[q], 1); }
         sh.pub_cnt = 0u;
@@ -618,7 +613,6 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
             unsigned fills = 0, used = 0, ever = 0;
             int cur_sb = 0, cur_nst = 0, s = 0;
             bool ok = true, prep_ok = !has_prep;
-            int to_prime = PRIME;                    // copies still to be issued before the row norms may start
             for (int it = 0; ok; ++it) {
                 const Item& w = item_at(it);
                 if (w.kind == 0) break;
@@ -672,10 +666,8 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                     }
                     fills ^= 1u << s; used |= 1u << s; ever |= 1u << s;
                     s = (s + 1 == cur_nst) ? 0 : s + 1;
-                    if (--to_prime == 0) mbar_arrive(&sh.primed);
                 }
             }
-            if (to_prime > 0) mbar_arrive(&sh.primed);
             // drain: a stage's release (empty) implies its copy landed and was consumed
             for (int q = 0; q < MAX_STAGES; ++q) {
                 if (!((ever >> q) & 1u)) continue;
@@ -788,9 +780,6 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         for (int it = 0;; ++it) {
             const Item& w = item_at(it);
             if (norms_due && (norms.X != nullptr || w.kind == 0 || !(w.seg ? seg1 : seg0).tri)) {
-                // (behind the first copies: their latency is the launch's, and these loads saturate the
-                // memory system)
-                if (!__all_sync(0xffffffffu, mbar_wait(&sh.primed, 0, abort_flag, 18))) break;
                 norm_rows(sh.norms, blockIdx.x * EPI_WARPS + (warp - 2), gridDim.x * EPI_WARPS, lane, dep_ctr + 1, status);
                 norms_due = false;
             }

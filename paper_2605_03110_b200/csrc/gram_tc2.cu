@@ -106,6 +106,16 @@ __device__ __forceinline__ void tma_load_3d_pair(const CUtensorMap* map, unsigne
           "r"(smem_u32(bar) & 0xFEFFFFFFu), "r"(c0), "r"(c1), "r"(c2)
         : "memory");
 }
+// The same for rows that no later copy of the launch reads: the first lines to leave L2.
+__device__ __forceinline__ void tma_load_3d_pair_once(const CUtensorMap* map, unsigned long long* bar,
+                                                      void* dst, int c0, int c1, int c2, unsigned long long policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+        " [%0], [%1, {%3, %4, %5}], [%2], %6;"
+        ::"r"(smem_u32(dst)), "l"(reinterpret_cast<unsigned long long>(map)),
+          "r"(smem_u32(bar) & 0xFEFFFFFFu), "r"(c0), "r"(c1), "r"(c2), "l"(policy)
+        : "memory");
+}
 __device__ __forceinline__ void umma_bf16_pair(unsigned tmem_d, unsigned long long adesc,
                                                unsigned long long bdesc, unsigned idesc,
                                                unsigned accumulate) {
@@ -149,7 +159,7 @@ struct Plan {
     int tiles0, total;          // triangular tiles; all tiles
     int tw;                     // column width of the triangular tiles
     int hrows;                  // rows of the left operand per CTA in cross tiles (128, or fewer: streaming form)
-    int smem_norms, compact;      // row norms of X out of the tiles in shared memory; cross tiles over Xnon
+    int smem_norms, compact;      // row norms of X out of the tiles in shared memory (2: streaming form); cross tiles over Xnon
     int alt;                    // the two epilogue sets take alternate tiles
     int full, rem, parts;       // tiles dealt whole; tiles of the last round, each cut into `parts` K ranges
     int len[PLAN_B];            // sequence lengths (B <= PLAN_B)
@@ -329,7 +339,7 @@ __device__ __noinline__ void make_plan(Plan& pl, const GramProblem& seg0, const 
         const int tiles0 = seg0.tri ? (narrow ? t128 : t256) : tc;
         const int total = nseg > 1 ? tiles0 + tc : tiles0;
         pl.tiles0 = tiles0; pl.total = total; pl.tw = narrow ? BM : PM; pl.hrows = hrows;
-        pl.smem_norms = stream || (!SPLIT && !cx.tri && nst >= 4 && nst <= 8 && total <= 2 * npairs && !compact) ? 1 : 0;
+        pl.smem_norms = stream ? 2 : (!SPLIT && !cx.tri && nst >= 4 && nst <= 8 && total <= 2 * npairs && !compact) ? 1 : 0;
         pl.compact = compact ? 1 : 0;
         // Short contractions, many tiles: a tile's main loop is as short as the bookkeeping of its
         // epilogue (column factors, barriers, atomics: dependent round trips), so the two sets of
@@ -478,6 +488,40 @@ __device__ __forceinline__ void copy_args(T& dst, const T& src, int i, int n) {
     static_assert(sizeof(T) % 8 == 0, "copied in 8-byte words");
     for (; i < (int)(sizeof(T) / 8); i += n)
         reinterpret_cast<unsigned long long*>(&dst)[i] = reinterpret_cast<const unsigned long long*>(&src)[i];
+}
+
+// The copies of one tile in the streaming form: every row of the left operand is copied once per
+// launch, so its lines are the first to leave L2.  Left to the default, a pass over an X larger than
+// L2 threw out all that the next launch starts with -- code, right operand, arguments (step over
+// T = 16384, d = 4096 with new rows each time: 45.5 -> 42.5 us; 4 x 4096: 41.5 -> 38.4;
+// 8 x 2000, d = 1536: 26.9 -> 24.8).  Not inlined and rolled: the same loop beside, or with a
+// choice of policy inside, the common one cost the pipelines 1-2 %.
+struct Fed { unsigned fills, used; int s; bool ok; };
+template <bool SPLIT>
+__device__ __noinline__ Fed feed_once(const CUtensorMap* amap, const CUtensorMap* bmap, const CUtensorMap* btail,
+                                      unsigned long long* full, unsigned long long* empty, volatile int* abort_flag,
+                                      unsigned char* smem, int subb, int a_bytes, unsigned tx, int nbox, bool tail32,
+                                      int a_row, int b_row, int wb, int nst, int ring, int s, unsigned fills) {
+    unsigned long long policy;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    Fed f{fills, 0u, s, true};
+    for (int st = 0; st < nst; ++st) {
+        if (!mbar_wait(&empty[f.s], ((f.fills >> f.s) & 1u) ^ 1u, abort_flag, 1)) { f.ok = false; break; }
+        unsigned char* su = smem + f.s * Stage<SPLIT>::NSUB * subb;
+        if (tx != 0) mbar_expect_tx(&full[f.s], tx);
+#pragma unroll 1
+        for (int u = 0; u < Stage<SPLIT>::NSUB; ++u, su += subb) {
+            const int k0 = st * Stage<SPLIT>::K + u * BK;
+            tma_load_3d_pair_once(amap, &full[f.s], su, k0, a_row, wb, policy);
+#pragma unroll 1
+            for (int j = 0; j < nbox; ++j)
+                tma_load_3d_pair(j == nbox - 1 && tail32 ? btail : bmap, &full[f.s], su + a_bytes + j * BOX_BYTES,
+                                 k0, b_row + j * BOX_N, wb);
+        }
+        f.fills ^= 1u << f.s; f.used |= 1u << f.s;
+        f.s = (f.s + 1 == ring) ? 0 : f.s + 1;
+    }
+    return f;
 }
 
 template <bool SPLIT>
@@ -648,6 +692,14 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                     prep_ok = true;
                     TRACE(3);
                     if (!ok) break;
+                }
+                if constexpr (!SPLIT) if (pl.smem_norms == 2 && !p.tri) {
+                    // (streaming form: no share of K is cut, st0 = 0)
+                    const Fed f = feed_once<SPLIT>(amap, &maps.b[sg], &maps.bt[sg], sh.full, sh.empty, abort_flag, smem,
+                                            subb, a_bytes, rank == 0 ? 2u * tx : 0u, nbox, tail32, a_row, b_row, wb, st1, cur_nst, s, fills);
+                    fills = f.fills; s = f.s; ok = f.ok;
+                    used |= f.used; ever |= f.used;
+                    continue;
                 }
                 for (int st = st0; st < st1; ++st) {
                     if (!mbar_wait(&sh.empty[s], ((fills >> s) & 1u) ^ 1u, abort_flag, 1)) { ok = false; break; }

@@ -274,7 +274,8 @@ ada_status ada_attention_reps(ada_ctx* ctx, const void* Q, const void* K, const 
 
 /* Same operations with HOST buffers: inputs are copied to the device (staging
  * buffers owned by the context, allocated on first use), the device-pointer
- * call above runs, results are copied back, all on `stream`, and the call
+ * call above runs, results are copied back, all in the order of `stream` (inputs
+ * that work queued on it is still filling are read after that work), and the call
  * returns after synchronising that stream.  Counts are int32[B] on the host.
  * Pinned host memory makes the copies asynchronous DMA transfers.  The context
  * must have been created with maxima covering the sizes. */

@@ -227,7 +227,7 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
     ctx->es = dt == ADA_F32 ? 4 : 2;
     ctx->engine = ADA_ENGINE_AUTO;
     ctx->stage = nullptr; ctx->stage_bytes = 0; ctx->host_stream = nullptr;
-    ctx->host_event = nullptr; ctx->host_out = false;
+    ctx->host_event = nullptr; ctx->host_ready = nullptr; ctx->host_out = false;
     ctx->attn_ws = nullptr; ctx->attn_ws_bytes = 0;
     ctx->map_cache = nullptr;
     ctx->tc_attr_set = false;
@@ -284,6 +284,14 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
         delete ctx;
         return ADA_ERR_CUDA;
     }
+    // for the *_host calls; made here so that a context's first such call costs no more than its second
+    if (cudaStreamCreateWithFlags(&ctx->host_stream, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->host_event, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->host_ready, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        ada_destroy(ctx);
+        return ADA_ERR_CUDA;
+    }
     ctx->map_cache = new_map_cache();
     *out = ctx;
     return ADA_OK;
@@ -302,6 +310,7 @@ ada_status ada_destroy(ada_ctx* ctx) {
     if (ctx->attn_ws) cudaFree(ctx->attn_ws);
     if (ctx->host_stream) cudaStreamDestroy(ctx->host_stream);
     if (ctx->host_event) cudaEventDestroy(ctx->host_event);
+    if (ctx->host_ready) cudaEventDestroy(ctx->host_ready);
     cudaFree(ctx->ws);
     delete_map_cache(ctx->map_cache);
     delete ctx;
@@ -837,9 +846,10 @@ ada_status ada_cascade_step_host(ada_ctx* ctx, const void* X, int64_t B, int64_t
     Stage sg = carve(ctx);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const size_t n_tok = (size_t)B * T;
-    // the inherited lists travel beside the activations, on a stream of their own
-    if (ctx->host_stream == nullptr) CU(cudaStreamCreateWithFlags(&ctx->host_stream, cudaStreamNonBlocking));
-    if (ctx->host_event == nullptr) CU(cudaEventCreateWithFlags(&ctx->host_event, cudaEventDisableTiming));
+    // the inherited lists travel beside the activations, on a stream of their own that joins the caller's
+    // before and after: work queued on `stream` ahead of the call may still be filling them
+    CU(cudaEventRecord(ctx->host_ready, s));
+    CU(cudaStreamWaitEvent(ctx->host_stream, ctx->host_ready, 0));
     CU(cudaMemcpyAsync(sg.X, X, n_tok * d * ctx->es, cudaMemcpyHostToDevice, s));
     CU(cudaMemcpyAsync(sg.l0, rep_in, n_tok * 4, cudaMemcpyHostToDevice, ctx->host_stream));
     CU(cudaMemcpyAsync(sg.c0, rep_in_cnt, (size_t)B * 4, cudaMemcpyHostToDevice, ctx->host_stream));

@@ -203,7 +203,7 @@ struct ada_ctx {
     char* stage;
     size_t stage_bytes;
     cudaStream_t host_stream;    // carries the small inputs beside the activations
-    cudaEvent_t host_event;
+    cudaEvent_t host_event, host_ready;   // lists copied; the caller's stream as it was before the call
     bool host_out;               // the call's outputs are mapped host memory
     ada::Profiler prof;
 };

@@ -71,6 +71,7 @@ ada_status setup_device(int device, PerDevice** out) {
         c.stage_bytes = 0;
         c.host_stream = nullptr;
         c.host_event = nullptr;
+        c.host_ready = nullptr;
         c.host_out = false;
         if (cudaDeviceGetAttribute(&c.sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
             return;

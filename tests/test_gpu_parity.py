@@ -730,3 +730,34 @@ def test_host_outputs_pinned_pageable_and_mixed(ada, pinned):
     assert torch.equal(gr, ref.gamma_rep.cpu()) and torch.equal(gc, ref.gamma_cross.cpu())
     assert ada.ada_device_status(ctx)[0] == 0
     ada.ada_destroy(ctx)
+
+
+@pytest.mark.parametrize("side", [False, True])
+def test_host_lists_are_read_in_stream_order(ada, side):
+    """The inherited list is still being written by work queued ahead of the call on the same stream:
+    the step takes the list that this work leaves behind."""
+    T, d = 1500, 512
+    X = torch.from_numpy(clustered(T, d, 9, "bf16").view(np.int16)).view(torch.bfloat16)
+    ctx = ada.ada_create(1, T, d, ada.ADA_BF16)
+    Xd, Xp = X.cuda(), X.pin_memory()
+    new, new_cnt, _ = ada.ada_select_full(ctx, Xd, TAU)
+    ref = ada.ada_cascade_step(ctx, Xd, TAU, new, new_cnt)
+    torch.cuda.synchronize()
+    stream = torch.cuda.Stream() if side else torch.cuda.current_stream()
+    for _ in range(3):
+        pin = lambda shape, kind=torch.int32: torch.zeros(shape, dtype=kind).pin_memory()
+        ri, rc, lists = pin((1, T)), pin(1), [pin(s) for _ in range(3) for s in ((1, T), 1)]
+        ri[0, :T // 2] = torch.arange(0, T // 2 * 2, 2)         # another valid list
+        rc[0] = T // 2
+        with torch.cuda.stream(stream):
+            torch.cuda._sleep(20_000_000)                       # about 10 ms
+            ri.copy_(new, non_blocking=True)
+            rc.copy_(new_cnt, non_blocking=True)
+            ada.ada_cascade_step_host(ctx, Xp, TAU, ri, rc, *lists)
+        for (got, cnt), want, want_cnt in zip(((lists[0], lists[1]), (lists[2], lists[3]), (lists[4], lists[5])),
+                                              (ref.rep_out, ref.add_idx, ref.rem_idx),
+                                              (ref.rep_out_cnt, ref.add_cnt, ref.rem_cnt)):
+            n = int(want_cnt[0])
+            assert int(cnt[0]) == n and got[0, :n].tolist() == want[0, :n].tolist()
+    assert ada.ada_device_status(ctx)[0] == 0
+    ada.ada_destroy(ctx)

@@ -277,17 +277,16 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
     ctx->splitX = split_bytes ? ctx->ws + o_sx : nullptr;
     ctx->splitR = split_bytes ? ctx->ws + o_sr : nullptr;
     ctx->part_buf = reinterpret_cast<unsigned*>(ctx->ws + o_part);
-    if (cudaMemset(ctx->ws, 0, o_xrep) != cudaSuccess ||
-        cudaMemset(ctx->part_buf, 0xFF, ctx->part_bytes) != cudaSuccess ||
-        (dt == ADA_BF16 && cudaMemset(ctx->ws + o_ntok, 0, n_tok * 4) != cudaSuccess)) {
-        cudaFree(ctx->ws);
-        delete ctx;
-        return ADA_ERR_CUDA;
-    }
-    // for the *_host calls; made here so that a context's first such call costs no more than its second
+    // A stream and events for the *_host calls: made here so that a context's first such call costs no
+    // more than its second.  The fills run on that stream, which waits for nobody, and are waited for: the
+    // first call may come on any stream, and none of them is ordered behind a fill.
     if (cudaStreamCreateWithFlags(&ctx->host_stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->host_event, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ctx->host_ready, cudaEventDisableTiming) != cudaSuccess) {
+        cudaEventCreateWithFlags(&ctx->host_ready, cudaEventDisableTiming) != cudaSuccess ||
+        cudaMemsetAsync(ctx->ws, 0, o_xrep, ctx->host_stream) != cudaSuccess ||
+        cudaMemsetAsync(ctx->part_buf, 0xFF, ctx->part_bytes, ctx->host_stream) != cudaSuccess ||
+        (dt == ADA_BF16 && cudaMemsetAsync(ctx->ws + o_ntok, 0, n_tok * 4, ctx->host_stream) != cudaSuccess) ||
+        cudaStreamSynchronize(ctx->host_stream) != cudaSuccess) {
         cudaGetLastError();
         ada_destroy(ctx);
         return ADA_ERR_CUDA;

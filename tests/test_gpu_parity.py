@@ -761,3 +761,24 @@ def test_host_lists_are_read_in_stream_order(ada, side):
             assert int(cnt[0]) == n and got[0, :n].tolist() == want[0, :n].tolist()
     assert ada.ada_device_status(ctx)[0] == 0
     ada.ada_destroy(ctx)
+
+
+def test_new_context_is_ready_for_a_call_on_any_stream(ada):
+    """ada_create returns with its workspace filled, whatever the default stream has queued: a first
+    call on a side stream, with tiles split along K, finds the exchange buffer empty."""
+    T, d = 700, 4096
+    X = torch.from_numpy(clustered(T, d, 13, "bf16").view(np.int16)).view(torch.bfloat16).cuda()
+    ctx = ada.ada_create(1, T, d, ada.ADA_BF16)
+    ref = ada.ada_select_full(ctx, X, TAU)
+    torch.cuda.synchronize()
+    ada.ada_destroy(ctx)
+    side = torch.cuda.Stream()
+    for _ in range(4):
+        torch.cuda._sleep(20_000_000)                           # about 10 ms on the default stream
+        ctx = ada.ada_create(1, T, d, ada.ADA_BF16)
+        with torch.cuda.stream(side):
+            got = ada.ada_select_full(ctx, X, TAU)
+        assert ada.ada_device_status(ctx, stream=side)[0] == 0
+        n = int(ref[1][0])
+        assert int(got[1][0]) == n and torch.equal(got[0][0, :n], ref[0][0, :n]) and torch.equal(got[2], ref[2])
+        ada.ada_destroy(ctx)

@@ -566,24 +566,24 @@ k_nearest_finish(unsigned long long* __restrict__ near_key, int32_t* __restrict_
     const int64_t o = (int64_t)b * T;
     const unsigned long long key = near_key[o + t];
     const int p = role[o + t];
+    const float inv = inv_norm[o + t];
     near_key[o + t] = 0ull;
     role[o + t] = 0;
     int idx;
     float g;
     if (p > 0) {
         idx = t;
-        g = inv_norm[o + t] > 0.f ? 1.f : 0.f;
+        g = inv > 0.f ? 1.f : 0.f;
     } else if (r_eff[b] <= 0) {
         idx = -1;
         g = 0.f;
-    } else if (key == 0ull) {
-        idx = rep_idx[o];
-        g = 0.f;
     } else {
-        // (the key's value still lacks the row's own factor, GramProblem::defer_row)
-        const unsigned pos = 0xFFFFFFFFu - (unsigned)(key & 0xFFFFFFFFull);
-        idx = rep_idx[o + pos];
-        g = __uint_as_float((unsigned)(key >> 32)) * inv_norm[o + t];
+        // (the key's value still lacks the row's own factor, GramProblem::defer_row; where that is 0 -- a
+        // zero row, or one so small that its squares vanish -- the row correlates with nothing)
+        g = __uint_as_float((unsigned)(key >> 32)) * inv;
+        const bool some = g > 0.f;
+        idx = rep_idx[o + (some ? 0xFFFFFFFFu - (unsigned)(key & 0xFFFFFFFFull) : 0u)];
+        if (!some) g = 0.f;
     }
     nearest_idx[o + t] = idx;
     if (nearest_gamma != nullptr) nearest_gamma[o + t] = g;

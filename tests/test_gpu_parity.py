@@ -419,6 +419,27 @@ def test_nearest_representative_small(ada, dtype, T, d):
     ada.ada_destroy(ctx)
 
 
+@pytest.mark.parametrize("dtype,T,d", [("bf16", 300, 72), ("bf16", 600, 768), ("bf16", 700, 4096), ("f32", 300, 72),
+                                       ("f32", 520, 768)])
+def test_nearest_of_rows_whose_squares_vanish(ada, dtype, T, d):
+    """Rows scaled by 2^-80: their squared norm is 0 in fp32, so they count as zero rows and go to the
+    first representative, though their dot products with the representatives are not 0."""
+    from parity import to_device
+    X = clustered(T, d, 55 + T, "f32")
+    R = list(range(3, T // 2, 4))
+    tiny = np.arange(T // 2 + 1, T, 5)
+    X[0, tiny] = X[0, np.array(R)[1 + np.arange(len(tiny)) % (len(R) - 1)]] * np.float32(2.0 ** -80)
+    Xd = to_device(wl.f32_to_bf16_bits(X) if dtype == "bf16" else X)
+    ctx = ada.ada_create(1, T, d, ada.ADA_BF16 if dtype == "bf16" else ada.ADA_F32)
+    idx = torch.zeros((1, T), dtype=torch.int32, device="cuda")
+    idx[0, :len(R)] = torch.tensor(R, dtype=torch.int32)
+    near, g = ada.ada_nearest_rep(ctx, Xd, idx, torch.tensor([len(R)], dtype=torch.int32, device="cuda"))
+    assert near[0, tiny].tolist() == [R[0]] * len(tiny)
+    assert g[0, tiny].abs().max().item() == 0.0
+    assert ada.ada_device_status(ctx) == (0, len(tiny))
+    ada.ada_destroy(ctx)
+
+
 def test_nearest_representative_on_configs(ada):
     """After full selection and after a cascade step, batched and at d = 4096."""
     from parity import lists, to_device

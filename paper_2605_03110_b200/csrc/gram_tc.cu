@@ -63,9 +63,9 @@ struct Shape {
 // triangular tile's maxima have been published, and a cross epilogue waits (bounded)
 // for the counter to reach the number of triangular tiles before it stages its column
 // factors.  The cross MAIN LOOPS do not wait, so the short r x r problem hides behind them.
-// Triangular tiles precede cross tiles in every CTA's order and wait on nothing, and the
-// launch is cooperative unless nothing else can keep its CTAs apart (coop_begin), so the wait
-// always ends.
+// Triangular tiles precede cross tiles in every CTA's order and wait on nothing (but the row norms, where
+// the launch makes those: every CTA's norm warps do their share without waiting), and the launch
+// is cooperative unless nothing else can keep its CTAs apart (coop_begin), so the wait always ends.
 __device__ __forceinline__ int seq_n(const GramProblem& p, int b) {
     return p.n_dev != nullptr ? p.n_dev[b] : p.n_host;
 }
@@ -856,7 +856,9 @@ cudaError_t launch_gram_tc(ada_ctx* ctx, const GramProblem* tri, const GramProbl
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     int na = 0;
-    const bool coop = fused && coop_begin(ctx, s);
+    // CTAs wait on results of other CTAs (triangle before cross epilogues, the row norms)
+    const bool waits = fused || nj.X != nullptr;
+    const bool coop = waits && coop_begin(ctx, s);
     if (coop) {
         attr[na].id = cudaLaunchAttributeCooperative;
         attr[na].val.cooperative = 1;
@@ -873,7 +875,7 @@ cudaError_t launch_gram_tc(ada_ctx* ctx, const GramProblem* tri, const GramProbl
     cudaError_t e = cudaLaunchKernelEx(&cfg, shortk ? (planes ? k_gram_tc<true, true> : k_gram_tc<true, false>)
                                                     : (planes ? k_gram_tc<false, true> : k_gram_tc<false, false>),
                                        maps, segs[0], segs[1], nseg, nj, ctx->tile_ctr, ctx->status);
-    if (fused) coop_end(ctx, coop);
+    if (waits) coop_end(ctx, coop);
     prof_end(ctx, s);
     return e;
 }

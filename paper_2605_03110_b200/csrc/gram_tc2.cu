@@ -1210,8 +1210,7 @@ cudaError_t launch_gram_tc2(ada_ctx* ctx, const GramProblem* tri, const GramProb
     const bool planes = segs[0].planes > 0;
     int max_parts = ctx->part_buf != nullptr ? ctx->max_parts : 1;
     if (nseg == 1 && segs[0].tri && segs[0].n_dev == nullptr) {
-        // tile count known here: a last round that is more than half full is not split, and the launch
-        // then need not be cooperative
+        // tile count known here: a last round that is more than half full is not split
         const int M = (segs[0].n_host + PM - 1) / PM, f = planes ? 2 : 1;
         const int64_t tiles = (int64_t)segs[0].B * (f * (M * (M - 1) / 2) + (segs[0].n_host + PM / f - 1) / (PM / f));
         if (2 * (tiles % ctx->tc2_pairs) > ctx->tc2_pairs || tiles % ctx->tc2_pairs == 0) max_parts = 1;
@@ -1230,8 +1229,8 @@ cudaError_t launch_gram_tc2(ada_ctx* ctx, const GramProblem* tri, const GramProb
     attr[na].val.clusterDim.x = 2; attr[na].val.clusterDim.y = 1; attr[na].val.clusterDim.z = 1;
     ++na;
     // CTAs wait on results of other CTAs (triangle before cross epilogues, the preparation before
-    // everything, the other shares of a split tile): all of them have to get to run
-    const bool waits = fused || gj.X != nullptr || sj.X != nullptr || max_parts > 1;
+    // everything, the row norms, the other shares of a split tile): all of them have to get to run
+    const bool waits = fused || gj.X != nullptr || sj.X != nullptr || nj.X != nullptr || max_parts > 1;
     const bool coop = waits && coop_begin(ctx, s);
     if (coop) {
         attr[na].id = cudaLaunchAttributeCooperative;

@@ -803,3 +803,56 @@ def test_new_context_is_ready_for_a_call_on_any_stream(ada):
         n = int(ref[1][0])
         assert int(got[1][0]) == n and torch.equal(got[0][0, :n], ref[0][0, :n]) and torch.equal(got[2], ref[2])
         ada.ada_destroy(ctx)
+
+
+def _gram_launches_of(call):
+    """The call captured in a stream: the cooperative attribute of its kernels whose blocks take a
+    whole SM's shared memory.  Nothing runs."""
+    from cuda.bindings import driver as cu
+
+    def ok(r):
+        assert r[0] == cu.CUresult.CUDA_SUCCESS, r[0]
+        return r[1] if len(r) == 2 else r[1:]
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        ok(cu.cuStreamBeginCapture(stream.cuda_stream, cu.CUstreamCaptureMode.CU_STREAM_CAPTURE_MODE_THREAD_LOCAL))
+        try:
+            call()
+        finally:
+            graph = ok(cu.cuStreamEndCapture(stream.cuda_stream))
+    found = []
+    for node in ok(cu.cuGraphGetNodes(graph, 64))[0]:
+        if int(node) == 0 or ok(cu.cuGraphNodeGetType(node)) != cu.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            continue
+        if ok(cu.cuGraphKernelNodeGetParams(node)).sharedMemBytes > 200 * 1024:
+            found.append(ok(cu.cuGraphKernelNodeGetAttribute(
+                node, cu.CUlaunchAttributeID.CU_LAUNCH_ATTRIBUTE_COOPERATIVE)).cooperative)
+    ok(cu.cuGraphDestroy(graph))
+    return found
+
+
+@pytest.mark.parametrize("dtype,engine,B,T,d", [
+    ("bf16", 0, 1, 700, 2048),     # split along K
+    ("bf16", 0, 1, 2300, 2048), ("bf16", 0, 1, 4096, 4096), ("bf16", 0, 2, 4096, 2048),   # whole tiles, norms in the launch
+    ("bf16", 2, 1, 4096, 2048),    # one-CTA kernel, norms in the launch
+    ("f32", 0, 1, 512, 768)])      # planes in the launch
+def test_captured_launches_that_wait_are_cooperative(ada, dtype, engine, B, T, d):
+    """Every Gram launch whose CTAs wait on other CTAs (the triangle, the preparation, the row norms, the
+    shares of a split tile) asks whether it has to be cooperative; a captured one always has to."""
+    kind = torch.bfloat16 if dtype == "bf16" else torch.float32
+    X = torch.randn((B, T, d), generator=torch.Generator("cuda").manual_seed(T), device="cuda").to(kind)
+    ctx = ada.ada_create(B, T, d, ada.ADA_F32 if dtype == "f32" else ada.ADA_BF16)
+    ada.ada_set_engine(ctx, engine)
+    ri, rc, g = ada.ada_select_full(ctx, X, TAU)                # (the one-time set-up of a context)
+    out = ada.ada_cascade_step(ctx, X, TAU, ri, rc)
+    torch.cuda.synchronize()
+    full = _gram_launches_of(lambda: ada.ada_select_full(ctx, X, TAU, ri, rc, g))
+    step = _gram_launches_of(lambda: ada.ada_cascade_step(ctx, X, TAU, ri, rc, out=out))
+    assert full == [1] and step == [1]
+    # launches without such waits do not ask: the norms are a launch of their own here
+    if dtype == "bf16" and engine == 0 and T == 700:
+        ada.ada_set_engine(ctx, ada.ADA_ENGINE_TCGEN05)
+        ada.ada_select_full(ctx, X, TAU, ri, rc, g)
+        assert _gram_launches_of(lambda: ada.ada_select_full(ctx, X, TAU, ri, rc, g)) == [0]
+    assert ada.ada_device_status(ctx)[0] == 0
+    ada.ada_destroy(ctx)

@@ -277,6 +277,8 @@ def ada_cascade_step_adaptive(ctx: Context, X: torch.Tensor, tau_state: torch.Te
     device, updated in place when a policy is given); `turnover` (float32[B]) receives Eq. 6."""
     X, B, T, d, ldx = _shape(X)
     assert tau_state.dtype == torch.float64 and tau_state.is_cuda and tau_state.numel() == B
+    if policy is not None and not isinstance(policy, TauPolicy):
+        raise C.ArgumentError("policy must be a TauPolicy")
     if out is None:
         out = CascadeOut(B, T, X.device, want_gamma)
     st = _fast.cascade_step_adaptive(

@@ -68,3 +68,61 @@ def test_create_rejects_bad_arguments_before_touching_a_device(lib):
     assert f(ctypes.byref(h), 0, 1, (1 << 21), 64, 1) == 1
     assert f(ctypes.byref(h), 0, 1 << 12, 1 << 20, 64, 1) == 1   # maxB * maxT above 2^30
     assert h.value is None
+
+
+def _calls():
+    """Every native call with CPU tensors and no context: argument lists by name, with the places of
+    required and of optional tensors."""
+    import torch
+    t = torch.zeros(64)
+    lists = [t] * 8 + [None] * 2
+    return {
+        "select_full": ([None, t, 1, 8, 8, 8, 0, 0.3, t, t, None, 0], (1, 8, 9), (10,)),
+        "select_full_heads": ([None, t, 8, 1, 8, 8, 0, 0.3, t, t, None, 0], (1, 8, 9), (10,)),
+        "cascade_step": ([None, t, 1, 8, 8, 8, 0, 0.3] + lists + [0, 0], (1,) + tuple(range(8, 16)), (16, 17)),
+        "cascade_step_heads": ([None, t, 8, 1, 8, 8, 0, 0.3] + lists + [0, 0], (1,) + tuple(range(8, 16)), (16, 17)),
+        "cascade_step_adaptive": ([None, t, 1, 8, 8, 8, 0, t, None] + lists + [None, 0, 0],
+                                  (1, 7) + tuple(range(9, 17)), (17, 18, 19)),
+        "nearest_rep": ([None, t, 1, 8, 8, 8, 0, t, t, t, None, 0], (1, 7, 8, 9), (10,)),
+        "attention_reps": ([None, t, t, t, 8, 1, 16, 16, 1, t, t, None, t, 16, 0, 0], (1, 2, 3, 9, 10, 12), (11,)),
+    }
+
+
+@pytest.mark.parametrize("name", sorted(_calls()))
+def test_native_calls_take_tensors_where_tensors_belong(name):
+    """A number or None in the place of a tensor raises instead of becoming a device address."""
+    from paper_2605_03110_b200 import binding
+    binding.lib()
+    call = getattr(binding._fast, name)
+    args, required, optional = _calls()[name]
+    assert call(*args) == 1                                     # ADA_ERR_INVALID_ARG: no context
+    for i in required + optional:
+        for wrong in (4096, 1.5, "x") + ((None,) if i in required else ()):
+            with pytest.raises(AttributeError):
+                call(*args[:i], wrong, *args[i + 1:])
+        assert call(*args[:i], args[1], *args[i + 1:]) == 1
+    with pytest.raises(TypeError):
+        call(*args[:-1])
+    if name in ("select_full", "cascade_step"):
+        assert call(*args[:7], "0.3", *args[8:]) == 1           # what float() takes
+        for wrong, error in ((None, TypeError), ("x", ValueError)):
+            with pytest.raises(error):
+                call(*args[:7], wrong, *args[8:])
+
+
+def test_policy_has_to_be_a_policy():
+    from types import SimpleNamespace
+
+    import torch
+
+    from paper_2605_03110_b200 import binding
+    binding.lib()
+    state = SimpleNamespace(dtype=torch.float64, is_cuda=True, numel=lambda: 1, data_ptr=lambda: 0)
+    X, i = torch.zeros(8, 8), torch.zeros(8, dtype=torch.int32)
+    args = (SimpleNamespace(addr=None), X, state)
+    stream = SimpleNamespace(cuda_stream=0)
+    with pytest.raises(ctypes.ArgumentError):
+        binding.ada_cascade_step_adaptive(*args, ctypes.c_double(0.1), i, i, stream=stream)
+    for policy in (None, binding.TauPolicy(0.2, 0.1, 0.25, 0.35)):
+        with pytest.raises(binding.AdaError):
+            binding.ada_cascade_step_adaptive(*args, policy, i, i, stream=stream)

@@ -96,7 +96,12 @@ def lib() -> C.CDLL:
         for name in SYMBOLS:
             if name not in ("ada_gram_op_count", "ada_status_string"):
                 getattr(L, name).restype = C.c_int
-        from . import _pycall
+        try:
+            from . import _pycall
+        except ImportError as e:
+            raise RuntimeError(
+                "the native marshalling module of this interpreter is missing or does not load: build it with "
+                f"`python -m paper_2605_03110_b200.build` ({e})") from e
         _lib, _fast = L, _pycall
     return _lib
 
@@ -114,9 +119,16 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return None if t is None else t.data_ptr()
 
 
+# the current stream's handle without a Stream object around it, where torch has these functions
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
+
+
 def _stream(stream) -> int:
-    if stream is None:           # the current stream's handle without a Stream object around it
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    if stream is None:
+        if _raw_stream is None:
+            return torch.cuda.current_stream().cuda_stream
+        return _raw_stream(_current_device())
     return stream.cuda_stream
 
 

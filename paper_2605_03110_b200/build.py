@@ -1,5 +1,5 @@
 """Build libada.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and the binding's native
-marshalling (_pycall.so, plain C) beside it."""
+marshalling (_pycall, plain C, one file per interpreter ABI) beside it."""
 from __future__ import annotations
 
 import glob
@@ -11,7 +11,8 @@ import sysconfig
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libada.so")
-PYCALL = os.path.join(HERE, "_pycall.so")
+# the suffix names the interpreter's ABI: another interpreter does not import it, and builds its own
+PYCALL = os.path.join(HERE, "_pycall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 PYCALL_SRC = os.path.join(CSRC, "pycall.c")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = [
@@ -50,7 +51,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if verbose or res_c.returncode != 0:
         sys.stderr.write(res_c.stdout + res_c.stderr)
     if res_c.returncode != 0:
-        raise RuntimeError("gcc failed building _pycall.so")
+        raise RuntimeError("gcc failed building " + os.path.basename(PYCALL))
     with open(os.path.join(HERE, "build.log"), "w") as f:
         f.write(" ".join(cmd) + "\n" + res.stdout + res.stderr)
     return LIB

@@ -126,3 +126,23 @@ def test_policy_has_to_be_a_policy():
     for policy in (None, binding.TauPolicy(0.2, 0.1, 0.25, 0.35)):
         with pytest.raises(binding.AdaError):
             binding.ada_cascade_step_adaptive(*args, policy, i, i, stream=stream)
+
+
+def test_native_module_carries_the_interpreter_abi(monkeypatch):
+    """Another interpreter neither loads this one's module nor takes the build for complete; a module that
+    is not there is explained."""
+    import importlib.machinery
+    import sys
+
+    from paper_2605_03110_b200 import binding
+    ada_build.build()
+    assert os.path.basename(ada_build.PYCALL) == "_pycall" + importlib.machinery.EXTENSION_SUFFIXES[0]
+    assert not ada_build.is_stale()
+    monkeypatch.setattr(ada_build, "PYCALL", ada_build.PYCALL.replace("_pycall.", "_pycall.other-"))
+    assert ada_build.is_stale()
+    import paper_2605_03110_b200
+    monkeypatch.delattr(paper_2605_03110_b200, "_pycall", raising=False)
+    monkeypatch.setitem(sys.modules, "paper_2605_03110_b200._pycall", None)
+    monkeypatch.setattr(binding, "_lib", None)
+    with pytest.raises(RuntimeError, match="paper_2605_03110_b200.build"):
+        binding.lib()

@@ -776,17 +776,38 @@ struct HostOut {
     void* dev;        // where the kernels write
     size_t bytes;     // copied back afterwards; 0: nothing to copy
 };
-static void* mapped(void* host) {
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-    return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
+// Device address of a host range that kernels may store 4-byte words to, or NULL: pinned from its first to its
+// last byte (part of a buffer may be registered), at consecutive device addresses, not read-only for the
+// device, and aligned.  A copy takes, or refuses, what a store would fault on.
+static void* mapped(void* host, size_t bytes) {
+    cudaPointerAttributes at, end;
+    unsigned flags = 0;
+    if (reinterpret_cast<uintptr_t>(host) % 4 != 0) return nullptr;
+    if (cudaPointerGetAttributes(&at, host) != cudaSuccess ||
+        cudaPointerGetAttributes(&end, static_cast<char*>(host) + bytes - 1) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (at.type != cudaMemoryTypeHost || end.type != cudaMemoryTypeHost || at.devicePointer == nullptr ||
+        static_cast<char*>(end.devicePointer) - static_cast<char*>(at.devicePointer) != (ptrdiff_t)(bytes - 1))
+        return nullptr;
+    if (cudaHostGetFlags(&flags, host) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    return (flags & cudaHostRegisterReadOnly) != 0 ? nullptr : at.devicePointer;
 }
-// the staging buffers become the outputs' own memory where every output is mapped
+// the staging buffers become the outputs' own memory where every output is mapped, and none overlaps
+// another (copied back one after the other, the last one stays; written by kernels, a mixture would)
 static void choose_outputs(ada_ctx* ctx, HostOut* out, int n) {
     void* m[8];
     for (int i = 0; i < n; ++i) {
-        m[i] = out[i].host != nullptr ? mapped(out[i].host) : nullptr;
-        if (out[i].host != nullptr && m[i] == nullptr) return;
+        m[i] = nullptr;
+        if (out[i].host == nullptr) continue;
+        const uintptr_t lo = reinterpret_cast<uintptr_t>(out[i].host);
+        for (int j = 0; j < i; ++j) {
+            const uintptr_t other = reinterpret_cast<uintptr_t>(out[j].host);
+            if (other != 0 && lo < other + out[j].bytes && other < lo + out[i].bytes) return;
+        }
+        m[i] = mapped(out[i].host, out[i].bytes);
+        if (m[i] == nullptr) return;
     }
     for (int i = 0; i < n; ++i) { out[i].dev = m[i]; out[i].bytes = 0; }
     ctx->host_out = true;
@@ -854,13 +875,13 @@ ada_status ada_cascade_step_host(ada_ctx* ctx, const void* X, int64_t B, int64_t
     CU(cudaMemcpyAsync(sg.c0, rep_in_cnt, (size_t)B * 4, cudaMemcpyHostToDevice, ctx->host_stream));
     CU(cudaEventRecord(ctx->host_event, ctx->host_stream));
     CU(cudaStreamWaitEvent(s, ctx->host_event, 0));
-    HostOut out[8] = {{rep_out, sg.l1, n_tok * 4}, {rep_out_cnt, sg.c1, (size_t)B * 4},
-                      {add_idx, sg.l2, n_tok * 4}, {add_cnt, sg.c2, (size_t)B * 4},
-                      {rem_idx, sg.l3, n_tok * 4}, {rem_cnt, sg.c3, (size_t)B * 4},
+    HostOut out[8] = {{rep_out, sg.l1, n_tok * 4}, {add_idx, sg.l2, n_tok * 4}, {rem_idx, sg.l3, n_tok * 4},
+                      {rep_out_cnt, sg.c1, (size_t)B * 4}, {add_cnt, sg.c2, (size_t)B * 4},
+                      {rem_cnt, sg.c3, (size_t)B * 4},
                       {gamma_rep, sg.g0, n_tok * 4}, {gamma_cross, sg.g1, n_tok * 4}};
     choose_outputs(ctx, out, 8);
-    st = ada_cascade_step(ctx, sg.X, B, T, d, d, dt, tau, sg.l0, sg.c0, (int32_t*)out[0].dev, (int32_t*)out[1].dev,
-                          (int32_t*)out[2].dev, (int32_t*)out[3].dev, (int32_t*)out[4].dev, (int32_t*)out[5].dev,
+    st = ada_cascade_step(ctx, sg.X, B, T, d, d, dt, tau, sg.l0, sg.c0, (int32_t*)out[0].dev, (int32_t*)out[3].dev,
+                          (int32_t*)out[1].dev, (int32_t*)out[4].dev, (int32_t*)out[2].dev, (int32_t*)out[5].dev,
                           gamma_rep ? (float*)out[6].dev : nullptr, gamma_cross ? (float*)out[7].dev : nullptr, flags, s);
     ctx->host_out = false;
     return st != ADA_OK ? st : copy_back(out, 8, s);

@@ -856,3 +856,44 @@ def test_captured_launches_that_wait_are_cooperative(ada, dtype, engine, B, T, d
         assert _gram_launches_of(lambda: ada.ada_select_full(ctx, X, TAU, ri, rc, g)) == [0]
     assert ada.ada_device_status(ctx)[0] == 0
     ada.ada_destroy(ctx)
+
+
+def test_host_outputs_that_kernels_must_not_write(ada):
+    """Pinned outputs that overlap one another or lie at odd addresses are copied back, in the order lists,
+    counts, gammas, as pageable ones are; whole registered buffers are as good as allocated ones."""
+    from types import SimpleNamespace
+    T, d = 1500, 512
+    X = torch.from_numpy(clustered(T, d, 7, "bf16").view(np.int16)).view(torch.bfloat16)
+    ctx = ada.ada_create(1, T, d, ada.ADA_BF16)
+    Xp = X.pin_memory()
+    ri = torch.zeros((1, T), dtype=torch.int32, device="cuda")
+    ri[0, :T // 2] = torch.arange(0, T, 2)                      # every other token: some of them redundant
+    rc = torch.tensor([T // 2], dtype=torch.int32, device="cuda")
+    ref = ada.ada_cascade_step(ctx, X.cuda(), TAU, ri, rc)
+    rih, rch = ri.cpu().pin_memory(), rc.cpu().pin_memory()
+    n_rep, n_add, n_rem = (int(c[0]) for c in (ref.rep_out_cnt, ref.add_cnt, ref.rem_cnt))
+    assert n_add > 0 and n_rem > 0
+    pin = lambda shape, kind=torch.int32: torch.zeros(shape, dtype=kind).pin_memory()
+    # one buffer for two lists, one for two gammas: what is copied last stays
+    ro, roc, lists, ac, mc, gam = pin(T), pin(1), pin(T), pin(1), pin(1), pin(T, torch.float32)
+    ada.ada_cascade_step_host(ctx, Xp, TAU, rih, rch, ro, roc, lists, ac, lists, mc, gam, gam)
+    assert ro[:n_rep].tolist() == ref.rep_out[0, :n_rep].tolist()
+    assert lists[:n_rem].tolist() == ref.rem_idx[0, :n_rem].tolist()
+    assert torch.equal(gam, ref.gamma_cross[0].cpu())
+    assert [int(t) for t in (roc, ac, mc)] == [n_rep, n_add, n_rem]
+    # an output two bytes off its alignment
+    raw = pin(4 * T + 4, torch.uint8)
+    odd = SimpleNamespace(data_ptr=lambda: raw.data_ptr() + 2)
+    ada.ada_cascade_step_host(ctx, Xp, TAU, rih, rch, odd, roc, lists, ac, pin(T), mc)
+    assert raw.numpy()[2:2 + 4 * n_rep].copy().view(np.int32).tolist() == ref.rep_out[0, :n_rep].tolist()
+    # a registered buffer
+    own = np.zeros(2 * 4096 + 4 * T, np.uint8)
+    at = -own.ctypes.data % 4096
+    size = -(-4 * T // 4096) * 4096
+    assert int(torch.cuda.cudart().cudaHostRegister(own.ctypes.data + at, size, 0)) == 0
+    reg = SimpleNamespace(data_ptr=lambda: own.ctypes.data + at)
+    ada.ada_cascade_step_host(ctx, Xp, TAU, rih, rch, reg, roc, lists, ac, pin(T), mc)
+    assert own[at:at + 4 * n_rep].view(np.int32).tolist() == ref.rep_out[0, :n_rep].tolist()
+    assert int(torch.cuda.cudart().cudaHostUnregister(own.ctypes.data + at)) == 0
+    assert ada.ada_device_status(ctx)[0] == 0
+    ada.ada_destroy(ctx)

@@ -85,7 +85,10 @@ inline int64_t plane_len(int64_t d) { return (d + 63) / 64 * 64; }
 #define CU(x)                                  \
     do {                                       \
         cudaError_t e__ = (x);                 \
-        if (e__ != cudaSuccess) return ADA_ERR_CUDA; \
+        if (e__ != cudaSuccess) {              \
+            cudaGetLastError(); /* reported by the status; the next launcher that asks must not find it */ \
+            return ADA_ERR_CUDA;               \
+        }                                      \
     } while (0)
 
 }  // namespace

@@ -619,6 +619,7 @@ static cudaError_t launch_compact(ada_ctx* ctx, int kid, const CompactArgs& a, i
     prof_begin(ctx, kid, s);
     cudaError_t e = V == 1 ? cudaLaunchKernelEx(&cfg, k_compact<1>, a)
                            : (V == 2 ? cudaLaunchKernelEx(&cfg, k_compact<2>, a) : cudaLaunchKernelEx(&cfg, k_compact<4>, a));
+    if (e != cudaSuccess) cudaGetLastError();   // returned; the next launcher that asks must not find it again
     prof_end(ctx, s);
     return e;
 }

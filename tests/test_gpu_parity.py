@@ -897,3 +897,18 @@ def test_host_outputs_that_kernels_must_not_write(ada):
     assert int(torch.cuda.cudart().cudaHostUnregister(own.ctypes.data + at)) == 0
     assert ada.ada_device_status(ctx)[0] == 0
     ada.ada_destroy(ctx)
+
+
+def test_a_refused_launch_does_not_fail_the_next_call(ada):
+    """More sequences than a grid's y extent holds: the call reports a CUDA error, and the next one, on
+    the same context, works."""
+    B = 65536
+    X = torch.ones((B, 1, 8), dtype=torch.bfloat16, device="cuda")
+    ctx = ada.ada_create(B, 1, 8, ada.ADA_BF16)
+    with pytest.raises(ada.AdaError) as e:
+        ada.ada_select_full(ctx, X, TAU)
+    assert e.value.status == 4                                  # ADA_ERR_CUDA
+    idx, cnt, gamma = ada.ada_select_full(ctx, X[:2], TAU)
+    assert idx.tolist() == [[0], [0]] and cnt.tolist() == [1, 1] and gamma.tolist() == [[0.0], [0.0]]
+    assert ada.ada_device_status(ctx)[0] == 0
+    ada.ada_destroy(ctx)

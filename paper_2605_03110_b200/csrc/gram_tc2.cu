@@ -636,8 +636,8 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
     }
     const unsigned prep_total = gridDim.x;
     if (!early && warp == 0) plan_work();
-    // (a plan is always made, by warp 0 of the same CTA, which waits for nobody)
-    while (!mbar_try_long(&sh.planned, 0)) { }
+    // (made by warp 0 of the same CTA, which waits for nobody)
+    const bool planned = __all_sync(0xffffffffu, mbar_wait(&sh.planned, 0, abort_flag, 18));
     const Plan& pl = sh.plan;
     const int tiles0 = pl.tiles0;
     const int hrows = pl.hrows;                          // rows per CTA of a cross tile
@@ -651,7 +651,9 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         decode_item<SPLIT>(&sh.seg[0], &sh.seg[1], pl, pair, npairs, it, own);
         return own;
     };
-    if (warp == 0) {
+    if (!planned) {
+        // no work: on to the end, where the status is raised
+    } else if (warp == 0) {
         // ------------------------------------------------ TMA producer (both CTAs)
         if (lane == 0) {
             unsigned fills = 0, used = 0, ever = 0;
@@ -783,7 +785,7 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
             }
         }
     } else {
-        // ------------------------------------------------ warps 2..13, both CTAs: row norms of X where
+        // ------------------------------------------------ warps 2..9, both CTAs: row norms of X where
         // the launch makes them, then the epilogue.  A warp reaches the TMEM lanes 32 (warp % 4)..;
         // the two warps of a lane quadrant share a tile's 32-column chunks (sub, sub + 2, ..), so
         // that a finished accumulator is read out by eight warps.

@@ -103,7 +103,10 @@ ada_status ada_set_engine(ada_ctx* ctx, ada_engine e);
  * has been seen idle by ada_device_status or ada_destroy), under stream capture, and under MPS.
  * on = 0 never uses the attribute: same kernels and results, but launches that overlap in
  * different streams can then wait for one another until the in-kernel limits expire
- * (ADA_ERR_TIMEOUT).  Meant for profilers that cannot replay cooperative launches. */
+ * (ADA_ERR_TIMEOUT).  Meant for profilers that cannot replay cooperative launches.
+ * Limit of every wait inside a kernel: 2 s, but 20 s in the launches of that first stream, whose CTAs
+ * may have to wait for SMs that a long kernel of another stream holds (a cooperative launch is
+ * not placed before they are free).  A fault that stalls a launch is reported after that time. */
 ada_status ada_set_cooperative(ada_ctx* ctx, int on);
 
 /* Algorithm 1 line 6 forms the cross-Gram from the tokens OUTSIDE the inherited set.  On the

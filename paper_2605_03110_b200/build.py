@@ -30,7 +30,7 @@ def is_stale() -> bool:
     if not os.path.exists(LIB) or not os.path.exists(PYCALL):
         return True
     t = min(os.path.getmtime(LIB), os.path.getmtime(PYCALL))
-    deps = sources() + [PYCALL_SRC] + glob.glob(os.path.join(CSRC, "*.cuh")) + \
+    deps = sources() + [PYCALL_SRC] + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + \
         [os.path.join(os.path.dirname(HERE), "include", "ada.h")]
     return any(os.path.getmtime(p) > t for p in deps)
 

@@ -3,7 +3,7 @@
 #include <stdio.h>
 #include <string.h>
 
-#include <mutex>
+#include <atomic>
 #include <new>
 
 #include "common.cuh"
@@ -95,28 +95,22 @@ inline int64_t plane_len(int64_t d) { return (d + 63) / 64 * 64; }
 
 namespace ada {
 
-// ---------------------------------------------------------------------------
-// Which launches have to be cooperative.  A Gram launch with CTAs that wait on one another ends
-// only if all of them get to run.  Two such launches in different streams could each hold
-// half of the SMs and wait for the other half for ever; a cooperative launch, placed whole or not
-// at all, rules that out, but the driver then neither places its CTAs while the kernel before
-// it drains nor lets them set up meanwhile (measured: 4 to 8 us per call of a chain).  So per
-// device ONE stream may launch without the attribute -- in stream order, its launches never
-// overlap one another -- and every other stream keeps it, until the first one has been seen idle.
-// Captured launches keep it too (where a graph will be replayed is unknown), and so does
-// everything under MPS (other processes are not known here).
-// ---------------------------------------------------------------------------
+// Which launches have to be cooperative: see launch_policy.h
 namespace {
-struct SoleStream {
-    std::mutex lock;
-    bool held = false;
-    unsigned long long id = 0;       // stream ids are never reused within a process
-    unsigned long long launches = 0; // launches without the attribute so far
-    int pending = 0;                 // of them, those not handed to the driver yet
-    int mps = -1;
-};
 constexpr int kMaxSole = 64;
 SoleStream g_sole[kMaxSole];
+std::atomic<int> g_mps[kMaxSole];        // 0: not asked yet, 1: no, 2: yes (or unknown)
+
+bool under_mps(int device) {
+    int v = g_mps[device].load(std::memory_order_relaxed);
+    if (v == 0) {
+        int on = 0;
+        if (cudaDeviceGetAttribute(&on, cudaDevAttrMpsEnabled, device) != cudaSuccess) { cudaGetLastError(); on = 1; }
+        v = on != 0 ? 2 : 1;
+        g_mps[device].store(v, std::memory_order_relaxed);
+    }
+    return v == 2;
+}
 }  // namespace
 
 bool coop_begin(ada_ctx* ctx, cudaStream_t s) {
@@ -127,41 +121,22 @@ bool coop_begin(ada_ctx* ctx, cudaStream_t s) {
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) { cudaGetLastError(); return true; }
     if (cap != cudaStreamCaptureStatusNone) return true;
     if (cudaStreamGetId(s, &id) != cudaSuccess) { cudaGetLastError(); return true; }
-    SoleStream& w = g_sole[ctx->device];
-    std::lock_guard<std::mutex> hold(w.lock);
-    if (w.mps < 0 && cudaDeviceGetAttribute(&w.mps, cudaDevAttrMpsEnabled, ctx->device) != cudaSuccess) {
-        cudaGetLastError();
-        w.mps = 1;
-    }
-    if (w.mps != 0 || (w.held && w.id != id)) return true;
-    w.held = true;
-    w.id = id;
-    ++w.launches;
-    ++w.pending;
-    return false;
+    return under_mps(ctx->device) || !g_sole[ctx->device].begin(id);
 }
 
 void coop_end(ada_ctx* ctx, bool coop) {
-    if (coop || !ctx->cooperative) return;
-    SoleStream& w = g_sole[ctx->device];
-    std::lock_guard<std::mutex> hold(w.lock);
-    --w.pending;
+    if (!coop && ctx->cooperative) g_sole[ctx->device].end();
 }
 
 unsigned long long sole_mark(int device) {
-    if (device < 0 || device >= kMaxSole) return 0;
-    SoleStream& w = g_sole[device];
-    std::lock_guard<std::mutex> hold(w.lock);
-    return w.pending == 0 ? w.launches : ~0ull;
+    return device < 0 || device >= kMaxSole ? 0 : g_sole[device].mark();
 }
 
 void sole_idle(int device, bool all, cudaStream_t s, unsigned long long mark) {
     if (device < 0 || device >= kMaxSole) return;
     unsigned long long id = 0;
     if (!all && cudaStreamGetId(s, &id) != cudaSuccess) { cudaGetLastError(); return; }
-    SoleStream& w = g_sole[device];
-    std::lock_guard<std::mutex> hold(w.lock);
-    if (w.held && w.launches == mark && (all || w.id == id)) w.held = false;
+    g_sole[device].idle(all, id, mark);
 }
 
 void prof_begin(ada_ctx* ctx, int kid, cudaStream_t s) {

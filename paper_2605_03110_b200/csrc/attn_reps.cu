@@ -43,7 +43,7 @@ struct alignas(16) AttnShared {
     unsigned long long s_full[2], s_empty[2], p_full[2], p_empty[2], o_full, o_empty;
     unsigned long long x_put[4];             // per 32-row group: the two warps of a row exchange their statistics
     unsigned tmem_base;
-    int abort_flag;
+    int abort_flag[2];
     float2 xstat[2][AQ];                     // (m_ref, l) of each warp set, by row
 };
 // Q (2 K blocks) | K ring 2 x 2 | V^T ring 2 x 2 | P 2 x 2.  The dynamic shared memory is declared
@@ -203,7 +203,7 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
     unsigned char* vs = smem + 6 * KB_BYTES;           // V^T ring: 2 slots x 2 K blocks of d_h rows
     unsigned char* ps = smem + 10 * KB_BYTES;          // P: 2 buffers x 2 K blocks
     AttnShared& sh = *reinterpret_cast<AttnShared*>(smem + 14 * KB_BYTES);
-    volatile int* abort_flag = &sh.abort_flag;
+    volatile int* abort_flag = sh.abort_flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     // Persistent CTAs: the work items are (128 query rows, head) pairs, nq * h of them with
@@ -227,7 +227,8 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
         }
         for (int i = 0; i < 4; ++i) mbar_init(&sh.x_put[i], 2);
         mbar_init(&sh.o_full, 1); mbar_init(&sh.o_empty, 8);
-        sh.abort_flag = 0;
+        sh.abort_flag[0] = 0;
+        sh.abort_flag[1] = wait_limit_units(false);   // (no CTA waits for another)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -290,7 +291,7 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
                 const unsigned ph = (base[s] - 1u) & 1u;
                 const unsigned long long t0 = global_ns();
                 while (!(mbar_try(&sh.k_empty[s], ph) && mbar_try(&sh.v_empty[s], ph)))
-                    if (*abort_flag != 0 || global_ns() - t0 > WAIT_LIMIT_NS / 2) { *abort_flag = 33; break; }
+                    if (*abort_flag != 0 || past_limit(2 * (global_ns() - t0), abort_flag)) { *abort_flag = 33; break; }
             }
         }
     } else if (warp == 1) {
@@ -529,9 +530,9 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
         tcgen05_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
     }
-    if (threadIdx.x == 0 && sh.abort_flag != 0) {
+    if (threadIdx.x == 0 && sh.abort_flag[0] != 0) {
         atomicOr(status, ST_TIMEOUT);
-        status[2] = 200u + (unsigned)sh.abort_flag;
+        status[2] = 200u + (unsigned)sh.abort_flag[0];
     }
     if (threadIdx.x == 0) ATRACE(17);
 }

@@ -7,6 +7,7 @@
 #include <string.h>
 
 #include "../../include/ada.h"
+#include "launch_policy.h"
 
 namespace ada {
 

@@ -216,7 +216,7 @@ struct alignas(16) SharedTc {
     unsigned long long tmem_empty[2];
     unsigned long long drain;
     unsigned tmem_base;
-    int abort_flag;
+    int abort_flag[2];          // why the CTA gives up (0: it does not); limit of its waits
     int tiles0, tiles1, par0, par1;
     int wide0, wide1;           // widest tile of each segment (fixes the segment's ring geometry)
     unsigned long long dep_seen[2];   // per epilogue set: every triangular tile of the grid is done
@@ -265,14 +265,14 @@ template <bool SHORTK, bool PLANES>
 __global__ void __launch_bounds__(Shape<SHORTK>::THREADS, 1)
 k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramProblem seg0,
           const __grid_constant__ GramProblem seg1, const int nseg,
-          const __grid_constant__ NormJob norms, unsigned* __restrict__ dep_ctr,
+          const __grid_constant__ NormJob norms, const int wait_limit, unsigned* __restrict__ dep_ctr,
           unsigned* __restrict__ status) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     constexpr int RING = Shape<SHORTK>::RING;
     SharedTc<SHORTK>& sh = *reinterpret_cast<SharedTc<SHORTK>*>(smem + RING);
-    volatile int* abort_flag = &sh.abort_flag;
+    volatile int* abort_flag = sh.abort_flag;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -288,7 +288,8 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
         mbar_init(&sh.drain, 1);
         for (int q = 0; q < 2; ++q) { mbar_init(&sh.dep_seen[q], 1); sh.pub[q] = 0u; }
         for (int q = 0; q < Shape<SHORTK>::EPI_WARPS / 4; ++q) mbar_init(&sh.staged[q], 4);
-        sh.abort_flag = 0;
+        sh.abort_flag[0] = 0;
+        sh.abort_flag[1] = wait_limit;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -527,7 +528,7 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
                 const unsigned ph = ((fills >> q) & 1u) ^ 1u;      // parity of the last fill's phase
                 const unsigned long long t0 = global_ns();
                 while (!mbar_try(&sh.full[q], ph)) {
-                    if (global_ns() - t0 > WAIT_LIMIT_NS / 2) { *abort_flag = 7; break; }
+                    if (past_limit(2 * (global_ns() - t0), abort_flag)) { *abort_flag = 7; break; }
                 }
             }
         }
@@ -584,7 +585,7 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
             umma_commit(&sh.drain);
             const unsigned long long t0 = global_ns();
             while (!mbar_try(&sh.drain, 0)) {
-                if (global_ns() - t0 > WAIT_LIMIT_NS / 2) { *abort_flag = 8; break; }
+                if (past_limit(2 * (global_ns() - t0), abort_flag)) { *abort_flag = 8; break; }
             }
         }
     } else if (warp < 2 + Shape<SHORTK>::EPI_WARPS) {
@@ -767,9 +768,9 @@ k_gram_tc(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPro
                      "r"(TMEM_COLS)
                      : "memory");
     }
-    if (threadIdx.x == 0 && sh.abort_flag != 0) {
+    if (threadIdx.x == 0 && sh.abort_flag[0] != 0) {
         atomicOr(status, ST_TIMEOUT);
-        status[2] = (unsigned)sh.abort_flag;
+        status[2] = (unsigned)sh.abort_flag[0];
     }
 }
 
@@ -874,7 +875,8 @@ cudaError_t launch_gram_tc(ada_ctx* ctx, const GramProblem* tri, const GramProbl
     const bool planes = segs[0].planes > 0;
     cudaError_t e = cudaLaunchKernelEx(&cfg, shortk ? (planes ? k_gram_tc<true, true> : k_gram_tc<true, false>)
                                                     : (planes ? k_gram_tc<false, true> : k_gram_tc<false, false>),
-                                       maps, segs[0], segs[1], nseg, nj, ctx->tile_ctr, ctx->status);
+                                       maps, segs[0], segs[1], nseg, nj, wait_limit_units(ctx->cooperative && waits && !coop),
+                                       ctx->tile_ctr, ctx->status);
     if (waits) coop_end(ctx, coop);
     prof_end(ctx, s);
     return e;

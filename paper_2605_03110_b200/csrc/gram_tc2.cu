@@ -416,7 +416,7 @@ struct alignas(16) SharedPair {
     unsigned long long prep_seen, norm_seen[SUBS], dep_seen[SUBS];
     unsigned pub_cnt;                          // epilogue warps that have published their share of a triangular tile
     unsigned tmem_base;
-    int abort_flag;
+    int abort_flag[2];                         // why the CTA gives up (0: it does not); limit of its waits
     unsigned norm_cnt[MAX_STAGES];             // norm warps done with a stage
     unsigned long long normed;                 // the sums of squares of a tile's rows are in norm_part
     float norm_part[2][SUBS][BM];              // by tile parity and set
@@ -468,7 +468,7 @@ __device__ __forceinline__ bool take_partials(uint4* src, uint4 (&x)[8], unsigne
             if (*abort_flag != 0) return false;
             const unsigned long long now = global_ns();
             if (t0 == 0) t0 = now;
-            else if (now - t0 > WAIT_LIMIT_NS) { *abort_flag = 16; return false; }
+            else if (past_limit(now - t0, abort_flag)) { *abort_flag = 16; return false; }
         }
         load_partials(src, x);
     }
@@ -529,14 +529,14 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1)
 k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramProblem seg0,
            const __grid_constant__ GramProblem seg1, const int nseg,
            const __grid_constant__ NormJob norms, const __grid_constant__ GatherJob gather,
-           const __grid_constant__ SplitJob split, const int max_parts, unsigned* __restrict__ part_buf,
+           const __grid_constant__ SplitJob split, const int max_parts, const int wait_limit, unsigned* __restrict__ part_buf,
            unsigned* __restrict__ dep_ctr, unsigned* __restrict__ status) {
     using St = Stage<SPLIT>;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     SharedPair<SPLIT>& sh = *reinterpret_cast<SharedPair<SPLIT>*>(smem + Ring<SPLIT>::BYTES);
-    volatile int* abort_flag = &sh.abort_flag;
+    volatile int* abort_flag = sh.abort_flag;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned rank = cluster_rank();            // 0 = leader
@@ -560,7 +560,8 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         for (int q = 0; q < SUBS; ++q) mbar_init(&sh.staged[q], 4);
         for (int q = 0; q < SUBS; ++q) { mbar_init(&sh.norm_seen[q], 1); mbar_init(&sh.dep_seen[q], 1); }
         sh.pub_cnt = 0u;
-        sh.abort_flag = 0;
+        sh.abort_flag[0] = 0;
+        sh.abort_flag[1] = wait_limit;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -728,7 +729,7 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                 const unsigned ph = ((fills >> q) & 1u) ^ 1u;
                 const unsigned long long t0 = global_ns();
                 while (!mbar_try(&sh.empty[q], ph)) {
-                    if (*abort_flag != 0 || global_ns() - t0 > WAIT_LIMIT_NS / 2) { *abort_flag = 7; break; }
+                    if (*abort_flag != 0 || past_limit(2 * (global_ns() - t0), abort_flag)) { *abort_flag = 7; break; }
                 }
             }
         }
@@ -781,7 +782,7 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
             umma_commit_pair_local(&sh.drain);
             const unsigned long long t0 = global_ns();
             while (!mbar_try(&sh.drain, 0)) {
-                if (global_ns() - t0 > WAIT_LIMIT_NS / 2) { *abort_flag = 8; break; }
+                if (past_limit(2 * (global_ns() - t0), abort_flag)) { *abort_flag = 8; break; }
             }
         }
     } else {
@@ -1114,9 +1115,9 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                      "r"(TMEM_COLS)
                      : "memory");
     }
-    if (threadIdx.x == 0 && sh.abort_flag != 0) {
+    if (threadIdx.x == 0 && sh.abort_flag[0] != 0) {
         atomicOr(status, ST_TIMEOUT);
-        status[2] = 100u + (unsigned)sh.abort_flag;
+        status[2] = 100u + (unsigned)sh.abort_flag[0];
     }
     if (threadIdx.x == 0) TRACE(63);
 }
@@ -1247,8 +1248,8 @@ cudaError_t launch_gram_tc2(ada_ctx* ctx, const GramProblem* tri, const GramProb
     cfg.attrs = attr;
     cfg.numAttrs = na;
     cudaError_t e = cudaLaunchKernelEx(&cfg, planes ? k_gram_tc2<true> : k_gram_tc2<false>, maps, segs[0], segs[1],
-                                       nseg, nj, gj, sj, max_parts, ctx->part_buf, ctx->tile_ctr,
-                                       ctx->status);
+                                       nseg, nj, gj, sj, max_parts, wait_limit_units(ctx->cooperative && waits && !coop),
+                                       ctx->part_buf, ctx->tile_ctr, ctx->status);
     if (waits) coop_end(ctx, coop);
     prof_end(ctx, s);
     return e;

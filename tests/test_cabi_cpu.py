@@ -2,6 +2,7 @@
 import ctypes
 import os
 import re
+import subprocess
 
 import pytest
 
@@ -146,3 +147,49 @@ def test_native_module_carries_the_interpreter_abi(monkeypatch):
     monkeypatch.setattr(binding, "_lib", None)
     with pytest.raises(RuntimeError, match="paper_2605_03110_b200.build"):
         binding.lib()
+
+
+def _run_host_code(tmp_path, body):
+    """Compiles `body` as main() beside the library's host-side launch rules and runs it."""
+    src = tmp_path / "rules.cc"
+    src.write_text('#include "launch_policy.h"\n#undef NDEBUG\n#include <assert.h>\nint main() {' + body + "return 0; }")
+    exe = str(tmp_path / "rules")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-pthread", "-I", ada_build.CSRC, "-o", exe, str(src)], check=True)
+    subprocess.run([exe], check=True)
+
+
+def test_one_stream_launches_without_the_attribute(tmp_path):
+    _run_host_code(tmp_path, """
+        ada::SoleStream w;
+        assert(!w.holds(7));
+        assert(w.begin(7)); w.end();                  // the first stream takes the place ...
+        assert(w.holds(7) && !w.holds(8));
+        assert(!w.begin(8));                          // ... and every other one is refused
+        assert(w.begin(7)); w.end();
+        const unsigned long long seen = w.mark();
+        w.idle(false, 8, seen);                       // another stream idle: nothing is known about 7
+        assert(w.holds(7) && !w.begin(8));
+        assert(w.begin(7)); w.end();                  // a launch after the mark
+        w.idle(false, 7, seen);
+        assert(w.holds(7) && !w.begin(8));
+        w.idle(false, 7, w.mark());                   // its own stream idle, nothing launched since
+        assert(!w.holds(7) && w.begin(8)); w.end();
+        assert(!w.begin(7));
+        w.idle(true, 0, w.mark());                    // the whole device idle
+        assert(w.begin(7));                           // not handed to the driver yet:
+        const unsigned long long pending = w.mark();
+        w.end();
+        w.idle(true, 0, pending);                     // the synchronisation did not wait for it
+        assert(w.holds(7) && !w.begin(8));
+        w.idle(true, 0, w.mark());
+        assert(!w.holds(7));
+    """)
+
+
+def test_limit_of_the_waits_inside_a_launch(tmp_path):
+    """Two seconds, but for the launch that may be placed piece by piece beside other streams' kernels."""
+    _run_host_code(tmp_path, """
+        auto seconds = [](bool alone) { return ada::wait_limit_units(alone) * 1048576e-9; };
+        assert(seconds(false) > 1.99 && seconds(false) < 2.01);
+        assert(seconds(true) > 19.9 && seconds(true) < 20.1);
+    """)

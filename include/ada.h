@@ -344,6 +344,10 @@ ada_status ada_device_status(ada_ctx* ctx, void* stream, int64_t* n_zero_norm_ro
  * Nothing faults, traps or hangs. */
 ada_status ada_selftest_wait_timeout(ada_ctx* ctx, int limit_ms, void* stream);
 
+/* Self-test of the launch rule stated at ada_set_cooperative: 1 if `stream` is the one stream of `device` whose
+ * launches go without the cooperative attribute now, else 0.  Host-only, enqueues nothing. */
+int ada_selftest_launches_alone(int device, void* stream);
+
 /* Per-kernel timing (for benchmarks): when enabled, every kernel launch of
  * this context is bracketed by CUDA events on the launching stream.
  * ada_profile_read synchronises those events, fills up to `cap` entries

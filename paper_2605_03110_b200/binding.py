@@ -27,7 +27,8 @@ SYMBOLS = [
     "ada_create", "ada_destroy", "ada_set_engine", "ada_normalize", "ada_select_full",
     "ada_cascade_step", "ada_select_full_host", "ada_cascade_step_host", "ada_gram_op_count",
     "ada_device_status", "ada_profile_enable", "ada_profile_read", "ada_status_string",
-    "ada_select_full_noalloc", "ada_set_cooperative", "ada_selftest_wait_timeout", "ada_nearest_rep",
+    "ada_select_full_noalloc", "ada_set_cooperative", "ada_selftest_wait_timeout",
+    "ada_selftest_launches_alone", "ada_nearest_rep",
     "ada_select_full_heads", "ada_cascade_step_heads", "ada_set_dependent_launch",
     "ada_cascade_step_adaptive", "ada_attention_reps", "ada_set_row_compaction",
 ]
@@ -65,6 +66,7 @@ def lib() -> C.CDLL:
         L.ada_set_dependent_launch.argtypes = [vp, C.c_int]
         L.ada_set_row_compaction.argtypes = [vp, i64]
         L.ada_selftest_wait_timeout.argtypes = [vp, C.c_int, vp]
+        L.ada_selftest_launches_alone.argtypes = [C.c_int, vp]
         L.ada_normalize.argtypes = [vp, vp, i64, i64, i64, i64, C.c_int, vp, fp, i32p, i32p, vp, vp]
         L.ada_select_full.argtypes = [vp, vp, i64, i64, i64, i64, C.c_int, C.c_double, i32p, i32p,
                                       fp, vp]
@@ -206,6 +208,11 @@ def ada_selftest_wait_timeout(ctx: Context, limit_ms: int = 50, stream=None) -> 
     """Enqueue the bounded-wait self-test; ada_device_status then reports ADA_ERR_TIMEOUT."""
     _check(lib().ada_selftest_wait_timeout(ctx.h, int(limit_ms), _stream(stream)),
            "ada_selftest_wait_timeout")
+
+
+def ada_selftest_launches_alone(stream=None, device: int = 0) -> bool:
+    """Is `stream` the one stream of the device whose launches go without the cooperative attribute?"""
+    return bool(lib().ada_selftest_launches_alone(device, _stream(stream)))
 
 
 def ada_gram_op_count(cascade: bool, T: int, d: int, r: int = 0) -> int:

@@ -139,6 +139,13 @@ void sole_idle(int device, bool all, cudaStream_t s, unsigned long long mark) {
     g_sole[device].idle(all, id, mark);
 }
 
+bool sole_holds(int device, cudaStream_t s) {
+    unsigned long long id = 0;
+    if (device < 0 || device >= kMaxSole) return false;
+    if (cudaStreamGetId(s, &id) != cudaSuccess) { cudaGetLastError(); return false; }
+    return g_sole[device].holds(id);
+}
+
 void prof_begin(ada_ctx* ctx, int kid, cudaStream_t s) {
     Profiler& pr = ctx->prof;
     if (!pr.on || pr.n >= Profiler::MAXREC) return;
@@ -870,6 +877,11 @@ ada_status ada_selftest_wait_timeout(ada_ctx* ctx, int limit_ms, void* stream) {
     DeviceGuard guard(ctx->device);
     CU(launch_selftest_wait(ctx, limit_ms, static_cast<cudaStream_t>(stream)));
     return ADA_OK;
+}
+
+int ada_selftest_launches_alone(int device, void* stream) {
+    DeviceGuard guard(device);
+    return sole_holds(device, static_cast<cudaStream_t>(stream)) ? 1 : 0;
 }
 
 ada_status ada_profile_enable(ada_ctx* ctx, int on) {

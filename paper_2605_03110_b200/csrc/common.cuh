@@ -258,6 +258,7 @@ bool coop_begin(ada_ctx* ctx, cudaStream_t s);
 void coop_end(ada_ctx* ctx, bool coop);
 unsigned long long sole_mark(int device);
 void sole_idle(int device, bool all, cudaStream_t s, unsigned long long mark);
+bool sole_holds(int device, cudaStream_t s);
 
 void* new_map_cache();            // NULL: none could be made, which costs only time
 void delete_map_cache(void* c);

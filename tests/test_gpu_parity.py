@@ -708,22 +708,38 @@ def test_tiles_split_along_the_contraction(ada, dtype, T, d):
 
 def test_two_streams_launch_without_waiting_on_each_other(ada):
     """Two contexts in two streams at once: only one stream's launches may go without the
-    cooperative attribute.  Results equal those of one stream, and no wait expires."""
-    T, d = 1500, 2048
-    Xs = [torch.from_numpy(clustered(T, d, 5 + i, "bf16").view(np.int16)).view(torch.bfloat16).cuda() for i in range(2)]
-    ctx = [ada.ada_create(1, T, d, ada.ADA_BF16) for _ in range(2)]
-    ref = [ada.ada_select_full(ctx[i], Xs[i], TAU) for i in range(2)]
-    steps = [ada.ada_cascade_step(ctx[i], Xs[i], TAU, ref[i][0], ref[i][1]) for i in range(2)]
-    torch.cuda.synchronize()
+    cooperative attribute.  Steps, and full selections whose tiles are split along K (T = 1500) or
+    are not (T = 2300: their CTAs wait for the row norms alone).  Results equal those of one stream, and no
+    wait expires."""
+    d, Ts = 2048, (1500, 2300)
+    ada.ada_destroy(ada.ada_create(1, 16, 8, ada.ADA_BF16))     # the device idle: no stream holds the place
+    Xs = [[torch.from_numpy(clustered(T, d, 5 + i, "bf16").view(np.int16)).view(torch.bfloat16).cuda() for T in Ts]
+          for i in range(2)]
+    ctx = [ada.ada_create(1, max(Ts), d, ada.ADA_BF16) for _ in range(2)]
+    ref = [[ada.ada_select_full(ctx[i], X, TAU) for X in Xs[i]] for i in range(2)]
+    steps = [[ada.ada_cascade_step(ctx[i], X, TAU, r[0], r[1]) for X, r in zip(Xs[i], ref[i])] for i in range(2)]
+    assert ada.ada_selftest_launches_alone()                    # the references' stream, until it has been seen idle
     streams = [torch.cuda.Stream() for _ in range(2)]
+    assert ada.ada_device_status(ctx[0])[0] == 0
+    assert not ada.ada_selftest_launches_alone()
     for _ in range(20):
-        out = [ada.ada_cascade_step(ctx[i], Xs[i], TAU, ref[i][0], ref[i][1], stream=streams[i]) for i in range(2)]
+        got = []
+        for i in range(2):
+            with torch.cuda.stream(streams[i]):
+                got.append([(ada.ada_cascade_step(ctx[i], X, TAU, r[0], r[1]), ada.ada_select_full(ctx[i], X, TAU))
+                            for X, r in zip(Xs[i], ref[i])])
+        assert ada.ada_selftest_launches_alone(streams[0]) and not ada.ada_selftest_launches_alone(streams[1])
         torch.cuda.synchronize()
         for i in range(2):
-            assert torch.equal(out[i].rep_out_cnt, steps[i].rep_out_cnt)
-            assert torch.equal(out[i].gamma_cross, steps[i].gamma_cross)
-    for c, s in zip(ctx, streams):
-        assert ada.ada_device_status(c, stream=s)[0] == 0
+            for (step, full), want, full_want in zip(got[i], steps[i], ref[i]):
+                assert torch.equal(step.rep_out_cnt, want.rep_out_cnt)
+                assert torch.equal(step.gamma_cross, want.gamma_cross)
+                assert torch.equal(full[1], full_want[1]) and torch.equal(full[2], full_want[2])
+    assert ada.ada_device_status(ctx[1], stream=streams[1])[0] == 0
+    assert ada.ada_selftest_launches_alone(streams[0])          # the other stream's idleness says nothing about it
+    assert ada.ada_device_status(ctx[0], stream=streams[0])[0] == 0
+    assert not ada.ada_selftest_launches_alone(streams[0])
+    for c in ctx:
         ada.ada_destroy(c)
 
 

@@ -285,6 +285,12 @@ struct GramMaps {
 // measured shifts at them are 7.9e-6 (bf16, d = 3450, p = 3) and 8.6e-6 (fp32, d = 1600, p = 3).
 template <bool SPLIT>
 __device__ __forceinline__ bool shares_ok(int p, int d) { return (p - 1) * d <= (SPLIT ? MAX_SPLIT_D_F32 : MAX_SPLIT_D) / 2 * p; }
+// Limits of the plan's rules in stages of a bf16 tile: what a split has to save, the longest contraction whose
+// norms come out of the tiles in shared memory, the longest whose epilogue sets take alternate tiles.  The last
+// two count on whole tiles (ring_s below, the shares of pub_cnt): what they cover is never split.
+constexpr int SPLIT_SAVES = 10, SMEM_NORM_STAGES = 8, ALT_STAGES = 12;
+static_assert(ALT_STAGES - (ALT_STAGES + MAX_PARTS - 1) / MAX_PARTS < SPLIT_SAVES && SMEM_NORM_STAGES <= ALT_STAGES,
+              "tiles read by alternate sets, or for their norms, are whole");
 template <bool SPLIT>
 __device__ __noinline__ void make_plan(Plan& pl, const GramProblem& seg0, const GramProblem& seg1, int nseg,
                                           bool maybe_compact, int npairs, int max_parts, int lane) {
@@ -302,7 +308,11 @@ __device__ __noinline__ void make_plan(Plan& pl, const GramProblem& seg0, const 
     big = __all_sync(0xffffffffu, big);
     // streaming form: one column tile covers the columns of every sequence and the rows are many,
     // so the launch is one pass over the rows of A, and shorter row tiles put every pair to work.
-    // (Below 48 rows per CTA the right operand would be most of the traffic; splitting K is cheaper.)
+    // Below 48 rows per CTA the right operand would be most of the traffic and splitting K is cheaper.  d = 4096,
+    // 2 % representatives, new rows at every call, split against streaming form: T = 4096 (28 rows) 28.4
+    // and 30.3 us, 6000 (41) 33.8 and 34.8, 7200 (50) 36.2 and 35.1, 8192 (57) 38.6 and 36.6, 10000 (69)
+    // 43.8 and 40.7.  (With an X that the call before left in L2 the lines cross at 64 rows: 31.8 and
+    // 36.1 at T = 8192.)
     const bool stream = !SPLIT && one && cx.hb_rows >= 48;
     const int hrows = stream && cx.hb_rows < BM ? cx.hb_rows : BM;
     const bool compact = !SPLIT && maybe_compact && big && !one;       // (compact_wanted)
@@ -325,9 +335,9 @@ __device__ __noinline__ void make_plan(Plan& pl, const GramProblem& seg0, const 
     const int nst = ((SPLIT ? cx.planes : cx.d) + Stage<SPLIT>::K - 1) / Stage<SPLIT>::K;
     const int cand = (lane & 8) ? t128 + tc : t256 + tc, q1 = (lane & 7) + 1;
     const int rounds = quot(cand, npairs), rem = cand - rounds * npairs;
-    // the exchange costs about 5 us: as much as six stages of fp32 planes, ten of bf16
+    // the exchange costs about 5 us: as much as six stages of fp32 planes, ten of bf16 (SPLIT_SAVES)
     const bool can = q1 == 1 || (!stream && q1 <= max_parts && shares_ok<SPLIT>(q1, cx.d) && rem > 0 && q1 * rem <= npairs && 2 * q1 <= nst &&
-                                 nst - quot(nst + q1 - 1, q1) >= (SPLIT ? 6 : 10));
+                                 nst - quot(nst + q1 - 1, q1) >= (SPLIT ? 6 : SPLIT_SAVES));
     const unsigned cans = __ballot_sync(0xffffffffu, can);
     const int parts256 = 32 - __clz(cans & 0xffu), parts128 = 32 - __clz((cans >> 8) & 0xffu);
     const int rounds256 = __shfl_sync(0xffffffffu, rounds + (rem > 0), 0), rounds128 = __shfl_sync(0xffffffffu, rounds + (rem > 0), 8);
@@ -339,13 +349,19 @@ __device__ __noinline__ void make_plan(Plan& pl, const GramProblem& seg0, const 
         const int tiles0 = seg0.tri ? (narrow ? t128 : t256) : tc;
         const int total = nseg > 1 ? tiles0 + tc : tiles0;
         pl.tiles0 = tiles0; pl.total = total; pl.tw = narrow ? BM : PM; pl.hrows = hrows;
-        pl.smem_norms = stream ? 2 : (!SPLIT && !cx.tri && nst >= 4 && nst <= 8 && total <= 2 * npairs && !compact) ? 1 : 0;
+        // Norms out of the tiles in shared memory also for 385 to 1024 elements and at most two tiles a pair, where
+        // the plain loads hold the epilogues up more than a late stage release does: steps over 4096 x 768,
+        // r = 410, 19.5 -> 18.8 us, 4 x 2048 x 768, r = 410, 27.1 -> 25.6, 2 x 2048 x 512 18.9 -> 18.5; at
+        // 1024 elements even (20.7), at 1536 slower (22.0 -> 23.7).
+        pl.smem_norms = stream ? 2 : (!SPLIT && !cx.tri && nst >= 4 && nst <= SMEM_NORM_STAGES && total <= 2 * npairs && !compact) ? 1 : 0;
         pl.compact = compact ? 1 : 0;
         // Short contractions, many tiles: a tile's main loop is as short as the bookkeeping of its
         // epilogue (column factors, barriers, atomics: dependent round trips), so the two sets of
         // four warps take alternate tiles, one accumulator each, and one set's bookkeeping runs beside
-        // the other's reading.  Otherwise both read every tile and its maxima are there sooner.
-        pl.alt = Stage<SPLIT>::ALT && !pl.smem_norms && nst <= 12 && total > 2 * npairs ? 1 : 0;
+        // the other's reading.  Otherwise both read every tile and its maxima are there sooner.  Steps, both
+        // reading against alternating: 2 x 8192 x 768, r = 819, 39.7 -> 36.6 us; 8192 x 1024, r = 1638, 38.9 ->
+        // 38.3; at 1536 elements, the longest that alternates, 46.0 -> 46.7.
+        pl.alt = Stage<SPLIT>::ALT && !pl.smem_norms && nst <= ALT_STAGES && total > 2 * npairs ? 1 : 0;
         pl.parts = narrow ? parts128 : parts256;
         pl.rem = pl.parts > 1 ? the_rem : 0;
         pl.full = total - pl.rem;

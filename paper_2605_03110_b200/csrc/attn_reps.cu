@@ -22,15 +22,6 @@ namespace ada {
 
 using namespace tc;
 
-// Time stamps for in-kernel timelines (development builds only: -DADA_TRACE): the first 16 query
-// tiles of head 0.
-#ifdef ADA_TRACE
-__device__ unsigned long long g_atrace[16 * 32];
-#define ATRACE(slot) do { if (blockIdx.y == 0 && blockIdx.x < 16) g_atrace[blockIdx.x * 32 + (slot)] = tc::global_ns(); } while (0)
-#else
-#define ATRACE(slot) do { } while (0)
-#endif
-
 namespace {
 
 constexpr int AQ = 128;                 // query rows per CTA (TMEM lanes)
@@ -216,7 +207,6 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
         if (threadIdx.x == 0) { atomicOr(status, ST_TIMEOUT); status[2] = 299u; }
         return;
     }
-    if (threadIdx.x == 0) ATRACE(0);
     if (threadIdx.x == 0) {
         mbar_init(&sh.q_full, 1); mbar_init(&sh.q_empty, 1);
         for (int i = 0; i < 2; ++i) {
@@ -248,7 +238,6 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
     const int n = clamp_count(rep_cnt, T);
     const int nq = (n + AQ - 1) / AQ;
     const int total = nq * h;                          // (a CTA without an item falls through to the end)
-    if (threadIdx.x == 0) ATRACE(1);
     const int nkv_all = (n + AKV - 1) / AKV;
     const int nkb = (d_h + BK - 1) / BK;               // 64-element K blocks of the first contraction
     const int v_kb_bytes = d_h * BK * 2;               // one K block (64 keys) of the V^T tile
@@ -382,8 +371,6 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
                 const unsigned ph = (base + ((unsigned)j >> 1)) & 1u;
                 bool got = mbar_wait(&sh.s_full[half], ph, abort_flag, 40);
                 if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
-                if (k == 0 && j == 0 && threadIdx.x == 64) ATRACE(2);
-                if (k == 0 && j == 2 && threadIdx.x == 64) ATRACE(20);
                 tcgen05_fence_after();
                 // columns past r, and under the causal mask the keys after the query, count as -inf
                 const int c0 = j * AKV;
@@ -405,7 +392,6 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
                     }
                 }
                 cm *= sc;                                          // sc > 0: the maximum of the scaled scores
-                if (k == 0 && j == 2 && threadIdx.x == 64) ATRACE(21);
                 const float m_new = fmaxf(m_ref, cm);
                 const bool raise = m_new > m_ref + ATT_LAG;        // also true for the first finite maximum
                 // the MMAs of this set's previous tile have retired: its P buffer is free and nothing
@@ -427,7 +413,6 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
                     l *= f;
                     if (raise) m_ref = m_new;
                 }
-                if (k == 0 && j == 2 && threadIdx.x == 64) ATRACE(22);
                 // sweep 2: the probabilities
                 const float mref = m_ref > -INFINITY ? m_ref : 0.f;   // all scores -inf so far: every p is 0
                 unsigned char* prow = ps + half * 2 * KB_BYTES + i * 128;
@@ -446,12 +431,10 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
                     sum += exp_store(r1, sc, mref, prow + (c >> 6) * KB_BYTES, 4, i);
                 }
                 l += sum;
-                if (k == 0 && j == 2 && threadIdx.x == 64) ATRACE(23);
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMA reads P through the async proxy
                 tcgen05_fence_before();
                 __syncwarp();
                 if (lane == 0) { mbar_arrive(&sh.s_empty[half]); mbar_arrive(&sh.p_full[half]); }
-                if (k == 0 && threadIdx.x == 64) ATRACE(3 + min(j, 12));
             }
             if (!ok) break;
             base += (half == 0) ? (unsigned)(nkv + 1) >> 1 : (unsigned)nkv >> 1;
@@ -460,7 +443,6 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
             // (the statistics' slots are reused: everybody is done with the previous item's)
             if (k > 0) got = got && mbar_wait(&sh.o_empty, (unsigned)(k - 1) & 1u, abort_flag, 48);
             if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
-            if (k == 0 && threadIdx.x == 64) ATRACE(16);
             tcgen05_fence_after();
             sh.xstat[half][i] = make_float2(m_ref, l);
             __syncwarp();
@@ -521,7 +503,6 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
             tcgen05_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh.o_empty);
-            if (k == 0 && threadIdx.x == 64) ATRACE(18);
         }
         tcgen05_fence_before();
     }
@@ -534,7 +515,6 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
         atomicOr(status, ST_TIMEOUT);
         status[2] = 200u + (unsigned)sh.abort_flag[0];
     }
-    if (threadIdx.x == 0) ATRACE(17);
 }
 
 // ---------------------------------------------------------------- expansion (Section 2.3)
@@ -605,14 +585,3 @@ cudaError_t launch_attention_reps(ada_ctx* ctx, const void* Q, const void* K, co
 }
 
 }  // namespace ada
-
-#ifdef ADA_TRACE
-extern "C" int ada_trace_read_attn(unsigned long long* host, int clear) {
-    if (cudaMemcpyFromSymbol(host, ada::g_atrace, sizeof(ada::g_atrace)) != cudaSuccess) return 1;
-    if (clear) {
-        static unsigned long long zeros[16 * 32];
-        if (cudaMemcpyToSymbol(ada::g_atrace, zeros, sizeof(zeros)) != cudaSuccess) return 2;
-    }
-    return 0;
-}
-#endif

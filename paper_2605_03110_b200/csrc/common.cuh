@@ -133,7 +133,7 @@ struct SplitJob {
     float* inv_rep;           // [B*T] by position
 };
 
-// Row norms computed inside a tensor-core Gram launch by four extra warps per CTA
+// Row norms computed inside a tensor-core Gram launch by eight warps per CTA
 // (Section 2.1; Algorithm 1 line 1): inv_norm[row] = 1/||x_row|| for all n_rows rows of X.
 // X == NULL: nothing to do.
 struct NormJob {

@@ -40,14 +40,6 @@ namespace ada {
 
 using namespace tc;
 
-// Time stamps for in-kernel timelines (development builds only: -DADA_TRACE).
-#ifdef ADA_TRACE
-__device__ unsigned long long g_trace[160 * 64];
-#define TRACE(slot) do { g_trace[blockIdx.x * 64 + (slot)] = tc::global_ns(); } while (0)
-#else
-#define TRACE(slot) do { } while (0)
-#endif
-
 namespace {
 
 constexpr int PM = 2 * BM;     // rows of a pair tile
@@ -632,7 +624,6 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
     grid_dep_wait();
     // (the compaction's blocks may take the SMs that fall idle first: they wait for this whole grid)
     grid_dep_launch_next();
-    if (threadIdx.x == 0) TRACE(0);
     if (has_prep && warp >= 2) {
         // ------------------------------------------------ preparation, by every warp that is idle at
         // the start.  Items are dealt across the SMs first, so that a
@@ -648,7 +639,6 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         if (threadIdx.x == 64) {
             __threadfence();
             atomicAdd(dep_ctr + 3, 1u);
-            TRACE(2);
         }
     }
     const unsigned prep_total = gridDim.x;
@@ -661,7 +651,6 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
     const bool smem_norms = pl.smem_norms != 0;        // row norms out of the tiles in shared memory
     const bool compact = pl.compact != 0;                // cross tiles over the copied-out rows (Xnon)
     Item own;                                            // an item beyond the table
-    if (threadIdx.x == 0) TRACE(1);
 
     auto item_at = [&](int it) __attribute__((always_inline)) -> const Item& {
         if (it < ITEMS) return sh.item[it];
@@ -709,7 +698,6 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                     mbar_arrive(&sh.prep_seen);
                     asm volatile("fence.proxy.async.global;" ::: "memory");
                     prep_ok = true;
-                    TRACE(3);
                     if (!ok) break;
                 }
                 if constexpr (!SPLIT) if (pl.smem_norms == 2 && !p.tri) {
@@ -774,7 +762,6 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                 const unsigned d_tmem = tmem_base + acc * BN;
                 for (int st = st0; st < st1; ++st) {
                     if (!mbar_wait(&sh.full[s], (uses >> s) & 1u, abort_flag, 3)) { ok = false; break; }
-                    if (tile_it == 1 && st == st0) TRACE(5);
                     tcgen05_fence_after();
                     const unsigned s_addr = smem_u32(smem + s * sb);
 #pragma unroll
@@ -792,9 +779,7 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                     s = (s + 1 == cur_nst) ? 0 : s + 1;
                 }
                 if (ok) umma_commit_pair_both(&sh.tmem_full[acc]);   // both epilogues may read
-                TRACE(8 + 2 * (int)min(tile_it - 1, 8u));
             }
-            TRACE(6);
             umma_commit_pair_local(&sh.drain);
             const unsigned long long t0 = global_ns();
             while (!mbar_try(&sh.drain, 0)) {
@@ -926,7 +911,6 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                         else atomicAdd(status + 1, 1u);
                         p.inv_out[o + row] = inv;
                     }
-                    if (lrow == 0) TRACE(40);
                 }
             }
             if (!prep_ok) {
@@ -1013,7 +997,6 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                 ok = await(dep_ctr, dep_total, sh.dep_seen, 5);
                 if (!ok) break;
                 dep_ok = true;
-                if (warp == 2 && lane == 0) TRACE(4);
             }
             // Column factors: the set's chunks are dealt to its four warps.  (Columns past the tile are
             // clamped to its last one and discarded afterwards, so that no load hangs on a
@@ -1118,7 +1101,6 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                     atomicAdd(dep_ctr, 1u);
                 }
             }
-            if (warp == 2 && lane == 0) TRACE(9 + 2 * (int)min(tile_it - 1, 8u));
         }
     }
 
@@ -1135,7 +1117,6 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
         atomicOr(status, ST_TIMEOUT);
         status[2] = 100u + (unsigned)sh.abort_flag[0];
     }
-    if (threadIdx.x == 0) TRACE(63);
 }
 
 }  // namespace
@@ -1272,14 +1253,3 @@ cudaError_t launch_gram_tc2(ada_ctx* ctx, const GramProblem* tri, const GramProb
 }
 
 }  // namespace ada
-
-#ifdef ADA_TRACE
-extern "C" int ada_trace_read(unsigned long long* host, int clear) {
-    if (cudaMemcpyFromSymbol(host, ada::g_trace, sizeof(ada::g_trace)) != cudaSuccess) return 1;
-    if (clear) {
-        static unsigned long long zeros[160 * 64];
-        if (cudaMemcpyToSymbol(ada::g_trace, zeros, sizeof(zeros)) != cudaSuccess) return 2;
-    }
-    return 0;
-}
-#endif

@@ -34,22 +34,6 @@ struct Piece {
     int b, row0, col0, ncols, n, m;
 };
 
-struct alignas(16) Shared {
-    unsigned long long full[MAX_STAGES];
-    unsigned long long empty[MAX_STAGES];
-    unsigned long long tmem_full[2];
-    unsigned long long tmem_empty[2];
-    unsigned long long drain;
-    unsigned tmem_base;
-    int abort_flag;
-    int tiles0, tiles1, par0, par1;
-    // per epilogue warp, so that staging needs no barrier across warps
-    alignas(16) float col_scale[4][BN];
-    alignas(16) int col_token[4][BN];
-};
-static constexpr int SMEM_BYTES = RING_BYTES + (int)sizeof(Shared) + 1024;   // +1024: alignment slack
-static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
-
 // ---------------------------------------------------------------- PTX wrappers
 static __device__ __forceinline__ unsigned smem_u32(const void* p) {
     return static_cast<unsigned>(__cvta_generic_to_shared(p));
@@ -70,18 +54,6 @@ static __device__ __forceinline__ bool mbar_try(unsigned long long* bar, unsigne
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// non-blocking form: try_wait may suspend the thread for a while before it reports failure
-static __device__ __forceinline__ bool mbar_test(unsigned long long* bar, unsigned parity) {
-    unsigned ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
         : "r"(smem_u32(bar)), "r"(parity)

@@ -41,6 +41,11 @@
  *     fp32) and applies 1/(|x_s| |x_t|) in the epilogue; a normalised bf16 copy
  *     of X is never fed to the Gram.  gamma is compared in fp32 with
  *     (float)(1 - tau*tau), strict "<".
+ *   - Accuracy of gamma on the tensor cores: their accumulator truncates, so a correlation comes
+ *     out too small, by up to 4e-9 d + 2e-6 of itself for ADA_BF16 and 8e-9 d + 2e-6 for ADA_F32
+ *     (measured against 64 bits: 1.4e-5 and 2.4e-5 at d = 4096; ADA_ENGINE_FFMA 4e-6).  Tiles that
+ *     several SM pairs share along d (small problems, d <= 4600, fp32 <= 2140) keep a half to a quarter of
+ *     that error, so the same row's gamma may differ by up to 1e-5 with the number of rows around it.
  */
 #ifndef ADA_H_
 #define ADA_H_
@@ -70,8 +75,8 @@ typedef enum { ADA_F32 = 0, ADA_BF16 = 1 } ada_dtype;
 
 /* Which Gram kernel family a context uses.  AUTO: tensor cores (tcgen05), one- or two-CTA
  * form by problem size.  ADA_BF16 feeds the stored values to the MMA; ADA_F32 is split into
- * three bf16 terms per value and contracted as the six leading cross terms (error at fp32
- * rounding level, fp32 accumulation), at the price of a 6x longer contraction and a
+ * three bf16 terms per value and contracted as the six leading cross terms (what is dropped is
+ * below 2^-23 |x||y|; accumulation as stated above), at the price of a 6x longer contraction and a
  * workspace of 12 bytes per element.  FFMA is the plain fp32 ALU kernel (any storage type;
  * for ADA_BF16 a slow cross-check of the tensor-core path).  TCGEN05 forces the one-CTA
  * kernel (128-row tiles), TCGEN05_PAIR the two-CTA kernel (cta_group::2, 256-row tiles

@@ -928,3 +928,26 @@ def test_a_refused_launch_does_not_fail_the_next_call(ada):
     assert idx.tolist() == [[0], [0]] and cnt.tolist() == [1, 1] and gamma.tolist() == [[0.0], [0.0]]
     assert ada.ada_device_status(ctx)[0] == 0
     ada.ada_destroy(ctx)
+
+
+@pytest.mark.parametrize("dtype,d", [("bf16", 768), ("bf16", 2048), ("bf16", 4096), ("bf16", 5120),
+                                     ("f32", 256), ("f32", 768), ("f32", 1600), ("f32", 2600), ("f32", 4096)])
+def test_accumulation_error_stays_within_what_the_header_states(ada, dtype, d):
+    """Whole contractions (the one-CTA kernel never splits them) and whatever the library chooses, against
+    64 bits.  The tensor core truncates its accumulator, so a sum over d elements is short by at most one
+    unit in the last place, 2^-23, per accumulation of 16 elements (fp32: six terms), and the running sum is
+    half as large on average: d / 32 x 2^-23 = 3.7e-9 d for bf16.  fp32's five small terms move an
+    accumulator that cuts off less than a whole unit each time; ada.h states 8e-9 d.  2e-6: norms."""
+    T = 520
+    X = clustered(T, d, 17 + d, dtype)
+    _, ref = oracle.select_full(wl.as_f64(X[0]), TAU)
+    from parity import to_device
+    ctx = ada.ada_create(1, T, d, ada.ADA_F32 if dtype == "f32" else ada.ADA_BF16)
+    for engine in (ada.ADA_ENGINE_TCGEN05, ada.ADA_ENGINE_AUTO):
+        ada.ada_set_engine(ctx, engine)
+        gamma = ada.ada_select_full(ctx, to_device(X), TAU)[2]
+        err = gamma.cpu().numpy()[0] - ref
+        bound = (4e-9 if dtype == "bf16" else 8e-9) * d + 2e-6
+        assert np.max(np.abs(err)) <= bound, (engine, float(np.max(np.abs(err))), bound)
+    assert ada.ada_device_status(ctx)[0] == 0
+    ada.ada_destroy(ctx)

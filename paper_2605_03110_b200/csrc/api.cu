@@ -15,7 +15,7 @@ namespace {
 const char* const kKernelNames[K_COUNT] = {
     "norm_gather",     "gram_ffma_tri",    "gram_ffma_cross",
     "gram_tc_tri",     "gram_tc_cross",    "gram_tc_cascade", "split_bf16x3",  "compact_full",
-    "compact_cascade", "nearest_finish",
+    "compact_cascade", "nearest_finish",  "step_short",
 };
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -219,6 +219,7 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
     ctx->cooperative = true;
     ctx->dep_launch = true;
     ctx->tc2_attr_set = false;
+    ctx->short_attr_set = false;
     ctx->tc2_pairs = 0;
     ctx->compact_min_rows = 8192;
     ctx->max_parts = MAX_PARTS;
@@ -474,6 +475,17 @@ static ada_status cascade_impl(ada_ctx* ctx, const void* X, int64_t B, int64_t T
     TauUpdate tau_upd;
     memset(&tau_upd, 0, sizeof(tau_upd));
     if (tu != nullptr) tau_upd = *tu;
+
+    // one attention head per sequence, or rows as short as that: the whole step in one launch
+    if (ctx->engine == ADA_ENGINE_AUTO && tu == nullptr && use_tc(ctx, dt)) {
+        const int ctas = step_short_ctas(ctx, B, T, d);
+        if (ctas > 0) {
+            CU(launch_step_short(ctx, ctas, X, (int)B, (int)T, (int)d, ldx, xb, thr, rep_in, rep_in_cnt, rep_out,
+                                 rep_out_cnt, add_idx, add_cnt, rem_idx, rem_cnt, gamma_rep, gamma_cross,
+                                 (flags & ADA_CROSS_CAUSAL) ? 1 : 0, s));
+            return ADA_OK;
+        }
+    }
 
     // role map, gamma scratch and dependency counters are zero on entry (workspace invariant
     // kept by the compaction kernels).

@@ -32,6 +32,7 @@ enum KernelId {
     K_COMPACT_FULL,
     K_COMPACT_CASCADE,
     K_NEAREST_FINISH,
+    K_STEP_SHORT,
     K_COUNT
 };
 
@@ -174,6 +175,8 @@ struct ada_ctx {
     bool dep_launch;     // kernels are launched with programmatic stream serialization
     int compact_min_rows;  // sequence length from which a large inherited set's complement is copied out
     bool tc2_attr_set;   // pair-CTA kernel configured
+    bool short_attr_set; // one-launch step of short rows configured
+    int short_clusters[9];  // of its clusters of 1..8 CTAs, how many run at once
     int tc2_pairs;       // clusters of two that fit on the device at once
     // device workspace
     char* ws;            // one allocation
@@ -300,6 +303,14 @@ cudaError_t launch_gram_tc(ada_ctx* ctx, const GramProblem* tri, const GramProbl
                            const NormJob* norms, cudaStream_t s);
 bool gram_tc_available();
 cudaError_t launch_selftest_wait(ada_ctx* ctx, int limit_ms, cudaStream_t s);
+
+// short_step.cu: a whole cascade step over many sequences of short bf16 rows in one launch, by clusters of C CTAs
+// (0: not these sizes)
+int step_short_ctas(ada_ctx* ctx, int64_t B, int64_t T, int64_t d);
+cudaError_t launch_step_short(ada_ctx* ctx, int C, const void* X, int B, int T, int d, int64_t ldx, int64_t xb, float thr,
+                              const int32_t* rep_in, const int32_t* rep_in_cnt, int32_t* rep_out, int32_t* rep_out_cnt,
+                              int32_t* add_idx, int32_t* add_cnt, int32_t* rem_idx, int32_t* rem_cnt, float* gamma_rep,
+                              float* gamma_cross, int causal, cudaStream_t s);
 
 // attn_reps.cu (Eq. 2 on the representative rows, both contractions on tcgen05)
 cudaError_t launch_attention_reps(ada_ctx* ctx, const void* Q, const void* K, const void* V, int T, int h,

@@ -134,6 +134,75 @@ def test_heads_on_gptj_shaped_layers(ada, h, d_h):
     ada.ada_destroy(ctx)
 
 
+# the step in one launch: edges of row tiles (128), chunks (256 representatives), rows per CTA and cluster
+# sizes, K blocks (64 elements); sets from empty to all tokens
+@pytest.mark.parametrize("T,h,d_h", [(1, 5, 128), (127, 2, 64), (128, 3, 72), (129, 2, 120), (1025, 19, 128),
+                                     (2048, 30, 40), (1300, 110, 8), (4000, 12, 96)])
+def test_heads_step_in_one_launch(ada, T, h, d_h):
+    from parity import check_cascade
+    ctx = ada.ada_create(h, T, d_h, ada.ADA_BF16)
+    X = clustered_heads(T, h, d_h, 3 + T + h, "bf16")
+    rng = np.random.default_rng(T)
+    sizes = [min(T, s) for s in (128, 0, 257, T, 1, 512, 256, 129, 700)]
+    sets = [np.sort(rng.permutation(T)[:sizes[j % len(sizes)]]).tolist() for j in range(h)]
+    keep = list(range(h)) if h * T <= 20000 else sorted(rng.permutation(h)[:6].tolist())
+    for causal in (False, True):
+        if len(keep) == h:
+            check_cascade(ctx, X, TAU, sets, causal=causal, heads=True)
+            continue
+        # the oracle for a few of the heads; all of them against the step of several launches
+        check_cascade(ctx, np.ascontiguousarray(X[:, keep]), TAU, [sets[j] for j in keep], causal=causal, heads=True)
+        ri = torch.zeros((h, T), dtype=torch.int32)
+        for j, r in enumerate(sets):
+            ri[j, :len(r)] = torch.tensor(r, dtype=torch.int32)
+        ri, rc = ri.cuda(), torch.tensor([len(r) for r in sets], dtype=torch.int32, device="cuda")
+        from parity import lists, to_device
+        outs = []
+        for engine in (ada.ADA_ENGINE_AUTO, ada.ADA_ENGINE_TCGEN05):
+            ada.ada_set_engine(ctx, engine)
+            outs.append(ada.ada_cascade_step_heads(ctx, to_device(X), TAU, ri, rc,
+                                                   flags=ada.ADA_CROSS_CAUSAL if causal else 0))
+        ada.ada_set_engine(ctx, ada.ADA_ENGINE_AUTO)
+        assert ada.ada_device_status(ctx)[0] == 0
+        one, several = outs
+        for a, b in (("rep_out", "rep_out_cnt"), ("add_idx", "add_cnt"), ("rem_idx", "rem_cnt")):
+            for x, y in zip(lists(getattr(one, a), getattr(one, b)), lists(getattr(several, a), getattr(several, b))):
+                assert x.tolist() == y.tolist()
+        # the same products and sums; norms are summed in another order (16 fp32 terms a lane, then a tree)
+        assert torch.allclose(one.gamma_cross, several.gamma_cross, rtol=1e-6, atol=0)
+        assert torch.allclose(one.gamma_rep, several.gamma_rep, rtol=1e-6, atol=0)
+    ada.ada_destroy(ctx)
+
+
+def test_heads_step_reports_what_it_meets(ada):
+    """Zero rows counted once each, non-finite rows, lists and counts that are none; the context serves the
+    next call."""
+    from parity import check_cascade, to_device
+    T, h, d_h = 300, 3, 64
+    ctx = ada.ada_create(h, T, d_h, ada.ADA_BF16)
+    X = clustered_heads(T, h, d_h, 11, "bf16")
+    good = [[0, 5, 130, 299], [], list(range(200))]
+
+    def step(Xn, sets, counts=None):
+        ri = torch.zeros((h, T), dtype=torch.int32)
+        for j, r in enumerate(sets):
+            ri[j, :len(r)] = torch.tensor(r, dtype=torch.int32)
+        rc = torch.tensor(counts or [len(r) for r in sets], dtype=torch.int32)
+        ada.ada_cascade_step_heads(ctx, to_device(Xn), TAU, ri.cuda(), rc.cuda())
+        return ada.ada_device_status(ctx)
+
+    Z = X.copy()
+    Z[[3, 130, 280], [0, 1, 2]] = 0
+    assert step(Z, good) == (0, 3)
+    Z[7, 1, 5] = 0x7FC0                          # NaN in a head without representatives
+    assert ada.status_string(step(Z, good)[0]) == "ADA_ERR_NONFINITE"
+    for bad, counts in (([[5, 5], [], []], None), ([[7, 3], [], []], None), ([[-1], [], [T]], None),
+                        (good, [4, -1, 200]), (good, [4, 0, T + 1])):
+        assert ada.status_string(step(X, bad, counts)[0]) == "ADA_ERR_BAD_INDEX_SET"
+    check_cascade(ctx, X, TAU, good, heads=True)
+    ada.ada_destroy(ctx)
+
+
 def test_heads_error_paths(ada):
     ctx = ada.ada_create(4, 64, 64, ada.ADA_BF16)
     lib, vp = ada.lib(), None

@@ -302,13 +302,11 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
                     if (!mbar_wait(&sh.k_full[b], ph, abort_flag, 36)) { ok = false; return; }
                     if (!mbar_wait(&sh.s_empty[b], ph ^ 1u, abort_flag, 37)) { ok = false; return; }
                     tcgen05_fence_after();
-                    for (int kb = 0; kb < nkb; ++kb) {
-                        const unsigned long long adesc = smem_desc_sw128(smem_u32(qs + kb * KB_BYTES));
-                        const unsigned long long bdesc = smem_desc_sw128(smem_u32(ks + (b * 2 + kb) * KB_BYTES));
-                        const int steps = min(BK, d_h - kb * BK) / UMMA_K;
-                        for (int q = 0; q < steps; ++q)
-                            umma_bf16(tmem_base + b * AKV, adesc + 2 * q, bdesc + 2 * q, idesc1, (kb | q) != 0);
-                    }
+                    // (unrolled, here and below: r = 4096, 32 heads of 128: 421 -> 374 us, r = 1377: 87.2 -> 80.9)
+                    const unsigned long long adesc = smem_desc_sw128(smem_u32(qs));
+                    const unsigned long long bdesc = smem_desc_sw128(smem_u32(ks + b * 2 * KB_BYTES));
+                    if (nkb == 2) umma_blocks<2>(tmem_base + b * AKV, adesc, bdesc, KB_BYTES, KB_BYTES, idesc1);
+                    else umma_blocks<1>(tmem_base + b * AKV, adesc, bdesc, 0, 0, idesc1);
                     umma_commit(&sh.k_empty[b]);
                     umma_commit(&sh.s_full[b]);
                     if (j == nkv - 1) umma_commit(&sh.q_empty);          // Q may be replaced
@@ -324,9 +322,11 @@ k_attn_reps(const __grid_constant__ AttnMaps maps, int T, int d_h, int h,
                     // the accumulators are overwritten: the previous item's rows have been read out
                     if (j == 0 && k > 0 && !mbar_wait(&sh.o_empty, (unsigned)(k - 1) & 1u, abort_flag, 47)) { ok = false; break; }
                     tcgen05_fence_after();
+#pragma unroll
                     for (int u = 0; u < 2; ++u) {                        // O[j & 1] += P_j V_j
                         const unsigned long long adesc = smem_desc_sw128(smem_u32(ps + (b * 2 + u) * KB_BYTES));
                         const unsigned long long bdesc = smem_desc_sw128(smem_u32(vs + b * 2 * KB_BYTES + u * v_kb_bytes));
+#pragma unroll
                         for (int q = 0; q < BK / UMMA_K; ++q)
                             umma_bf16(tmem_base + (2 + b) * AKV, adesc + 2 * q, bdesc + 2 * q, idesc2,
                                       ((j >> 1) | u | q) != 0);

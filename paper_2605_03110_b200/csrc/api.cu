@@ -228,8 +228,8 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
     const size_t n_tok = (size_t)maxB * (size_t)maxT;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
-    // role, g_tok, g_rep are contiguous so that one memset clears them
-    const size_t o_role = take(n_tok * 4), o_gtok = take(n_tok * 4), o_grep = take(n_tok * 4);
+    // role, g_tok, g_rep, g_rep_tok are contiguous so that one memset clears them
+    const size_t o_role = take(n_tok * 4), o_gtok = take(n_tok * 4), o_grep = take(n_tok * 4), o_grept = take(n_tok * 4);
     const size_t o_ctr = take(32);
     const size_t o_near = take(n_tok * 8);
     const size_t o_inv = take(n_tok * 4), o_invr = take(n_tok * 4);
@@ -251,6 +251,7 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
     ctx->role = reinterpret_cast<int32_t*>(ctx->ws + o_role);
     ctx->g_tok = reinterpret_cast<unsigned*>(ctx->ws + o_gtok);
     ctx->g_rep = reinterpret_cast<unsigned*>(ctx->ws + o_grep);
+    ctx->g_rep_tok = reinterpret_cast<unsigned*>(ctx->ws + o_grept);
     ctx->inv_norm = reinterpret_cast<float*>(ctx->ws + o_inv);
     ctx->inv_rep = reinterpret_cast<float*>(ctx->ws + o_invr);
     ctx->r_eff = reinterpret_cast<int32_t*>(ctx->ws + o_reff);
@@ -520,6 +521,9 @@ static ada_status cascade_impl(ada_ctx* ctx, const void* X, int64_t B, int64_t T
     p.a_batch = T * d; p.b_batch = T * d;
     p.inv_a = ctx->inv_rep; p.inv_b = ctx->inv_rep;
     p.out = ctx->g_rep;
+    // (by token too: the compaction then reads everything of a token at once instead of by its position)
+    p.out_tok = inl ? ctx->g_rep_tok : nullptr;
+    p.col_token = rep_in;
     p.n_dev = inl ? rep_in_cnt : ctx->r_eff; p.n_host = 0;
     p.n_clamp = inl ? 1 : 0;
     p.rows = (int)T; p.cap = (int)T; p.d = (int)d; p.B = (int)B;
@@ -560,7 +564,7 @@ static ada_status cascade_impl(ada_ctx* ctx, const void* X, int64_t B, int64_t T
     else CU(launch_gram_ffma(ctx, q, dt, s));
     // lines 5, 9, 10-11
     CU(launch_compact_cascade(ctx, (int)B, (int)T, thr, rep_out, rep_out_cnt, add_idx, add_cnt,
-                              rem_idx, rem_cnt, gamma_rep, gamma_cross, tau_upd, q.defer_row != 0, s));
+                              rem_idx, rem_cnt, gamma_rep, gamma_cross, tau_upd, q.defer_row != 0, inl, s));
     return ADA_OK;
 }
 

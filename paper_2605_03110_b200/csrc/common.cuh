@@ -54,6 +54,7 @@ struct GramProblem {
     const float* inv_a;       // [B*cap]
     const float* inv_b;       // [B*cap]
     unsigned* out;            // [B*cap] gamma bit patterns (zero-initialised)
+    unsigned* out_tok;        // pair kernel, tri over a list: the same by token (col_token), or NULL
     const int32_t* n_dev;     // [B] device-resident column/row count, or NULL
     int n_host;               // used when n_dev == NULL
     int rows;                 // number of A rows (cross); ignored for tri
@@ -184,6 +185,7 @@ struct ada_ctx {
     float* inv_rep;      // [maxB*maxT] 1/||x|| of gathered rows, by position
     unsigned* g_tok;     // [maxB*maxT] gamma (full) or gamma_cross, by token, bit patterns
     unsigned* g_rep;     // [maxB*maxT] gamma_rep by position, bit patterns
+    unsigned* g_rep_tok; // [maxB*maxT] the same by token (pair kernel)
     int32_t* role;       // [maxB*maxT] 0 = not inherited, p+1 = position p in the inherited list
     int32_t* r_eff;      // [maxB] sanitised inherited counts
     unsigned* status;    // [8]
@@ -288,11 +290,12 @@ struct TauUpdate {
     int update;            // 0: leave tau_state as it is
     double target, gain, tau_min, tau_max;
 };
-// row_scale: the cross maxima in the scratch still lack the factor 1/||x_t|| (GramProblem::defer_row)
+// row_scale: the cross maxima in the scratch still lack the factor 1/||x_t|| (GramProblem::defer_row); by_tok: the
+// inherited ones' are there by token as well (GramProblem::out_tok)
 cudaError_t launch_compact_cascade(ada_ctx* ctx, int B, int T, float thr, int32_t* rep_out,
                                    int32_t* rep_out_cnt, int32_t* add_idx, int32_t* add_cnt,
                                    int32_t* rem_idx, int32_t* rem_cnt, float* gamma_rep,
-                                   float* gamma_cross, const TauUpdate& tu, bool row_scale,
+                                   float* gamma_cross, const TauUpdate& tu, bool row_scale, bool by_tok,
                                    cudaStream_t s);
 
 // gram_ffma.cu

@@ -370,6 +370,7 @@ constexpr unsigned long long COUNT_MASK = (1ull << COUNT_BITS) - 1;
 struct CompactArgs {
     unsigned* g_tok;             // gamma (full) / gamma_cross by token, bit patterns
     unsigned* g_rep;             // gamma_rep by position (cascade) or NULL
+    unsigned* g_rep_tok;         // the same by token, or NULL: read by position, behind the role map
     int32_t* role;               // 0 / position+1 (cascade) or NULL
     unsigned* dep_ctr;           // dependency counters of the Gram launch (cleared here)
     unsigned* status;
@@ -436,9 +437,12 @@ __global__ void __launch_bounds__(1024) k_compact(const CompactArgs a) {
             pos[v] = (cascade && in) ? a.role[o + t] : 0;
             gt[v] = in ? a.g_tok[o + t] : 0u;
             rs[v] = (in && a.row_scale != nullptr) ? a.row_scale[o + t] : 1.0f;
+            gp[v] = (in && a.g_rep_tok != nullptr) ? a.g_rep_tok[o + t] : 0u;
         }
+        if (a.g_rep_tok == nullptr) {
 #pragma unroll
-        for (int v = 0; v < V; ++v) gp[v] = pos[v] > 0 ? a.g_rep[o + pos[v] - 1] : 0u;
+            for (int v = 0; v < V; ++v) gp[v] = pos[v] > 0 ? a.g_rep[o + pos[v] - 1] : 0u;
+        }
         unsigned bk[V], ba[V], br[V];                          // ballots: kept, added, removed
 #pragma unroll
         for (int v = 0; v < V; ++v) {
@@ -451,6 +455,7 @@ __global__ void __launch_bounds__(1024) k_compact(const CompactArgs a) {
                     keep = ga < thr;
                     rem = !keep;
                     a.g_rep[o + pos[v] - 1] = 0u;
+                    if (a.g_rep_tok != nullptr) a.g_rep_tok[o + t] = 0u;
                     a.role[o + t] = 0;
                 } else {                          // Definition 1 / line 9
                     // (an untouched entry is a maximum over nothing: 0 whatever the row's norm)
@@ -462,7 +467,10 @@ __global__ void __launch_bounds__(1024) k_compact(const CompactArgs a) {
                 if (cascade) {
                     if (a.gamma_a != nullptr) a.gamma_a[o + t] = ga;
                     if (a.gamma_b != nullptr) a.gamma_b[o + t] = gb;
-                    if (faulted != 0u) a.g_rep[o + t] = 0u;   // a rejected list leaves positions without a token
+                    if (faulted != 0u) {              // a rejected list leaves positions without a token
+                        a.g_rep[o + t] = 0u;
+                        if (a.g_rep_tok != nullptr) a.g_rep_tok[o + t] = 0u;
+                    }
                 } else if (a.gamma_a != nullptr) {
                     a.gamma_a[o + t] = gb;
                 }
@@ -627,7 +635,7 @@ static cudaError_t launch_compact(ada_ctx* ctx, int kid, const CompactArgs& a, i
 cudaError_t launch_compact_full(ada_ctx* ctx, int B, int T, float thr, int32_t* rep_idx,
                                 int32_t* rep_cnt, float* gamma, cudaStream_t s) {
     CompactArgs a;
-    a.g_tok = ctx->g_tok; a.g_rep = nullptr; a.role = nullptr;
+    a.g_tok = ctx->g_tok; a.g_rep = nullptr; a.g_rep_tok = nullptr; a.role = nullptr;
     a.dep_ctr = ctx->tile_ctr; a.status = ctx->status;
     a.T = T; a.thr = thr; a.prefetch = ctx->host_out ? 0 : 1;
     a.keep_idx = rep_idx; a.keep_cnt = rep_cnt;
@@ -641,10 +649,10 @@ cudaError_t launch_compact_full(ada_ctx* ctx, int B, int T, float thr, int32_t* 
 cudaError_t launch_compact_cascade(ada_ctx* ctx, int B, int T, float thr, int32_t* rep_out,
                                    int32_t* rep_out_cnt, int32_t* add_idx, int32_t* add_cnt,
                                    int32_t* rem_idx, int32_t* rem_cnt, float* gamma_rep,
-                                   float* gamma_cross, const TauUpdate& tu, bool row_scale,
+                                   float* gamma_cross, const TauUpdate& tu, bool row_scale, bool by_tok,
                                    cudaStream_t s) {
     CompactArgs a;
-    a.g_tok = ctx->g_tok; a.g_rep = ctx->g_rep; a.role = ctx->role;
+    a.g_tok = ctx->g_tok; a.g_rep = ctx->g_rep; a.g_rep_tok = by_tok ? ctx->g_rep_tok : nullptr; a.role = ctx->role;
     a.dep_ctr = ctx->tile_ctr; a.status = ctx->status;
     a.T = T; a.thr = thr; a.prefetch = ctx->host_out ? 0 : 1;
     a.keep_idx = rep_out; a.keep_cnt = rep_out_cnt;

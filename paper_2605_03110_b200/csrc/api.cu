@@ -228,8 +228,8 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
     const size_t n_tok = (size_t)maxB * (size_t)maxT;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
-    // role, g_tok, g_rep, g_rep_tok are contiguous so that one memset clears them
-    const size_t o_role = take(n_tok * 4), o_gtok = take(n_tok * 4), o_grep = take(n_tok * 4), o_grept = take(n_tok * 4);
+    // role, g_tok, g_rep are contiguous so that one memset clears them
+    const size_t o_role = take(n_tok * 4), o_gtok = take(n_tok * 4), o_grep = take(n_tok * 4);
     const size_t o_ctr = take(32);
     const size_t o_near = take(n_tok * 8);
     const size_t o_inv = take(n_tok * 4), o_invr = take(n_tok * 4);
@@ -243,6 +243,7 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
     // one 256-column fp32 accumulator per SM
     ctx->part_bytes = (size_t)ctx->sm_count * 128 * 256 * 4;
     const size_t o_part = take(ctx->part_bytes);
+    const size_t o_grept = take(n_tok * 4);
     if (cudaMalloc(&ctx->ws, off) != cudaSuccess) {
         cudaGetLastError();
         delete ctx;
@@ -272,6 +273,7 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
         cudaEventCreateWithFlags(&ctx->host_ready, cudaEventDisableTiming) != cudaSuccess ||
         cudaMemsetAsync(ctx->ws, 0, o_xrep, ctx->host_stream) != cudaSuccess ||
         cudaMemsetAsync(ctx->part_buf, 0xFF, ctx->part_bytes, ctx->host_stream) != cudaSuccess ||
+        cudaMemsetAsync(ctx->g_rep_tok, 0, n_tok * 4, ctx->host_stream) != cudaSuccess ||
         (dt == ADA_BF16 && cudaMemsetAsync(ctx->ws + o_ntok, 0, n_tok * 4, ctx->host_stream) != cudaSuccess) ||
         cudaStreamSynchronize(ctx->host_stream) != cudaSuccess) {
         cudaGetLastError();
@@ -522,7 +524,8 @@ static ada_status cascade_impl(ada_ctx* ctx, const void* X, int64_t B, int64_t T
     p.inv_a = ctx->inv_rep; p.inv_b = ctx->inv_rep;
     p.out = ctx->g_rep;
     // (by token too: the compaction then reads everything of a token at once instead of by its position)
-    p.out_tok = inl ? ctx->g_rep_tok : nullptr;
+    const bool by_tok = inl && !split;
+    p.out_tok = by_tok ? ctx->g_rep_tok : nullptr;
     p.col_token = rep_in;
     p.n_dev = inl ? rep_in_cnt : ctx->r_eff; p.n_host = 0;
     p.n_clamp = inl ? 1 : 0;
@@ -564,7 +567,7 @@ static ada_status cascade_impl(ada_ctx* ctx, const void* X, int64_t B, int64_t T
     else CU(launch_gram_ffma(ctx, q, dt, s));
     // lines 5, 9, 10-11
     CU(launch_compact_cascade(ctx, (int)B, (int)T, thr, rep_out, rep_out_cnt, add_idx, add_cnt,
-                              rem_idx, rem_cnt, gamma_rep, gamma_cross, tau_upd, q.defer_row != 0, inl, s));
+                              rem_idx, rem_cnt, gamma_rep, gamma_cross, tau_upd, q.defer_row != 0, by_tok, s));
     return ADA_OK;
 }
 
@@ -715,6 +718,7 @@ ada_status ada_device_status(ada_ctx* ctx, void* stream, int64_t* n_zero_norm_ro
         // a faulted call may have left scratch behind: restore the workspace invariants
         CU(cudaMemsetAsync(ctx->role, 0, (size_t)((char*)ctx->inv_norm - (char*)ctx->role), s));
         CU(cudaMemsetAsync(ctx->part_buf, 0xFF, ctx->part_bytes, s));
+        CU(cudaMemsetAsync(ctx->g_rep_tok, 0, (size_t)ctx->maxB * ctx->maxT * 4, s));
         CU(cudaStreamSynchronize(s));
     }
     if (h[0] & ST_TIMEOUT) return ADA_ERR_TIMEOUT;

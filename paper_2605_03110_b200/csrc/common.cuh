@@ -54,7 +54,6 @@ struct GramProblem {
     const float* inv_a;       // [B*cap]
     const float* inv_b;       // [B*cap]
     unsigned* out;            // [B*cap] gamma bit patterns (zero-initialised)
-    unsigned* out_tok;        // pair kernel, tri over a list: the same by token (col_token), or NULL
     const int32_t* n_dev;     // [B] device-resident column/row count, or NULL
     int n_host;               // used when n_dev == NULL
     int rows;                 // number of A rows (cross); ignored for tri
@@ -72,9 +71,13 @@ struct GramProblem {
     // set when inv_a / inv_b are produced inside the same launch (NormJob): the epilogue
     // waits for the norm warps before it reads them
     int wait_norm_a, wait_norm_b;
-    // nearest-representative mode (cross only): instead of `out`, combine per row the packed
-    // key (value bits << 32 | ~column) with a 64-bit atomicMax: largest value, lowest column
-    unsigned long long* out_arg;
+    union {
+        // nearest-representative mode (cross only): instead of `out`, combine per row the packed
+        // key (value bits << 32 | ~column) with a 64-bit atomicMax: largest value, lowest column
+        unsigned long long* out_arg;
+        // pair kernel, bf16, tri over a list: `out` once more, by token (col_token), or NULL
+        unsigned* out_tok;
+    };
     // n_dev holds the caller's raw counts: clamp them to [0, cap] (nobody has sanitised them yet)
     int n_clamp;
     // cross only --------------------------------------------------------------------------------

@@ -937,7 +937,7 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
             const bool skip = row_live && !p.tri && !defer && p.row_role[o + row] != 0;
             const bool inv_early = defer || !(p.wait_norm_a && !norm_ok);
             float inv_row = defer ? 1.0f : ((row_live && inv_early) ? __ldcg(p.inv_a + o + row) : 0.f);
-            const int rep_tok = p.out_tok != nullptr && row_live ? __ldg(p.col_token + o + row) : -1;
+            const int rep_tok = !SPLIT && p.tri && p.out_tok != nullptr && row_live ? __ldg(p.col_token + o + row) : -1;
             const unsigned tbase = tmem_base + ((unsigned)(quad * 32) << 16) + acc * BN;
             int own0 = 0, own1 = nch;                    // chunks that this share of the tile answers for
             // Two steps: the column factors (for a cross tile they wait for the triangle's verdict), and for a
@@ -1033,7 +1033,7 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                 tcgen05_fence_after();
             }
             const bool need_cmp = p.tri ? (col0 + ncols > row_base) : (p.causal != 0);
-            const bool want_arg = p.out_arg != nullptr;
+            const bool want_arg = (SPLIT || !p.tri) && p.out_arg != nullptr;
             float mx0 = 0.f, mx1 = 0.f;
             int arg = 0;                                     // nearest-representative mode: column of the maximum
             // 32 columns (chunk c) of this thread's row
@@ -1103,8 +1103,8 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                 }
                 // By token too, behind the arrival, since nobody in this launch waits for it: the compaction then reads all
                 // that it needs of a token at once (8 x 2048 x 768 chain of twelve 314 -> 309 us, 2005 x 4096 of 28
-                // 796 -> 786).  (An entry of a rejected list may be anything.)
-                if (mx > 0.f && (unsigned)rep_tok < (unsigned)p.cap) atomicMax(p.out_tok + o + rep_tok, __float_as_uint(mx));
+                // 796 -> 786; nothing for fp32, whose steps do without).  (An entry of a rejected list may be anything.)
+                if (!SPLIT && mx > 0.f && (unsigned)rep_tok < (unsigned)p.cap) atomicMax(p.out_tok + o + rep_tok, __float_as_uint(mx));
             }
         }
     }

@@ -45,7 +45,7 @@
  *     out too small, by up to 4e-9 d + 2e-6 of itself for ADA_BF16 and 8e-9 d + 2e-6 for ADA_F32
  *     (measured against 64 bits: 1.4e-5 and 2.4e-5 at d = 4096; ADA_ENGINE_FFMA 4e-6).  Tiles that
  *     several SM pairs share along d (small problems, d <= 4600, fp32 <= 2140) keep a half to a quarter of
- *     that error, so the same row's gamma may differ by up to 1e-5 with the number of rows around it.
+ *     that error, so the same row's gamma may differ by up to 1.2e-5 with the number of rows around it.
  */
 #ifndef ADA_H_
 #define ADA_H_

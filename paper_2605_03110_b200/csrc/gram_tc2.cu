@@ -272,11 +272,15 @@ struct GramMaps {
 // How many shares a tile may have.  The tensor core's accumulator truncates, so a sum over K comes out
 // too small, by about 3.6e-9 d of itself for bf16 storage (measured at d = 2600 and 4096; more past 4096,
 // where the sums of unit-variance rows enter the next binade) and by up to 8e-9 d for the six
-// terms of fp32 storage; cutting it in p shares takes 1 - 1/p of that away.  The same row must
-// not move by more than 1e-5 when the number of tiles around it changes, hence the limits:
-// measured shifts at them are 7.9e-6 (bf16, d = 3450, p = 3) and 8.6e-6 (fp32, d = 1600, p = 3).
+// terms of fp32 storage; cutting it in p shares takes 1 - 1/p of that away.  The same row moves by that much
+// when the number of tiles around it changes, which is to stay near 1e-5, hence the limits: largest shifts at
+// them 1.08e-5 (bf16, d = 4096, p = 3), 1.15e-5 (bf16, d = 4600, p = 2) and 8.6e-6 (fp32, d = 1600, p = 3), the
+// split sum being the better one (error against 64 bits at d = 4096: 4.1e-6 in three shares, 1.4e-5 whole).
+// Three instead of two at d = 4096: chain over 2005 tokens 795 -> 776 us, full selection at T = 8192 215.8 -> 214.6.
 template <bool SPLIT>
-__device__ __forceinline__ bool shares_ok(int p, int d) { return (p - 1) * d <= (SPLIT ? MAX_SPLIT_D_F32 : MAX_SPLIT_D) / 2 * p; }
+__device__ __forceinline__ bool shares_ok(int p, int d) {
+    return (p - 1) * d <= (SPLIT ? MAX_SPLIT_D_F32 / 2 : (d <= 4096 ? 2731 : MAX_SPLIT_D / 2)) * p;
+}
 // Limits of the plan's rules in stages of a bf16 tile: what a split has to save, the longest contraction whose
 // norms come out of the tiles in shared memory, the longest whose epilogue sets take alternate tiles.  The last
 // two count on whole tiles (ring_s below, the shares of pub_cnt): what they cover is never split.

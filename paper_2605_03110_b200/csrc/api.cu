@@ -237,13 +237,13 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
     const size_t o_xrep = take(n_tok * (size_t)maxd * ctx->es + 1024);
     // bf16: the rows outside a large inherited set, copied out for the cross step (Algorithm 1 line 6)
     const size_t o_ntok = take(dt == ADA_BF16 ? n_tok * 4 : 0);
+    const size_t o_grept = take(dt == ADA_BF16 ? n_tok * 4 : 0);      // (cleared together with the one before it)
     const size_t o_xnon = take(dt == ADA_BF16 ? n_tok * (size_t)maxd * 2 + 1024 : 0);
     const size_t split_bytes = dt == ADA_F32 ? n_tok * (size_t)plane_len(maxd) * 6 + 1024 : 0;
     const size_t o_sx = take(split_bytes), o_sr = take(split_bytes);
     // one 256-column fp32 accumulator per SM
     ctx->part_bytes = (size_t)ctx->sm_count * 128 * 256 * 4;
     const size_t o_part = take(ctx->part_bytes);
-    const size_t o_grept = take(n_tok * 4);
     if (cudaMalloc(&ctx->ws, off) != cudaSuccess) {
         cudaGetLastError();
         delete ctx;
@@ -252,7 +252,7 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
     ctx->role = reinterpret_cast<int32_t*>(ctx->ws + o_role);
     ctx->g_tok = reinterpret_cast<unsigned*>(ctx->ws + o_gtok);
     ctx->g_rep = reinterpret_cast<unsigned*>(ctx->ws + o_grep);
-    ctx->g_rep_tok = reinterpret_cast<unsigned*>(ctx->ws + o_grept);
+    ctx->g_rep_tok = dt == ADA_BF16 ? reinterpret_cast<unsigned*>(ctx->ws + o_grept) : nullptr;
     ctx->inv_norm = reinterpret_cast<float*>(ctx->ws + o_inv);
     ctx->inv_rep = reinterpret_cast<float*>(ctx->ws + o_invr);
     ctx->r_eff = reinterpret_cast<int32_t*>(ctx->ws + o_reff);
@@ -273,8 +273,7 @@ ada_status ada_create(ada_ctx** out, int device, int64_t maxB, int64_t maxT, int
         cudaEventCreateWithFlags(&ctx->host_ready, cudaEventDisableTiming) != cudaSuccess ||
         cudaMemsetAsync(ctx->ws, 0, o_xrep, ctx->host_stream) != cudaSuccess ||
         cudaMemsetAsync(ctx->part_buf, 0xFF, ctx->part_bytes, ctx->host_stream) != cudaSuccess ||
-        cudaMemsetAsync(ctx->g_rep_tok, 0, n_tok * 4, ctx->host_stream) != cudaSuccess ||
-        (dt == ADA_BF16 && cudaMemsetAsync(ctx->ws + o_ntok, 0, n_tok * 4, ctx->host_stream) != cudaSuccess) ||
+        (dt == ADA_BF16 && cudaMemsetAsync(ctx->ws + o_ntok, 0, o_xnon - o_ntok, ctx->host_stream) != cudaSuccess) ||
         cudaStreamSynchronize(ctx->host_stream) != cudaSuccess) {
         cudaGetLastError();
         ada_destroy(ctx);
@@ -718,7 +717,7 @@ ada_status ada_device_status(ada_ctx* ctx, void* stream, int64_t* n_zero_norm_ro
         // a faulted call may have left scratch behind: restore the workspace invariants
         CU(cudaMemsetAsync(ctx->role, 0, (size_t)((char*)ctx->inv_norm - (char*)ctx->role), s));
         CU(cudaMemsetAsync(ctx->part_buf, 0xFF, ctx->part_bytes, s));
-        CU(cudaMemsetAsync(ctx->g_rep_tok, 0, (size_t)ctx->maxB * ctx->maxT * 4, s));
+        if (ctx->g_rep_tok != nullptr) CU(cudaMemsetAsync(ctx->g_rep_tok, 0, (size_t)ctx->maxB * ctx->maxT * 4, s));
         CU(cudaStreamSynchronize(s));
     }
     if (h[0] & ST_TIMEOUT) return ADA_ERR_TIMEOUT;

@@ -140,6 +140,13 @@ struct Walk {
     __device__ __forceinline__ int width(int ph, int c, int x) const {
         return ph ? cols(c) : min(cols(c), (x + 1) * BM - c * SS_COLS);
     }
+    // Has a column to be compared with the row, or does the whole chunk lie before the tile?  (Causal: every
+    // token of a chunk is below the next one's first.  Compared everywhere, a tile of a causal step took 1.6 us
+    // instead of 1.25: 32 heads x 2048, r = 1024 58.0 -> 51.6, which three launches do in 69.)
+    __device__ __forceinline__ bool mixed(int ph, int c, int x) const {
+        if (!ph) return c * SS_COLS + width(0, c, x) > x * BM;
+        return causal && !(c + 1 < nch && tok0[c + 1] <= t0 + x * BM);
+    }
 };
 
 __global__ void __launch_bounds__(SS_THREADS, 1)
@@ -428,7 +435,7 @@ k_step_short(const __grid_constant__ StepMaps maps, const __grid_constant__ Step
                     if (!ok) break;
                     tcgen05_fence_after();
                     const int ncols = w.width(ph, c, x);
-                    const bool need_cmp = ph ? a.causal != 0 : c * SS_COLS + ncols > x * BM;
+                    const bool need_cmp = w.mixed(ph, c, x);
                     const unsigned tbase = tmem_base + ((unsigned)(quad * 32) << 16) + p * SS_COLS;
                     auto consume = [&](const unsigned (&r)[32], int c0) {
                         if (!need_cmp) {

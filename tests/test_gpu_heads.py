@@ -262,3 +262,50 @@ def test_heads_on_long_sequence_past_the_tile_table(ada):
         assert np.max(np.abs(gc[j] - ref.gamma_cross)) <= tol
         assert reps1[j].tolist() == ref.rep.tolist()
     ada.ada_destroy(ctx)
+
+
+def both_forms(ada, ctx, X, sets, flags):
+    """The step as the library chooses it, and by the one-CTA kernel's launches; which kernels the first one used."""
+    from parity import to_device
+    T, h = X.shape[0], X.shape[1]
+    ri = torch.zeros((h, T), dtype=torch.int32)
+    for j, r in enumerate(sets):
+        ri[j, :len(r)] = torch.tensor(r, dtype=torch.int32)
+    ri, rc = ri.cuda(), torch.tensor([len(r) for r in sets], dtype=torch.int32, device="cuda")
+    Xd, outs, kernels = to_device(X), [], []
+    for engine in (ada.ADA_ENGINE_AUTO, ada.ADA_ENGINE_TCGEN05):
+        ada.ada_set_engine(ctx, engine)
+        ada.ada_profile_enable(ctx, True)
+        outs.append(ada.ada_cascade_step_heads(ctx, Xd, TAU, ri, rc, flags=flags))
+        kernels.append({k for k, (n, _) in ada.ada_profile_read(ctx).items() if n > 0})
+        ada.ada_profile_enable(ctx, False)
+    ada.ada_set_engine(ctx, ada.ADA_ENGINE_AUTO)
+    assert ada.ada_device_status(ctx)[0] == 0
+    assert "step_short" not in kernels[1]
+    return outs[0], outs[1], kernels[0]
+
+
+def assert_same_step(one, several):
+    from parity import lists
+    for a, b in (("rep_out", "rep_out_cnt"), ("add_idx", "add_cnt"), ("rem_idx", "rem_cnt")):
+        for x, y in zip(lists(getattr(one, a), getattr(one, b)), lists(getattr(several, a), getattr(several, b))):
+            assert x.tolist() == y.tolist()
+    # the same products and sums; norms are summed in another order (16 fp32 terms a lane, then a tree)
+    assert torch.allclose(one.gamma_cross, several.gamma_cross, rtol=1e-6, atol=0)
+    assert torch.allclose(one.gamma_rep, several.gamma_rep, rtol=1e-6, atol=0)
+
+
+def test_heads_causal_step_where_chunks_and_tiles_meet(ada):
+    """Causal: a chunk of 256 representatives that ends before a tile's first row is not compared with the rows.
+    Runs of consecutive tokens put the next chunk's first one at a tile's first row, one before and one behind it."""
+    from parity import check_cascade
+    T, h, d_h = 1300, 16, 64
+    ctx = ada.ada_create(h, T, d_h, ada.ADA_BF16)
+    X = clustered_heads(T, h, d_h, 5, "bf16")
+    sets = [list(range(k, min(k + 700, T))) for k in (0, 1, 127, 128, 129, 255, 256, 257, 383, 384, 385, 640, 767, 768, 1043, 1044)]
+    one, several, kernels = both_forms(ada, ctx, X, sets, ada.ADA_CROSS_CAUSAL)
+    assert kernels == {"step_short"}
+    assert_same_step(one, several)
+    some = [0, 3, 4, 6, 11]
+    check_cascade(ctx, np.ascontiguousarray(X[:, some]), TAU, [sets[j] for j in some], causal=True, heads=True)
+    ada.ada_destroy(ctx)

@@ -115,8 +115,11 @@ __device__ __forceinline__ void ss_workers_sync() { asm volatile("bar.sync 1, %0
 // Within a group a chunk that has something for a row tile has something for all later ones.
 struct Walk {
     int n, nch, nrt, C, rank, tiles, t0, causal;
+    // columns and chunks of the cross tiles.  Where every token is inherited no maximum of theirs is read, and one narrow
+    // chunk is left, with which the row norms come (one such head beside 31 with 20 of 2048 tokens: 90 -> 57 us).
+    int nx, nchx;
     const int* tok0;
-    __device__ __forceinline__ int groups(int ph) const { return ph ? max((nch + 1) >> 1, 1) : (nch + 1) >> 1; }
+    __device__ __forceinline__ int groups(int ph) const { return ph ? max((nchx + 1) >> 1, 1) : (nch + 1) >> 1; }
     __device__ __forceinline__ int first(int ph, int g) const {
         if (ph) return 0;
         const int lo = 4 * g;                            // (nothing of chunk 2g left of row tile 4g)
@@ -133,12 +136,14 @@ struct Walk {
     __device__ __forceinline__ bool live(int ph, int c, int x) const {
         if (!ph) return c < nch && x >= 2 * c;
         const int lim = t0 + (x + 1) * BM;
-        return c == 0 || (c < nch && !(causal && (tok0[c] >= lim || (c > 1 && tok0[c & ~1] >= lim))));
+        return c == 0 || (c < nchx && !(causal && (tok0[c] >= lim || (c > 1 && tok0[c & ~1] >= lim))));
     }
-    __device__ __forceinline__ int cols(int c) const { return max(16, (min(n - c * SS_COLS, SS_COLS) + 15) & ~15); }
+    __device__ __forceinline__ int cols(int ph, int c) const {
+        return max(16, (min((ph ? nx : n) - c * SS_COLS, SS_COLS) + 15) & ~15);
+    }
     // (nothing right of a triangular tile's last row)
     __device__ __forceinline__ int width(int ph, int c, int x) const {
-        return ph ? cols(c) : min(cols(c), (x + 1) * BM - c * SS_COLS);
+        return ph ? cols(1, c) : min(cols(0, c), (x + 1) * BM - c * SS_COLS);
     }
     // Has a column to be compared with the row, or does the whole chunk lie before the tile?  (Causal: every
     // token of a chunk is below the next one's first.  Compared everywhere, a tile of a causal step took 1.6 us
@@ -220,6 +225,7 @@ k_step_short(const __grid_constant__ StepMaps maps, const __grid_constant__ Step
     const int nkb = (d + BK - 1) / BK;               // 64-element K blocks (one or two)
     Walk w;
     w.n = n; w.nch = (n + SS_COLS - 1) / SS_COLS; w.nrt = (n + BM - 1) / BM;
+    w.nx = n == T ? 1 : n; w.nchx = n == T ? 1 : w.nch;
     w.C = C; w.rank = rank; w.tiles = (own + BM - 1) / BM; w.t0 = t0; w.causal = a.causal;
     w.tok0 = sh.tok0;
 
@@ -295,7 +301,7 @@ k_step_short(const __grid_constant__ StepMaps maps, const __grid_constant__ Step
                         for (int e = 0; e < 2 && ok; ++e) {
                             const int c = 2 * g + e;
                             if (!w.live(ph, c, x1)) continue;
-                            const int nbox = (w.cols(c) + BOX_N - 1) / BOX_N;
+                            const int nbox = (w.cols(ph, c) + BOX_N - 1) / BOX_N;
                             ok = mbar_wait(&sh.b_empty[e], (nb[e] & 1u) ^ 1u, abort_flag, 51);
                             if (!ok) break;
                             ++nb[e];

@@ -309,3 +309,32 @@ def test_heads_causal_step_where_chunks_and_tiles_meet(ada):
     some = [0, 3, 4, 6, 11]
     check_cascade(ctx, np.ascontiguousarray(X[:, some]), TAU, [sets[j] for j in some], causal=True, heads=True)
     ada.ada_destroy(ctx)
+
+
+@pytest.mark.parametrize("T,h,d_h", [(1, 3, 8), (130, 4, 128), (1000, 23, 128), (2048, 30, 40)])
+def test_heads_step_with_heads_of_inherited_tokens_only(ada, T, h, d_h):
+    """A head all of whose tokens are inherited has no cross maxima, but its rows' norms are still looked at."""
+    from parity import check_cascade
+    ctx = ada.ada_create(h, T, d_h, ada.ADA_BF16)
+    X = clustered_heads(T, h, d_h, 23 + T, "bf16")
+    sets = [list(range(T)) if j % 3 == 0 else list(range(j % T, T, 5)) for j in range(h)]
+    for flags in (0, ada.ADA_CROSS_CAUSAL):
+        one, several, kernels = both_forms(ada, ctx, X, sets, flags)
+        assert kernels == {"step_short"}
+        assert_same_step(one, several)
+        assert not one.gamma_cross[::3].any()
+    check_cascade(ctx, np.ascontiguousarray(X[:, :4]), TAU, sets[:4], heads=True)
+    # one zero row in such a head, and then a NaN in one
+    from parity import to_device
+    Z = X.copy()
+    Z[T - 1, 3 * ((h - 1) // 3)] = 0
+    ri = torch.zeros((h, T), dtype=torch.int32)
+    for j, r in enumerate(sets):
+        ri[j, :len(r)] = torch.tensor(r, dtype=torch.int32)
+    ri, rc = ri.cuda(), torch.tensor([len(r) for r in sets], dtype=torch.int32, device="cuda")
+    ada.ada_cascade_step_heads(ctx, to_device(Z), TAU, ri, rc)
+    assert ada.ada_device_status(ctx) == (0, 1)
+    Z[T // 2, 0, d_h - 1] = 0x7FC0
+    ada.ada_cascade_step_heads(ctx, to_device(Z), TAU, ri, rc)
+    assert ada.status_string(ada.ada_device_status(ctx)[0]) == "ADA_ERR_NONFINITE"
+    ada.ada_destroy(ctx)

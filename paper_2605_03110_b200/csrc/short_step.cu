@@ -21,7 +21,7 @@
 // stamps): 5 us until the rows are gathered, 1.5 us to the first MMA, 5 us for the triangle and its verdict,
 // 10 us for eight cross tiles, 4 us for the lists, 1 us between launches.  A cross tile (128 x 256 x 128) takes
 // 1.25 us where its MMAs need 0.55: the epilogue reads an accumulator in 0.75 us, a quarter of it column factors
-// out of shared memory (without those reads 420 -> 342 us at T = 8192, r = 4096; without the epilogue 283).
+// out of shared memory.
 #include "gram_tc_dev.cuh"
 
 namespace ada {
@@ -36,10 +36,10 @@ constexpr int SS_COLS = 256;                         // representatives per chun
 constexpr int SS_B_SLOT = SS_COLS * 128 * 2;         // two 64-element K blocks of 256 rows
 constexpr int SS_A_SLOT = BM * 128 * 2;
 constexpr int SS_CLUSTER = 8;                        // largest portable cluster
-constexpr int SS_MAX_ROWS = 2048;                    // tokens per CTA
+constexpr int SS_MAX_T = 2048;                       // tokens of a sequence (see step_short_ctas), and of a CTA
 constexpr int SS_TAB = 1024;                         // representatives whose factors are passed through shared memory
-static_assert(SS_CLUSTER * SS_MAX_ROWS < 1 << 16, "positions fit role[]");
-constexpr int SS_CHUNKS = SS_CLUSTER * SS_MAX_ROWS / SS_COLS;
+static_assert(SS_MAX_T < 1 << 16, "positions fit role[]");
+constexpr int SS_CHUNKS = SS_MAX_T / SS_COLS;
 
 struct alignas(16) StepShared {
     unsigned long long a_full[2], a_empty[2], b_full[2], b_empty[2], t_full[2], t_empty[2], drain;
@@ -52,11 +52,11 @@ struct alignas(16) StepShared {
     alignas(16) float col_f[2][2 * SS_COLS];         // column factors (and tokens) of a group, in alternating buffers
     alignas(16) int col_t[2][2 * SS_COLS];
     float tab[SS_TAB];                               // cross factors of the first representatives, written by their owners
-    unsigned long long off[SS_MAX_ROWS / 32];        // counts, then exclusive offsets, by 32 tokens
+    unsigned long long off[SS_MAX_T / 32];           // counts, then exclusive offsets, by 32 tokens
     unsigned long long total[SS_CLUSTER];            // of every CTA of the cluster
-    unsigned short role[SS_MAX_ROWS];                // this CTA's tokens: 0, or position + 1 in the inherited list
-    unsigned mx[SS_MAX_ROWS];                        // maxima (bit patterns): of its representatives, then of its tokens
-    float inv[SS_MAX_ROWS];                          // 1/||x_t||
+    unsigned short role[SS_MAX_T];                   // this CTA's tokens: 0, or position + 1 in the inherited list
+    unsigned mx[SS_MAX_T];                           // maxima (bit patterns): of its representatives, then of its tokens
+    float inv[SS_MAX_T];                             // 1/||x_t||
 };
 constexpr int SS_SMEM = 2 * SS_B_SLOT + 2 * SS_A_SLOT + (int)sizeof(StepShared) + 1024;
 static_assert(SS_SMEM <= 227 * 1024, "shared memory budget");
@@ -148,8 +148,8 @@ struct Walk {
     // Has a column to be compared with the row, or does the whole chunk lie before the tile?  (Causal: every
     // token of a chunk is below the next one's first.  Compared everywhere, a tile of a causal step took 1.6 us
     // instead of 1.25: 32 heads x 2048, r = 1024 58.0 -> 51.6, which three launches do in 69.)
-    __device__ __forceinline__ bool mixed(int ph, int c, int x) const {
-        if (!ph) return c * SS_COLS + width(0, c, x) > x * BM;
+    __device__ __forceinline__ bool mixed(int ph, int c, int x, int ncols) const {
+        if (!ph) return c * SS_COLS + ncols > x * BM;
         return causal && !(c + 1 < nch && tok0[c + 1] <= t0 + x * BM);
     }
 };
@@ -366,7 +366,7 @@ k_step_short(const __grid_constant__ StepMaps maps, const __grid_constant__ Step
         const int wk = (int)threadIdx.x - 64, wl = warp - 2;
         const int quad = warp & 3, set = wl >> 2;
         const int lrow = quad * 32 + lane;               // this thread's row of a tile
-        constexpr int V = SS_MAX_ROWS / SS_WORKERS;
+        constexpr int V = SS_MAX_T / SS_WORKERS;
         const int slices = (own + SS_WORKERS - 1) / SS_WORKERS;
         unsigned k = 0, ka = 0, staged = 0;              // tiles, left operands, groups so far
         float gp[V];                                     // gamma_rep of this thread's tokens, where they are inherited
@@ -441,7 +441,7 @@ k_step_short(const __grid_constant__ StepMaps maps, const __grid_constant__ Step
                     if (!ok) break;
                     tcgen05_fence_after();
                     const int ncols = w.width(ph, c, x);
-                    const bool need_cmp = w.mixed(ph, c, x);
+                    const bool need_cmp = w.mixed(ph, c, x, ncols);
                     const unsigned tbase = tmem_base + ((unsigned)(quad * 32) << 16) + p * SS_COLS;
                     auto consume = [&](const unsigned (&r)[32], int c0) {
                         if (!need_cmp) {
@@ -511,7 +511,7 @@ k_step_short(const __grid_constant__ StepMaps maps, const __grid_constant__ Step
         }
         ss_workers_sync();
         // ------------------------------------------------ lists (lines 5, 9-11 and Eq. 6); the three counts of a
-        // sequence share a word (20 bits each: T is at most 16384 here)
+        // sequence share a word (20 bits each)
         constexpr unsigned BITS = 20;
         constexpr unsigned MASK = (1u << BITS) - 1u;
         {
@@ -545,7 +545,7 @@ k_step_short(const __grid_constant__ StepMaps maps, const __grid_constant__ Step
             }
             ss_workers_sync();
             if (warp == 2) {                             // lane l scans entries 2l and 2l + 1 (token order)
-                static_assert(SS_MAX_ROWS / 32 == 64, "two entries per lane");
+                static_assert(SS_MAX_T / 32 == 64, "two entries per lane");
                 const int ne = slices * (SS_WORKERS / 32);
                 const unsigned long long c0 = 2 * lane < ne ? sh.off[2 * lane] : 0ull, c1 = 2 * lane + 1 < ne ? sh.off[2 * lane + 1] : 0ull;
                 unsigned long long incl = c0 + c1;
@@ -632,23 +632,37 @@ static cudaError_t ensure_short(ada_ctx* ctx) {
 }
 
 // CTAs per sequence of the one-launch step, or 0: not this step.  As many as let all clusters run at once, at most
-// eight (with one more round of clusters 16 heads x 2048 took 27.6 us instead of 17.0).  Against the three
-// launches, whose tiles go to all SMs whatever the number of sequences (d = 128; us, three launches ->
-// one; r = T/100, T/10, T/2):
-//     8 heads x 1000    17.9 -> 13.7   19.4 -> 14.9   21.2 -> 18.6      32 x 1000   22.4 -> 15.7   24.1 -> 16.8   32.3 -> 22.8
-//     8 x 2048          19.2 -> 14.9   21.5 -> 17.6   29.1 -> 30.7      32 x 2048   28.3 -> 18.3   33.1 -> 21.8   61.7 -> 47.9
-//     8 x 8192          29.8 -> 23.5   50.4 -> 54.7    148 -> 230       32 x 8192   67.7 -> 34.9    149 -> 95      629 -> 423
-//     12 x 8192         35.9 -> 23.8   67.5 -> 54.8    225 -> 227      148 x 2048    105 -> 32.7    121 -> 47.4    278 -> 149
-// It is the faster one, whatever the sets, where its CTAs cover three fifths of the SMs, and with one row tile per
-// CTA (2 heads x 1000, r = T/2: 18.6 -> 18.2).
+// eight (with one more round of clusters 16 heads x 2048 took 27.6 us instead of 17.0).
+//
+// A sequence has its cluster and no other CTA, while the tiles of the three launches go to all SMs: the one launch lasts as
+// long as its largest set, the others as long as the average.  Both forms (d = 128; us, one launch / three) where all sets
+// hold T/100, T/10, T/5, T/2 of the tokens, where one holds T/5, T/2, or all, the others T/100, and where they are
+// spread evenly in the logarithm over T/100..T/5 and T/100..0.6 T:
+//                  T/100       T/10        T/5         T/2       one T/5     one T/2      one T       ..T/5     ..0.6 T
+//    8 x 1000   14.1/18.5   15.1/19.7   16.1/20.1   18.7/21.2   15.7/19.1   18.1/20.0   20.7/20.4   15.4/19.9   18.0/20.4
+//   32 x 1000   15.9/22.9   17.1/24.7   18.6/26.1   22.9/32.5   17.2/23.5   21.0/23.9   27.8/24.0   17.2/24.8   27.8/29.2
+//  100 x 1000   22.5/57.5   25.6/62.2   33.5/66.5   55.0/86.0   32.5/57.2   53.7/57.1   74.4/57.7   32.2/62.2   67.8/68.0
+//   12 x 2048   15.4/21.7   17.9/24.0   20.8/27.2   30.9/34.5   19.9/22.6   29.6/23.1   36.9/25.6   19.5/24.3   29.7/29.0
+//   16 x 2048   17.1/23.4   20.0/25.5   23.7/30.3   40.3/41.4   22.8/24.5   39.0/25.3   46.1/27.2   22.2/27.1   38.7/30.7
+//   32 x 2048   18.4/29.4   22.0/34.2   26.9/42.1   47.1/61.8   25.1/30.0   45.1/30.7   56.6/33.4   25.4/34.8   58.2/42.3
+//  148 x 2048   32.7/107    47.7/123    72.8/157    149/278     70.3/109    143/109     179/109     71.1/123    185/156
+//   32 x 3000   20.8/35.4   29.5/49.2   44.0/59.4   82.8/103    41.8/36.4   80.3/37.7   92.8/40.7   41.4/45.1   96.6/61.7
+// (ADA_CROSS_CAUSAL changes both by up to a sixth, and no comparison up to T/5.)  The set sizes live on the device, so the
+// line is drawn where no set of up to a fifth of its sequence, whatever the others hold, makes the step slower: at 2048
+// tokens.  Where one set is larger than that and the others are not, the three launches would be faster, by up to 1.5
+// times at T/2.  (At 8192 tokens a single set of T/2 beside 31 small ones took 411 us instead of 87.)  Sharing such a head's tiles among all CTAs, counted out through global memory, was tried: 8192 tokens 411 -> 93,
+// but 2048 tokens 45 -> 43, and its code costs every other step 0.5 to 5 %.
+//
+// Within that, used where its CTAs cover three fifths of the SMs, or have one row tile each (8 x 2048, r = T/2: 30.7 / 29.1;
+// 2 x 1000, r = T/2: 18.2 / 18.6), and up to as many sequences as there are SMs (more rounds of clusters: not measured).
 int step_short_ctas(ada_ctx* ctx, int64_t B, int64_t T, int64_t d) {
-    if (d > 128 || ensure_short(ctx) != cudaSuccess) return 0;
+    if (d > 128 || T > SS_MAX_T || ensure_short(ctx) != cudaSuccess) return 0;
     const int64_t tiles = (T + BM - 1) / BM;
     for (int64_t C = SS_CLUSTER; C >= 1; --C) {
         if (C > tiles || ctx->short_clusters[C] < B) continue;
         const int64_t per = (tiles + C - 1) / C;                       // row tiles per CTA
         C = (tiles + per - 1) / per;                                   // (no CTA without rows)
-        if (per * BM > SS_MAX_ROWS || (per > 1 && 5 * B * C < 3 * ctx->sm_count)) return 0;
+        if (per > 1 && 5 * B * C < 3 * ctx->sm_count) return 0;
         return (int)C;
     }
     return 0;

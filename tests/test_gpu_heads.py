@@ -338,3 +338,18 @@ def test_heads_step_with_heads_of_inherited_tokens_only(ada, T, h, d_h):
     ada.ada_cascade_step_heads(ctx, to_device(Z), TAU, ri, rc)
     assert ada.status_string(ada.ada_device_status(ctx)[0]) == "ADA_ERR_NONFINITE"
     ada.ada_destroy(ctx)
+
+
+@pytest.mark.parametrize("T,one", [(2048, True), (2049, False), (4096, False)])
+def test_heads_step_takes_one_launch_up_to_2048_tokens(ada, T, one):
+    """Longer sequences go to the launches whose tiles all SMs share: a head's cluster has nobody to help it with
+    a set that is larger than the others'."""
+    h, d_h = 32, 32
+    ctx = ada.ada_create(h, T, d_h, ada.ADA_BF16)
+    X = clustered_heads(T, h, d_h, 9, "bf16")
+    sets = [list(range(0, T, 2)) if j == 11 else list(range(j, T, 100)) for j in range(h)]
+    for flags in (0, ada.ADA_CROSS_CAUSAL):
+        a, b, kernels = both_forms(ada, ctx, X, sets, flags)
+        assert ("step_short" in kernels) == one
+        assert_same_step(a, b)
+    ada.ada_destroy(ctx)

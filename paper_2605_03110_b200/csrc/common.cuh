@@ -154,7 +154,7 @@ struct NormJob {
 };
 
 // contraction lengths up to which a tile may be split in two (pair kernel, shares_ok)
-constexpr int MAX_SPLIT_D = 4600, MAX_SPLIT_D_F32 = 2140;
+constexpr int MAX_SPLIT_D = 5500, MAX_SPLIT_D_F32 = 2140;
 constexpr int MAX_PARTS = 4;      // most shares of one tile
 
 struct Profiler {

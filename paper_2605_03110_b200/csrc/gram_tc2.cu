@@ -269,17 +269,20 @@ struct GramMaps {
 // chain to a part of it, and a wide tile split over K draws fewer bytes per SM than narrow tiles
 // would.  Measured: full selection at T = 2048, d = 4096 31.0 -> 26.1 us, at T = 512, d = 768 fp32 30.2 ->
 // 17.7 us, cascade steps at T = 2005, d = 4096 43 -> 31 us.
-// How many shares a tile may have.  The tensor core's accumulator truncates, so a sum over K comes out
-// too small, by about 3.6e-9 d of itself for bf16 storage (measured at d = 2600 and 4096; more past 4096,
-// where the sums of unit-variance rows enter the next binade) and by up to 8e-9 d for the six
-// terms of fp32 storage; cutting it in p shares takes 1 - 1/p of that away.  The same row moves by that much
-// when the number of tiles around it changes, which is to stay near 1e-5, hence the limits: largest shifts at
-// them 1.08e-5 (bf16, d = 4096, p = 3), 1.15e-5 (bf16, d = 4600, p = 2) and 8.6e-6 (fp32, d = 1600, p = 3), the
-// split sum being the better one (error against 64 bits at d = 4096: 4.1e-6 in three shares, 1.4e-5 whole).
-// Three instead of two at d = 4096: chain over 2005 tokens 795 -> 776 us, full selection at T = 8192 215.8 -> 214.6.
+// How many shares a tile may have.  The tensor core's accumulator truncates, so a sum over d elements comes out too small,
+// and cutting it in p shares takes part of that away: the same row moves by as much when the number of tiles around it
+// changes, the split sum being the better one.  That is to stay below 1.5e-5 for bf16 (1e-5 for the six terms of fp32
+// storage, whose contraction is cut earlier) whatever the scale of the rows.
+// An accumulation loses in proportion to the unit in the last place of the running sum, so with elements of one scale a
+// whole sum loses e d f of itself, f = 1/s - 2/(3 s^2) for a sum that ends at s (1 <= s < 2) in its binade: 1/3 at
+// its ends, 3/8 at s = 4/3.  A share ends p times lower, at f': the row moves by e d (f - f'/p), at worst
+// 0.19, 0.26, 0.28 e d for p = 2, 3, 4, which is 3/8 e d (1 - 1/p) within a few per cent, hence one limit on d (1 - 1/p).
+// Measured e = 1.2e-8 .. 1.38e-8; largest shifts over rows of scale 0.7 .. 1.3: 1.32e-5 (d = 5120, p = 2), 1.34e-5 (4096, 3),
+// 1.23e-5 (3640, 4); fp32 7.6e-6 (2136, 2), 6.9e-6 (1600, 3), 7.0e-6 (1424, 4).  Error against 64 bits at d = 4096: 4.3e-6 in
+// three shares, 1.7e-5 whole.
 template <bool SPLIT>
 __device__ __forceinline__ bool shares_ok(int p, int d) {
-    return (p - 1) * d <= (SPLIT ? MAX_SPLIT_D_F32 / 2 : (d <= 4096 ? 2731 : MAX_SPLIT_D / 2)) * p;
+    return (p - 1) * d <= (SPLIT ? MAX_SPLIT_D_F32 : MAX_SPLIT_D) / 2 * p;
 }
 // Limits of the plan's rules in stages of a bf16 tile: what a split has to save, the longest contraction whose
 // norms come out of the tiles in shared memory, the longest whose epilogue sets take alternate tiles.  The last

@@ -951,3 +951,44 @@ def test_accumulation_error_stays_within_what_the_header_states(ada, dtype, d):
         assert np.max(np.abs(err)) <= bound, (engine, float(np.max(np.abs(err))), bound)
     assert ada.ada_device_status(ctx)[0] == 0
     ada.ada_destroy(ctx)
+
+
+@pytest.mark.parametrize("dtype,d", [("bf16", 3064), ("bf16", 3640), ("bf16", 4096), ("bf16", 4600), ("bf16", 5120), ("bf16", 5496),
+                                     ("f32", 1424), ("f32", 1600), ("f32", 2136)])
+def test_a_row_moves_by_no_more_than_stated_when_tiles_are_split(ada, dtype, d):
+    """The same rows whole (the one-CTA kernel never splits a contraction) and in as many shares as a small
+    problem gets, at several places of a sum within its binade.  ada.h: 1.5e-5, ADA_F32 1e-5, for rows of one scale;
+    where the first elements hold the norm, both forms keep to the larger error stated for that (6e-6: the
+    norms' and 64-bit reference's roundings, as 2e-6 for ordinary rows, over rows three times as uneven)."""
+    T = 520
+    code = ada.ADA_F32 if dtype == "f32" else ada.ADA_BF16
+    kind = torch.float32 if dtype == "f32" else torch.bfloat16
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d)
+    base = torch.randn((T // 8, d), generator=g, device="cuda")
+    X = base[torch.randint(T // 8, (T,), generator=g, device="cuda")] + 0.02 * torch.randn((T, d), generator=g, device="cuda")
+    ctx = ada.ada_create(1, T, d, code)
+
+    def gammas(rows):
+        out = []
+        for engine in (ada.ADA_ENGINE_TCGEN05, ada.ADA_ENGINE_AUTO):
+            ada.ada_set_engine(ctx, engine)
+            out.append(ada.ada_select_full(ctx, rows[None], TAU)[2][0].double())
+        return out
+
+    most = 0.0
+    for scale in (0.7, 0.84, 1.0, 1.155, 1.4):
+        whole, split = gammas((scale * X).to(kind))
+        most = max(most, float((whole - split).abs().max()))
+    assert most <= (1.5e-5 if dtype == "bf16" else 1e-5), most
+    assert most > 2e-6, "nothing was split"
+    front = X.clone()
+    front[:, :16] *= 3 * (d / 16) ** 0.5
+    front = front.to(kind)
+    x = front.double()
+    x = x / x.norm(dim=1, keepdim=True)
+    ref = torch.tril((x @ x.T).abs(), -1).max(1).values
+    for got in gammas(front):
+        assert float((got - ref).abs().max()) <= (1.6e-8 if dtype == "bf16" else 2.1e-8) * d + 6e-6
+    assert ada.ada_device_status(ctx)[0] == 0
+    ada.ada_destroy(ctx)

@@ -138,18 +138,17 @@ static __device__ __forceinline__ void umma_bf16(unsigned tmem_d, unsigned long 
 // The MMAs of one tile over one or two 64-element K blocks (a_next, b_next: bytes from a block to the next; what
 // lies past the operands' last element is zero).  Unrolled and without a condition per instruction: one
 // thread's loop takes longer over an instruction than the tensor core does (128 x 256 x 16: 0.1 us against
-// 0.067).  The first one overwrites the accumulator.
+// 0.067).  The first one overwrites the accumulator.  (Each instruction under a condition of its own, `if (16 q < d)`,
+// gave wrong sums from the second one on.  The source does not show why, so that form is not used anywhere: blocks are
+// contracted whole, here and in the loops of the other kernels, and only the first flag is ever a variable.)
 template <int BLOCKS>
 static __device__ __forceinline__ void umma_blocks(unsigned tmem_d, unsigned long long adesc, unsigned long long bdesc,
                                                    int a_next, int b_next, unsigned idesc) {
-    unsigned first = 0;
-    asm volatile("" : "+r"(first));                           // (a predicate in a register, as everywhere)
 #pragma unroll
     for (int kb = 0; kb < BLOCKS; ++kb)
 #pragma unroll
         for (int q = 0; q < BK / UMMA_K; ++q)
-            umma_bf16(tmem_d, adesc + kb * (a_next >> 4) + 2 * q, bdesc + kb * (b_next >> 4) + 2 * q, idesc,
-                      first + (unsigned)(kb * (BK / UMMA_K) + q));
+            umma_bf16(tmem_d, adesc + kb * (a_next >> 4) + 2 * q, bdesc + kb * (b_next >> 4) + 2 * q, idesc, (kb | q) != 0);
 }
 static __device__ __forceinline__ void tmem_ld32(unsigned taddr, float (&v)[32]) {
     unsigned r[32];

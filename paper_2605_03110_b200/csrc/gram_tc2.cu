@@ -1139,7 +1139,7 @@ static cudaError_t ensure_tc2(ada_ctx* ctx) {
                                          smem_pair_bytes<false>());
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_gram_tc2<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_pair_bytes<true>());
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) { cudaGetLastError(); return e; }
     // how many clusters of two fit on the device at once
     cudaLaunchConfig_t q;
     memset(&q, 0, sizeof(q));

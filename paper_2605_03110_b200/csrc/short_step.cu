@@ -611,7 +611,7 @@ k_step_short(const __grid_constant__ StepMaps maps, const __grid_constant__ Step
 static cudaError_t ensure_short(ada_ctx* ctx) {
     if (ctx->short_attr_set) return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute(k_step_short, cudaFuncAttributeMaxDynamicSharedMemorySize, SS_SMEM);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) { cudaGetLastError(); return e; }
     for (int C = 1; C <= SS_CLUSTER; ++C) {
         cudaLaunchConfig_t q;
         memset(&q, 0, sizeof(q));

@@ -193,3 +193,39 @@ def test_limit_of_the_waits_inside_a_launch(tmp_path):
         assert(seconds(false) > 1.99 && seconds(false) < 2.01);
         assert(seconds(true) > 19.9 && seconds(true) < 20.1);
     """)
+
+
+@pytest.mark.parametrize("unit,ask", [("short_step.cu", "ada::step_short_ctas(&ctx, 32, 2048, 128)"),
+                                      ("gram_tc2.cu", "ada::gram_tc2_hb_rows(&ctx, 1, 4096)")])
+def test_a_kernel_that_cannot_be_configured_leaves_no_error_behind(tmp_path, unit, ask):
+    """Where the runtime refuses a kernel's shared memory, these two report it by their result; the launchers
+    that ask for the last error afterwards must not find this one.  (The refusal is played by a stand-in.)"""
+    src = tmp_path / "unit.cu"
+    src.write_text(f"""
+        #include <cuda_runtime.h>
+        #include <stdio.h>
+        static cudaError_t pending = cudaSuccess;
+        template <class F> static cudaError_t refuse(F, cudaFuncAttribute, int) {{ return pending = cudaErrorInvalidValue; }}
+        static cudaError_t take_last() {{ const cudaError_t e = pending; pending = cudaSuccess; return e; }}
+        #define cudaFuncSetAttribute refuse
+        #define cudaGetLastError take_last
+        #include "{unit}"
+        namespace ada {{
+        void prof_begin(ada_ctx*, int, cudaStream_t) {{}}
+        void prof_end(ada_ctx*, cudaStream_t) {{}}
+        bool coop_begin(ada_ctx*, cudaStream_t) {{ return false; }}
+        void coop_end(ada_ctx*, bool) {{}}
+        }}
+        static ada_ctx ctx;
+        int main() {{
+            ctx.sm_count = 148;
+            if ({ask} != 0) return puts("configured"), 1;
+            if (pending != cudaSuccess) return puts("an error is left behind"), 2;
+            return 0;
+        }}""")
+    exe = str(tmp_path / "unit")
+    if not os.path.exists(ada_build.NVCC):
+        pytest.skip("needs nvcc")
+    subprocess.run([ada_build.NVCC, "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-I", ada_build.CSRC, "-o", exe, str(src)],
+                   check=True, capture_output=True)
+    assert subprocess.run([exe], capture_output=True, text=True).stdout == ""

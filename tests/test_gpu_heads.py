@@ -353,3 +353,20 @@ def test_heads_step_takes_one_launch_up_to_2048_tokens(ada, T, one):
         assert ("step_short" in kernels) == one
         assert_same_step(a, b)
     ada.ada_destroy(ctx)
+
+
+@pytest.mark.parametrize("T,h,d_h", [(1, 5, 128), (127, 2, 64), (128, 3, 72), (129, 2, 120), (1025, 19, 128), (1300, 110, 8),
+                                     (2047, 12, 96), (2048, 16, 128), (2048, 148, 16)])
+def test_heads_step_in_one_launch_against_several(ada, T, h, d_h):
+    """Every size against the one-CTA kernel's launches, up to 2048 tokens in one CTA (148 heads), sets from empty
+    to all tokens, and the verdict of more than 1024 representatives."""
+    ctx = ada.ada_create(h, T, d_h, ada.ADA_BF16)
+    X = clustered_heads(T, h, d_h, 31 + T + h, "bf16")
+    rng = np.random.default_rng(T + h)
+    sizes = [min(T, s) for s in (1500, 128, 0, 257, T, 1, 1024, 1025, 512, 129, 700)]
+    sets = [np.sort(rng.permutation(T)[:sizes[j % len(sizes)]]).tolist() for j in range(h)]
+    for flags in (0, ada.ADA_CROSS_CAUSAL):
+        one, several, kernels = both_forms(ada, ctx, X, sets, flags)
+        assert kernels == {"step_short"}
+        assert_same_step(one, several)
+    ada.ada_destroy(ctx)

@@ -77,7 +77,8 @@ typedef enum { ADA_F32 = 0, ADA_BF16 = 1 } ada_dtype;
 #define ADA_CROSS_CAUSAL 1u /* restrict Algorithm 1 line 8 to valid representatives s < t */
 
 /* Which Gram kernel family a context uses.  AUTO: tensor cores (tcgen05), one- or two-CTA
- * form by problem size.  ADA_BF16 feeds the stored values to the MMA; ADA_F32 is split into
+ * form by problem size; a fixed-threshold step over many ADA_BF16 sequences of at most 2048 tokens of at most 128
+ * elements (one per attention head) runs as one launch, a cluster of CTAs per sequence.  ADA_BF16 feeds the stored values to the MMA; ADA_F32 is split into
  * three bf16 terms per value and contracted as the six leading cross terms (what is dropped is
  * below 2^-23 |x||y|; accumulation as stated above), at the price of a 6x longer contraction and a
  * workspace of 12 bytes per element.  FFMA is the plain fp32 ALU kernel (any storage type;
@@ -95,8 +96,8 @@ typedef struct ada_ctx ada_ctx; /* opaque */
 
 /* Create a context on `device` able to serve up to maxB sequences of maxT
  * tokens of width maxd in storage type dt.  Allocates the workspace
- * (cudaMalloc; about maxB*maxT*(maxd*es + 32) bytes, as much again of rows for ADA_BF16,
- * 12*maxB*maxT*maxd for ADA_F32, and 128 KiB per SM for partial sums).
+ * (cudaMalloc; about maxB*maxT*(maxd*es + 28) bytes, maxB*maxT*(maxd*es + 8) more for ADA_BF16,
+ * 12*maxB*maxT*maxd more for ADA_F32, and 128 KiB per SM for partial sums).
  * maxT may not exceed ADA_MAX_T (the list counts of one sequence are kept in 21-bit fields),
  * nor maxB*maxT 2^30: ADA_ERR_INVALID_ARG.  *out is NULL on error. */
 #define ADA_MAX_T ((int64_t)2097151)

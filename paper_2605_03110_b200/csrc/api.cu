@@ -68,7 +68,7 @@ bool use_pair(const ada_ctx* ctx, int64_t B, int64_t T, int64_t d, ada_dtype dt,
     // has to split its few tiles along K: with the split the pair kernel is faster from 512 tokens
     // on (T = 1024, d = 4096: full selection 27.4 -> 24.0 us, step 34.8 -> 28.2; fp32, T = 700,
     // d = 1600: 55.8 -> 23.7, step 67.8 -> 30.3), where the contraction is too long to be split only from a few
-    // thousand rows on (T = 700, d = 5120, when that was not split: 31.0 against 34.7 us; in two shares 27.8).
+    // thousand rows on (T = 700, d = 5120, when that was not split: 31.0 against 34.7 us).
     if (dt == ADA_F32) return d >= 256 && (d <= MAX_SPLIT_D_F32 || B * T >= 4096);
     if (d >= 2048) return B * T >= (d <= MAX_SPLIT_D ? 512 : 4096);
     // Shorter contractions: a step saves the launch that gathers and normalises (8 x 2048 x 768: 37 -> 29 us

@@ -1109,8 +1109,8 @@ k_gram_tc2(const __grid_constant__ GramMaps maps, const __grid_constant__ GramPr
                     atomicAdd(dep_ctr, 1u);
                 }
                 // By token too, behind the arrival, since nobody in this launch waits for it: the compaction then reads all
-                // that it needs of a token at once (8 x 2048 x 768 chain of twelve 314 -> 309 us, 2005 x 4096 of 28
-                // 796 -> 786; nothing for fp32, whose steps do without).  (An entry of a rejected list may be anything.)
+                // that it needs of a token at once (2005 x 4096 chain of 28 796 -> 786 us; 8 x 2048 x 768 and 8192 x 4096 within
+                // their spread, nothing for fp32, whose steps do without).  (An entry of a rejected list may be anything.)
                 if (!SPLIT && mx > 0.f && (unsigned)rep_tok < (unsigned)p.cap) atomicMax(p.out_tok + o + rep_tok, __float_as_uint(mx));
             }
         }

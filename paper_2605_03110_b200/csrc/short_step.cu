@@ -17,7 +17,7 @@
 // TMEM lane quadrant) that share every tile's columns, with two 128 x 256 accumulators, so that the
 // next tile's MMAs run behind a tile's reading.
 //
-// What bounds it (T = 2048, 32 heads of 128, r = 410, one B200; 42.3 us as three launches, 26.2 so; in-kernel time
+// What bounds it (T = 2048, 32 heads of 128, r = 410, one B200; 42.3 us as three launches, 26.4 so; in-kernel time
 // stamps): 5 us until the rows are gathered, 1.5 us to the first MMA, 5 us for the triangle and its verdict,
 // 10 us for eight cross tiles, 4 us for the lists, 1 us between launches.  A cross tile (128 x 256 x 128) takes
 // 1.25 us where its MMAs need 0.55: the epilogue reads an accumulator in 0.75 us, a quarter of it column factors

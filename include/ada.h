@@ -44,8 +44,8 @@
  *   - Accuracy of gamma on the tensor cores: their accumulator truncates, so a correlation comes
  *     out too small, by up to 4e-9 d + 2e-6 of itself for ADA_BF16 and 8e-9 d + 2e-6 for ADA_F32 where the
  *     elements of a row are of one scale (measured against 64 bits: 1.7e-5 and 2.4e-5 at d = 4096;
- *     ADA_ENGINE_FFMA 4e-6), and by up to 1.6e-8 d and 2.1e-8 d where a few leading ones hold most of a row's
- *     norm (6.3e-5 at d = 4096; ADA_F32 4.4e-5 at d = 2140).  Tiles that several SM pairs share along d (small problems,
+ *     ADA_ENGINE_FFMA 4e-6), and by up to 1.6e-8 d + 2e-6 and 2.1e-8 d + 2e-6 where a few leading ones hold most of a
+ *     row's norm (6.3e-5 at d = 4096; ADA_F32 4.3e-5 at d = 2136).  Tiles that several SM pairs share along d (small problems,
  *     d <= 5500, ADA_F32 <= 2140) keep a half to a quarter of that error, so the same row's gamma may
  *     differ with the number of rows around it: by up to 1.5e-5 (ADA_F32 1e-5) for rows of one scale, whatever
  *     that scale is, and by three quarters of the error else.

@@ -958,8 +958,9 @@ def test_accumulation_error_stays_within_what_the_header_states(ada, dtype, d):
 def test_a_row_moves_by_no_more_than_stated_when_tiles_are_split(ada, dtype, d):
     """The same rows whole (the one-CTA kernel never splits a contraction) and in as many shares as a small
     problem gets, at several places of a sum within its binade.  ada.h: 1.5e-5, ADA_F32 1e-5, for rows of one scale;
-    where the first elements hold the norm, both forms keep to the larger error stated for that (6e-6: the
-    norms' and 64-bit reference's roundings, as 2e-6 for ordinary rows, over rows three times as uneven)."""
+    where the first elements hold the norm, both forms keep to the larger error stated for that: there an accumulation of
+    16 elements cuts off up to two units in the last place of a sum that is full from the start, d / 16 x 2 x 2^-23 =
+    1.5e-8 d (ADA_F32: six terms, 2.1e-8 d as measured), and 2e-6 for the norms."""
     T = 520
     code = ada.ADA_F32 if dtype == "f32" else ada.ADA_BF16
     kind = torch.float32 if dtype == "f32" else torch.bfloat16
@@ -989,6 +990,6 @@ def test_a_row_moves_by_no_more_than_stated_when_tiles_are_split(ada, dtype, d):
     x = x / x.norm(dim=1, keepdim=True)
     ref = torch.tril((x @ x.T).abs(), -1).max(1).values
     for got in gammas(front):
-        assert float((got - ref).abs().max()) <= (1.6e-8 if dtype == "bf16" else 2.1e-8) * d + 6e-6
+        assert float((got - ref).abs().max()) <= (1.6e-8 if dtype == "bf16" else 2.1e-8) * d + 2e-6
     assert ada.ada_device_status(ctx)[0] == 0
     ada.ada_destroy(ctx)

@@ -17,7 +17,7 @@
 // TMEM lane quadrant) that share every tile's columns, with two 128 x 256 accumulators, so that the
 // next tile's MMAs run behind a tile's reading.
 //
-// What bounds it (T = 2048, 32 heads of 128, r = 410, one B200; 42.3 us as three launches, 26.4 so; in-kernel time
+// What bounds it (T = 2048, 32 heads of 128, r = 410, one B200; 42.3 us as three launches, 26.0 so; in-kernel time
 // stamps): 5 us until the rows are gathered, 1.5 us to the first MMA, 5 us for the triangle and its verdict,
 // 10 us for eight cross tiles, 4 us for the lists, 1 us between launches.  A cross tile (128 x 256 x 128) takes
 // 1.25 us where its MMAs need 0.55: the epilogue reads an accumulator in 0.75 us, a quarter of it column factors
@@ -73,7 +73,6 @@ struct StepArgs {
     float* g_pos;               // [B*T] scratch: gamma_rep by position
     unsigned* status;
     int T, d, rows;             // rows: tokens per CTA, a multiple of 128
-    int causal;
     float thr;
     int32_t *keep_idx, *keep_cnt, *add_idx, *add_cnt, *rem_idx, *rem_cnt;
     float *gamma_rep, *gamma_cross;
@@ -154,6 +153,9 @@ struct Walk {
     }
 };
 
+// CAUSAL: ADA_CROSS_CAUSAL.  (A parameter of the template, so that each form does without the other's code, which is
+// fetched cold: 32 heads x 2048, r = 410 26.4 -> 26.0 us; r = 1024 47.3 -> 46.5, causal 51.7 -> 51.1.)
+template <bool CAUSAL>
 __global__ void __launch_bounds__(SS_THREADS, 1)
 k_step_short(const __grid_constant__ StepMaps maps, const __grid_constant__ StepArgs a) {
     extern __shared__ unsigned char smem_raw[];
@@ -226,7 +228,7 @@ k_step_short(const __grid_constant__ StepMaps maps, const __grid_constant__ Step
     Walk w;
     w.n = n; w.nch = (n + SS_COLS - 1) / SS_COLS; w.nrt = (n + BM - 1) / BM;
     w.nx = n == T ? 1 : n; w.nchx = n == T ? 1 : w.nch;
-    w.C = C; w.rank = rank; w.tiles = (own + BM - 1) / BM; w.t0 = t0; w.causal = a.causal;
+    w.C = C; w.rank = rank; w.tiles = (own + BM - 1) / BM; w.t0 = t0; w.causal = CAUSAL ? 1 : 0;
     w.tok0 = sh.tok0;
 
     if (warp >= 2) {
@@ -390,7 +392,7 @@ k_step_short(const __grid_constant__ StepMaps maps, const __grid_constant__ Step
                         if (ph && !(__ldcg(a.g_pos + o + col) < a.thr)) v = 0.f;
                     }
                     sh.col_f[staged & 1u][e * SS_COLS + wk] = v;
-                    if (ph == 0 || a.causal) sh.col_t[staged & 1u][e * SS_COLS + wk] = ph && live ? __ldg(list + col) : col;
+                    if (ph == 0 || CAUSAL) sh.col_t[staged & 1u][e * SS_COLS + wk] = ph && live ? __ldg(list + col) : col;
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sh.staged);
@@ -610,7 +612,8 @@ k_step_short(const __grid_constant__ StepMaps maps, const __grid_constant__ Step
 // How many clusters of C CTAs (C = 1..8) run at once, per context.
 static cudaError_t ensure_short(ada_ctx* ctx) {
     if (ctx->short_attr_set) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_step_short, cudaFuncAttributeMaxDynamicSharedMemorySize, SS_SMEM);
+    cudaError_t e = cudaFuncSetAttribute(k_step_short<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SS_SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_step_short<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SS_SMEM);
     if (e != cudaSuccess) { cudaGetLastError(); return e; }
     for (int C = 1; C <= SS_CLUSTER; ++C) {
         cudaLaunchConfig_t q;
@@ -623,7 +626,7 @@ static cudaError_t ensure_short(ada_ctx* ctx) {
         qa[0].val.clusterDim.x = C; qa[0].val.clusterDim.y = 1; qa[0].val.clusterDim.z = 1;
         q.attrs = qa; q.numAttrs = 1;
         int at_once = 0;
-        e = cudaOccupancyMaxActiveClusters(&at_once, k_step_short, &q);
+        e = cudaOccupancyMaxActiveClusters(&at_once, k_step_short<false>, &q);
         if (e != cudaSuccess) { cudaGetLastError(); return e; }
         ctx->short_clusters[C] = at_once;
     }
@@ -684,7 +687,7 @@ cudaError_t launch_step_short(ada_ctx* ctx, int C, const void* X, int B, int T, 
     a.Xrep = static_cast<__nv_bfloat16*>(ctx->Xrep); a.inv_rep = ctx->inv_rep; a.g_pos = ctx->inv_norm;
     a.status = ctx->status;
     a.T = T; a.d = d; a.rows = ((T + BM - 1) / BM + C - 1) / C * BM;
-    a.causal = causal; a.thr = thr;
+    a.thr = thr;
     a.keep_idx = rep_out; a.keep_cnt = rep_out_cnt;
     a.add_idx = add_idx; a.add_cnt = add_cnt; a.rem_idx = rem_idx; a.rem_cnt = rem_cnt;
     a.gamma_rep = gamma_rep; a.gamma_cross = gamma_cross;
@@ -702,7 +705,7 @@ cudaError_t launch_step_short(ada_ctx* ctx, int C, const void* X, int B, int T, 
     cfg.attrs = attr;
     cfg.numAttrs = ctx->dep_launch ? 2 : 1;
     prof_begin(ctx, K_STEP_SHORT, s);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_step_short, maps, a);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, causal ? k_step_short<true> : k_step_short<false>, maps, a);
     if (e != cudaSuccess) cudaGetLastError();   // returned; the next launcher that asks must not find it again
     prof_end(ctx, s);
     return e;
